@@ -18,7 +18,7 @@
 //     else they read. Two calls whose work overlaps on the GPU (different streams or host
 //     threads without ordering) race on the array and give wrong results: serialize them.
 //   - The first call on each device does a one-time set-up with that device current (the
-//     array's device address, kernel attributes, occupancy). Every call copies its segment
+//     array's device address, kernel attributes). Every call copies its segment
 //     descriptor from host memory and waits for its stream, so no call can be captured into a
 //     CUDA graph: a call on a capturing stream is refused with CV_EINVAL before any work.
 //   - On an error return the output buffer's contents are undefined; when the scan failed (a
@@ -59,7 +59,6 @@ struct NoAllocDev {
   bool ready = false;
   uint8_t* scratch = nullptr;  // device address of g_noalloc_scratch on this device
   int sms = 0;
-  int blocks_per_sm = 0;
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
 };
 
@@ -90,8 +89,6 @@ int setup(int dev, NoAllocDev** out) {
       e = cudaFuncSetAttribute(cfg.scan_fn[kind], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.smem);
       if (e != cudaSuccess) return fail(e);
     }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.blocks_per_sm, cfg.scan_fn[0], cfg.threads, cfg.smem);
-    if (e != cudaSuccess || d.blocks_per_sm < 1) return fail(e);
     cudaDriverEntryPointQueryResult q;
     void* fn = nullptr;
     e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
@@ -187,9 +184,8 @@ extern "C" int cv_scan_noalloc(const cv_master* m, const void* image, uint64_t n
   p.tile_nhit = tile_nhit;
   p.tile_ntrip = tile_ntrip;
   p.status = status_d;
-  const uint64_t grid = n_tiles < (uint64_t)d->sms * d->blocks_per_sm ? n_tiles : (uint64_t)d->sms * d->blocks_per_sm;
   void* sargs[] = {&p};
-  if ((e = cudaLaunchKernel(cfg.scan_fn[table_kind(tab)], dim3((unsigned)grid), dim3(cfg.threads), sargs, cfg.smem,
+  if ((e = cudaLaunchKernel(cfg.scan_fn[table_kind(tab)], dim3((unsigned)n_tiles), dim3(cfg.threads), sargs, cfg.smem,
                             stream)) !=
       cudaSuccess)
     return fail(e);

@@ -7,7 +7,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <array>
 #include <mutex>
 #include <vector>
 
@@ -61,8 +60,6 @@ struct DevCtx {
   cudaStream_t copy_stream = nullptr;  // host-to-device copies of streamed images
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   PFN_cuMemGetAddressRange_v3020 address_range = nullptr;
-  std::vector<std::array<int, kTableKinds>> blocks_per_sm;  // per scan configuration and table kind
-  std::vector<int> blocks_per_sm_digest;  // per scan configuration (0: no digest-mode kernels)
   int cfg_index = -1;  // scan configuration forced by CV_SCAN_CONFIG, or -1: per table kind
 
   // The scan configuration for a table kind when the caller asks for the default.

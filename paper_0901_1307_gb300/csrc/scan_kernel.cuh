@@ -9,7 +9,13 @@
 // XOR swizzle, which plays the role of Figure 9's skew; thread t then hashes sector t of the
 // tile (one sector per thread, Section 3.2), reading its words with conflict-free 16-byte
 // shared loads. A dedicated producer warp keeps NS stages in flight through an mbarrier ring,
-// so the hashing warps never issue a global load. Tiles are spread over a persistent grid.
+// so the hashing warps never issue a global load.
+//
+// Tiles are handed out as blocks get to them: the grid has one block per tile, the blocks that
+// become resident stay, and each takes the next tile over from a block that has not started yet
+// (cluster launch control), asking for it one tile ahead. With a fixed share of the tiles per
+// block the scheduler's preference among the blocks of an SM let some finish early, and the SM
+// ran a quarter short of warps on average (27.5 of 36 active; 1 GiB image).
 //
 // Every mbarrier wait is bounded in time: on expiry the kernel sets kStTimeout in the status
 // word, stops waiting (its results are then discarded by the host), lets the producer wait
@@ -206,15 +212,55 @@ __device__ __forceinline__ void crc64_block(uint32_t& rh, uint32_t& rl, const ui
   }
 }
 
+// Cluster launch control: ask for the index of a block of this grid that has not started (it then
+// never does); the 16-byte answer lands at resp and completes 16 bytes on bar.
+__device__ __forceinline__ void clc_ask(uint32_t resp, uint32_t bar) {
+  mbar_arrive_expect_tx(bar, 16);
+  asm volatile(
+      "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(resp),
+      "r"(bar)
+      : "memory");
+}
+
+// The answer: true and the block's index, or false when every block has started.
+__device__ __forceinline__ bool clc_answer(uint32_t resp, uint32_t& block) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .b128 a;\n\t.reg .pred p;\n\t"
+      "ld.shared.b128 a, [%2];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t"
+      "mov.u32 %1, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, a;\n\t}"
+      : "=r"(ok), "=r"(block)
+      : "r"(resp)
+      : "memory");
+  return ok != 0;
+}
+
 enum : int { kModeScan = 0, kModeDigest = 1 };
+
+// What the producer tells the hashing warps about a tile.
+struct TileInfo {
+  uint64_t tile;         // global index; kNoTile: no more tiles
+  uint64_t sector0;      // index within its image of the tile's first sector
+  const uint8_t* bytes;  // its address (byte confirmation)
+  uint32_t rows;         // sectors of the tile inside the segment
+  uint32_t pad;
+};
+constexpr uint64_t kNoTile = ~0ull;
 
 template <int T, int NS, int BOXB>
 struct ScanSmem {
   static constexpr uint32_t kStageBytes = T * BOXB;
-  // stages first (1024-byte aligned), then the barriers and the abort flag
+  // stages first (1024-byte aligned), then the barriers; the abort flag, the barrier and the
+  // 16-byte answer of the tile requests; two tile records
   static constexpr uint32_t kBarOff = NS * kStageBytes;
   static constexpr uint32_t kMiscOff = kBarOff + 2 * NS * 8;
-  static constexpr uint32_t kBytes = kMiscOff + 16;
+  static constexpr uint32_t kClcBarOff = kMiscOff + 8;
+  static constexpr uint32_t kClcOff = kMiscOff + 16;
+  static constexpr uint32_t kInfoOff = kMiscOff + 32;
+  static constexpr uint32_t kBytes = kInfoOff + 2 * sizeof(TileInfo);
   static constexpr uint32_t kAlloc = kBytes + 1024;  // room to align the base
 };
 
@@ -247,10 +293,9 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
   const uint32_t bar_full = base + L::kBarOff;  // NS x 8 bytes
   const uint32_t bar_empty = bar_full + NS * 8;
   volatile uint32_t* const s_abort = reinterpret_cast<uint32_t*>(gbase + L::kMiscOff);
-  // The segment of the block's k-th tile, found by the producer (a binary search over the
-  // launch's segments) and read by the hashing warps after the tile's first stage, so that they
-  // do not each repeat the search: two entries, by the parity of k.
-  volatile uint32_t* const s_seg = reinterpret_cast<uint32_t*>(gbase + L::kMiscOff + 8);
+  // The block's k-th tile as the producer found it (a binary search over the launch's segments),
+  // read by the hashing warps after the tile's first stage: two entries, by the parity of k.
+  volatile TileInfo* const s_info = reinterpret_cast<TileInfo*>(gbase + L::kInfoOff);
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
@@ -261,8 +306,13 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
       mbar_init(bar_full + 8 * s, 1);
       mbar_init(bar_empty + 8 * s, C);
     }
+    mbar_init(base + L::kClcBarOff, 1);
     *s_abort = 0u;
-    s_seg[0] = s_seg[1] = 0u;  // in range even if a wait gives up before the producer writes
+    // in range even if a wait gives up before the producer writes
+    for (int k = 0; k < 2; k++) {
+      s_info[k].tile = kNoTile;
+      s_info[k].rows = 0u;
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -271,14 +321,16 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
     // ------------------------------------------------------------------ producer warp
     if (lane != 0) return;
     const uint64_t policy = l2_evict_first_policy();
-    uint32_t j = 0;
-    bool ok = true;
-    for (uint64_t lt = blockIdx.x; lt < p.n_tiles && ok; lt += gridDim.x) {
+    const uint32_t bar_clc = base + L::kClcBarOff;
+    uint32_t j = 0, lt = blockIdx.x, answers = 0;
+    bool ok = true, more = true;
+    while (more && ok) {
+      clc_ask(base + L::kClcOff, bar_clc);  // the next tile; answered while this one is staged
       const uint64_t tile = p.tile_begin + lt;
-      const uint32_t sg = find_segment(p.segs, p.n_segs, tile);
-      const Segment& seg = p.segs[sg];
+      const Segment& seg = p.segs[find_segment(p.segs, p.n_segs, tile)];
       const CUtensorMap* map = &p.maps[seg.map - p.map_base];
-      const int32_t row0 = (int32_t)(seg.row_base + (tile - seg.tile_base) * T);
+      const uint64_t first = (tile - seg.tile_base) * T;  // the tile's first sector within the segment
+      const int32_t row0 = (int32_t)(seg.row_base + first);
       for (int c = 0; c < kChunks; c++, j++) {
         const uint32_t s = j % NS;
         if (j >= (uint32_t)NS && !mbar_wait(bar_empty + 8 * s, ((j / NS) - 1) & 1, s_abort, p.status)) {
@@ -288,13 +340,30 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
         // published by the arrive below (release), seen after the matching wait (acquire); the
         // entry is rewritten for the tile after next, whose first copy waits for every hashing
         // thread to release a stage of the next tile, long after it read this one
-        if (c == 0) s_seg[(j / kChunks) & 1] = sg;
+        if (c == 0) {
+          volatile TileInfo& info = s_info[(j / kChunks) & 1];
+          info.tile = tile;
+          info.sector0 = seg.sector_base + first;
+          info.bytes = seg.bytes + first * kSector;
+          info.rows = (uint32_t)(seg.n_sectors - first < (uint64_t)T ? seg.n_sectors - first : (uint64_t)T);
+        }
         mbar_arrive_expect_tx(bar_full + 8 * s, L::kStageBytes);
 #pragma unroll
         for (int k = 0; k < kBoxes; k++)
           tma_load_2d(base + s * L::kStageBytes + k * kBoxRows * BOXB, map, c * (BOXB / 4), row0 + k * kBoxRows,
                       bar_full + 8 * s, policy);
       }
+      // the answer, also when giving up: it must not land after the block exits
+      if (!mbar_wait(bar_clc, answers & 1, s_abort, p.status)) {
+        volatile uint32_t never = 0;
+        mbar_wait(bar_clc, answers & 1, &never, p.status);
+        ok = false;
+        break;
+      }
+      answers++;
+      more = clc_answer(base + L::kClcOff, lt);
+      // read (generic proxy) before the next answer is written (async proxy)
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     // Wait (bounded) for the copies still in flight so none lands after the block exits.
     const uint32_t issued = j;
@@ -308,6 +377,11 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
           break;
         }
       }
+    }
+    // No more tiles: one more phase of the next stage, without a copy.
+    if (ok && (j < (uint32_t)NS || mbar_wait(bar_empty + 8 * (j % NS), ((j / NS) - 1) & 1, s_abort, p.status))) {
+      s_info[(j / kChunks) & 1].tile = kNoTile;
+      mbar_arrive(bar_full + 8 * (j % NS));
     }
     return;
   }
@@ -323,12 +397,9 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
   }
   const uint32_t lane_lt = (1u << lane) - 1u;
   uint32_t j = 0;
-  for (uint64_t lt = blockIdx.x; lt < p.n_tiles; lt += gridDim.x) {
-    const uint64_t tile = p.tile_begin + lt;
-    // No-pad MD5 has no padding compression between the last stage and the lookup to hide the
-    // segment's loads behind, and measured faster finding its segment itself at the tile start.
-    uint32_t sgi = 0;
-    if constexpr (SIG == kSigMd5NoPad) sgi = find_segment(p.segs, p.n_segs, tile);
+  bool ok = true;
+  for (uint32_t par = 0;; par ^= 1u) {
+    const volatile TileInfo& info = s_info[par];
     uint32_t st[SPT][4];
     uint64_t h[SPT];  // djb2 / CRC64 accumulators
     uint32_t diff[SPT], ref[SPT];
@@ -349,10 +420,9 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
 #pragma unroll(kUnroll)
     for (int c = 0; c < kChunks; c++, j++) {
       const uint32_t s = (kChunks % NS == 0) ? (uint32_t)c % NS : j % NS;
-      mbar_wait(bar_full + 8 * s, (j / NS) & 1, s_abort, p.status);
-      if constexpr (SIG != kSigMd5NoPad) {
-        if (c == 0) sgi = s_seg[(j / kChunks) & 1];
-      }
+      ok = mbar_wait(bar_full + 8 * s, (j / NS) & 1, s_abort, p.status) && ok;
+      // the end, or an earlier wait that gave up: the whole warp leaves together
+      if (c == 0 && !__all_sync(0xFFFFFFFFu, ok && info.tile != kNoTile)) return;
       const uint32_t stage = base + s * L::kStageBytes;
 #pragma unroll
       for (int b = 0; b < kBlocksPerChunk; b++) {
@@ -406,22 +476,22 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
       if constexpr (sig_is_weak(SIG)) sig64_words(h[k], st[k]);
     }
 
-    const Segment& seg = p.segs[sgi];
-    const uint64_t row0 = (tile - seg.tile_base) * T;  // within the segment
+    const uint64_t tile = info.tile, sector0 = info.sector0;
+    const uint32_t rows = info.rows;
 #pragma unroll
     for (int k = 0; k < SPT; k++) {
-      const uint64_t r = row0 + (uint64_t)(tid + k * C);
-      const bool valid = r < seg.n_sectors;
+      const uint32_t r = (uint32_t)(tid + k * C);
+      const bool valid = r < rows;
       if constexpr (MODE == kModeDigest) {
         if (valid) {
-          const uint64_t g = seg.sector_base + r;
+          const uint64_t g = sector0 + r;
           p.digests[g] = make_uint4(st[k][0], st[k][1], st[k][2], st[k][3]);
           if (p.trivial) p.trivial[g] = diff[k] == 0u ? 1 : 0;
         }
       } else {
         uint32_t post_off = 0, post_cnt = 0;
         // the disk sector's position in its cluster (0 for a table over all positions)
-        const uint32_t tau = (uint32_t)(seg.sector_base + r + p.tab.tau_add) & p.tab.tau_mask;
+        const uint32_t tau = (uint32_t)(sector0 + r + p.tab.tau_add) & p.tab.tau_mask;
         if (valid && (!p.tab.use_bloom || bloom_test(p.tab, st[k][1], st[k][2], st[k][3], tau)))
           post_cnt = LAYOUT == kLayoutSorted
                          ? sorted_probe(p.tab, st[k][0], st[k][1], st[k][2], st[k][3], tau, post_off)
@@ -431,7 +501,7 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
         uint32_t n_emit = post_cnt;
         if constexpr (sig_is_weak(SIG)) {
           if (post_cnt) {
-            const uint8_t* mine = seg.bytes + r * kSector;
+            const uint8_t* mine = info.bytes + r * kSector;
             n_emit = 0;
             for (uint32_t q = 0; q < post_cnt; q++)
               n_emit += sectors_equal(mine, p.tab.confirm + (uint64_t)(post_off + q) * kSector) ? 1u : 0u;

@@ -138,11 +138,13 @@ typedef struct {
   uint32_t flags;             /* CV_KEEP_ON_DEVICE */
   void* stream;               /* cudaStream_t */
   uint64_t chunk_bytes;       /* host images are streamed in chunks of this size; 0 = 256 MiB */
-  uint32_t kernel_config;     /* 0 = the default for the table's signature (MD5 and MD5 without
-                                 padding: configuration 0; djb2-64 and CRC64, whose scans are
-                                 bound by the staging of the image: 128-byte stages of
-                                 128-sector tiles), or the CV_SCAN_CONFIG environment variable's
-                                 configuration (by name) when set; k + 1 selects configuration k */
+  uint32_t kernel_config;     /* 0 = the default for the table's signature and the sectors scanned
+                                 (small scans with MD5 or MD5 without padding: configuration 0;
+                                 larger ones, djb2-64 and CRC64: 128-byte stages of 128-sector
+                                 tiles; MD5 without padding from 1 GiB on: 256-sector tiles with
+                                 an even split of the additions), or the CV_SCAN_CONFIG
+                                 environment variable's configuration (by name) when set; k + 1
+                                 selects configuration k */
   uint32_t reserved;
   uint64_t base_offset;       /* position-keyed tables: disk sector of the first cluster (only its
                                  value mod 8 matters); ignored for CV_POSITION_ANY tables. The

@@ -230,7 +230,9 @@ int cv_batch_create(const cv_master* m, const cv_buf* images, uint32_t n_images,
     if (k != kDevice) return CV_EINVAL;
   }
   const bool bloom_avail = tab.use_bloom != 0;
-  int cfg_i = ctx->default_config(table_kind(tab));
+  uint64_t all_sectors = 0;
+  for (uint32_t i = 0; i < n_images; i++) all_sectors += images[i].n_bytes / kSector;
+  int cfg_i = ctx->default_config(table_kind(tab), all_sectors);
   int bloom = bloom_avail ? 1 : 0;
   if (opts && opts->kernel_config) {
     if (opts->kernel_config > (uint32_t)ncfg) return CV_EINVAL;

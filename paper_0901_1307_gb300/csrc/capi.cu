@@ -339,7 +339,10 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
   if (m->tab.unit == kUnitFragment) return frag_scan(ctx, m, images, n_images, flags, stream, out);
   int ncfg;
   scan_configs(&ncfg);
-  int cfg_i = ctx->default_config(table_kind(m->tab));
+  // what one launch scans: every device image, or a host image's chunk
+  uint64_t launch_sectors = 0;
+  for (uint32_t i = 0; i < n_images; i++) launch_sectors += images[i].n_bytes / kSector;
+  int cfg_i = ctx->default_config(table_kind(m->tab), launch_sectors);
   if (opts && opts->kernel_config) {
     if (opts->kernel_config > (uint32_t)ncfg) return CV_EINVAL;
     cfg_i = (int)opts->kernel_config - 1;

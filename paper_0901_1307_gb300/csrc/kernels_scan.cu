@@ -135,8 +135,7 @@ __global__ void wait_timeout_selftest_kernel(uint32_t* status, uint64_t timeout_
 }
 
 
-// The configurations in table order. The first is the default (the fastest measured on GB300
-// for the 32 GiB image workload) and the only one with digest-mode kernels; every one has scan
+// The configurations in table order. The first is the only one with digest-mode kernels; every one has scan
 // kernels for all eight table kinds (four signatures x two layouts), so the batch autotuner can
 // pick any of them for any table. The kernels are instantiated in scan_cfgs_{a,b,c}.cu, which
 // compile in parallel.
@@ -167,21 +166,33 @@ const ScanCfg& scan_config_for(int cfg_i, int kind, int* used) {
   return c[cfg_i];
 }
 
-int preferred_config(int kind) {
-  // Measured on GB300 (32 GiB image, 4,194,304-sector table, kernel time per call): MD5 and
-  // MD5 without padding are bound by integer issue and fastest with the first configuration;
-  // djb2-64 and CRC64 do far less arithmetic and are bound by the staging of the image, which
-  // 128-byte stages of 128-sector tiles serve best (djb2-64 6,241 against 5,146 GB/s; CRC64 5,889
-  // against 5,151).
-  static const int light = [] {
-    int n;
-    const ScanCfg* c = scan_configs(&n);
-    for (int i = 0; i < n; i++)
-      if (strcmp(c[i].name, "t128_x1_s2_b128_p2") == 0) return i;
-    return 0;
-  }();
+int preferred_config(int kind, uint64_t sectors, int sms) {
+  // Measured on GB300, kernel time per call. djb2-64 and CRC64 do little arithmetic and are bound
+  // by the staging of the image, which 128-byte stages of 128-sector tiles serve best (djb2-64 on
+  // 8 GiB: 7,006 GB/s against 5,781 with configuration 0). MD5 is bound by the register file: a
+  // step's four or five instructions read ten or eleven distinct registers and a scheduler gets
+  // about two operand reads a clock (a register-only loop of any mix of the addition forms, with 16
+  // to 48 warps, ends at 18 to 19.4 steps a clock per SM; the scan does 19.5). There the same
+  // configuration, with its additions split evenly, is the fastest once the image is more than one
+  // round of 256-sector tiles on four blocks per SM: 32 GiB 5,497 against 5,355 GB/s, 1 GiB 5,112
+  // against 4,894, 100 MiB 2,867 against 2,388, but 64 MiB 2,076 against 2,444. Without the padding
+  // block the 256-sector form of that split overtakes it from about 1 GiB on (4 GiB: 5,837 against
+  // 5,738, and 5,718 for configuration 0; 128 MiB: 3,007, 3,347 and 3,075).
+  static const struct Picks {
+    int light, nopad;
+    Picks() : light(0), nopad(0) {
+      int n;
+      const ScanCfg* c = scan_configs(&n);
+      for (int i = 0; i < n; i++) {
+        if (strcmp(c[i].name, "t128_x1_s2_b128_p2") == 0) light = i;
+        if (strcmp(c[i].name, "t256_x1_s2_b64_p2") == 0) nopad = i;
+      }
+    }
+  } picks;
   const int sig = kind % 4;
-  return (sig == kSigDjb2 || sig == kSigCrc64) ? light : 0;
+  if (sig == kSigDjb2 || sig == kSigCrc64) return picks.light;
+  if (sectors <= (uint64_t)sms * 4 * 256) return 0;
+  return sig == kSigMd5NoPad && sectors >= (1ull << 21) ? picks.nopad : picks.light;
 }
 
 const ScanCfg& digest_config_for(int cfg_i, int sig, int* used) {

@@ -60,10 +60,13 @@ struct DevCtx {
   cudaStream_t copy_stream = nullptr;  // host-to-device copies of streamed images
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   PFN_cuMemGetAddressRange_v3020 address_range = nullptr;
-  int cfg_index = -1;  // scan configuration forced by CV_SCAN_CONFIG, or -1: per table kind
+  int cfg_index = -1;  // scan configuration forced by CV_SCAN_CONFIG, or -1: by table kind and size
 
-  // The scan configuration for a table kind when the caller asks for the default.
-  int default_config(int kind) const { return cfg_index >= 0 ? cfg_index : preferred_config(kind); }
+  // The scan configuration for a table kind and sectors per launch when the caller asks for the
+  // default.
+  int default_config(int kind, uint64_t sectors) const {
+    return cfg_index >= 0 ? cfg_index : preferred_config(kind, sectors, sms);
+  }
 
   // Timing events of finished calls, kept for later calls: creating and destroying four events
   // per scan cost host time while the device waited for the next call.

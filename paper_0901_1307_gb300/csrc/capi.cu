@@ -187,12 +187,11 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
   Temps staging(ctx, stream);
   std::vector<const uint8_t*> dptr(n_images, nullptr);
   std::vector<uint64_t> nbytes(n_images, 0), tile_base(n_images + 1, 0);
-  uint64_t windows = 0, max_tiles = 0;
+  uint64_t windows = 0;
   for (uint32_t i = 0; i < n_images; i++) {
     nbytes[i] = images[i].n_bytes;
     const uint64_t t = frag_tiles((int)m->tab.sig, nbytes[i]);
     tile_base[i + 1] = tile_base[i] + t;
-    max_tiles = std::max(max_tiles, t);
     windows += frag_windows(nbytes[i]);
     if (!t) continue;
     if (!images[i].data) return CV_EINVAL;
@@ -232,13 +231,16 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       CV_TRY(ctx->take_events(ev, 4));
       CV_CUDA(cudaEventRecord(ev[0], stream));
       uint64_t *tile_ntrip, *tile_off, *seg_off_d, *scratch;
-      uint32_t* list;
+      FragHits hits;
       Segment* segs_d;
       CV_TRY(tmp.alloc(&tile_ntrip, std::max<uint64_t>(T, 1) * 8));
       CV_TRY(tmp.alloc(&tile_off, std::max<uint64_t>(T, 1) * 8));
-      CV_TRY(tmp.alloc(&seg_off_d, (n_images + 3) * 8));  // seg_off[n], total, status, rejected
+      // seg_off[n], total, status, rejected, listed tiles of every image
+      CV_TRY(tmp.alloc(&seg_off_d, (2ull * n_images + 3) * 8));
       CV_TRY(tmp.alloc(&scratch, tile_offsets_scratch_words(T) * 8 + 8));
-      CV_TRY(tmp.alloc(&list, (max_tiles + 1) * 4));
+      CV_TRY(tmp.alloc(&hits.tiles, T * 4));
+      hits.mask_tiles = std::min(T, kFragMaskTiles);
+      CV_TRY(tmp.alloc(&hits.masks, hits.mask_tiles * 32 * 4));
       CV_TRY(tmp.alloc(&segs_d, std::max<uint32_t>(n_images, 1) * sizeof(Segment)));
       std::vector<Segment> segs(n_images);
       memset(segs.data(), 0, segs.size() * sizeof(Segment));
@@ -250,12 +252,14 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
         CV_CUDA(cudaMemcpyAsync(segs_d, segs.data(), n_images * sizeof(Segment), cudaMemcpyHostToDevice, stream));
       uint32_t* status = (uint32_t*)(seg_off_d + n_images + 1);
       unsigned long long* rejected = (unsigned long long*)(seg_off_d + n_images + 2);
-      CV_CUDA(cudaMemsetAsync(status, 0, 16, stream));
+      uint64_t* listed = seg_off_d + n_images + 3;
+      CV_CUDA(cudaMemsetAsync(status, 0, 16 + n_images * 8ull, stream));
       CV_CUDA(cudaEventRecord(ev[1], stream));
       for (uint32_t i = 0; i < n_images; i++) {
         if (tile_base[i + 1] == tile_base[i]) continue;
-        CV_CUDA((cudaError_t)frag_count(m->tab, dptr[i], nbytes[i], tile_base[i], tile_ntrip, status, rejected,
-                                        ctx->sms, stream));
+        hits.count = (uint32_t*)(listed + i);
+        CV_CUDA((cudaError_t)frag_count(m->tab, dptr[i], nbytes[i], tile_base[i], tile_ntrip, hits, status,
+                                        rejected, ctx->sms, stream));
         r->launches++;
       }
       CV_CUDA(cudaEventRecord(ev[2], stream));
@@ -274,8 +278,10 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
         CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, total * sizeof(MatchOut), ctx->pool, stream));
         for (uint32_t i = 0; i < n_images; i++) {
           if (tile_base[i + 1] == tile_base[i]) continue;
-          CV_CUDA((cudaError_t)frag_emit(m->tab, dptr[i], nbytes[i], tile_base[i], tile_ntrip, tile_off, list,
-                                         r->dev_out, total, status, ctx->sms, stream, &r->launches));
+          hits.count = (uint32_t*)(listed + i);
+          CV_CUDA((cudaError_t)frag_emit(m->tab, dptr[i], nbytes[i], tile_base[i], tile_off, hits, r->dev_out, total,
+                                         status, ctx->sms, stream));
+          r->launches++;
         }
       }
       for (uint32_t i = 0; i < n_images; i++) r->off[i] = seg_off[i];

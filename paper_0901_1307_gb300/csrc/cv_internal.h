@@ -48,7 +48,7 @@ __host__ __device__ constexpr bool sig_is_weak(int sig) { return sig == kSigDjb2
 //          comparison of the records whose h0 is equal.
 enum : uint32_t { kLayoutHash = 0, kLayoutSorted = 1 };
 // What a table's keys are: 512-byte sectors, or 64-byte fragments (a fragment table's Bloom
-// filter is one u32 word per block, 3 bits per key: word d3 & bloom_mask, bits from d2).
+// filter is one u32 word per block, 3 bits per key: frag_bloom_word and frag_bloom_bits).
 enum : uint32_t { kUnitSector = 0, kUnitFragment = 1 };
 
 struct TableView {
@@ -95,13 +95,12 @@ __host__ __device__ inline void sig64_words(uint64_t h, uint32_t w[4]) {
 // the whole 64-byte fragments of the master files.
 constexpr uint32_t kFrag = 64;
 constexpr uint32_t kFragStride = 4;
-// The shared-memory filter of a fragment table: 2^20 bits (128 KiB), bit = top 20 bits of d1.
-constexpr uint32_t kFragL1Log2Bits = 20;
-constexpr uint32_t kFragL1Bytes = (1u << kFragL1Log2Bits) / 8;
+// The shared-memory filter of a fragment table: 2^20 bits (128 KiB).
+constexpr uint32_t kFragL1Bytes = (1u << 20) / 8;
 
 // The four table words of a fragment's 64-bit signature h: h itself (low word first: the home
-// slot is given by the signature's least significant bits, Eq. 3) and h times an odd constant,
-// whose high bits (mixing every bit of h) choose the Bloom word and bits. Equal words <=> equal h.
+// slot is given by the signature's least significant bits, Eq. 3) and h times an odd constant.
+// Equal words <=> equal h.
 __host__ __device__ inline void frag64_words(uint64_t h, uint32_t w[4]) {
   const uint64_t f = h * 0x9E3779B97F4A7C15ull;
   w[0] = (uint32_t)h;

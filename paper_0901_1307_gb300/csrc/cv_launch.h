@@ -65,20 +65,30 @@ bool frag_sig_supported(int sig);         // MD5, MD5 without padding, djb2-64
 int frag_digests(int sig, const uint8_t* arena, uint64_t n, uint4* dig, uint8_t* trivial, int sms, void* stream);
 // The filters of a fragment table (zeroed by the caller): the one-word Bloom filter (words, null
 // for none; mask = words - 1) and the shared-memory filter l1 (kFragL1Bytes).
-int frag_bloom(const uint4* slots, uint32_t n_slots, uint32_t* words, uint32_t mask, uint32_t* l1, int sms,
+int frag_bloom(int sig, const uint4* slots, uint32_t n_slots, uint32_t* words, uint32_t mask, uint32_t* l1, int sms,
                void* stream);
-// Triples per tile of one device image (16-byte aligned) into tile_ntrip[tile_base ..);
-// djb2 candidates dropped by the byte comparison are added to *rejected (when non-null).
+// The hit lists of a scan's images: tiles has room for every tile of the scan, masks (32 words per
+// tile) for the first mask_tiles of them, an image's entries starting at its first tile; count is
+// the image's own counter.
+struct FragHits {
+  uint32_t* tiles;
+  uint32_t* masks;
+  uint64_t mask_tiles;
+  uint32_t* count;
+};
+constexpr uint64_t kFragMaskTiles = 1ull << 22;
+// Triples per tile of one device image (16-byte aligned) into tile_ntrip[tile_base ..) and its
+// hit list (*hits.count zero before); djb2 candidates dropped by the byte comparison are added to
+// *rejected (when non-null).
 int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base, uint64_t* tile_ntrip,
-               uint32_t* status, unsigned long long* rejected, int sms, void* stream);
+               const FragHits& hits, uint32_t* status, unsigned long long* rejected, int sms, void* stream);
 // The 16-byte key of every 64-byte window at a 4-byte offset of a device image, through the
 // fragment kernels' own signature code (MD5, MD5 without padding, rolled djb2-64).
 int frag_window_sigs(int sig, const uint8_t* image, uint64_t n_bytes, uint4* out, int sms, void* stream);
-// The triples of the image's tiles that have any, at out[tile_off[tile]..]. list: scratch of
-// frag_tiles(n_bytes) + 1 u32 words. *launches counts the kernels launched.
+// The triples of the image's listed tiles, at out[tile_off[tile]..].
 int frag_emit(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base,
-              const uint64_t* tile_ntrip, const uint64_t* tile_off, uint32_t* list, MatchOut* out, uint64_t out_cap,
-              uint32_t* status, int sms, void* stream, int* launches);
+              const uint64_t* tile_off, const FragHits& hits, MatchOut* out, uint64_t out_cap, uint32_t* status, int sms,
+              void* stream);
 
 // One block whose single waiting thread waits on an mbarrier nothing completes (bounded by
 // timeout_ns): the status word gets the timeout bit. Returns a CUDA error code.

@@ -14,18 +14,20 @@
 //   g = h - 5381 * 33^64, a window W_k of words x_k .. x_{k+15} has g(W_k) = sum_q
 //   P(x_{k+q}) 33^{4 (15 - q)}, so g(W_{k+1}) = 33^4 g(W_k) - 33^64 P(x_k) + P(x_{k+16})
 //   (mod 2^64): after a lane's first window each one costs one word and a few multiply-adds.
-//   A rolled window is cheap enough that its Bloom lookup, not its hash, sets the pace, and an
-//   SM keeps only so many L2 misses in flight: so the djb2 kernel first tests a 2^20-bit filter
-//   held in shared memory (loaded once per block) and sends only the windows that pass it to
-//   the one-word Bloom filter in global memory.
+//   The same recurrence holds mod 2^32, so the count kernel rolls only the low word of h: two
+//   multiply-adds a window. Its filters are functions of that word: two bits of one word of a
+//   2^20-bit filter in shared memory (loaded once per block), then, for the windows that pass, one
+//   word of a Bloom filter in global memory. What is left computes its whole h and is looked up.
 //   MD5 is computed per window (two compressions, or one without the padding block); there the
 //   hash dominates and the global Bloom word is tested directly.
 //
-// Passes (no worst-case hit buffer). The count kernel hashes every window, filters it, resolves
-// the candidates (probe; byte confirmation for djb2) and writes each tile's triple count; an
-// exclusive scan gives every tile its output offset; the emit kernel redoes only the tiles
-// that have triples and writes them in window order. Filters never drop a match, so the emit
-// kernel, which skips the shared-memory filter, finds exactly the counted triples.
+// Passes. The count kernel hashes every window, filters it, resolves the candidates (probe; byte
+// confirmation for djb2), writes each tile's triple count and, for a tile with triples, an entry
+// of the image's hit list: which windows of each lane have any. An exclusive scan gives every tile
+// its output offset; the emit kernel looks the listed windows up again and writes their triples
+// in window order. (Hit records instead of lookups done twice would need room for every window.)
+// The lists' masks take 128 bytes per tile, 4.3% of the image for djb2 and 3.2% for MD5, and at
+// most 512 MiB; a listed tile beyond that has all its windows looked up again.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -34,40 +36,27 @@
 #include "cv_launch.h"
 #include "scan_kernel.cuh"
 
-// The djb2 count kernel's block size, tile buffers per warp and Bloom pipeline depth: the
-// fastest measured on GB300 (4 GiB fragment workload, count kernel, all exact): 512 threads, two
-// buffers, depth 12: 1,431 GB/s; depth 8: 1,425; depth 17: 1,298. With more warps per SM the
-// kernel exceeds its register share and spills: 1024 threads, one buffer, depth 6 / 8 / 12:
-// 1,312 / 971 / 834; 640 threads, two buffers, depth 8: 892; 768, one buffer, depth 8: 883.
-#ifndef CV_FRAG_DJB2_THREADS
-#define CV_FRAG_DJB2_THREADS 512
-#endif
-#ifndef CV_FRAG_DJB2_BUFS
-#define CV_FRAG_DJB2_BUFS 2
-#endif
-#ifndef CV_FRAG_DJB2_BLOOM_DEPTH
-#define CV_FRAG_DJB2_BLOOM_DEPTH 12
-#endif
-
 namespace cvk {
 
 // Tile geometry per signature (a tile is one warp's work).
 template <int SIG>
 struct FragGeom {
   static constexpr bool kRolled = SIG == kSigDjb2;
-  static constexpr int kThreads = kRolled ? CV_FRAG_DJB2_THREADS : 256;  // block size
+  static constexpr int kThreads = kRolled ? 1024 : 256;  // block size
   static constexpr int kWarps = kThreads / 32;
-  static constexpr int kWPT = kRolled ? 17 : 33;        // windows per lane per tile (odd)
-  static constexpr int kBufs = kRolled ? CV_FRAG_DJB2_BUFS : 2;  // tile buffers per warp (count kernel)
-  static constexpr int kBloomDepth = CV_FRAG_DJB2_BLOOM_DEPTH;  // Bloom words in flight per lane
+  static constexpr int kWPT = kRolled ? 23 : 31;  // windows per lane per tile (odd)
+  static constexpr int kBufs = kRolled ? 1 : 2;   // tile buffers per warp (count kernel)
+  // Rolled: windows per lane that can wait for the second filter. They wait in the lane's part of
+  // the tile, from its word 15 on, where the words are read by this lane alone, each before the
+  // entry that takes its place is written.
+  static constexpr int kQueue = kWPT - 15;
   static constexpr uint32_t kTileWin = 32 * kWPT;
   static constexpr uint32_t kTileStep = kTileWin * kFragStride;  // bytes between tile starts
   static constexpr uint32_t kTileBytes = kTileStep + 64;         // bytes staged per tile
   static constexpr bool kL1 = kRolled;                           // shared-memory filter
   static constexpr uint32_t kL1Off = kBufs * kWarps * kTileBytes;  // filter after the warps' buffers
   static constexpr uint32_t kSmemCount = kL1Off + (kL1 ? kFragL1Bytes : 0);
-  static constexpr uint32_t kSmemEmit = kWarps * kTileBytes;
-  static_assert(kWPT % 2 == 1 && kWPT <= 64 && (!kRolled || kWPT <= 32), "odd window count, masks of 64/32 bits");
+  static_assert(kWPT % 2 == 1 && kWPT <= 32 && (!kRolled || kQueue > 0), "odd window count, masks of 32 bits");
   static_assert(kTileBytes % 16 == 0 && kTileStep % 16 == 0, "bulk copies of whole 16-byte chunks");
   static_assert(kBufs == 1 || kBufs == 2, "one or two tile buffers per warp");
   static_assert(kSmemCount <= 227 * 1024, "shared memory of one block");
@@ -91,8 +80,10 @@ struct FragParams {
   uint64_t tile_base;            // index of this image's first tile in tile_ntrip / tile_off
   uint64_t* tile_ntrip;          // count: triples per tile
   const uint64_t* tile_off;      // emit: output offset per tile
-  const uint32_t* hit_tiles;     // emit: this image's tiles with triples (local indices)
-  const uint32_t* n_hit_tiles;   // emit: their number (device)
+  uint32_t* hit_tiles;           // this image's tiles with triples, in any order (local indices)
+  uint32_t* hit_masks;           // per listed tile and lane: its windows with triples
+  uint32_t* n_hit_tiles;         // their number (device), zero before the count
+  uint32_t mask_cap;             // listed tiles that have masks
   MatchOut* out;
   uint64_t out_cap;
   uint32_t* status;
@@ -109,45 +100,72 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
       : "memory");
 }
 
-__device__ __forceinline__ uint32_t frag_bloom_bits(uint32_t d2) {
-  return (1u << (d2 & 31)) | (1u << ((d2 >> 5) & 31)) | (1u << ((d2 >> 10) & 31));
+// The one-word Bloom filter of a fragment table. MD5 keys are mixed already; a djb2-64 key is represented by g, the low word of h less
+// the initial value's share (what the scan rolls), spread by two odd multipliers.
+template <int SIG>
+__device__ __forceinline__ uint32_t frag_bloom_word(uint32_t g, uint32_t d3, uint32_t mask) {
+  if constexpr (SIG == kSigDjb2) return __umulhi(g * 0x9E3779B1u + 0x7F4A7C15u, mask + 1u);
+  return d3 & mask;
 }
 
-__device__ __forceinline__ bool frag_bloom_test(const TableView& tab, uint32_t d2, uint32_t d3) {
-  const uint32_t bits = frag_bloom_bits(d2);
-  return (__ldg(reinterpret_cast<const uint32_t*>(tab.bloom) + (d3 & tab.bloom_mask)) & bits) == bits;
+// The key's bits of its word: three bit numbers, for djb2-64 (where the test is off the scan's
+// inner loop) five, each taken mod 32.
+template <int SIG>
+constexpr int kFragBloomBits = SIG == kSigDjb2 ? 5 : 3;
+
+template <int SIG>
+__device__ __forceinline__ uint32_t frag_bloom_bit(uint32_t g, uint32_t d2, int k) {
+  if constexpr (SIG == kSigDjb2) return (g * 0x85EBCA77u + 0x27D4EB2Fu) >> (27 - 5 * k);  // g = 0: zero windows
+  return d2 >> (5 * k);
+}
+
+template <int SIG>
+__device__ __forceinline__ bool frag_bloom_hit(uint32_t v, uint32_t g, uint32_t d2) {
+  uint32_t t = 1u;
+#pragma unroll
+  for (int k = 0; k < kFragBloomBits<SIG>; k++) t &= __funnelshift_r(v, 0u, frag_bloom_bit<SIG>(g, d2, k));
+  return t != 0u;
+}
+
+// The shared-memory filter of a djb2 fragment table: two bits, from the low ten bits of g, of the
+// word that its top 15 bits select. Both bits are set for 0.09 of the windows at 173,751 keys,
+// against 0.15 for one bit.
+__device__ __forceinline__ uint32_t frag_l1_word(uint32_t g) { return g >> 17; }
+__device__ __forceinline__ uint32_t frag_l1_bits(uint32_t g) { return (1u << (g & 31)) | (1u << ((g >> 5) & 31)); }
+__device__ __forceinline__ uint32_t frag_l1_hit(uint32_t v, uint32_t g) {
+  return __funnelshift_r(v, 0u, g) & __funnelshift_r(v, 0u, g >> 5) & 1u;
 }
 
 // djb2-64 of consecutive windows w0, w0 + 1, ... (ws: 32-bit words in shared memory), rolled:
-// first() computes window w0 from its 16 words, then next(i) moves to window w0 + i (called for
+// first() computes window w0 from its 16 words, then next(x, i) moves to window w0 + i (called for
 // i = 1, 2, ... in order) with one new word. P holds the Horner values of the current window's
-// words, g = h - 5381 * 33^64.
+// words, g = h - 5381 * 33^64. U: uint64_t, or uint32_t for the low word of g alone.
+template <class U>
 struct Djb2Roll {
   uint32_t P[16];
-  uint64_t g;
-  __device__ __forceinline__ uint64_t first(const uint32_t* ws, uint32_t w0) {
+  U g;
+  __device__ __forceinline__ void first(const uint32_t* ws, uint32_t w0) {
     g = 0;
 #pragma unroll
     for (int q = 0; q < 16; q++) {
       P[q] = horner33(ws[w0 + q]);
-      g = g * kD33x4 + P[q];
+      g = g * (U)kD33x4 + P[q];
     }
-    return g + kDjbInit;
   }
-  __device__ __forceinline__ uint64_t next(const uint32_t* ws, uint32_t w0, int i) {
-    const uint32_t pin = horner33(ws[w0 + i + 15]);
-    g = g * kD33x4 - (uint64_t)P[(i - 1) & 15] * kD33x64 + pin;
+  // x: the new window's last word (ws[w0 + i + 15])
+  __device__ __forceinline__ void next(uint32_t x, int i) {
+    const uint32_t pin = horner33(x);
+    g = g * (U)kD33x4 + (P[(i - 1) & 15] * (U)(0 - kD33x64) + pin);
     P[(i - 1) & 15] = pin;
-    return g + kDjbInit;
   }
 };
 
-// Key words of the window whose first word is ws[w] (shared memory), computed directly.
+// Key words of the window whose 16 words start at x, computed directly.
 template <int SIG>
-__device__ __forceinline__ void frag_key(const uint32_t* ws, uint32_t w, uint32_t (&d)[4], uint32_t one) {
+__device__ __forceinline__ void frag_key(const uint32_t* x, uint32_t (&d)[4], uint32_t one) {
   uint32_t X[16];
 #pragma unroll
-  for (int q = 0; q < 16; q++) X[q] = ws[w + q];
+  for (int q = 0; q < 16; q++) X[q] = x[q];
   if constexpr (SIG == kSigDjb2) {
     frag64_words(djb2_block(5381ull, X), d);
   } else {
@@ -157,102 +175,167 @@ __device__ __forceinline__ void frag_key(const uint32_t* ws, uint32_t w, uint32_
   }
 }
 
-// 64 bytes of the window at ws[w] (shared, 4-byte aligned) against a master fragment (global,
-// 16-byte aligned).
-__device__ __forceinline__ bool frag_equal(const uint32_t* ws, uint32_t w, const uint8_t* m) {
+// The 64 bytes at x (4-byte aligned) against a master fragment (16-byte aligned).
+__device__ __forceinline__ bool frag_equal(const uint32_t* x, const uint8_t* m) {
   const uint4* y = reinterpret_cast<const uint4*>(m);
   uint32_t diff = 0;
 #pragma unroll
   for (int q = 0; q < 4; q++) {
     const uint4 v = __ldg(y + q);
-    diff |= (ws[w + 4 * q] ^ v.x) | (ws[w + 4 * q + 1] ^ v.y) | (ws[w + 4 * q + 2] ^ v.z) | (ws[w + 4 * q + 3] ^ v.w);
+    diff |= (x[4 * q] ^ v.x) | (x[4 * q + 1] ^ v.y) | (x[4 * q + 2] ^ v.z) | (x[4 * q + 3] ^ v.w);
   }
   return diff == 0;
 }
 
 // Candidate windows of this thread (bit i: window w0 + i passed the filters; every valid window
-// when the table has no Bloom filter). n_valid: the thread's windows inside the image. l1: the
-// shared-memory filter, or null to skip it (then every window goes to the global Bloom word).
+// when the table has no Bloom filter and no first filter). n_valid: the thread's windows inside the
+// image. l1: the first filter, in shared or global memory (rolled kernels only). ws is the warp's
+// tile; the rolled kernels' waiting windows overwrite parts of it (FragGeom::kQueue).
+//
+// Rolled: the cost is instructions, not memory. A window takes one shared-memory word, two dp2a,
+// two multiply-adds and the filter (word address, load, two shifts by the low bits of g, which wrap
+// by themselves); its random load, 3.6 shared-memory cycles on average, sets the pace. The windows
+// that pass (one in twelve at 173,751 keys) only store their g; their Bloom words are requested
+// afterwards. 1 GiB image, count kernel: the loop alone takes 225 us (shared memory 85% busy), the
+// Bloom words 105 more, the lookups 55: 388 us, against 800 with 64-bit h, one filter bit and the
+// Bloom test inside the loop, where its dozen instructions are executed for every window because
+// some lane nearly always has one to test. Dealing the waiting windows out evenly over the warp
+// (a scan and searches by shuffles) took 392 us: shuffles use the same pipe.
+// A window with the g of the window before it (fills, patterns of four bytes) shares that one's
+// entry, so such runs need one place; a lane with more passing windows than places sends the rest
+// on unfiltered. The stores are predicated by hand (a branch per window cost more than they do),
+// and each word is read a window ahead because no load may move past them.
 template <int SIG>
-__device__ __forceinline__ uint64_t frag_candidates(const FragParams& p, const uint32_t* ws, uint32_t w0,
-                                                    uint32_t n_valid, const uint32_t* l1) {
+__device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_t* ws, uint32_t w0, uint32_t n_valid,
+                                                    const uint32_t* l1) {
   using G = FragGeom<SIG>;
-  uint64_t cand = 0;
   if constexpr (G::kRolled) {
-    // Window by window: the rolled hash, its shared-memory filter bit (from h's high word, d1,
-    // with no further mixing) and, when that passes, the request of its one-word Bloom filter
-    // word (mixed words d2, d3); each Bloom word is tested kBloomDepth windows later, so that
-    // many requests are in flight per lane while only kBloomDepth are held in registers. A window
-    // that did not pass keeps (word 0, bits 1), which fails the test.
-    constexpr int D = G::kBloomDepth < G::kWPT ? G::kBloomDepth : G::kWPT;
-    const uint32_t* bloom = reinterpret_cast<const uint32_t*>(p.tab.bloom);
-    const bool use_bloom = p.tab.use_bloom != 0u;
-    Djb2Roll roll;
-    uint32_t wv[D], wbits[D];
+    const uint32_t queue = smem_addr(ws + w0 + 15), queue_end = queue + 4u * G::kQueue;
+    Djb2Roll<uint32_t> roll;
+    uint32_t pass = 0, fresh = 0, at = queue, x = 0, before = 0;
 #pragma unroll
-    for (int i = 0; i < G::kWPT + D; i++) {
-      if (use_bloom && i >= D) {  // window i - D's word, before window i takes its ring slot
-        const int j = i - D;
-        if ((wv[j % D] & wbits[j % D]) == wbits[j % D]) cand |= 1ull << j;
+    for (int i = 0; i < G::kWPT; i++) {
+      if (i == 0) {
+        roll.first(ws, w0);
+        before = ~roll.g;
+      } else {
+        before = roll.g;
+        roll.next(x, i);
       }
-      if (i < G::kWPT) {
-        const uint64_t h = i == 0 ? roll.first(ws, w0) : roll.next(ws, w0, i);
-        const uint32_t b = (uint32_t)(h >> 32) >> (32 - kFragL1Log2Bits);
-        const bool pass = (uint32_t)i < n_valid && (!l1 || ((l1[b >> 5] >> (b & 31)) & 1u));
-        if (!use_bloom) {
-          if (pass) cand |= 1ull << i;
-        } else {
-          wv[i % D] = 0u;
-          wbits[i % D] = 1u;
-          if (pass) {
-            uint32_t d[4];
-            frag64_words(h, d);
-            wbits[i % D] = frag_bloom_bits(d[2]);
-            wv[i % D] = __ldg(bloom + (d[3] & p.tab.bloom_mask));
-          }
-        }
+      if (i + 1 < G::kWPT) x = ws[w0 + i + 16];
+      asm volatile(
+          "{\n\t.reg .pred hit, first, room;\n\t"
+          "setp.ne.u32 hit, %3, 0;\n\t"
+          "setp.ne.and.u32 first, %4, %5, hit;\n\t"
+          "setp.lt.and.u32 room, %0, %6, first;\n\t"
+          "@room st.shared.u32 [%0], %4;\n\t"
+          "@first add.u32 %0, %0, 4;\n\t"
+          "@first or.b32 %1, %1, %7;\n\t"
+          "@hit or.b32 %2, %2, %7;\n\t}"
+          : "+r"(at), "+r"(fresh), "+r"(pass)
+          : "r"(frag_l1_hit(l1[frag_l1_word(roll.g)], roll.g)), "r"(roll.g), "r"(before), "r"(queue_end), "r"(1u << i)
+          : "memory");
+    }
+    // windows past the image's end come last
+    if (n_valid < (uint32_t)G::kWPT) {
+      pass &= (1u << n_valid) - 1u;
+      fresh &= (1u << n_valid) - 1u;
+    }
+    if (!p.tab.use_bloom) return pass;
+    const uint32_t* bloom = reinterpret_cast<const uint32_t*>(p.tab.bloom);
+    const uint32_t* const waiting = ws + w0 + 15;
+    const uint32_t same = pass ^ fresh, n = min((uint32_t)__popc(fresh), (uint32_t)G::kQueue);
+    uint32_t cand = 0;
+    for (uint32_t k = 0; k < n; k += 2) {  // two requests at a time
+      const bool two = k + 1 < n;
+      const uint32_t g0 = waiting[k], g1 = two ? waiting[k + 1] : 0u;
+      const uint32_t v0 = __ldg(bloom + frag_bloom_word<SIG>(g0, 0u, p.tab.bloom_mask));
+      const uint32_t v1 = two ? __ldg(bloom + frag_bloom_word<SIG>(g1, 0u, p.tab.bloom_mask)) : 0u;
+      const uint32_t b0 = fresh & (0u - fresh);
+      fresh ^= b0;
+      if (frag_bloom_hit<SIG>(v0, g0, 0u)) cand |= b0;
+      if (two) {
+        const uint32_t b1 = fresh & (0u - fresh);
+        fresh ^= b1;
+        if (frag_bloom_hit<SIG>(v1, g1, 0u)) cand |= b1;
       }
     }
+    cand |= fresh;
+    // the windows after a candidate that share its entry: a carry through each run of them
+    return cand | (((same + (same & (cand << 1))) ^ same) & same);
   } else {
+    uint32_t cand = 0;
 #pragma unroll 1
     for (uint32_t i = 0; i < n_valid; i++) {
       uint32_t d[4];
-      frag_key<SIG>(ws, w0 + i, d, p.one);
-      if (!p.tab.use_bloom || frag_bloom_test(p.tab, d[2], d[3])) cand |= 1ull << i;
+      frag_key<SIG>(ws + w0 + i, d, p.one);
+      if (!p.tab.use_bloom || frag_bloom_hit<SIG>(__ldg(reinterpret_cast<const uint32_t*>(p.tab.bloom) +
+                                                        frag_bloom_word<SIG>(d[0], d[3], p.tab.bloom_mask)),
+                                                  d[0], d[2]))
+        cand |= 1u << i;
     }
+    return cand;
   }
-  return cand;
 }
 
-// Probe one candidate window; returns the triples it yields (postings, confirmed byte for byte
-// for djb2) and the posting range.
+// The 16 words of this thread's window w0 + i of the tile: in the tile, or, where the tile may be
+// overwritten, in the image.
+template <int SIG>
+__device__ __forceinline__ const uint32_t* frag_words(const FragParams& p, uint64_t tile, const uint32_t* ws,
+                                                      uint32_t w) {
+  if constexpr (FragGeom<SIG>::kRolled)
+    return reinterpret_cast<const uint32_t*>(p.image) + (tile * FragGeom<SIG>::kTileWin + w);
+  return ws + w;
+}
+
+// One candidate window per lane (has; x: its words) looked up; returns the triples it yields
+// (postings, confirmed byte for byte for djb2) and its posting range. The lanes of the warp
+// compare the postings of a window that has several together: a header that hundreds of files
+// share has hundreds. Every lane of the warp calls it.
 template <int SIG, int LAYOUT>
-__device__ __forceinline__ uint32_t frag_resolve(const FragParams& p, const uint32_t* ws, uint32_t w,
-                                                 uint32_t& post_off, uint32_t& post_cnt) {
-  uint32_t d[4];
-  frag_key<SIG>(ws, w, d, p.one);
+__device__ __forceinline__ uint32_t frag_resolve(const FragParams& p, const uint32_t* x, bool has, uint32_t& post_off,
+                                                 uint32_t& post_cnt) {
   post_off = 0;
-  post_cnt = LAYOUT == kLayoutSorted ? sorted_probe(p.tab, d[0], d[1], d[2], d[3], 0u, post_off)
-                                     : table_probe(p.tab, d[0], d[1], d[2], d[3], 0u, post_off);
-  if (!sig_is_weak(SIG) || post_cnt == 0) return post_cnt;
+  post_cnt = 0;
+  if (has) {
+    uint32_t d[4];
+    frag_key<SIG>(x, d, p.one);
+    post_cnt = LAYOUT == kLayoutSorted ? sorted_probe(p.tab, d[0], d[1], d[2], d[3], 0u, post_off)
+                                       : table_probe(p.tab, d[0], d[1], d[2], d[3], 0u, post_off);
+  }
+  if constexpr (!sig_is_weak(SIG)) return post_cnt;
   uint32_t n = 0;
-  for (uint32_t q = 0; q < post_cnt; q++) n += frag_equal(ws, w, p.tab.confirm + (uint64_t)(post_off + q) * 64) ? 1u : 0u;
+  if (post_cnt == 1u) n = frag_equal(x, p.tab.confirm + (uint64_t)post_off * 64) ? 1u : 0u;
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t several = __ballot_sync(0xFFFFFFFFu, post_cnt > 1u); several; several &= several - 1) {
+    const int src = __ffs(several) - 1;
+    const uint32_t* xs = reinterpret_cast<const uint32_t*>(
+        __shfl_sync(0xFFFFFFFFu, reinterpret_cast<uintptr_t>(x), src));
+    const uint32_t off = __shfl_sync(0xFFFFFFFFu, post_off, src), cnt = __shfl_sync(0xFFFFFFFFu, post_cnt, src);
+    uint32_t k = 0;
+    for (uint32_t q = lane; q < cnt; q += 32) k += frag_equal(xs, p.tab.confirm + (uint64_t)(off + q) * 64) ? 1u : 0u;
+    k = __reduce_add_sync(0xFFFFFFFFu, k);
+    if ((int)lane == src) n = k;
+  }
   return n;
 }
 
-// Triples of this thread's candidate windows; *rejected (when given) adds the candidates that
-// the byte comparison dropped.
+// Triples of this thread's candidate windows; hits: the windows with any; *rejected adds the
+// candidates that the byte comparison dropped. Every lane of the warp calls it.
 template <int SIG, int LAYOUT>
-__device__ __forceinline__ uint64_t frag_thread_count(const FragParams& p, const uint32_t* ws, uint32_t w0,
-                                                      uint64_t cand, uint32_t* rejected = nullptr) {
+__device__ __forceinline__ uint64_t frag_thread_count(const FragParams& p, uint64_t tile, const uint32_t* ws,
+                                                      uint32_t w0, uint32_t cand, uint32_t& hits, uint32_t* rejected) {
   uint64_t n = 0;
-  while (cand) {
-    const int i = __ffsll((long long)cand) - 1;
+  hits = 0;
+  while (__any_sync(0xFFFFFFFFu, cand != 0)) {
+    const bool has = cand != 0;
+    const uint32_t i = has ? (uint32_t)__ffs(cand) - 1u : 0u;
     cand &= cand - 1;
     uint32_t off, cnt;
-    const uint32_t k = frag_resolve<SIG, LAYOUT>(p, ws, w0 + (uint32_t)i, off, cnt);
+    const uint32_t k = frag_resolve<SIG, LAYOUT>(p, frag_words<SIG>(p, tile, ws, w0 + i), has, off, cnt);
     n += k;
-    if (rejected) *rejected += cnt - k;
+    if (k) hits |= 1u << i;
+    *rejected += cnt - k;
   }
   return n;
 }
@@ -362,14 +445,22 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, 1) frag_count_kernel(
       break;
     }
     if ((tile + 1) * G::kTileStep + 64 > p.n_bytes) frag_tail<SIG>(p, tile, buf);  // warp-uniform
-    const uint32_t* ws = reinterpret_cast<const uint32_t*>(buf);
+    uint32_t* ws = reinterpret_cast<uint32_t*>(buf);
     const uint32_t w0 = (uint32_t)lane * G::kWPT;
-    const uint64_t cand = frag_candidates<SIG>(p, ws, w0, frag_valid<SIG>(p, tile, w0), l1);
+    const uint32_t cand = frag_candidates<SIG>(p, ws, w0, frag_valid<SIG>(p, tile, w0), l1);
     uint32_t rej = 0;
-    uint64_t n = frag_thread_count<SIG, LAYOUT>(p, ws, w0, cand, &rej);
+    uint32_t hits;
+    uint64_t n = frag_thread_count<SIG, LAYOUT>(p, tile, ws, w0, cand, hits, &rej);
     if (sig_is_weak(SIG) && rej && p.rejected) atomicAdd(p.rejected, (unsigned long long)rej);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) n += __shfl_xor_sync(0xFFFFFFFFu, n, d);
+    if (n) {  // the sum over the warp
+      uint32_t q = 0;
+      if (lane == 0) q = atomicAdd(p.n_hit_tiles, 1u);
+      q = __shfl_sync(0xFFFFFFFFu, q, 0);
+      if (lane == 0) p.hit_tiles[q] = (uint32_t)tile;
+      if (q < p.mask_cap) p.hit_masks[32ull * q + lane] = hits;
+    }
     __syncwarp();  // every lane is done with the buffer
     if (lane == 0) {
       p.tile_ntrip[p.tile_base + tile] = n;
@@ -391,73 +482,80 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, 1) frag_count_kernel(
   }
 }
 
-// Tiles of one image with triples, as a list of local tile indices (any order).
-__global__ void frag_hit_list_kernel(const uint64_t* tile_ntrip, uint64_t n_tiles, uint32_t* list, uint32_t* count) {
-  for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n_tiles; t += (uint64_t)gridDim.x * blockDim.x)
-    if (tile_ntrip[t]) list[atomicAdd(count, 1u)] = (uint32_t)t;
+// Triple `pos` of the output: window k and posting `post`.
+__device__ __forceinline__ void frag_put(const FragParams& p, uint64_t pos, uint64_t k, uint32_t post) {
+  if (pos < p.out_cap) {
+    const uint2 e = __ldg(p.tab.postings + post);
+    p.out[pos] = MatchOut{k, e.x, e.y};
+  } else {
+    atomicOr(p.status, kStOverflow);
+  }
 }
 
+// A warp per listed tile: its windows with triples are numbered in window order (a lane's windows
+// follow one another) and taken 32 at a time, one per lane, so that the dependent loads of 32 of
+// them (words, slot, confirmation, posting) are in flight together. Bound by that latency.
+constexpr int kEmitThreads = 256;
+
 template <int SIG, int LAYOUT>
-__global__ void __launch_bounds__(FragGeom<SIG>::kThreads, 1) frag_emit_kernel(const __grid_constant__ FragParams p) {
+__global__ void __launch_bounds__(kEmitThreads) frag_emit_kernel(const __grid_constant__ FragParams p) {
   using G = FragGeom<SIG>;
-  extern __shared__ __align__(128) uint8_t fsm[];
-  __shared__ __align__(8) uint64_t bars[G::kWarps];
-  __shared__ uint32_t abort_flag[G::kWarps];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint8_t* buf = fsm + warp * G::kTileBytes;
-  const uint32_t bar = smem_addr(&bars[warp]);
-  if (lane == 0) {
-    abort_flag[warp] = 0;
-    mbar_init(bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncwarp();
-  const uint64_t policy = l2_evict_first_policy();
+  if (*(volatile const uint32_t*)p.status & (kStTimeout | kStProbeBound | kStBadTable)) return;
+  constexpr uint32_t kFull = 0xFFFFFFFFu;
+  const uint32_t lane = threadIdx.x & 31;
   const uint32_t n_list = *(volatile const uint32_t*)p.n_hit_tiles;
-  const uint32_t n_warps = gridDim.x * G::kWarps;
-  uint32_t phase = 0;
-  for (uint32_t j = blockIdx.x * G::kWarps + warp; j < n_list; j += n_warps) {
+  const uint32_t n_warps = gridDim.x * (kEmitThreads / 32);
+  for (uint32_t j = blockIdx.x * (kEmitThreads / 32) + (threadIdx.x >> 5); j < n_list; j += n_warps) {
     const uint64_t tile = p.hit_tiles[j];
-    if (lane == 0) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      frag_issue<SIG>(p, tile, smem_addr(buf), bar, policy);
+    // beyond the masks' room every window is looked up
+    const uint32_t valid = frag_valid<SIG>(p, tile, lane * G::kWPT);
+    const uint32_t mask = j < p.mask_cap ? p.hit_masks[32ull * j + lane] : (uint32_t)((1ull << valid) - 1u);
+    uint64_t at = p.tile_off[p.tile_base + tile];
+    const uint32_t n = (uint32_t)__popc(mask);
+    uint32_t first = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t v = __shfl_up_sync(kFull, first, d);
+      if (lane >= (uint32_t)d) first += v;
     }
-    const bool ok = mbar_wait(bar, phase & 1u, &abort_flag[warp], p.status);
-    if (!__all_sync(0xFFFFFFFFu, ok)) {
-      if (lane == 0) {  // the copy may still land: wait for it (bounded) before leaving
-        volatile uint32_t never = 0;
-        mbar_wait(bar, phase & 1u, &never, p.status);
-      }
-      return;
-    }
-    phase++;
-    if ((tile + 1) * G::kTileStep + 64 > p.n_bytes) frag_tail<SIG>(p, tile, buf);
-    const uint32_t* ws = reinterpret_cast<const uint32_t*>(buf);
-    const uint32_t w0 = (uint32_t)lane * G::kWPT;
-    const uint64_t cand = frag_candidates<SIG>(p, ws, w0, frag_valid<SIG>(p, tile, w0), nullptr);
-    const uint64_t n = frag_thread_count<SIG, LAYOUT>(p, ws, w0, cand);
-    uint64_t total;
-    uint64_t pos = p.tile_off[p.tile_base + tile] + warp_exclusive_u64(n, &total);
-    uint64_t c = cand;
-    while (c) {
-      const int i = __ffsll((long long)c) - 1;
-      c &= c - 1;
-      const uint32_t w = w0 + (uint32_t)i;
+    const uint32_t total = __shfl_sync(kFull, first, 31);
+    first -= n;
+    for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+      // window number e: the k-th window of the last lane whose first number is at or before e
+      const uint32_t e = e0 + lane;
+      uint32_t src = 0;
+#pragma unroll
+      for (uint32_t step = 16; step > 0; step >>= 1)
+        if (__shfl_sync(kFull, first, src + step) <= e) src += step;
+      const bool has = e < total;
+      uint32_t k = e - __shfl_sync(kFull, first, src);
+      uint32_t m = __shfl_sync(kFull, mask, src);
+      if (!has) k = 0;
+      for (; k > 0; k--) m &= m - 1;
+      const uint64_t w = tile * G::kTileWin + src * G::kWPT + (has ? (uint32_t)__ffs(m) - 1u : 0u);
+      const uint32_t* x = reinterpret_cast<const uint32_t*>(p.image) + w;
       uint32_t off, cnt;
-      if (!frag_resolve<SIG, LAYOUT>(p, ws, w, off, cnt)) continue;
-      const uint64_t k = tile * G::kTileWin + w;
-      for (uint32_t q = 0; q < cnt; q++) {
-        if (sig_is_weak(SIG) && !frag_equal(ws, w, p.tab.confirm + (uint64_t)(off + q) * 64)) continue;
-        if (pos < p.out_cap) {
-          const uint2 e = __ldg(p.tab.postings + off + q);
-          p.out[pos] = MatchOut{k, e.x, e.y};
-        } else {
-          atomicOr(p.status, kStOverflow);
+      const uint32_t put = frag_resolve<SIG, LAYOUT>(p, x, has, off, cnt);
+      uint64_t sum;
+      const uint64_t pos = at + warp_exclusive_u64(put, &sum);
+      at += sum;
+      if (cnt == 1u && put == 1u) frag_put(p, pos, w, off);
+      // the postings of a window with several, 32 at a time
+      for (uint32_t several = __ballot_sync(kFull, cnt > 1u); several; several &= several - 1) {
+        const int from = __ffs(several) - 1;
+        const uint32_t* xs = reinterpret_cast<const uint32_t*>(__shfl_sync(kFull, reinterpret_cast<uintptr_t>(x), from));
+        const uint32_t o = __shfl_sync(kFull, off, from), c = __shfl_sync(kFull, cnt, from);
+        const uint64_t ww = __shfl_sync(kFull, (unsigned long long)w, from);
+        uint64_t to = __shfl_sync(kFull, (unsigned long long)pos, from);
+        for (uint32_t q0 = 0; q0 < c; q0 += 32) {
+          const uint32_t q = q0 + lane;
+          const bool equal = q < c && (!sig_is_weak(SIG) || frag_equal(xs, p.tab.confirm + (uint64_t)(o + q) * 64));
+          const uint32_t who = __ballot_sync(kFull, equal);
+          if (equal) frag_put(p, to + __popc(who & ((1u << lane) - 1u)), ww, o + q);
+          to += __popc(who);
         }
-        pos++;
       }
     }
-    __syncwarp();  // the buffer is free again
   }
 }
 
@@ -492,19 +590,20 @@ __global__ void __launch_bounds__(256) frag_window_sig_kernel(const uint8_t* ima
     const uint32_t w0 = (uint32_t)lane * G::kWPT;
     const uint64_t k0 = tile * G::kTileWin + w0;
     if constexpr (G::kRolled) {
-      Djb2Roll roll;
+      Djb2Roll<uint64_t> roll;
 #pragma unroll
       for (int i = 0; i < G::kWPT; i++) {
-        const uint64_t h = i == 0 ? roll.first(ws, w0) : roll.next(ws, w0, i);
+        if (i == 0) roll.first(ws, w0);
+        else roll.next(ws[w0 + i + 15], i);
         uint32_t d[4];
-        frag64_words(h, d);
+        frag64_words(roll.g + kDjbInit, d);
         if (k0 + i < n_windows) out[k0 + i] = make_uint4(d[0], d[1], d[2], d[3]);
       }
     } else {
       for (int i = 0; i < G::kWPT; i++) {
         if (k0 + i >= n_windows) break;
         uint32_t d[4];
-        frag_key<SIG>(ws, w0 + (uint32_t)i, d, one);
+        frag_key<SIG>(ws + w0 + i, d, one);
         out[k0 + i] = make_uint4(d[0], d[1], d[2], d[3]);
       }
     }
@@ -545,17 +644,21 @@ __global__ void frag_digest_kernel(const uint8_t* arena, uint64_t n, uint4* dig,
   }
 }
 
-// The filters of a fragment table from its occupied slots: the one-word Bloom filter (3 bits
-// from d2 in word d3 & mask; none when words is null) and the 2^20-bit shared-memory filter
-// (bit: the top 20 bits of d1).
+// The filters of a fragment table from its occupied slots: the one-word Bloom filter (none when
+// words is null) and the shared-memory filter.
+template <int SIG>
 __global__ void frag_bloom_kernel(const uint4* slots, uint32_t n_slots, uint32_t* words, uint32_t mask,
                                   uint32_t* l1) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_slots; i += gridDim.x * blockDim.x) {
     if (slots[2ull * i + 1].y == 0u) continue;
     const uint4 d = slots[2ull * i];
-    if (words) atomicOr(words + (d.w & mask), frag_bloom_bits(d.z));
-    const uint32_t b = d.y >> (32 - kFragL1Log2Bits);
-    atomicOr(l1 + (b >> 5), 1u << (b & 31));
+    const uint32_t g = SIG == kSigDjb2 ? d.x - (uint32_t)kDjbInit : d.x;
+    if (words) {
+      uint32_t bits = 0;
+      for (int k = 0; k < kFragBloomBits<SIG>; k++) bits |= 1u << (frag_bloom_bit<SIG>(g, d.z, k) & 31);
+      atomicOr(words + frag_bloom_word<SIG>(g, d.w, mask), bits);
+    }
+    atomicOr(l1 + frag_l1_word(g), frag_l1_bits(g));
   }
 }
 
@@ -567,7 +670,7 @@ using KernelFn = const void*;
 struct Geom {
   KernelFn count, emit;
   int threads;
-  uint32_t tile_win, smem_count, smem_emit;
+  uint32_t tile_win, smem_count;
 };
 
 template <int SIG>
@@ -576,7 +679,7 @@ Geom geom_t(uint32_t layout) {
   const bool s = layout == kLayoutSorted;
   return Geom{s ? (KernelFn)frag_count_kernel<SIG, kLayoutSorted> : (KernelFn)frag_count_kernel<SIG, kLayoutHash>,
               s ? (KernelFn)frag_emit_kernel<SIG, kLayoutSorted> : (KernelFn)frag_emit_kernel<SIG, kLayoutHash>,
-              G::kThreads, G::kTileWin, G::kSmemCount, G::kSmemEmit};
+              G::kThreads, G::kTileWin, G::kSmemCount};
 }
 
 bool geom(int sig, uint32_t layout, Geom* g) {
@@ -611,9 +714,6 @@ int frag_device(FragDev** out) {
         if ((e = cudaFuncSetAttribute(g.count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem_count)) !=
             cudaSuccess)
           return (int)e;
-        if ((e = cudaFuncSetAttribute(g.emit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem_emit)) !=
-            cudaSuccess)
-          return (int)e;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.count_blocks[sig][l], g.count, g.threads,
                                                                g.smem_count)) != cudaSuccess)
           return (int)e;
@@ -626,7 +726,7 @@ int frag_device(FragDev** out) {
 }
 
 FragParams make_params(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base,
-                       uint32_t* status) {
+                       const FragHits& hits, uint32_t* status) {
   FragParams p;
   memset(&p, 0, sizeof p);
   p.tab = tab;
@@ -635,6 +735,10 @@ FragParams make_params(const TableView& tab, const uint8_t* image, uint64_t n_by
   p.n_windows = frag_windows(n_bytes);
   p.n_tiles = frag_tiles((int)tab.sig, n_bytes);
   p.tile_base = tile_base;
+  p.hit_tiles = hits.tiles + tile_base;
+  p.hit_masks = hits.masks + 32 * std::min(tile_base, hits.mask_tiles);
+  p.mask_cap = (uint32_t)std::min(p.n_tiles, hits.mask_tiles - std::min(tile_base, hits.mask_tiles));
+  p.n_hit_tiles = hits.count;
   p.status = status;
   p.one = 1u;
   return p;
@@ -663,10 +767,13 @@ int frag_digests(int sig, const uint8_t* arena, uint64_t n, uint4* dig, uint8_t*
   return (int)cudaGetLastError();
 }
 
-int frag_bloom(const uint4* slots, uint32_t n_slots, uint32_t* words, uint32_t mask, uint32_t* l1, int sms,
+int frag_bloom(int sig, const uint4* slots, uint32_t n_slots, uint32_t* words, uint32_t mask, uint32_t* l1, int sms,
                void* stream) {
-  const unsigned g = (unsigned)std::min<uint64_t>((n_slots + 255) / 256, (uint64_t)sms * 8);
-  frag_bloom_kernel<<<g, 256, 0, (cudaStream_t)stream>>>(slots, n_slots, words, mask, l1);
+  const unsigned g = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(((uint64_t)n_slots + 255) / 256, (uint64_t)sms * 8));
+  if (sig == kSigDjb2)
+    frag_bloom_kernel<kSigDjb2><<<g, 256, 0, (cudaStream_t)stream>>>(slots, n_slots, words, mask, l1);
+  else
+    frag_bloom_kernel<kSigMd5><<<g, 256, 0, (cudaStream_t)stream>>>(slots, n_slots, words, mask, l1);
   return (int)cudaGetLastError();
 }
 
@@ -704,8 +811,8 @@ int frag_window_sigs(int sig, const uint8_t* image, uint64_t n_bytes, uint4* out
 }
 
 int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base, uint64_t* tile_ntrip,
-               uint32_t* status, unsigned long long* rejected, int sms, void* stream) {
-  FragParams p = make_params(tab, image, n_bytes, tile_base, status);
+               const FragHits& hits, uint32_t* status, unsigned long long* rejected, int sms, void* stream) {
+  FragParams p = make_params(tab, image, n_bytes, tile_base, hits, status);
   p.rejected = rejected;
   if (!p.n_tiles) return 0;
   FragDev* d;
@@ -723,34 +830,20 @@ int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uin
 }
 
 int frag_emit(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base,
-              const uint64_t* tile_ntrip, const uint64_t* tile_off, uint32_t* list, MatchOut* out, uint64_t out_cap,
-              uint32_t* status, int sms, void* stream, int* launches) {
-  FragParams p = make_params(tab, image, n_bytes, tile_base, status);
+              const uint64_t* tile_off, const FragHits& hits, MatchOut* out, uint64_t out_cap, uint32_t* status, int sms,
+              void* stream) {
+  FragParams p = make_params(tab, image, n_bytes, tile_base, hits, status);
   if (!p.n_tiles) return 0;
-  FragDev* d;
-  int rc = frag_device(&d);
-  if (rc) return rc;
   Geom g;
   if (!geom((int)tab.sig, tab.layout, &g)) return (int)cudaErrorInvalidValue;
-  cudaStream_t st = (cudaStream_t)stream;
-  uint32_t* count = list + p.n_tiles;
-  cudaError_t e = cudaMemsetAsync(count, 0, 4, st);
-  if (e != cudaSuccess) return (int)e;
-  const unsigned gl = (unsigned)std::min<uint64_t>((p.n_tiles + 255) / 256, (uint64_t)sms * 4);
-  frag_hit_list_kernel<<<gl, 256, 0, st>>>(tile_ntrip + tile_base, p.n_tiles, list, count);
-  if ((e = cudaGetLastError()) != cudaSuccess) return (int)e;
   p.tile_off = tile_off;
-  p.hit_tiles = list;
-  p.n_hit_tiles = count;
   p.out = out;
   p.out_cap = out_cap;
-  const uint64_t warps_per_block = (uint64_t)g.threads / 32;
+  const uint64_t warps_per_block = kEmitThreads / 32;
   const unsigned grid = (unsigned)std::min<uint64_t>((p.n_tiles + warps_per_block - 1) / warps_per_block,
-                                                     (uint64_t)sms * 2);
+                                                     (uint64_t)sms * 8);
   void* args[] = {&p};
-  e = cudaLaunchKernel(g.emit, dim3(grid), dim3(g.threads), args, g.smem_emit, st);
-  if (launches) *launches += 2;
-  return (int)e;
+  return (int)cudaLaunchKernel(g.emit, dim3(grid), dim3(kEmitThreads), args, 0, (cudaStream_t)stream);
 }
 
 }  // namespace cvk

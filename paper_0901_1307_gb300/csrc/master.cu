@@ -389,7 +389,7 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
           CV_CUDA(cudaGetLastError());
         }
         if (frag) {
-          CV_CUDA((cudaError_t)frag_bloom((const uint4*)m->slots, (uint32_t)n_slots, (uint32_t*)m->bloom,
+          CV_CUDA((cudaError_t)frag_bloom(sig, (const uint4*)m->slots, (uint32_t)n_slots, (uint32_t*)m->bloom,
                                           bpk ? (uint32_t)(n_blocks - 1) : 0u, (uint32_t*)m->frag_l1, ctx->sms,
                                           stream));
         } else if (bpk) {
@@ -632,6 +632,15 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
     CV_CUDA(cudaFreeAsync(status, stream));
     CV_CUDA(cudaStreamSynchronize(stream));
     if (st) return CV_ECORRUPT;
+    if (h.unit == kUnitFragment) {
+      // a fragment table's filters are made again from its records: their hash functions belong to
+      // the scan kernel of this build, not to the file format
+      CV_CUDA(cudaMemsetAsync(m->frag_l1, 0, h.bytes_l1, stream));
+      if (h.bytes_bloom) CV_CUDA(cudaMemsetAsync(m->bloom, 0, h.bytes_bloom, stream));
+      CV_CUDA((cudaError_t)frag_bloom((int)h.sig, (const uint4*)m->slots, (uint32_t)n_records, (uint32_t*)m->bloom,
+                                      h.bloom_mask, (uint32_t*)m->frag_l1, ctx->sms, stream));
+      CV_CUDA(cudaStreamSynchronize(stream));
+    }
     m->tab.slots = (const uint4*)m->slots;
     m->tab.postings = (const uint2*)m->postings;
     m->tab.bloom = (const uint4*)m->bloom;

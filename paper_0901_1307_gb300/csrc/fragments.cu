@@ -3,12 +3,11 @@
 // find small files (logos, small images) embedded in other files at any 32-bit offset.
 //
 // Work layout. A tile is one warp's work: 32 x WPT consecutive windows. Each warp stages its own
-// tiles (the window starts plus the last window's 60-byte tail) into its own two shared-memory
-// buffers with 1-D bulk TMA copies issued by its lane 0, completion on the warp's own mbarriers,
+// tiles (the window starts plus the last window's 60-byte tail) into its own shared-memory
+// buffer with 1-D bulk TMA copies issued by its lane 0, completion on the warp's own mbarrier,
 // every wait bounded; warps of a block never wait for one another, so a warp that meets a
 // candidate (an L2 probe) holds up no one. Lane l takes windows [WPT l, WPT l + WPT) of the tile;
-// with WPT odd the 32 lanes read 32 different banks at every step. Tiles are spread over every
-// warp of a persistent grid.
+// with WPT odd the 32 lanes read 32 different banks at every step.
 //
 //   djb2-64 (Eq. 1) is rolled. With P(x) the base-33 Horner value of a 4-byte word x and
 //   g = h - 5381 * 33^64, a window W_k of words x_k .. x_{k+15} has g(W_k) = sum_q
@@ -42,10 +41,14 @@ namespace cvk {
 template <int SIG>
 struct FragGeom {
   static constexpr bool kRolled = SIG == kSigDjb2;
-  static constexpr int kThreads = kRolled ? 1024 : 256;  // block size
+  // 32 warps per SM. The rolled kernel's blocks stay and share one copy of the filter; an MD5 warp
+  // hashes one tile (some 70 us) and a block of four such warps ends, so that the hardware deals the
+  // blocks out: with a fixed share of the tiles per warp the same kernel took 1,660 against 1,506 us
+  // (256 MiB), because the scheduler favours some warps of an SM.
+  static constexpr int kThreads = kRolled ? 1024 : 128;  // block size
+  static constexpr int kMinBlocks = kRolled ? 1 : 8;     // resident blocks per SM
   static constexpr int kWarps = kThreads / 32;
   static constexpr int kWPT = kRolled ? 23 : 31;  // windows per lane per tile (odd)
-  static constexpr int kBufs = kRolled ? 1 : 2;   // tile buffers per warp (count kernel)
   // Rolled: windows per lane that can wait for the second filter. They wait in the lane's part of
   // the tile, from its word 15 on, where the words are read by this lane alone, each before the
   // entry that takes its place is written.
@@ -54,11 +57,10 @@ struct FragGeom {
   static constexpr uint32_t kTileStep = kTileWin * kFragStride;  // bytes between tile starts
   static constexpr uint32_t kTileBytes = kTileStep + 64;         // bytes staged per tile
   static constexpr bool kL1 = kRolled;                           // shared-memory filter
-  static constexpr uint32_t kL1Off = kBufs * kWarps * kTileBytes;  // filter after the warps' buffers
+  static constexpr uint32_t kL1Off = kWarps * kTileBytes;  // filter after the warps' buffers
   static constexpr uint32_t kSmemCount = kL1Off + (kL1 ? kFragL1Bytes : 0);
   static_assert(kWPT % 2 == 1 && kWPT <= 32 && (!kRolled || kQueue > 0), "odd window count, masks of 32 bits");
   static_assert(kTileBytes % 16 == 0 && kTileStep % 16 == 0, "bulk copies of whole 16-byte chunks");
-  static_assert(kBufs == 1 || kBufs == 2, "one or two tile buffers per warp");
   static_assert(kSmemCount <= 227 * 1024, "shared memory of one block");
 };
 
@@ -170,7 +172,7 @@ __device__ __forceinline__ void frag_key(const uint32_t* x, uint32_t (&d)[4], ui
     frag64_words(djb2_block(5381ull, X), d);
   } else {
     md5_init(d);
-    md5_compress<3>(d, X, one);
+    md5_compress<0>(d, X, one);
     if constexpr (SIG == kSigMd5) md5_compress_block_padding(d, one);
   }
 }
@@ -398,19 +400,18 @@ __device__ __forceinline__ uint32_t frag_valid(const FragParams& p, uint64_t til
 }
 
 template <int SIG, int LAYOUT>
-__global__ void __launch_bounds__(FragGeom<SIG>::kThreads, 1) frag_count_kernel(const __grid_constant__ FragParams p) {
+__global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBlocks) frag_count_kernel(const __grid_constant__ FragParams p) {
   using G = FragGeom<SIG>;
   extern __shared__ __align__(128) uint8_t fsm[];
-  constexpr int B = G::kBufs;
-  __shared__ __align__(8) uint64_t bars[B * G::kWarps + 1];  // B per warp, the shared-memory filter
+  __shared__ __align__(8) uint64_t bars[G::kWarps + 1];  // one per warp, the shared-memory filter
   __shared__ uint32_t abort_flag[G::kWarps + 1];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t* l1 = G::kL1 ? reinterpret_cast<const uint32_t*>(fsm + G::kL1Off) : nullptr;
-  uint8_t* mybuf = fsm + B * warp * G::kTileBytes;
-  const uint32_t bar0 = smem_addr(&bars[B * warp]);
-  const uint32_t bar_l1 = smem_addr(&bars[B * G::kWarps]);
+  uint8_t* buf = fsm + warp * G::kTileBytes;
+  const uint32_t bar = smem_addr(&bars[warp]);
+  const uint32_t bar_l1 = smem_addr(&bars[G::kWarps]);
   if (tid == 0) {
-    for (int b = 0; b < B * G::kWarps + 1; b++) mbar_init(smem_addr(&bars[b]), 1);
+    for (int b = 0; b < G::kWarps + 1; b++) mbar_init(smem_addr(&bars[b]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid <= G::kWarps) abort_flag[tid] = 0;
@@ -418,18 +419,13 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, 1) frag_count_kernel(
   const uint64_t policy = l2_evict_first_policy();
   const uint64_t n_warps = (uint64_t)gridDim.x * G::kWarps;
   const uint64_t first = (uint64_t)blockIdx.x * G::kWarps + warp;
-  // Buffer s of a warp holds the tiles of its iterations i with i mod B == s; the k-th of them
-  // completes phase k of the buffer's barrier. Lane 0 issues the first B tiles, then each tile
-  // B iterations ahead.
+  // The warp's i-th tile completes phase i of its buffer's barrier; lane 0 issues the next tile when
+  // every lane is done with the buffer (the other warps of the SM cover the copy).
   if (tid == 0 && G::kL1) {
     mbar_arrive_expect_tx(bar_l1, kFragL1Bytes);
     bulk_load(smem_addr(fsm + G::kL1Off), p.tab.frag_l1, kFragL1Bytes, bar_l1, policy);
   }
-  if (lane == 0)
-    for (int s = 0; s < B; s++) {
-      const uint64_t t = first + s * n_warps;
-      if (t < p.n_tiles) frag_issue<SIG>(p, t, smem_addr(mybuf + s * G::kTileBytes), bar0 + 8 * s, policy);
-    }
+  if (lane == 0 && first < p.n_tiles) frag_issue<SIG>(p, first, smem_addr(buf), bar, policy);
   bool ok = true;
   if constexpr (G::kL1) ok = mbar_wait(bar_l1, 0u, &abort_flag[G::kWarps], p.status);
   bool aborted = !__syncthreads_and(ok);  // the only block-wide barrier: the filter is in place
@@ -437,9 +433,7 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, 1) frag_count_kernel(
   for (; !aborted; i++) {
     const uint64_t tile = first + i * n_warps;
     if (tile >= p.n_tiles) break;
-    const int s = (int)(i % B);
-    uint8_t* buf = mybuf + s * G::kTileBytes;
-    ok = mbar_wait(bar0 + 8 * s, (uint32_t)(i / B) & 1u, &abort_flag[warp], p.status);
+    ok = mbar_wait(bar, (uint32_t)i & 1u, &abort_flag[warp], p.status);
     if (!__all_sync(0xFFFFFFFFu, ok)) {
       aborted = true;
       break;
@@ -464,21 +458,20 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, 1) frag_count_kernel(
     __syncwarp();  // every lane is done with the buffer
     if (lane == 0) {
       p.tile_ntrip[p.tile_base + tile] = n;
-      const uint64_t next = tile + B * n_warps;
+      const uint64_t next = tile + n_warps;
       if (next < p.n_tiles) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        frag_issue<SIG>(p, next, smem_addr(buf), bar0 + 8 * s, policy);
+        frag_issue<SIG>(p, next, smem_addr(buf), bar, policy);
       }
     }
     __syncwarp();
   }
   if (aborted && lane == 0) {
-    // The filter (lane 0 of warp 0) and this warp's iterations i .. i + B - 1 may have copies
-    // issued and not waited for: let them land, each wait bounded, before shared memory goes away.
+    // The filter (lane 0 of warp 0) and this warp's tile may have copies issued and not waited for:
+    // let them land, each wait bounded, before shared memory goes away.
     volatile uint32_t never = 0;
     if (G::kL1 && tid == 0) mbar_wait(bar_l1, 0u, &never, p.status);
-    for (uint64_t j = i; j < i + B && first + j * n_warps < p.n_tiles; j++)
-      if (!mbar_wait(bar0 + 8 * (j % B), (uint32_t)(j / B) & 1u, &never, p.status)) break;
+    if (first + i * n_warps < p.n_tiles) mbar_wait(bar, (uint32_t)i & 1u, &never, p.status);
   }
 }
 
@@ -822,7 +815,7 @@ int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uin
   if (!geom((int)tab.sig, tab.layout, &g)) return (int)cudaErrorInvalidValue;
   if (tab.sig == kSigDjb2 && !tab.frag_l1) return (int)cudaErrorInvalidValue;  // the kernel copies it in
   p.tile_ntrip = tile_ntrip;
-  const uint64_t cap = (uint64_t)sms * (uint64_t)d->count_blocks[tab.sig][tab.layout];
+  const uint64_t cap = tab.sig == kSigDjb2 ? (uint64_t)sms * (uint64_t)d->count_blocks[tab.sig][tab.layout] : INT32_MAX;
   const uint64_t warps_per_block = (uint64_t)g.threads / 32;
   const unsigned grid = (unsigned)std::min<uint64_t>((p.n_tiles + warps_per_block - 1) / warps_per_block, cap);
   void* args[] = {&p};

@@ -149,16 +149,15 @@ __device__ __forceinline__ void md5_compress_x2(uint32_t (&s0)[4], const uint32_
 
 // The padding block of a message of L bits (a multiple of 512 below 2^32): one 1 bit, zeros, then
 // L as a little-endian 64-bit word, i.e. words 0x80, 0, ..., 0, L, 0. Every word is a constant, so
-// X[k] + T[i] folds into one constant per operation. Two of every three operations add it on the
-// FMA pipe (mad.lo with the run-time `one`, as PIPE 3 does for the data blocks): on the
-// ALU-bound sector scan that measured 1% faster than adding it with the integer ALU throughout.
+// X[k] + T[i] folds into one constant per operation. It is added on the FMA pipe (mad.lo with the
+// run-time `one`): the fragment scan, half of whose work is this block, took 1,353 us with that in
+// every operation, 1,395 in two of three, 1,411 in every other one and 1,474 with three-input adds
+// (256 MiB); the sector scan, where it is a ninth, 1.562, 1.566, 1.565 ms and no more (8 GiB).
 template <uint32_t L, int I>
 __device__ __forceinline__ void md5_step_padding(uint32_t& a, uint32_t b, uint32_t c, uint32_t d, uint32_t one) {
   constexpr int k = md5_word(I);
   constexpr uint32_t C = (k == 0 ? 0x80u : k == 14 ? L : 0u) + kMd5Sines.v[I];
-  uint32_t t;
-  if constexpr (I % 3 != 0) t = mad_one_imm<C>(one, a) + md5_aux<I / 16>(b, c, d);
-  else t = a + C + md5_aux<I / 16>(b, c, d);
+  const uint32_t t = mad_one_imm<C>(one, a) + md5_aux<I / 16>(b, c, d);
   a = b + __funnelshift_l(t, t, md5_rot(I));
 }
 

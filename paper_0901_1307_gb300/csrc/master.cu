@@ -22,6 +22,16 @@ using namespace cvk;
 
 namespace {
 
+// In-place exclusive scan of n u32 values (sums: (n + kScanChunk - 1) / kScanChunk words).
+int scan_u32(uint32_t* v, uint64_t n, uint32_t* sums, cudaStream_t stream) {
+  const uint32_t nc = (uint32_t)((n + kScanChunk - 1) / kScanChunk);
+  scan_chunk_sums_u32_kernel<<<nc, kScanThreads, 0, stream>>>(v, n, sums);
+  scan_sums_u32_kernel<<<1, 1024, 0, stream>>>(sums, nc);
+  scan_chunks_u32_kernel<<<nc, kScanThreads, 0, stream>>>(v, n, sums);
+  CV_CUDA(cudaGetLastError());
+  return CV_OK;
+}
+
 // Stable LSD radix sort of n (key, value) pairs by the low `bits` bits of the key, 8 bits per
 // pass, ping-ponging between (k0, v0) and (k1, v1); *kres/*vres receive the pair holding the
 // result.
@@ -35,9 +45,7 @@ int radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uin
   CV_TRY(tmp.alloc(&sums, (uint64_t)nc * 4));
   for (int shift = 0; shift < bits && n; shift += 8) {
     rs_hist_kernel<<<nb, kRsThreads, 0, stream>>>(k0, n, shift, hist, nb);
-    scan_chunk_sums_u32_kernel<<<nc, kScanThreads, 0, stream>>>(hist, (uint64_t)nb * 256, sums);
-    scan_sums_u32_kernel<<<1, 1024, 0, stream>>>(sums, nc);
-    scan_chunks_u32_kernel<<<nc, kScanThreads, 0, stream>>>(hist, (uint64_t)nb * 256, sums);
+    CV_TRY(scan_u32(hist, (uint64_t)nb * 256, sums, stream));
     rs_scatter_kernel<<<nb, kRsThreads, 0, stream>>>(k0, v0, k1, v1, n, shift, hist, nb);
     CV_CUDA(cudaGetLastError());
     std::swap(k0, k1);
@@ -45,6 +53,28 @@ int radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uin
   }
   *kres = k0;
   *vres = v0;
+  return CV_OK;
+}
+
+// The postings of keys with several members (n_several members in all): in master order within a key.
+int several_members(DevCtx* ctx, const uint32_t* slot_of, uint64_t M, uint64_t n_slots, const uint64_t* words,
+                    const uint4* slots, uint32_t n_several, uint32_t n_kept, const uint2* post, uint2* postings,
+                    uint32_t* member, Temps& tmp, cudaStream_t stream) {
+  uint32_t *at, *sums, *k0, *v0, *k1, *v1, *kr, *vr;
+  CV_TRY(tmp.alloc(&at, M * 4));
+  CV_TRY(tmp.alloc(&sums, (M + kScanChunk - 1) / kScanChunk * 4));
+  for (uint32_t** q : {&k0, &v0, &k1, &v1}) CV_TRY(tmp.alloc(q, (uint64_t)n_several * 4));
+  const unsigned g = grid_for(M, 256, ctx->sms), gs = grid_for(n_several, 256, ctx->sms);
+  several_flags_kernel<<<g, 256, 0, stream>>>(slot_of, M, (uint32_t)n_slots, words, at);
+  CV_CUDA(cudaGetLastError());
+  CV_TRY(scan_u32(at, M, sums, stream));
+  several_keys_kernel<<<g, 256, 0, stream>>>(slot_of, M, (uint32_t)n_slots, slots, at, k0, v0);
+  CV_CUDA(cudaGetLastError());
+  int bits = 1;
+  while ((1ull << bits) < n_kept) bits++;
+  CV_TRY(radix_sort_pairs(k0, v0, k1, v1, n_several, bits, tmp, stream, &kr, &vr));
+  several_postings_kernel<<<gs, 256, 0, stream>>>(kr, vr, n_several, post, postings, member);
+  CV_CUDA(cudaGetLastError());
   return CV_OK;
 }
 
@@ -318,29 +348,31 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       const uint8_t* arena;  // the master units, back to back in file order (device memory)
       uint4* dig;
       uint8_t* trivial;
-      uint32_t *owner, *cnt, *slot_of, *keys2, *vals, *vals2, *counters;
+      uint32_t *slot_of, *counters, *member = nullptr;
+      uint32_t *first, *sums;
+      unsigned long long* words;
+      uint2* post;
+      const uint32_t chunks = (uint32_t)((n_slots + kSlotChunk - 1) / kSlotChunk);
       uint64_t* file_base_d;
       CV_TRY(tmp.alloc(&dig, M * sizeof(uint4)));
       CV_TRY(tmp.alloc(&trivial, M));
-      CV_TRY(tmp.alloc(&owner, n_slots * 4));
-      CV_TRY(tmp.alloc(&cnt, n_slots * 4));
+      CV_TRY(tmp.alloc(&words, n_slots * 8));
+      CV_TRY(tmp.alloc(&first, chunks * 4ull));
+      CV_TRY(tmp.alloc(&sums, (chunks / kScanChunk + 1) * 4ull));
       CV_TRY(tmp.alloc(&slot_of, M * 4));
-      CV_TRY(tmp.alloc(&keys2, M * 4));
-      CV_TRY(tmp.alloc(&vals, M * 4));
-      CV_TRY(tmp.alloc(&vals2, M * 4));
-      CV_TRY(tmp.alloc(&counters, 16));  // max_disp, n_kept, n_unique, status
+      CV_TRY(tmp.alloc(&post, M * sizeof(uint2)));
+      if (sig_is_weak(sig)) CV_TRY(tmp.alloc(&member, M * 4));
+      CV_TRY(tmp.alloc(&counters, 32));  // max_disp, n_kept, n_unique, members of keys with several, status
       CV_TRY(tmp.alloc(&file_base_d, (n_files + 1) * 8));
       uint8_t* tau = nullptr;  // per master sector cluster position (position-keyed tables)
       if (by_tau) CV_TRY(tmp.alloc(&tau, std::max<uint64_t>(M, 1)));
-      CV_CUDA(cudaMemsetAsync(owner, 0, n_slots * 4, stream));
-      CV_CUDA(cudaMemsetAsync(cnt, 0, n_slots * 4, stream));
-      CV_CUDA(cudaMemsetAsync(counters, 0, 16, stream));
+      CV_CUDA(cudaMemsetAsync(words, 0, n_slots * 8, stream));
+      CV_CUDA(cudaMemsetAsync(counters, 0, 32, stream));
       CV_CUDA(cudaMemcpyAsync(file_base_d, file_base.data(), (n_files + 1) * 8, cudaMemcpyHostToDevice, stream));
       CV_TRY(gather_master_units(ctx, files, n_files, file_base, U, tmp, stream, &arena));
       // long-lived table memory
       CV_CUDA(cudaMalloc(&m->slots, n_slots * 32));
       CV_CUDA(cudaMalloc(&m->postings, std::max<uint64_t>(M, 1) * 8));
-      CV_CUDA(cudaMemsetAsync(m->slots, 0, n_slots * 32, stream));
       // Bloom blocks: 32 bytes for sector tables, one 32-bit word for fragment tables
       const uint64_t block_bytes = frag ? 4 : 32;
       uint64_t n_blocks = 0;
@@ -361,50 +393,44 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
         } else {
           Job job;
           CV_TRY(job.add(ctx, cfg, arena, M, 0, 0, false));
-          CV_TRY(digest_job(ctx, cfg_i, sig, job, dig, trivial, counters + 3, stream, tmp));
+          CV_TRY(digest_job(ctx, cfg_i, sig, job, dig, trivial, counters + 4, stream, tmp));
         }
         const unsigned g = grid_for(M, 256, ctx->sms);
-        if (tau) {
-          tau_kernel<<<g, 256, 0, stream>>>(file_base_d, n_files, M, tau);
-          CV_CUDA(cudaGetLastError());
-        }
-        insert_kernel<<<g, 256, 0, stream>>>(dig, trivial, tau, M, owner, cnt, slot_of, mask, counters, counters + 1,
-                                            counters + 3);
+        unit_postings_kernel<<<grid_for((M + kPostRun - 1) / kPostRun * 32, 256, ctx->sms), 256, 0, stream>>>(
+            file_base_d, n_files, M, post, tau);
         CV_CUDA(cudaGetLastError());
-        iota_kernel<<<g, 256, 0, stream>>>(vals, M);
+        insert_kernel<<<g, 256, 0, stream>>>(dig, trivial, tau, M, words, slot_of, mask, counters, counters + 1,
+                                            counters + 4);
         CV_CUDA(cudaGetLastError());
-        // stable LSD radix sort of (slot_of, m) by slot_of; keys <= n_slots
-        int bits = 1;
-        while ((1ull << bits) <= n_slots) bits++;
-        uint32_t *kin, *vin;
-        CV_TRY(radix_sort_pairs(slot_of, vals, keys2, vals2, M, bits, tmp, stream, &kin, &vin));
-        fill_kernel<<<g, 256, 0, stream>>>(kin, vin, M, (uint32_t)n_slots, owner, cnt, dig, tau, file_base_d,
-                                          n_files, (uint4*)m->slots, (uint2*)m->postings, counters + 2);
-        CV_CUDA(cudaGetLastError());
-        if (sig_is_weak(sig)) {
-          // a copy of the kept master units in posting order, to confirm matches byte for byte
-          CV_CUDA(cudaMalloc(&m->confirm, M * U));
-          gather_units_kernel<<<grid_for(M * (U / 16), 256, ctx->sms), 256, 0, stream>>>(
-              (const uint4*)arena, kin, vin, M, (uint32_t)n_slots, (uint32_t)(U / 16), (uint4*)m->confirm);
-          CV_CUDA(cudaGetLastError());
-        }
-        if (frag) {
-          CV_CUDA((cudaError_t)frag_bloom(sig, (const uint4*)m->slots, (uint32_t)n_slots, (uint32_t*)m->bloom,
-                                          bpk ? (uint32_t)(n_blocks - 1) : 0u, (uint32_t*)m->frag_l1, ctx->sms,
-                                          stream));
-        } else if (bpk) {
-          bloom_kernel<<<grid_for(n_slots, 256, ctx->sms), 256, 0, stream>>>((const uint4*)m->slots,
-                                                                             (uint32_t)n_slots, (uint32_t*)m->bloom,
-                                                                             (uint32_t)(n_blocks - 1));
+      }
+      // also when there is no master unit: it clears the slots
+      slot_sums_kernel<<<chunks, kSlotThreads, 0, stream>>>((const uint64_t*)words, (uint32_t)n_slots, first);
+      CV_CUDA(cudaGetLastError());
+      CV_TRY(scan_u32(first, chunks, sums, stream));
+      table_slots_kernel<<<chunks, kSlotThreads, 0, stream>>>(
+          (const uint64_t*)words, (uint32_t)n_slots, first, dig, tau, post, (uint4*)m->slots, (uint2*)m->postings,
+          member, frag ? nullptr : (uint32_t*)m->bloom, bpk ? (uint32_t)(n_blocks - 1) : 0u, counters + 2);
+      CV_CUDA(cudaGetLastError());
+      if (M && frag)
+        CV_CUDA((cudaError_t)frag_bloom(sig, (const uint4*)m->slots, (uint32_t)n_slots, (uint32_t*)m->bloom,
+                                        bpk ? (uint32_t)(n_blocks - 1) : 0u, (uint32_t*)m->frag_l1, ctx->sms, stream));
+      uint32_t hc[5];
+      CV_CUDA(cudaMemcpyAsync(hc, counters, 20, cudaMemcpyDeviceToHost, stream));
+      CV_CUDA(cudaStreamSynchronize(stream));
+      if (hc[4] & kStTableFull) return CV_ETABLEFULL;
+      if (hc[4] & kStTimeout) return CV_ETIMEOUT;
+      if (hc[4]) return CV_ECORRUPT;
+      if (hc[3]) CV_TRY(several_members(ctx, slot_of, M, n_slots, (const uint64_t*)words, (const uint4*)m->slots, hc[3], hc[1], post,
+                                        (uint2*)m->postings, member, tmp, stream));
+      if (M && sig_is_weak(sig)) {
+        // a copy of the kept master units in posting order, to confirm matches byte for byte
+        CV_CUDA(cudaMalloc(&m->confirm, M * U));
+        if (hc[1]) {
+          gather_units_kernel<<<grid_for(hc[1] * (U / 16), 256, ctx->sms), 256, 0, stream>>>(
+              (const uint4*)arena, member, hc[1], (uint32_t)(U / 16), (uint4*)m->confirm);
           CV_CUDA(cudaGetLastError());
         }
       }
-      uint32_t hc[4];
-      CV_CUDA(cudaMemcpyAsync(hc, counters, 16, cudaMemcpyDeviceToHost, stream));
-      CV_CUDA(cudaStreamSynchronize(stream));
-      if (hc[3] & kStTableFull) return CV_ETABLEFULL;
-      if (hc[3] & kStTimeout) return CV_ETIMEOUT;
-      if (hc[3]) return CV_ECORRUPT;
       if (layout == CV_LAYOUT_AUTO)  // thresholds from the occupancy sweep (Bloom on / off)
         layout = (double)hc[2] > (bpk ? 0.8 : 0.5) * (double)n_slots ? CV_LAYOUT_SORTED : CV_LAYOUT_HASH;
       uint32_t steps = 0;  // binary-search steps of the sorted layout

@@ -3,14 +3,16 @@
 // linear probing, Eq. 3).
 //
 // Steps (one launch each):
+//   postings the (file_id, file_sector) of every master sector, in master order.
 //   insert   one thread per master sector: claim the first free slot from the digest's home
-//            slot on (atomicCAS of an owner word), or join the slot that already holds an
-//            equal digest; record the slot, count its members, track the longest probe run.
-//   sort     stable LSD radix sort of (slot, master index) pairs by slot, so every slot's
-//            members end up contiguous and in master order, i.e. by (file_id, file_sector).
-//   fill     the sorted pairs become the postings; the first pair of each run writes its
-//            slot {digest, post_off, post_cnt}.
-//   bloom    every occupied slot sets its 8 bits in the blocked Bloom filter.
+//            slot on (atomicCAS of a word holding the owner and the member count), or join the
+//            slot that already holds an equal digest; record the slot, track the longest probe run.
+//   slots    an exclusive scan of the member counts gives every key its postings; one pass over the
+//            slots writes their records, the postings of keys with one member and the Bloom
+//            filter's bits.
+//   members  (only for keys with several members) these members, in master order, are sorted by
+//            their key's first posting (stable LSD radix sort) and take the postings from there
+//            on, so they are in master order, i.e. by (file_id, file_sector).
 //   sorted   (sorted layout only) the occupied slots, compacted in slot order, are sorted by
 //            h0 and become the searched array.
 // Position-keyed tables (one S_tau per cluster position, Section 3.1) key every slot by
@@ -23,24 +25,47 @@
 
 namespace cvk {
 
-// Position of every master sector in its file's clusters: tau[m] = file_sector mod 8, the
-// file found by binary search of file_base (n_files + 1 entries: first master index of every
-// file, then the total).
-__global__ void tau_kernel(const uint64_t* file_base, uint32_t n_files, uint64_t n, uint8_t* tau) {
-  for (uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; m < n; m += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t lo = 0, hi = n_files;  // largest f with file_base[f] <= m
-    while (hi - lo > 1) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (file_base[mid] <= m) lo = mid; else hi = mid;
+// Posting of every master sector: its file, by binary search of file_base (n_files + 1 entries:
+// first master index of every file, then the total), and its sector in the file. With tau (position-
+// keyed tables), tau[m] = file_sector mod 8.
+// A warp takes kPostRun consecutive sectors: two searches over all files for its first and last one,
+// then short ones between them.
+constexpr uint32_t kPostRun = 512;
+
+__device__ __forceinline__ uint32_t file_of(const uint64_t* file_base, uint32_t lo, uint32_t hi, uint64_t m) {
+  while (hi - lo > 1) {  // largest f in [lo, hi) with file_base[f] <= m
+    const uint32_t mid = (lo + hi) >> 1;
+    if (file_base[mid] <= m) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+__global__ void unit_postings_kernel(const uint64_t* file_base, uint32_t n_files, uint64_t n, uint2* post,
+                                     uint8_t* tau) {
+  const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+  for (uint64_t m0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kPostRun; m0 < n;
+       m0 += warps * kPostRun) {
+    const uint64_t end = m0 + kPostRun < n ? m0 + kPostRun : n;
+    const uint32_t f0 = file_of(file_base, 0, n_files, m0), f1 = file_of(file_base, f0, n_files, end - 1) + 1;
+    for (uint64_t m = m0 + (threadIdx.x & 31); m < end; m += 32) {
+      const uint32_t f = file_of(file_base, f0, f1, m);
+      const uint32_t s = (uint32_t)(m - file_base[f]);
+      post[m] = make_uint2(f, s);
+      if (tau) tau[m] = (uint8_t)(s & 7u);
     }
-    tau[m] = (uint8_t)((m - file_base[lo]) & 7u);
   }
 }
 
+// A slot while the table is built: the master index of its key's first member + 1 (0: empty) in the
+// low word, the number of members in the high word.
+__host__ __device__ inline uint32_t build_owner(uint64_t w) { return (uint32_t)w; }
+__host__ __device__ inline uint32_t build_count(uint64_t w) { return (uint32_t)(w >> 32); }
+
 // tau: per master sector position (position-keyed tables), or null for one table over all
-// positions (every tau 0). The key is (digest, tau).
+// positions (every tau 0). The key is (digest, tau). One atomic per key and slot looked at: the
+// claim also counts the first member.
 __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const uint8_t* tau, uint64_t n,
-                              uint32_t* owner, uint32_t* cnt, uint32_t* slot_of, uint32_t mask, uint32_t* max_disp,
+                              unsigned long long* words, uint32_t* slot_of, uint32_t mask, uint32_t* max_disp,
                               uint32_t* n_kept, uint32_t* status) {
   const uint32_t none = mask + 1u;
   uint32_t kept = 0, longest = 0;  // this thread's, added to the shared counters once per warp
@@ -55,7 +80,7 @@ __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const ui
     uint32_t c = 0;
     bool placed = false;
     for (; c <= mask; c++) {
-      const uint32_t prev = atomicCAS(owner + idx, 0u, (uint32_t)m + 1u);
+      const uint32_t prev = build_owner(atomicCAS(words + idx, 0ull, (1ull << 32) | ((uint32_t)m + 1u)));
       if (prev == 0u) {
         placed = true;
         break;
@@ -63,6 +88,7 @@ __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const ui
       const uint4 e = dig[prev - 1u];
       const uint32_t te = tau ? tau[prev - 1u] : 0u;
       if (e.x == d.x && e.y == d.y && e.z == d.z && e.w == d.w && te == t) {
+        atomicAdd(words + idx, 1ull << 32);
         placed = true;
         break;
       }
@@ -74,7 +100,6 @@ __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const ui
       continue;
     }
     slot_of[m] = idx;
-    atomicAdd(cnt + idx, 1u);
     longest = c > longest ? c : longest;
     kept++;
   }
@@ -85,11 +110,6 @@ __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const ui
     atomicAdd(n_kept, kept);
     atomicMax(max_disp, longest);
   }
-}
-
-__global__ void iota_kernel(uint32_t* v, uint64_t n) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-    v[i] = (uint32_t)i;
 }
 
 // ------------------------------------------------------------------ stable radix sort pass
@@ -252,46 +272,171 @@ __global__ void __launch_bounds__(kRsThreads) rs_scatter_kernel(const uint32_t* 
   }
 }
 
-// ------------------------------------------------------------------------------ fill
-// Sorted (slot, master index) pairs -> postings and slot records. file_base has n_files + 1
-// entries: the first master index of every file, then the total.
-__global__ void fill_kernel(const uint32_t* keys, const uint32_t* vals, uint64_t n, uint32_t n_slots,
-                            const uint32_t* owner, const uint32_t* cnt, const uint4* dig, const uint8_t* tau,
-                            const uint64_t* file_base, uint32_t n_files, uint4* slots, uint2* postings,
-                            uint32_t* n_unique) {
-  uint32_t uniq = 0;
-  for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t key = keys[q];
-    if (key >= n_slots) continue;
-    const uint32_t m = vals[q];
-    uint32_t lo = 0, hi = n_files;  // largest f with file_base[f] <= m
-    while (hi - lo > 1) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (file_base[mid] <= m) lo = mid; else hi = mid;
-    }
-    postings[q] = make_uint2(lo, (uint32_t)(m - file_base[lo]));
-    if (q == 0 || keys[q - 1] != key) {
-      const uint32_t o = owner[key] - 1u;
-      slots[2ull * key] = dig[o];
-      slots[2ull * key + 1] = make_uint4((uint32_t)q, cnt[key], tau ? (uint32_t)tau[o] : 0u, 0u);
-      uniq++;
-    }
+// ------------------------------------------------------------------------------ slots
+// The slots in chunks of kSlotChunk, a block each; a warp has 128 consecutive slots, in four rows of
+// 32. first[c] holds the members of the chunks before chunk c: the chunks' sums, read in a pass of
+// their own (8 bytes a slot) and scanned. With decoupled look-back instead, in one pass, the kernel took
+// 400 us for the same table: some 300 chunks are under way at a time, none of them with an
+// inclusive prefix yet, and each walked back over all of them.
+//
+// Bound by memory: 8 bytes read and 32 written per slot (4,194,304 keys in 2^24 slots: 671 MB),
+// two random sectors read per key, a Bloom block updated per key. A slot record is one 32-byte store.
+// Of a key's eight Bloom bits eight lanes each set one, so that the block is one update in L2. This
+// and the sums take 245 us, where sorting (slot, master) pairs, filling postings and slots, a pass
+// for the Bloom filter and clearing the slots and counts took 804.
+constexpr int kSlotThreads = 256;
+constexpr int kSlotRows = 4;
+constexpr uint32_t kSlotChunk = kSlotThreads * kSlotRows;
+
+// sums[c] = members of the keys in chunk c.
+__global__ void __launch_bounds__(kSlotThreads) slot_sums_kernel(const uint64_t* words, uint32_t n_slots,
+                                                                 uint32_t* sums) {
+  const uint64_t base = (uint64_t)blockIdx.x * kSlotChunk + threadIdx.x;
+  uint32_t s = 0;
+#pragma unroll
+  for (int k = 0; k < kSlotRows; k++) {
+    const uint64_t i = base + (uint64_t)k * kSlotThreads;
+    if (i < n_slots) s += build_count(words[i]);
   }
-  uniq = __reduce_add_sync(0xFFFFFFFFu, uniq);
-  if ((threadIdx.x & 31) == 0 && uniq) atomicAdd(n_unique, uniq);
+  uint32_t total;
+  block_exclusive_u32<kSlotThreads>(s, &total);
+  if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-// Kept master units (sectors or fragments of wpu 16-byte words) in posting order: posting q
-// (sorted pair q, key < n_slots) is master unit vals[q]; its words go to out + wpu q. One thread
-// per 16-byte word.
-__global__ void gather_units_kernel(const uint4* arena, const uint32_t* keys, const uint32_t* vals, uint64_t n,
-                                    uint32_t n_slots, uint32_t wpu, uint4* out) {
-  const uint64_t words = n * wpu;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t q = i / wpu;
-    if (keys[q] >= n_slots) continue;
-    out[i] = arena[(uint64_t)vals[q] * wpu + i % wpu];
+__device__ __forceinline__ void store_slot(uint4* p, uint4 a, uint4 b) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+               "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+               : "memory");
+}
+
+// counters: [0] keys, [1] members of keys with several. post: posting per master index; member: the
+// master index of every posting (null: not wanted). bloom: null for none.
+__global__ void __launch_bounds__(kSlotThreads) table_slots_kernel(
+    const uint64_t* words, uint32_t n_slots, const uint32_t* first, const uint4* dig, const uint8_t* tau,
+    const uint2* post, uint4* slots, uint2* postings, uint32_t* member, uint32_t* bloom, uint32_t bloom_mask,
+    uint32_t* counters) {
+  constexpr int kWarps = kSlotThreads / 32;
+  constexpr uint32_t kFull = 0xFFFFFFFFu;
+  __shared__ uint32_t s_warp[kWarps];
+  __shared__ uint32_t s_key[kWarps][32 * kSlotRows][3];  // d1, d2, Bloom block of the warp's keys
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint64_t base = (uint64_t)blockIdx.x * kSlotChunk + warp * 32u * kSlotRows + lane;
+  uint32_t owner[kSlotRows], cnt[kSlotRows], before[kSlotRows], t[kSlotRows];
+  uint4 d[kSlotRows];
+  uint2 po[kSlotRows];
+#pragma unroll
+  for (int k = 0; k < kSlotRows; k++) {
+    const uint64_t w = base + 32u * k < n_slots ? words[base + 32u * k] : 0ull;
+    owner[k] = build_owner(w);
+    cnt[k] = build_count(w);
   }
+#pragma unroll
+  for (int k = 0; k < kSlotRows; k++) {
+    d[k] = owner[k] ? dig[owner[k] - 1u] : make_uint4(0, 0, 0, 0);
+    po[k] = owner[k] ? post[owner[k] - 1u] : make_uint2(0, 0);
+    t[k] = owner[k] && tau ? tau[owner[k] - 1u] : 0u;
+  }
+  // exclusive scan of the counts within the warp's slots, then over the warps
+  uint32_t sum = 0, keys = 0, several = 0;
+#pragma unroll
+  for (int k = 0; k < kSlotRows; k++) {
+    uint32_t incl = cnt[k];
+#pragma unroll
+    for (int q = 1; q < 32; q <<= 1) {
+      const uint32_t v = __shfl_up_sync(kFull, incl, q);
+      if (lane >= (uint32_t)q) incl += v;
+    }
+    before[k] = sum + incl - cnt[k];
+    sum += __shfl_sync(kFull, incl, 31);
+    several += cnt[k] > 1u ? cnt[k] : 0u;
+  }
+  if (lane == 0) s_warp[warp] = sum;
+  __syncthreads();
+  uint32_t off0 = first[blockIdx.x];
+  for (uint32_t w = 0; w < warp; w++) off0 += s_warp[w];
+#pragma unroll
+  for (int k = 0; k < kSlotRows; k++) {
+    const uint64_t i = base + 32u * k;
+    const uint32_t off = off0 + before[k];
+    const uint32_t has = __ballot_sync(kFull, owner[k] != 0u);
+    if (i < n_slots) store_slot(slots + 2 * i, d[k], make_uint4(owner[k] ? off : 0u, cnt[k], t[k], 0u));
+    if (cnt[k] == 1u) {
+      postings[off] = po[k];
+      if (member) member[off] = owner[k] - 1u;
+    }
+    if (bloom && owner[k]) {
+      uint32_t* e = s_key[warp][keys + __popc(has & ((1u << lane) - 1u))];
+      e[0] = d[k].y;
+      e[1] = d[k].z;
+      e[2] = tau_block(d[k].w, t[k]) & bloom_mask;
+    }
+    keys += __popc(has);
+  }
+  if (bloom) {
+    __syncwarp();
+    const uint32_t word = lane & 7u;  // the Bloom bit in word j: d1 >> 5j for j < 6, d2 >> 5(j - 6) else
+    for (uint32_t e = lane >> 3; e < keys; e += 4) {
+      const uint32_t* key = s_key[warp][e];
+      const uint32_t b = word < 6u ? key[0] >> (5u * word) : key[1] >> (5u * (word - 6u));
+      atomicOr(bloom + 8ull * key[2] + word, 1u << (b & 31u));
+    }
+  }
+  several = __reduce_add_sync(kFull, several);
+  __shared__ uint32_t s_keys, s_several;
+  if (threadIdx.x == 0) s_keys = s_several = 0;
+  __syncthreads();
+  if (lane == 0 && keys) {
+    atomicAdd(&s_keys, keys);
+    if (several) atomicAdd(&s_several, several);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && s_keys) {  // one update per block
+    atomicAdd(counters, s_keys);
+    if (s_several) atomicAdd(counters + 1, s_several);
+  }
+}
+
+// ---------------------------------------------------------------------------- members
+// 1 for every master unit whose key has several members, else 0.
+__global__ void several_flags_kernel(const uint32_t* slot_of, uint64_t n, uint32_t n_slots, const uint64_t* words,
+                                     uint32_t* flags) {
+  for (uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; m < n; m += (uint64_t)gridDim.x * blockDim.x)
+    flags[m] = slot_of[m] < n_slots && build_count(words[slot_of[m]]) > 1u ? 1u : 0u;
+}
+
+// These units in master order (at: the exclusive scan of the flags), keyed by their key's first posting.
+__global__ void several_keys_kernel(const uint32_t* slot_of, uint64_t n, uint32_t n_slots, const uint4* slots,
+                                    const uint32_t* at, uint32_t* keys, uint32_t* vals) {
+  for (uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; m < n; m += (uint64_t)gridDim.x * blockDim.x) {
+    if (slot_of[m] >= n_slots) continue;
+    const uint4 val = slots[2ull * slot_of[m] + 1];
+    if (val.y <= 1u) continue;
+    keys[at[m]] = val.x;
+    vals[at[m]] = (uint32_t)m;
+  }
+}
+
+// Sorted by key: the members of a key take its postings in this order.
+__global__ void several_postings_kernel(const uint32_t* keys, const uint32_t* vals, uint32_t n, const uint2* post,
+                                        uint2* postings, uint32_t* member) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t key = keys[i];
+    uint32_t lo = 0, hi = i;  // the key's first place
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (keys[mid] < key) lo = mid + 1; else hi = mid;
+    }
+    postings[key + i - lo] = post[vals[i]];
+    if (member) member[key + i - lo] = vals[i];
+  }
+}
+
+// Kept master units (sectors or fragments of wpu 16-byte words) in posting order: posting q is
+// master unit member[q]; its words go to out + wpu q. One thread per 16-byte word.
+__global__ void gather_units_kernel(const uint4* arena, const uint32_t* member, uint64_t n, uint32_t wpu, uint4* out) {
+  const uint64_t words = n * wpu;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x)
+    out[i] = arena[(uint64_t)member[i / wpu] * wpu + i % wpu];
 }
 
 // ------------------------------------------------------------------- sorted layout

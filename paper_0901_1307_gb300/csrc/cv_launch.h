@@ -34,8 +34,9 @@ inline int table_kind(const TableView& t) { return (int)t.sig + 4 * (int)t.layou
 const ScanCfg& scan_config_for(int cfg_i, int kind, int* used);
 // The default scan configuration for a table kind and a number of sectors (the fastest measured).
 int preferred_config(int kind, uint64_t sectors, int sms);
-// Configuration cfg_i if it has a digest-mode kernel for signature sig, else the default one.
-const ScanCfg& digest_config_for(int cfg_i, int sig, int* used);
+// Configuration cfg_i (-1: the preferred one for the signature and the sectors) if it has a
+// digest-mode kernel for signature sig, else the first one.
+const ScanCfg& digest_config_for(int cfg_i, int sig, uint64_t sectors, int sms, int* used);
 
 // The expand pass over n_out_tiles output tiles (see expand_kernel). Returns a CUDA error code.
 int launch_expand(const ScanCfg& cfg, const uint4* hit_rec, const uint32_t* tile_nhit, const uint64_t* tile_off,

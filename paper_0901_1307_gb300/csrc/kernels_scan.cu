@@ -135,7 +135,7 @@ __global__ void wait_timeout_selftest_kernel(uint32_t* status, uint64_t timeout_
 }
 
 
-// The configurations in table order. The first is the only one with digest-mode kernels; every one has scan
+// The configurations in table order. The first and the 128-byte-stage one have digest-mode kernels; every one has scan
 // kernels for all eight table kinds (four signatures x two layouts), so the batch autotuner can
 // pick any of them for any table. The kernels are instantiated in scan_cfgs_{a,b,c}.cu, which
 // compile in parallel.
@@ -195,10 +195,11 @@ int preferred_config(int kind, uint64_t sectors, int sms) {
   return sig == kSigMd5NoPad && sectors >= (1ull << 21) ? picks.nopad : picks.light;
 }
 
-const ScanCfg& digest_config_for(int cfg_i, int sig, int* used) {
+const ScanCfg& digest_config_for(int cfg_i, int sig, uint64_t sectors, int sms, int* used) {
   int n;
   const ScanCfg* c = scan_configs(&n);
-  if (cfg_i < 0 || cfg_i >= n || sig < 0 || sig > kSigCrc64 || !c[cfg_i].digest_fn[sig]) cfg_i = 0;
+  if (cfg_i < 0) cfg_i = preferred_config(sig, sectors, sms);
+  if (cfg_i >= n || sig < 0 || sig > kSigCrc64 || !c[cfg_i].digest_fn[sig]) cfg_i = 0;
   if (used) *used = cfg_i;
   return c[cfg_i];
 }

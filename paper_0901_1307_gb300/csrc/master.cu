@@ -57,7 +57,7 @@ int radix_sort_pairs(uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uin
 }
 
 // The postings of keys with several members (n_several members in all): in master order within a key.
-int several_members(DevCtx* ctx, const uint32_t* slot_of, uint64_t M, uint64_t n_slots, const uint64_t* words,
+int several_members(DevCtx* ctx, const uint32_t* slot_of, uint64_t M, uint64_t n_slots, const uint32_t* extra,
                     const uint4* slots, uint32_t n_several, uint32_t n_kept, const uint2* post, uint2* postings,
                     uint32_t* member, Temps& tmp, cudaStream_t stream) {
   uint32_t *at, *sums, *k0, *v0, *k1, *v1, *kr, *vr;
@@ -65,7 +65,7 @@ int several_members(DevCtx* ctx, const uint32_t* slot_of, uint64_t M, uint64_t n
   CV_TRY(tmp.alloc(&sums, (M + kScanChunk - 1) / kScanChunk * 4));
   for (uint32_t** q : {&k0, &v0, &k1, &v1}) CV_TRY(tmp.alloc(q, (uint64_t)n_several * 4));
   const unsigned g = grid_for(M, 256, ctx->sms), gs = grid_for(n_several, 256, ctx->sms);
-  several_flags_kernel<<<g, 256, 0, stream>>>(slot_of, M, (uint32_t)n_slots, words, at);
+  several_flags_kernel<<<g, 256, 0, stream>>>(slot_of, M, (uint32_t)n_slots, extra, at);
   CV_CUDA(cudaGetLastError());
   CV_TRY(scan_u32(at, M, sums, stream));
   several_keys_kernel<<<g, 256, 0, stream>>>(slot_of, M, (uint32_t)n_slots, slots, at, k0, v0);
@@ -322,9 +322,6 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
   cudaStream_t stream = opts ? (cudaStream_t)opts->stream : nullptr;
   DevCtx* ctx;
   CV_TRY(get_ctx(&ctx));
-  int cfg_i;
-  const ScanCfg& cfg = digest_config_for(ctx->cfg_index, sig, &cfg_i);
-
   // whole units (sectors or fragments) of every file, concatenated
   std::vector<uint64_t> file_base(n_files + 1, 0);
   for (uint32_t f = 0; f < n_files; f++) {
@@ -333,6 +330,8 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
   }
   const uint64_t M = file_base[n_files];
   if (M >= (1ull << 27)) return CV_EINVAL;
+  int cfg_i;
+  const ScanCfg& cfg = digest_config_for(ctx->cfg_index, sig, M, ctx->sms, &cfg_i);
 
   cv_master* m = (cv_master*)calloc(1, sizeof(cv_master));
   if (!m) return CV_ENOMEM;
@@ -350,13 +349,14 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       uint8_t* trivial;
       uint32_t *slot_of, *counters, *member = nullptr;
       uint32_t *first, *sums;
-      unsigned long long* words;
+      uint32_t *owner, *extra;
       uint2* post;
       const uint32_t chunks = (uint32_t)((n_slots + kSlotChunk - 1) / kSlotChunk);
       uint64_t* file_base_d;
       CV_TRY(tmp.alloc(&dig, M * sizeof(uint4)));
       CV_TRY(tmp.alloc(&trivial, M));
-      CV_TRY(tmp.alloc(&words, n_slots * 8));
+      CV_TRY(tmp.alloc(&owner, n_slots * 8));  // and extra
+      extra = owner + n_slots;
       CV_TRY(tmp.alloc(&first, chunks * 4ull));
       CV_TRY(tmp.alloc(&sums, (chunks / kScanChunk + 1) * 4ull));
       CV_TRY(tmp.alloc(&slot_of, M * 4));
@@ -366,7 +366,7 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       CV_TRY(tmp.alloc(&file_base_d, (n_files + 1) * 8));
       uint8_t* tau = nullptr;  // per master sector cluster position (position-keyed tables)
       if (by_tau) CV_TRY(tmp.alloc(&tau, std::max<uint64_t>(M, 1)));
-      CV_CUDA(cudaMemsetAsync(words, 0, n_slots * 8, stream));
+      CV_CUDA(cudaMemsetAsync(owner, 0, n_slots * 8, stream));
       CV_CUDA(cudaMemsetAsync(counters, 0, 32, stream));
       CV_CUDA(cudaMemcpyAsync(file_base_d, file_base.data(), (n_files + 1) * 8, cudaMemcpyHostToDevice, stream));
       CV_TRY(gather_master_units(ctx, files, n_files, file_base, U, tmp, stream, &arena));
@@ -399,17 +399,17 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
         unit_postings_kernel<<<grid_for((M + kPostRun - 1) / kPostRun * 32, 256, ctx->sms), 256, 0, stream>>>(
             file_base_d, n_files, M, post, tau);
         CV_CUDA(cudaGetLastError());
-        insert_kernel<<<g, 256, 0, stream>>>(dig, trivial, tau, M, words, slot_of, mask, counters, counters + 1,
+        insert_kernel<<<g, 256, 0, stream>>>(dig, trivial, tau, M, owner, extra, slot_of, mask, counters, counters + 1,
                                             counters + 4);
         CV_CUDA(cudaGetLastError());
       }
       // also when there is no master unit: it clears the slots
-      slot_sums_kernel<<<chunks, kSlotThreads, 0, stream>>>((const uint64_t*)words, (uint32_t)n_slots, first);
+      slot_sums_kernel<<<chunks, kSlotThreads, 0, stream>>>(owner, extra, (uint32_t)n_slots, first);
       CV_CUDA(cudaGetLastError());
       CV_TRY(scan_u32(first, chunks, sums, stream));
       table_slots_kernel<<<chunks, kSlotThreads, 0, stream>>>(
-          (const uint64_t*)words, (uint32_t)n_slots, first, dig, tau, post, (uint4*)m->slots, (uint2*)m->postings,
-          member, frag ? nullptr : (uint32_t*)m->bloom, bpk ? (uint32_t)(n_blocks - 1) : 0u, counters + 2);
+          owner, extra, (uint32_t)n_slots, first, dig, tau, post, (uint4*)m->slots, (uint2*)m->postings, member,
+          frag ? nullptr : (uint32_t*)m->bloom, bpk ? (uint32_t)(n_blocks - 1) : 0u, counters + 2);
       CV_CUDA(cudaGetLastError());
       if (M && frag)
         CV_CUDA((cudaError_t)frag_bloom(sig, (const uint4*)m->slots, (uint32_t)n_slots, (uint32_t*)m->bloom,
@@ -420,7 +420,7 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       if (hc[4] & kStTableFull) return CV_ETABLEFULL;
       if (hc[4] & kStTimeout) return CV_ETIMEOUT;
       if (hc[4]) return CV_ECORRUPT;
-      if (hc[3]) CV_TRY(several_members(ctx, slot_of, M, n_slots, (const uint64_t*)words, (const uint4*)m->slots, hc[3], hc[1], post,
+      if (hc[3]) CV_TRY(several_members(ctx, slot_of, M, n_slots, extra, (const uint4*)m->slots, hc[3], hc[1], post,
                                         (uint2*)m->postings, member, tmp, stream));
       if (M && sig_is_weak(sig)) {
         // a copy of the kept master units in posting order, to confirm matches byte for byte

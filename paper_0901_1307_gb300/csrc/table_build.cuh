@@ -5,8 +5,8 @@
 // Steps (one launch each):
 //   postings the (file_id, file_sector) of every master sector, in master order.
 //   insert   one thread per master sector: claim the first free slot from the digest's home
-//            slot on (atomicCAS of a word holding the owner and the member count), or join the
-//            slot that already holds an equal digest; record the slot, track the longest probe run.
+//            slot on (atomicCAS of its owner word), or join the slot that already holds an equal
+//            digest; record the slot, track the longest probe run.
 //   slots    an exclusive scan of the member counts gives every key its postings; one pass over the
 //            slots writes their records, the postings of keys with one member and the Bloom
 //            filter's bits.
@@ -56,16 +56,16 @@ __global__ void unit_postings_kernel(const uint64_t* file_base, uint32_t n_files
   }
 }
 
-// A slot while the table is built: the master index of its key's first member + 1 (0: empty) in the
-// low word, the number of members in the high word.
-__host__ __device__ inline uint32_t build_owner(uint64_t w) { return (uint32_t)w; }
-__host__ __device__ inline uint32_t build_count(uint64_t w) { return (uint32_t)(w >> 32); }
-
 // tau: per master sector position (position-keyed tables), or null for one table over all
-// positions (every tau 0). The key is (digest, tau). One atomic per key and slot looked at: the
-// claim also counts the first member.
+// positions (every tau 0). The key is (digest, tau). A slot's owner is the master index of its key's
+// first member + 1 (0: empty), its extra the number of other members. Bound by the random accesses:
+// 165 us for 4,194,304 keys while the owners (4 bytes a slot, 67 MB) stay in L2, against 248 us
+// with owner and count in one 8-byte word and 333 us with a second atomic that counts every member.
+// (Claiming slots from the kernel that hashes the sectors saved nothing: waited for at once, the
+// atomics held up the hashing by 220 us; looked at a tile later, by 100, and the keys whose home was
+// taken still took 153.)
 __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const uint8_t* tau, uint64_t n,
-                              unsigned long long* words, uint32_t* slot_of, uint32_t mask, uint32_t* max_disp,
+                              uint32_t* owner, uint32_t* extra, uint32_t* slot_of, uint32_t mask, uint32_t* max_disp,
                               uint32_t* n_kept, uint32_t* status) {
   const uint32_t none = mask + 1u;
   uint32_t kept = 0, longest = 0;  // this thread's, added to the shared counters once per warp
@@ -80,7 +80,7 @@ __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const ui
     uint32_t c = 0;
     bool placed = false;
     for (; c <= mask; c++) {
-      const uint32_t prev = build_owner(atomicCAS(words + idx, 0ull, (1ull << 32) | ((uint32_t)m + 1u)));
+      const uint32_t prev = atomicCAS(owner + idx, 0u, (uint32_t)m + 1u);
       if (prev == 0u) {
         placed = true;
         break;
@@ -88,7 +88,7 @@ __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const ui
       const uint4 e = dig[prev - 1u];
       const uint32_t te = tau ? tau[prev - 1u] : 0u;
       if (e.x == d.x && e.y == d.y && e.z == d.z && e.w == d.w && te == t) {
-        atomicAdd(words + idx, 1ull << 32);
+        atomicAdd(extra + idx, 1u);
         placed = true;
         break;
       }
@@ -289,14 +289,14 @@ constexpr int kSlotRows = 4;
 constexpr uint32_t kSlotChunk = kSlotThreads * kSlotRows;
 
 // sums[c] = members of the keys in chunk c.
-__global__ void __launch_bounds__(kSlotThreads) slot_sums_kernel(const uint64_t* words, uint32_t n_slots,
+__global__ void __launch_bounds__(kSlotThreads) slot_sums_kernel(const uint32_t* owner, const uint32_t* extra, uint32_t n_slots,
                                                                  uint32_t* sums) {
   const uint64_t base = (uint64_t)blockIdx.x * kSlotChunk + threadIdx.x;
   uint32_t s = 0;
 #pragma unroll
   for (int k = 0; k < kSlotRows; k++) {
     const uint64_t i = base + (uint64_t)k * kSlotThreads;
-    if (i < n_slots) s += build_count(words[i]);
+    if (i < n_slots) s += extra[i] + (owner[i] ? 1u : 0u);
   }
   uint32_t total;
   block_exclusive_u32<kSlotThreads>(s, &total);
@@ -312,7 +312,7 @@ __device__ __forceinline__ void store_slot(uint4* p, uint4 a, uint4 b) {
 // counters: [0] keys, [1] members of keys with several. post: posting per master index; member: the
 // master index of every posting (null: not wanted). bloom: null for none.
 __global__ void __launch_bounds__(kSlotThreads) table_slots_kernel(
-    const uint64_t* words, uint32_t n_slots, const uint32_t* first, const uint4* dig, const uint8_t* tau,
+    const uint32_t* owners, const uint32_t* extra, uint32_t n_slots, const uint32_t* first, const uint4* dig, const uint8_t* tau,
     const uint2* post, uint4* slots, uint2* postings, uint32_t* member, uint32_t* bloom, uint32_t bloom_mask,
     uint32_t* counters) {
   constexpr int kWarps = kSlotThreads / 32;
@@ -326,9 +326,9 @@ __global__ void __launch_bounds__(kSlotThreads) table_slots_kernel(
   uint2 po[kSlotRows];
 #pragma unroll
   for (int k = 0; k < kSlotRows; k++) {
-    const uint64_t w = base + 32u * k < n_slots ? words[base + 32u * k] : 0ull;
-    owner[k] = build_owner(w);
-    cnt[k] = build_count(w);
+    const bool in = base + 32u * k < n_slots;
+    owner[k] = in ? owners[base + 32u * k] : 0u;
+    cnt[k] = in ? extra[base + 32u * k] + (owner[k] ? 1u : 0u) : 0u;
   }
 #pragma unroll
   for (int k = 0; k < kSlotRows; k++) {
@@ -398,10 +398,10 @@ __global__ void __launch_bounds__(kSlotThreads) table_slots_kernel(
 
 // ---------------------------------------------------------------------------- members
 // 1 for every master unit whose key has several members, else 0.
-__global__ void several_flags_kernel(const uint32_t* slot_of, uint64_t n, uint32_t n_slots, const uint64_t* words,
+__global__ void several_flags_kernel(const uint32_t* slot_of, uint64_t n, uint32_t n_slots, const uint32_t* extra,
                                      uint32_t* flags) {
   for (uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; m < n; m += (uint64_t)gridDim.x * blockDim.x)
-    flags[m] = slot_of[m] < n_slots && build_count(words[slot_of[m]]) > 1u ? 1u : 0u;
+    flags[m] = slot_of[m] < n_slots && extra[slot_of[m]] > 0u ? 1u : 0u;
 }
 
 // These units in master order (at: the exclusive scan of the flags), keyed by their key's first posting.

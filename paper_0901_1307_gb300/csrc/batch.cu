@@ -23,6 +23,7 @@
 #include <string>
 #include <vector>
 
+#include "compact.cuh"
 #include "cv.h"
 #include "runtime.h"
 
@@ -94,13 +95,28 @@ int enqueue_run(DevCtx* ctx, int cfg_i, const TableView& tab, const Job& job, co
   if (ev0) CV_CUDA(cudaEventRecordWithFlags(ev0, stream, rec_flags));
   CV_TRY(launch_range(ctx, cfg_i, false, job, b.segs_d, 0, nseg, p, stream, launches));
   if (ev1) CV_CUDA(cudaEventRecordWithFlags(ev1, stream, rec_flags));
-  uint64_t* total_d = b.counters_d + nseg;
-  CV_CUDA((cudaError_t)launch_tile_offsets(b.tile_ntrip, n_out, b.tile_off, b.segs_d, (uint32_t)nseg,
-                                           (uint32_t)(cfg.T / 32), b.counters_d, total_d, b.off_scratch, stream,
-                                           status));
-  if (launches) *launches += 2;
-  CV_CUDA((cudaError_t)launch_expand(cfg, b.hit_rec, b.tile_nhit, b.tile_off, n_out, b.segs_d, (uint32_t)nseg, tab,
-                                     b.out_d, capacity, status, ctx->sms, stream));
+  CompactParams cp;
+  memset(&cp, 0, sizeof cp);
+  compact_table(&cp, tab);
+  cp.hit_rec = b.hit_rec;
+  cp.tile_nhit = b.tile_nhit;
+  cp.tile_ntrip = b.tile_ntrip;
+  cp.n_out_tiles = n_out;
+  cp.segs = seg_list(job.segs.data(), b.segs_d, nseg);
+  cp.out = b.out_d;
+  cp.out_cap = capacity;
+  cp.status = status;
+  cp.tile_off = b.tile_off;
+  cp.seg_off = b.counters_d;
+  cp.total = b.counters_d + nseg;
+  if (n_out <= kFinishTiles) {
+    CV_CUDA((cudaError_t)launch_finish(cfg, cp, ctx->sms, stream));
+  } else {
+    CV_CUDA((cudaError_t)launch_tile_offsets(b.tile_ntrip, n_out, b.tile_off, cp.segs, (uint32_t)(cfg.T / 32),
+                                             cp.seg_off, cp.total, b.off_scratch, stream, status));
+    if (launches) *launches += 2;
+    CV_CUDA((cudaError_t)launch_expand(cfg, cp, ctx->sms, stream));
+  }
   if (launches) *launches += 1;
   if (counters_h) CV_CUDA(cudaMemcpyAsync(counters_h, b.counters_d, (nseg + 2) * 8, cudaMemcpyDeviceToHost, stream));
   return CV_OK;

@@ -23,6 +23,7 @@
 
 #include "cv.h"
 #include "cv_internal.h"
+#include "compact.cuh"
 #include "cv_launch.h"
 #include "handles.h"
 #include "runtime.h"
@@ -91,8 +92,7 @@ const char* cv_kernel_config_name(int k) {
 int cvk::digest_job(DevCtx* ctx, int cfg_i, int sig, Job& job, uint4* digests, uint8_t* trivial, uint32_t* status,
                     cudaStream_t stream, Temps& tmp) {
   Segment* segs_d;
-  CV_TRY(tmp.alloc(&segs_d, job.segs.size() * sizeof(Segment)));
-  CV_CUDA(cudaMemcpyAsync(segs_d, job.segs.data(), job.segs.size() * sizeof(Segment), cudaMemcpyHostToDevice, stream));
+  CV_TRY(job.segs_device(&segs_d, tmp, stream));
   ScanParams p;
   memset(&p, 0, sizeof p);
   p.status = status;
@@ -232,7 +232,7 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       CV_CUDA(cudaEventRecord(ev[0], stream));
       uint64_t *tile_ntrip, *tile_off, *seg_off_d, *scratch;
       FragHits hits;
-      Segment* segs_d;
+      Segment* segs_d = nullptr;
       CV_TRY(tmp.alloc(&tile_ntrip, std::max<uint64_t>(T, 1) * 8));
       CV_TRY(tmp.alloc(&tile_off, std::max<uint64_t>(T, 1) * 8));
       // seg_off[n], total, status, rejected, listed tiles of every image
@@ -241,15 +241,16 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       CV_TRY(tmp.alloc(&hits.tiles, T * 4));
       hits.mask_tiles = std::min(T, kFragMaskTiles);
       CV_TRY(tmp.alloc(&hits.masks, hits.mask_tiles * 32 * 4));
-      CV_TRY(tmp.alloc(&segs_d, std::max<uint32_t>(n_images, 1) * sizeof(Segment)));
       std::vector<Segment> segs(n_images);
       memset(segs.data(), 0, segs.size() * sizeof(Segment));
       for (uint32_t i = 0; i < n_images; i++) {
         segs[i].tile_base = tile_base[i];
         segs[i].image = i;
       }
-      if (n_images)
+      if (n_images > kInlineSegs) {
+        CV_TRY(tmp.alloc(&segs_d, n_images * sizeof(Segment)));
         CV_CUDA(cudaMemcpyAsync(segs_d, segs.data(), n_images * sizeof(Segment), cudaMemcpyHostToDevice, stream));
+      }
       uint32_t* status = (uint32_t*)(seg_off_d + n_images + 1);
       unsigned long long* rejected = (unsigned long long*)(seg_off_d + n_images + 2);
       uint64_t* listed = seg_off_d + n_images + 3;
@@ -263,8 +264,8 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
         r->launches++;
       }
       CV_CUDA(cudaEventRecord(ev[2], stream));
-      CV_CUDA((cudaError_t)launch_tile_offsets(tile_ntrip, T, tile_off, segs_d, n_images, 1, seg_off_d,
-                                               seg_off_d + n_images, scratch, stream, status));
+      CV_CUDA((cudaError_t)launch_tile_offsets(tile_ntrip, T, tile_off, seg_list(segs.data(), segs_d, n_images), 1,
+                                               seg_off_d, seg_off_d + n_images, scratch, stream, status));
       r->launches += 2;
       std::vector<uint64_t> seg_off(n_images + 3, 0);
       CV_CUDA(cudaMemcpyAsync(seg_off.data(), seg_off_d, (n_images + 3) * 8, cudaMemcpyDeviceToHost, stream));
@@ -445,23 +446,25 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
         Segment* segs_d;
         uint4* hit_rec;
         uint32_t *tile_nhit, *status;
-        uint64_t *tile_ntrip, *tile_off, *seg_off_d, *off_scratch;
+        uint64_t *tile_ntrip, *tile_off = nullptr, *seg_off_d, *off_scratch = nullptr;
         // compaction works on output tiles of 32 sectors, T / 32 per scan tile
         const uint64_t n_out = nt * (uint64_t)(cfg.T / 32);
+        const bool small = n_out <= kFinishTiles;  // offsets and expansion in one launch
         Carve carve;
-        carve.add(&segs_d, nseg * sizeof(Segment));
         carve.add(&hit_rec, n_out * 32 * sizeof(uint4));
         carve.add(&tile_nhit, n_out * 4);
         carve.add(&tile_ntrip, n_out * 8);
-        carve.add(&tile_off, n_out * 8);
+        if (!small) {
+          carve.add(&tile_off, n_out * 8);
+          carve.add(&off_scratch, tile_offsets_scratch_words(n_out) * 8);
+        }
         // seg_off[nseg], total, status, hit sectors, rejected candidates
         carve.add(&seg_off_d, (nseg + 4) * 8);
-        carve.add(&off_scratch, tile_offsets_scratch_words(n_out) * 8);
         CV_TRY(carve.commit(tmp));
         status = (uint32_t*)(seg_off_d + nseg + 1);
         status_keep = status;
         CV_CUDA(cudaMemsetAsync(status, 0, 24, stream));
-        CV_CUDA(cudaMemcpyAsync(segs_d, job.segs.data(), nseg * sizeof(Segment), cudaMemcpyHostToDevice, stream));
+        CV_TRY(job.segs_device(&segs_d, tmp, stream));
         ScanParams p;
         memset(&p, 0, sizeof p);
         p.tab = tab;
@@ -498,26 +501,46 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
         CV_CUDA(cudaEventRecord(ev[2], stream));
         launches_range.end();
         NvtxRange offsets_range("cv.scan.offsets_expand");
-        uint64_t* total_d = seg_off_d + nseg;
-        uint32_t nseg32 = (uint32_t)nseg;
-        uint64_t nt_arg = n_out;
+        CompactParams cp;
+        memset(&cp, 0, sizeof cp);
+        compact_table(&cp, tab);
+        cp.hit_rec = hit_rec;
+        cp.tile_nhit = tile_nhit;
+        cp.tile_ntrip = tile_ntrip;
+        cp.n_out_tiles = n_out;
+        cp.segs = seg_list(job.segs.data(), segs_d, nseg);
+        cp.status = status;
+        cp.tile_off = tile_off;
+        cp.seg_off = seg_off_d;
+        cp.total = seg_off_d + nseg;
+        cp.nhit_sum = (unsigned long long*)(seg_off_d + nseg + 2);
+        auto expand = [&](uint64_t room) -> int {
+          CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, room * sizeof(MatchOut), ctx->pool, stream));
+          cp.out = r->dev_out;
+          cp.out_cap = room;
+          CV_CUDA((cudaError_t)(small ? launch_finish(cfg, cp, ctx->sms, stream)
+                                      : launch_expand(cfg, cp, ctx->sms, stream)));
+          r->launches += 1;
+          return CV_OK;
+        };
         // the offsets, and the sectors with a match summed in the same pass
-        CV_CUDA((cudaError_t)launch_tile_offsets(tile_ntrip, n_out, tile_off, segs_d, nseg32, (uint32_t)(cfg.T / 32),
-                                                 seg_off_d, total_d, off_scratch, stream, status, tile_nhit,
-                                                 seg_off_d + nseg + 2));
+        if (!small) {
+          CV_CUDA((cudaError_t)launch_tile_offsets(tile_ntrip, n_out, tile_off, cp.segs, (uint32_t)(cfg.T / 32),
+                                                   seg_off_d, cp.total, off_scratch, stream, status, tile_nhit,
+                                                   seg_off_d + nseg + 2));
+          r->launches += 2;
+        }
         // The expand pass needs an output buffer before the exact count is known on the host.
         // After a scan against the same table it is launched at once, with room for a quarter more
         // than that scan's matches (one wait for the whole call); the exact count then tells
         // whether the room sufficed (the pass writes nothing beyond it and flags the overflow),
-        // and only if not is it run again into an exact buffer.
+        // and only if not is it run again into an exact buffer. A small scan, whose offsets come
+        // from the same launch, has room for 4,096 matches at least.
         const uint64_t hint = __atomic_load_n(&const_cast<cv_master*>(m)->last_matches, __ATOMIC_RELAXED);
         uint64_t room = 0;
-        if (hint) {
-          room = hint + hint / 4 + 1024;
-          CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, room * sizeof(MatchOut), ctx->pool, stream));
-          CV_CUDA((cudaError_t)launch_expand(cfg, hit_rec, tile_nhit, tile_off, n_out, segs_d, nseg32, tab,
-                                             r->dev_out, room, status, ctx->sms, stream));
-          r->launches += 1;
+        if (hint || small) {
+          room = std::max<uint64_t>(hint + hint / 4 + 1024, small ? 4096 : 0);
+          CV_TRY(expand(room));
         }
         CV_CUDA(cudaMemcpyAsync(seg_off.data(), seg_off_d, (nseg + 4) * 8, cudaMemcpyDeviceToHost, stream));
         // the call's end unless more work follows (then recorded again after it): in the common
@@ -537,17 +560,14 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
             r->dev_out = nullptr;
           }
           CV_CUDA(cudaMemsetAsync(status, 0, 4, stream));
-          CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, total * sizeof(MatchOut), ctx->pool, stream));
-          CV_CUDA((cudaError_t)launch_expand(cfg, hit_rec, tile_nhit, tile_off, n_out, segs_d, nseg32, tab,
-                                             r->dev_out, total, status, ctx->sms, stream));
-          r->launches += 1;
+          cp.nhit_sum = nullptr;  // counted already
+          CV_TRY(expand(total));
         } else if (r->dev_out && !total) {
           CV_CUDA(cudaFreeAsync(r->dev_out, stream));
           r->dev_out = nullptr;
         } else {
           expanded_early = true;
         }
-        r->launches += 2;  // the offset pass
       }
       // per-image ranges; an image without sectors gets an empty range
       r->off[n_images] = total;

@@ -29,6 +29,25 @@ struct Segment {
   const uint8_t* bytes;  // device address of the segment's first sector (byte confirmation)
 };
 
+// A launch's segments, sorted by tile_base: up to kInlineSegs of them travel in the kernel's
+// parameters, so that scans of a few images copy no segment list to the device.
+constexpr uint32_t kInlineSegs = 4;
+struct SegList {
+  const Segment* dev;  // device memory; not used (may be null) when n <= kInlineSegs
+  uint32_t n;
+  uint32_t pad;
+  Segment in[kInlineSegs];
+  __host__ __device__ const Segment* get() const { return n <= kInlineSegs ? in : dev; }
+};
+inline SegList seg_list(const Segment* host, const Segment* dev, size_t n) {
+  SegList l;
+  l.dev = dev;
+  l.n = (uint32_t)n;
+  l.pad = 0;
+  for (size_t k = 0; k < kInlineSegs; k++) l.in[k] = n <= kInlineSegs && k < n ? host[k] : Segment{};
+  return l;
+}
+
 // Signature kinds (the values of CV_SIG_*).
 enum : int { kSigMd5 = 0, kSigMd5NoPad = 1, kSigDjb2 = 2, kSigCrc64 = 3 };
 
@@ -131,11 +150,9 @@ constexpr int kMapsPerLaunch = 64;
 // placed side by side in one device allocation).
 struct ScanParams {
   CUtensorMap maps[kMapsPerLaunch];  // the job's maps [map_base, map_base + kMapsPerLaunch)
-  const Segment* segs;               // device: this launch's segments, sorted by tile_base
-  uint32_t n_segs;
+  SegList segs;                      // this launch's segments
   uint32_t map_base;
   uint32_t one;         // always 1 (an opaque multiplier for the MD5 additions)
-  uint32_t pad;
   uint64_t tile_begin;  // global index of the first tile of this launch
   uint64_t n_tiles;     // tiles of this launch
   TableView tab;

@@ -16,6 +16,7 @@ struct ScanCfg {
   const void* scan_fn[8];    // scan_kernel per table kind (table_kind); null: not built for it
   const void* digest_fn[4];  // digest mode, per signature (kSig*)
   const void* expand_fn;     // expand_kernel<T>
+  const void* finish_fn;     // finish_kernel<T>
   uint32_t smem;             // dynamic shared memory bytes
 };
 
@@ -38,11 +39,13 @@ int preferred_config(int kind, uint64_t sectors, int sms);
 // digest-mode kernel for signature sig, else the first one.
 const ScanCfg& digest_config_for(int cfg_i, int sig, uint64_t sectors, int sms, int* used);
 
-// The expand pass over n_out_tiles output tiles (see expand_kernel). Returns a CUDA error code.
-int launch_expand(const ScanCfg& cfg, const uint4* hit_rec, const uint32_t* tile_nhit, const uint64_t* tile_off,
-                  uint64_t n_out_tiles, const Segment* segs, uint32_t n_segs, const TableView& tab, MatchOut* out,
-                  uint64_t out_cap, uint32_t* status, int sms, void* stream);
-
+// The expand pass (see expand_kernel). Returns a CUDA error code.
+struct CompactParams;
+int launch_expand(const ScanCfg& cfg, const CompactParams& p, int sms, void* stream);
+// Offsets and expansion in one launch, for at most kFinishTiles output tiles (see finish_kernel).
+int launch_finish(const ScanCfg& cfg, const CompactParams& p, int sms, void* stream);
+// The tables' side of CompactParams.
+void compact_table(CompactParams* p, const TableView& tab);
 
 // Scratch (u64 words) the offset pass needs for n tiles.
 uint64_t tile_offsets_scratch_words(uint64_t n_tiles);
@@ -52,10 +55,9 @@ uint64_t tile_offsets_scratch_words(uint64_t n_tiles);
 // tile_offsets_scratch_words(n_tiles) u64 words. status: the scan's status word (kStTimeout if
 // a wait of the pass gives up). With tile_nhit, the sum of the n_tiles hit counts is added to
 // *nhit_sum (device memory, zeroed by the caller). Returns a CUDA error code.
-int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* tile_off, const Segment* segs,
-                        uint32_t n_segs, uint32_t scale, uint64_t* seg_off, uint64_t* total, uint64_t* scratch,
-                        void* stream, uint32_t* status, const uint32_t* tile_nhit = nullptr,
-                        uint64_t* nhit_sum = nullptr);
+int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* tile_off, const SegList& segs,
+                        uint32_t scale, uint64_t* seg_off, uint64_t* total, uint64_t* scratch, void* stream,
+                        uint32_t* status, const uint32_t* tile_nhit = nullptr, uint64_t* nhit_sum = nullptr);
 
 // ---------------------------------------------------------------- fragment scans (Section 5)
 uint64_t frag_windows(uint64_t n_bytes);       // 64-byte windows at 4-byte offsets in n_bytes

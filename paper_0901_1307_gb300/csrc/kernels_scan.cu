@@ -2,6 +2,7 @@
 // second compaction pass.
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "compact.cuh"
@@ -112,9 +113,10 @@ __global__ void __launch_bounds__(kOffThreads) lookback_scan_kernel(const uint64
 }
 
 // seg_off[s] = offset of the first output tile of segment s (output tiles per scan tile: scale).
-__global__ void segment_offsets_kernel(const uint64_t* tile_off, uint64_t n, const Segment* segs, uint32_t n_segs,
+__global__ void segment_offsets_kernel(const uint64_t* tile_off, uint64_t n, const __grid_constant__ SegList list,
                                        uint32_t scale, const uint64_t* total, uint64_t* seg_off) {
-  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n_segs; s += gridDim.x * blockDim.x) {
+  const Segment* const segs = list.get();
+  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < list.n; s += gridDim.x * blockDim.x) {
     const uint64_t u = segs[s].tile_base * scale;
     seg_off[s] = u < n ? tile_off[u] : *total;
   }
@@ -204,17 +206,28 @@ const ScanCfg& digest_config_for(int cfg_i, int sig, uint64_t sectors, int sms, 
   return c[cfg_i];
 }
 
-int launch_expand(const ScanCfg& cfg, const uint4* hit_rec, const uint32_t* tile_nhit, const uint64_t* tile_off,
-                  uint64_t n_out_tiles, const Segment* segs, uint32_t n_segs, const TableView& tab, MatchOut* out,
-                  uint64_t out_cap, uint32_t* status, int sms, void* stream) {
-  const uint2* post = tab.postings;
-  const uint8_t* confirm = sig_is_weak((int)tab.sig) ? tab.confirm : nullptr;
-  uint64_t g = (n_out_tiles * 32 + 255) / 256;
+void compact_table(CompactParams* p, const TableView& tab) {
+  p->postings = tab.postings;
+  p->confirm = sig_is_weak((int)tab.sig) ? tab.confirm : nullptr;
+}
+
+int launch_expand(const ScanCfg& cfg, const CompactParams& p, int sms, void* stream) {
+  uint64_t g = (p.n_out_tiles + 255) / 256;
   if (g > (uint64_t)sms * 16) g = (uint64_t)sms * 16;
   if (g == 0) g = 1;
-  void* args[] = {&hit_rec, &tile_nhit, &tile_off, &n_out_tiles, &segs, &n_segs, &post, &out, &out_cap, &status,
-                  &confirm};
+  void* args[] = {const_cast<CompactParams*>(&p)};
   return (int)cudaLaunchKernel(cfg.expand_fn, dim3((unsigned)g), dim3(256), args, 0, (cudaStream_t)stream);
+}
+
+int launch_finish(const ScanCfg& cfg, const CompactParams& p, int sms, void* stream) {
+  if (p.n_out_tiles > kFinishTiles) return (int)cudaErrorInvalidValue;
+  const uint64_t groups = (p.n_out_tiles + 31) / 32;
+  // a warp per group, up to 64 blocks: each block reads every tile's count
+  uint64_t g = (groups + kFinishThreads / 32 - 1) / (kFinishThreads / 32);
+  g = std::max<uint64_t>(1, std::min<uint64_t>(g, std::min(sms, 64)));
+  void* args[] = {const_cast<CompactParams*>(&p)};
+  return (int)cudaLaunchKernel(cfg.finish_fn, dim3((unsigned)g), dim3(kFinishThreads), args, groups * 8,
+                               (cudaStream_t)stream);
 }
 
 int launch_wait_selftest(uint32_t* status, uint64_t timeout_ns, void* stream) {
@@ -245,9 +258,9 @@ int launch_lookback_selftest(uint64_t* words, uint32_t* status, uint64_t timeout
 
 uint64_t tile_offsets_scratch_words(uint64_t n_tiles) { return (n_tiles + kOffChunk - 1) / kOffChunk + 1; }
 
-int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* tile_off, const Segment* segs,
-                        uint32_t n_segs, uint32_t scale, uint64_t* seg_off, uint64_t* total, uint64_t* scratch,
-                        void* stream_, uint32_t* status, const uint32_t* tile_nhit, uint64_t* nhit_sum) {
+int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* tile_off, const SegList& segs,
+                        uint32_t scale, uint64_t* seg_off, uint64_t* total, uint64_t* scratch, void* stream_,
+                        uint32_t* status, const uint32_t* tile_nhit, uint64_t* nhit_sum) {
   cudaStream_t stream = (cudaStream_t)stream_;
   const uint64_t chunks = (n_tiles + kOffChunk - 1) / kOffChunk;
   cudaError_t e;
@@ -260,8 +273,8 @@ int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* 
   } else if ((e = cudaMemsetAsync(total, 0, 8, stream)) != cudaSuccess) {
     return (int)e;
   }
-  if (n_segs) segment_offsets_kernel<<<(n_segs + 255) / 256, 256, 0, stream>>>(tile_off, n_tiles, segs, n_segs, scale,
-                                                                               total, seg_off);
+  if (segs.n)
+    segment_offsets_kernel<<<(segs.n + 255) / 256, 256, 0, stream>>>(tile_off, n_tiles, segs, scale, total, seg_off);
   return (int)cudaGetLastError();
 }
 

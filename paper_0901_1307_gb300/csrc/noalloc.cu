@@ -18,9 +18,9 @@
 //     else they read. Two calls whose work overlaps on the GPU (different streams or host
 //     threads without ordering) race on the array and give wrong results: serialize them.
 //   - The first call on each device does a one-time set-up with that device current (the
-//     array's device address, kernel attributes). Every call copies its segment
-//     descriptor from host memory and waits for its stream, so no call can be captured into a
-//     CUDA graph: a call on a capturing stream is refused with CV_EINVAL before any work.
+//     array's device address, kernel attributes). Every call waits for its stream, so no call can
+//     be captured into a CUDA graph: a call on a capturing stream is refused with CV_EINVAL before
+//     any work.
 //   - On an error return the output buffer's contents are undefined; when the scan failed (a
 //     device wait timed out or a lookup ran past its bound) nothing is written to it.
 #include <cuda.h>
@@ -31,6 +31,7 @@
 
 #include <mutex>
 
+#include "compact.cuh"
 #include "cv.h"
 #include "cv_internal.h"
 #include "cv_launch.h"
@@ -43,13 +44,11 @@ namespace {
 // Scratch layout (offsets in bytes); sized for CV_NOALLOC_MAX_SECTORS with the smallest tile.
 constexpr uint64_t kMaxSectors = CV_NOALLOC_MAX_SECTORS;
 constexpr uint64_t kMaxTiles = kMaxSectors / 32 + 32;  // output tiles of 32 sectors, plus a ragged tile
-constexpr uint64_t kOffSeg = 128;                               // Segment
 constexpr uint64_t kOffCounters = 256;                          // seg_off[1], total, status
-constexpr uint64_t kOffSums = 512;                              // chunk sums of the offset pass
-constexpr uint64_t kOffNhit = kOffSums + 1024;                  // u32 per tile
-constexpr uint64_t kOffNtrip = kOffNhit + ((kMaxTiles * 4 + 255) / 256) * 256;   // u64 per tile
-constexpr uint64_t kOffToff = kOffNtrip + ((kMaxTiles * 8 + 255) / 256) * 256;   // u64 per tile
-constexpr uint64_t kOffHits = kOffToff + ((kMaxTiles * 8 + 255) / 256) * 256;    // uint4 per sector slot
+constexpr uint64_t kOffNhit = 512;                              // u32 per tile
+constexpr uint64_t kOffNtrip = kOffNhit + ((kMaxTiles * 4 + 255) / 256) * 256;  // u64 per tile
+constexpr uint64_t kOffHits = kOffNtrip + ((kMaxTiles * 8 + 255) / 256) * 256;  // uint4 per sector slot
+static_assert(kMaxTiles <= kFinishTiles, "offsets and expansion in one launch");
 constexpr uint64_t kHitSlots = kMaxTiles * 32;
 constexpr uint64_t kNoAllocScratchBytes = kOffHits + kHitSlots * 16;
 
@@ -134,17 +133,14 @@ extern "C" int cv_scan_noalloc(const cv_master* m, const void* image, uint64_t n
   const ScanCfg& cfg = scan_config_for(0, table_kind(tab), nullptr);
 
   uint8_t* sc = d->scratch;
-  Segment* seg_d = (Segment*)(sc + kOffSeg);
   uint64_t* seg_off_d = (uint64_t*)(sc + kOffCounters);
   uint64_t* total_d = seg_off_d + 1;
   uint32_t* status_d = (uint32_t*)(seg_off_d + 2);
   uint32_t* tile_nhit = (uint32_t*)(sc + kOffNhit);
   uint64_t* tile_ntrip = (uint64_t*)(sc + kOffNtrip);
-  uint64_t* tile_off = (uint64_t*)(sc + kOffToff);
   uint4* hit_rec = (uint4*)(sc + kOffHits);
 
-  // The tensor map travels in the kernel's parameters; the segment descriptor is also copied
-  // to the scratch array for the compaction kernels.
+  // The tensor map and the segment descriptor travel in the kernels' parameters.
   ScanParams p;
   memset(&p, 0, sizeof p);
   CUtensorMap& map = p.maps[0];
@@ -171,10 +167,8 @@ extern "C" int cv_scan_noalloc(const cv_master* m, const void* image, uint64_t n
 
   cudaError_t e;
   if ((e = cudaMemsetAsync(status_d, 0, 4, stream)) != cudaSuccess) return fail(e);
-  if ((e = cudaMemcpyAsync(seg_d, &seg, sizeof seg, cudaMemcpyHostToDevice, stream)) != cudaSuccess) return fail(e);
 
-  p.segs = seg_d;
-  p.n_segs = 1;
+  p.segs = seg_list(&seg, nullptr, 1);
   p.map_base = 0;
   p.one = 1u;
   p.tile_begin = 0;
@@ -189,16 +183,20 @@ extern "C" int cv_scan_noalloc(const cv_master* m, const void* image, uint64_t n
                             stream)) !=
       cudaSuccess)
     return fail(e);
-  uint32_t one = 1;
-  uint64_t nt = n_out_tiles;
-  const Segment* segc = seg_d;
-  static_assert((kMaxTiles + 4095) / 4096 + 1 <= 1024 / 8, "offset scratch");
-  if ((e = (cudaError_t)launch_tile_offsets(tile_ntrip, nt, tile_off, segc, one, (uint32_t)(cfg.T / 32), seg_off_d,
-                                            total_d, (uint64_t*)(sc + kOffSums), stream, status_d)) != cudaSuccess)
-    return fail(e);
-  if ((e = (cudaError_t)launch_expand(cfg, hit_rec, tile_nhit, tile_off, nt, segc, one, tab, (MatchOut*)out,
-                                      out_capacity, status_d, d->sms, stream)) != cudaSuccess)
-    return fail(e);
+  CompactParams cp;
+  memset(&cp, 0, sizeof cp);
+  compact_table(&cp, tab);
+  cp.hit_rec = hit_rec;
+  cp.tile_nhit = tile_nhit;
+  cp.tile_ntrip = tile_ntrip;
+  cp.n_out_tiles = n_out_tiles;
+  cp.segs = p.segs;
+  cp.out = (MatchOut*)out;
+  cp.out_cap = out_capacity;
+  cp.status = status_d;
+  cp.seg_off = seg_off_d;
+  cp.total = total_d;
+  if ((e = (cudaError_t)launch_finish(cfg, cp, d->sms, stream)) != cudaSuccess) return fail(e);
   uint64_t hc[2] = {0, 0};  // total, status
   if ((e = cudaMemcpyAsync(hc, total_d, 16, cudaMemcpyDeviceToHost, stream)) != cudaSuccess) return fail(e);
   if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return fail(e);

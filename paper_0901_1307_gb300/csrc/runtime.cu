@@ -227,6 +227,14 @@ int Job::add(DevCtx* ctx, const ScanCfg& cfg, const void* base, uint64_t n_in, u
   return CV_OK;
 }
 
+int Job::segs_device(Segment** out, Temps& tmp, cudaStream_t stream) const {
+  *out = nullptr;
+  if (segs.size() <= kInlineSegs) return CV_OK;
+  CV_TRY(tmp.alloc(out, segs.size() * sizeof(Segment)));
+  CV_CUDA(cudaMemcpyAsync(*out, segs.data(), segs.size() * sizeof(Segment), cudaMemcpyHostToDevice, stream));
+  return CV_OK;
+}
+
 int Job::set_map(DevCtx* ctx, const ScanCfg& cfg, size_t s, const void* base) {
   Segment& sg = segs[s];
   CV_TRY(make_tmap(ctx, cfg, base, sg.n_sectors, &maps[sg.map]));
@@ -267,8 +275,7 @@ int launch_range(DevCtx* ctx, int cfg_i, bool digest, const Job& job, const Segm
     for (uint32_t k = lo; k <= hi; k++) p.maps[k - lo] = job.maps[k];
     p.map_base = lo;
     p.one = 1u;
-    p.segs = segs_d + a;
-    p.n_segs = (uint32_t)(b - a);
+    p.segs = seg_list(job.segs.data() + a, segs_d ? segs_d + a : nullptr, b - a);
     p.tile_begin = job.segs[a].tile_base;
     const uint64_t tile_end = (b < job.segs.size()) ? job.segs[b].tile_base : job.n_tiles;
     p.n_tiles = tile_end - p.tile_begin;

@@ -138,12 +138,14 @@ struct Job {
   // whose map is set later (set_map).
   int add(DevCtx* ctx, const ScanCfg& cfg, const void* base, uint64_t n, uint64_t sector_base, uint32_t image,
           bool share_alloc);
+  // The segment list in device memory, or null when it travels in the kernels' parameters (SegList).
+  int segs_device(Segment** out, Temps& tmp, cudaStream_t stream) const;
   // Point segment s at a fresh map over base (streamed chunks).
   int set_map(DevCtx* ctx, const ScanCfg& cfg, size_t s, const void* base);
 };
 
 // Launch the scan (or digest) kernel over segments [s0, s1) of the job; segs_d is the job's
-// segment array in device memory. `base` carries the table and output pointers. Returns the
+// segment array in device memory (null: at most kInlineSegs segments). `base` carries the table and output pointers. Returns the
 // number of kernel launches through *launches when non-null.
 int launch_range(DevCtx* ctx, int cfg_i, bool digest, const Job& job, const Segment* segs_d, size_t s0, size_t s1,
                  const ScanParams& base, cudaStream_t stream, int* launches = nullptr);

@@ -24,7 +24,7 @@
   ::cvk::ScanCfg {                                                                             \
     "t" #T "_x" #SPT "_s" #NS "_b" #B "_p" #P, T, SPT, T / SPT + 32, NS, B,                   \
         CV_SCAN_KINDS(T, SPT, NS, B, P, MB), {nullptr, nullptr, nullptr, nullptr},           \
-        (const void*)::cvk::expand_kernel<T>, ::cvk::ScanSmem<T, NS, B>::kAlloc              \
+        (const void*)::cvk::expand_kernel<T>, (const void*)::cvk::finish_kernel<T>, ::cvk::ScanSmem<T, NS, B>::kAlloc              \
   }
 
 // The same with digest-mode kernels for every signature (table builds, cv_sector_signatures).
@@ -36,5 +36,5 @@
          CV_KS(T, SPT, NS, B, ::cvk::kModeDigest, P, MB, ::cvk::kSigMd5NoPad),                 \
          CV_KS(T, SPT, NS, B, ::cvk::kModeDigest, P, MB, ::cvk::kSigDjb2),                     \
          CV_KS(T, SPT, NS, B, ::cvk::kModeDigest, P, MB, ::cvk::kSigCrc64)},                   \
-        (const void*)::cvk::expand_kernel<T>, ::cvk::ScanSmem<T, NS, B>::kAlloc              \
+        (const void*)::cvk::expand_kernel<T>, (const void*)::cvk::finish_kernel<T>, ::cvk::ScanSmem<T, NS, B>::kAlloc              \
   }

@@ -324,10 +324,11 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
     const uint32_t bar_clc = base + L::kClcBarOff;
     uint32_t j = 0, lt = blockIdx.x, answers = 0;
     bool ok = true, more = true;
+    const Segment* const segs = p.segs.get();
     while (more && ok) {
       clc_ask(base + L::kClcOff, bar_clc);  // the next tile; answered while this one is staged
       const uint64_t tile = p.tile_begin + lt;
-      const Segment& seg = p.segs[find_segment(p.segs, p.n_segs, tile)];
+      const Segment& seg = segs[find_segment(segs, p.segs.n, tile)];
       const CUtensorMap* map = &p.maps[seg.map - p.map_base];
       const uint64_t first = (tile - seg.tile_base) * T;  // the tile's first sector within the segment
       const int32_t row0 = (int32_t)(seg.row_base + first);

@@ -35,6 +35,7 @@
 #include <thread>
 #include <vector>
 
+#include "compact.cuh"
 #include "cv.h"
 #include "runtime.h"
 
@@ -347,9 +348,9 @@ int cv_server::launch_scan(ScanBatch& b, const std::vector<Request*>& work, bool
   p.tile_ntrip = b.tile_ntrip;
   p.status = status;
   CV_TRY(launch_range(ctx, cfg_i, false, job, b.segs_d, 0, b.nseg, p, b.stream));
-  CV_CUDA((cudaError_t)launch_tile_offsets(b.tile_ntrip, b.n_out, b.tile_off, b.segs_d, (uint32_t)b.nseg,
-                                           (uint32_t)(cfg.T / 32), b.counters_d, b.counters_d + b.nseg,
-                                           b.off_scratch, b.stream, status));
+  CV_CUDA((cudaError_t)launch_tile_offsets(b.tile_ntrip, b.n_out, b.tile_off,
+                                           seg_list(b.segs_h, b.segs_d, b.nseg), (uint32_t)(cfg.T / 32), b.counters_d,
+                                           b.counters_d + b.nseg, b.off_scratch, b.stream, status));
   CV_CUDA(cudaMemcpyAsync(b.counters_h, b.counters_d, (b.nseg + 2) * 8, cudaMemcpyDeviceToHost, b.stream));
   CV_CUDA(cudaEventRecord(b.counts_ready, b.stream));
   b.state = ScanBatch::kCounting;
@@ -371,8 +372,18 @@ int cv_server::launch_expand_of(ScanBatch& b) {
     const ScanCfg& cfg = scan_configs(&n_ops)[cfg_i];
     CV_TRY(b.ensure_buffers(0, 0, b.total));
     uint32_t* status = (uint32_t*)(b.counters_d + b.nseg + 1);
-    CV_CUDA((cudaError_t)launch_expand(cfg, b.hit_rec, b.tile_nhit, b.tile_off, b.n_out, b.segs_d,
-                                       (uint32_t)b.nseg, tab, b.out_d, b.cap_out, status, ctx->sms, b.stream));
+    CompactParams cp;
+    memset(&cp, 0, sizeof cp);
+    compact_table(&cp, tab);
+    cp.hit_rec = b.hit_rec;
+    cp.tile_nhit = b.tile_nhit;
+    cp.n_out_tiles = b.n_out;
+    cp.segs = seg_list(b.segs_h, b.segs_d, b.nseg);
+    cp.out = b.out_d;
+    cp.out_cap = b.cap_out;
+    cp.status = status;
+    cp.tile_off = b.tile_off;
+    CV_CUDA((cudaError_t)launch_expand(cfg, cp, ctx->sms, b.stream));
     CV_CUDA(cudaMemcpyAsync(b.out_h, b.out_d, b.total * sizeof(MatchOut), cudaMemcpyDeviceToHost, b.stream));
   }
   CV_CUDA(cudaEventRecord(b.matches_ready, b.stream));

@@ -383,12 +383,12 @@ int cv_batch_create(const cv_master* m, const cv_buf* images, uint32_t n_images,
     if (layout_choice) CV_TRY(need_sorted());
     if (bloom && !bloom_avail) CV_TRY(need_bloom());
     if (!layout_choice && b->own_slots) {
-      cudaFree(b->own_slots);
-      cudaFree(b->own_keys0);
+      cudaFreeAsync(b->own_slots, stream);  // used on this stream only so far
+      cudaFreeAsync(b->own_keys0, stream);
       b->own_slots = b->own_keys0 = nullptr;
     }
     if (!bloom && b->own_bloom) {
-      cudaFree(b->own_bloom);
+      cudaFreeAsync(b->own_bloom, stream);
       b->own_bloom = nullptr;
     }
     const TableView chosen = variant(layout_choice, bloom);
@@ -521,8 +521,8 @@ void cvk_batch_free(void* h) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   b->buf.release();
-  for (void* p : {b->own_slots, b->own_keys0, b->own_bloom})
-    if (p) cudaFree(p);
+  void* const tables[] = {b->own_slots, b->own_keys0, b->own_bloom};
+  if (b->own_slots || b->own_keys0 || b->own_bloom) table_free(tables, 3, b->dev);
   if (b->counters_h) cudaFreeHost(b->counters_h);
   if (b->ev0) cudaEventDestroy(b->ev0);
   if (b->ev1) cudaEventDestroy(b->ev1);

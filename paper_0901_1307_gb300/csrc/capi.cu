@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <optional>
 #include <vector>
 
 #include "cv.h"
@@ -179,6 +180,46 @@ cv_result* make_host_result(int dev, const MatchOut* data, uint64_t n, uint64_t 
 
 namespace {
 
+// What a call reads back behind its last kernel: n counts, and the matches when they fit in a
+// stage. The counts land in `to` when wait() returns; staged matches stay in stage.matches.
+struct Readback {
+  DevCtx* ctx;
+  uint64_t* to;
+  const uint64_t* from;
+  uint64_t n;
+  cudaStream_t stream;
+  Stage stage;
+  uint64_t staged = 0;  // matches copied
+  Readback(DevCtx* c, uint64_t* host, const uint64_t* dev, uint64_t count, cudaStream_t s)
+      : ctx(c), to(host), from(dev), n(count), stream(s), stage(c->take_stage()) {}
+  ~Readback() {
+    if (!waited_) cudaStreamSynchronize(stream);  // an error in between: copies may be on their way
+    ctx->give_stage(&stage);
+  }
+  Readback(const Readback&) = delete;
+  Readback& operator=(const Readback&) = delete;
+  int counts() {
+    uint64_t* dst = stage.counts && n <= kStageCounts ? stage.counts : to;
+    CV_CUDA(cudaMemcpyAsync(dst, from, n * 8, cudaMemcpyDeviceToHost, stream));
+    return CV_OK;
+  }
+  int matches(const MatchOut* dev, uint64_t room) {
+    if (!stage.counts) return CV_OK;
+    staged = std::min(room, kStageMatches);
+    CV_CUDA(cudaMemcpyAsync(stage.matches, dev, staged * sizeof(MatchOut), cudaMemcpyDeviceToHost, stream));
+    return CV_OK;
+  }
+  int wait() {
+    CV_CUDA(cudaStreamSynchronize(stream));
+    waited_ = true;
+    if (stage.counts && n <= kStageCounts) memcpy(to, stage.counts, n * 8);
+    return CV_OK;
+  }
+
+ private:
+  bool waited_ = false;
+};
+
 // cv_scan over a fragment table (Section 5): count kernel per image, one offset scan over all
 // tiles, emit kernel per image over its tiles with triples. Host images are copied whole.
 int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_images, uint32_t flags,
@@ -267,23 +308,45 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       CV_CUDA((cudaError_t)launch_tile_offsets(tile_ntrip, T, tile_off, seg_list(segs.data(), segs_d, n_images), 1,
                                                seg_off_d, seg_off_d + n_images, scratch, stream, status));
       r->launches += 2;
-      std::vector<uint64_t> seg_off(n_images + 3, 0);
-      CV_CUDA(cudaMemcpyAsync(seg_off.data(), seg_off_d, (n_images + 3) * 8, cudaMemcpyDeviceToHost, stream));
-      CV_CUDA(cudaStreamSynchronize(stream));
-      const uint32_t st = (uint32_t)seg_off[n_images + 1];
-      if (st & kStTimeout) return CV_ETIMEOUT;
-      if (st) return CV_ECORRUPT;
-      const uint64_t total = seg_off[n_images];
-      r->st.confirm_rejected = seg_off[n_images + 2];
-      if (total) {
-        CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, total * sizeof(MatchOut), ctx->pool, stream));
+      auto emit = [&](uint64_t room) -> int {
+        CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, room * sizeof(MatchOut), ctx->pool, stream));
         for (uint32_t i = 0; i < n_images; i++) {
           if (tile_base[i + 1] == tile_base[i]) continue;
           hits.count = (uint32_t*)(listed + i);
-          CV_CUDA((cudaError_t)frag_emit(m->tab, dptr[i], nbytes[i], tile_base[i], tile_off, hits, r->dev_out, total,
+          CV_CUDA((cudaError_t)frag_emit(m->tab, dptr[i], nbytes[i], tile_base[i], tile_off, hits, r->dev_out, room,
                                          status, ctx->sms, stream));
           r->launches++;
         }
+        return CV_OK;
+      };
+      // As in the sector scan: the emit pass is launched with the room that the last scan against
+      // the table suggests, its outcome read back with the counts, and run again only if that
+      // was too little.
+      const uint64_t hint = __atomic_load_n(&const_cast<cv_master*>(m)->last_matches, __ATOMIC_RELAXED);
+      const uint64_t room = std::max<uint64_t>(hint + hint / 4 + 1024, 4096);
+      CV_TRY(emit(room));
+      std::vector<uint64_t> seg_off(n_images + 3, 0);
+      Readback rb(ctx, seg_off.data(), seg_off_d, n_images + 3, stream);
+      CV_TRY(rb.counts());
+      if (!r->on_device) CV_TRY(rb.matches(r->dev_out, room));
+      CV_CUDA(cudaEventRecord(ev[3], stream));
+      CV_TRY(rb.wait());
+      uint32_t st = (uint32_t)seg_off[n_images + 1];
+      if (st & kStTimeout) return CV_ETIMEOUT;
+      if (st & ~kStOverflow) return CV_ECORRUPT;
+      const uint64_t total = seg_off[n_images];
+      __atomic_store_n(&const_cast<cv_master*>(m)->last_matches, total, __ATOMIC_RELAXED);
+      r->st.confirm_rejected = seg_off[n_images + 2];
+      if (total == 0 || total > room) {
+        CV_CUDA(cudaFreeAsync(r->dev_out, stream));
+        r->dev_out = nullptr;
+      }
+      bool more = false;
+      if (total > room) {
+        CV_CUDA(cudaMemsetAsync(status, 0, 4, stream));
+        CV_TRY(emit(total));
+        rb.staged = 0;
+        more = true;
       }
       for (uint32_t i = 0; i < n_images; i++) r->off[i] = seg_off[i];
       r->off[n_images] = total;
@@ -291,14 +354,21 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       if (total && !r->on_device) {
         r->host = (MatchOut*)malloc(total * sizeof(MatchOut));
         if (!r->host) return CV_ENOMEM;
-        CV_CUDA(cudaMemcpyAsync(r->host, r->dev_out, total * sizeof(MatchOut), cudaMemcpyDeviceToHost, stream));
+        if (total <= rb.staged) {
+          memcpy(r->host, rb.stage.matches, total * sizeof(MatchOut));
+        } else {
+          CV_CUDA(cudaMemcpyAsync(r->host, r->dev_out, total * sizeof(MatchOut), cudaMemcpyDeviceToHost, stream));
+          more = true;
+        }
       }
-      uint32_t st2 = 0;
-      CV_CUDA(cudaMemcpyAsync(&st2, status, 4, cudaMemcpyDeviceToHost, stream));
-      CV_CUDA(cudaEventRecord(ev[3], stream));
-      CV_CUDA(cudaStreamSynchronize(stream));
-      if (st2 & kStTimeout) return CV_ETIMEOUT;
-      if (st2) return CV_ECORRUPT;
+      if (more) {
+        uint32_t st2 = 0;
+        CV_CUDA(cudaMemcpyAsync(&st2, status, 4, cudaMemcpyDeviceToHost, stream));
+        CV_CUDA(cudaEventRecord(ev[3], stream));
+        CV_CUDA(cudaStreamSynchronize(stream));
+        if (st2 & kStTimeout) return CV_ETIMEOUT;
+        if (st2) return CV_ECORRUPT;
+      }
       float ms = 0.f;
       CV_CUDA(cudaEventElapsedTime(&ms, ev[1], ev[2]));
       r->st.kernel_ms = ms;
@@ -424,6 +494,7 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
       uint64_t total = 0;
       std::vector<uint64_t> seg_off(nseg + 4, 0);
       uint32_t* status_keep = nullptr;
+      std::optional<Readback> rb;
       bool expanded_early = false;  // the expand pass ran before the count came back, and sufficed
       if (nseg) {
         void* ring[2] = {nullptr, nullptr};
@@ -542,11 +613,13 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
           room = std::max<uint64_t>(hint + hint / 4 + 1024, small ? 4096 : 0);
           CV_TRY(expand(room));
         }
-        CV_CUDA(cudaMemcpyAsync(seg_off.data(), seg_off_d, (nseg + 4) * 8, cudaMemcpyDeviceToHost, stream));
+        rb.emplace(ctx, seg_off.data(), seg_off_d, nseg + 4, stream);
+        CV_TRY(rb->counts());
+        if (room && !r->on_device) CV_TRY(rb->matches(r->dev_out, room));
         // the call's end unless more work follows (then recorded again after it): in the common
         // case this one wait for the stream is the call's only one
         CV_CUDA(cudaEventRecord(ev[3], stream));
-        CV_CUDA(cudaStreamSynchronize(stream));
+        CV_TRY(rb->wait());
         const uint32_t st = (uint32_t)seg_off[nseg + 1];
         if (st & kStTimeout) return CV_ETIMEOUT;
         if (st & ~kStOverflow) return CV_ECORRUPT;
@@ -578,8 +651,12 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
       if (total && !r->on_device) {
         r->host = (MatchOut*)malloc(total * sizeof(MatchOut));
         if (!r->host) return CV_ENOMEM;
-        CV_CUDA(cudaMemcpyAsync(r->host, r->dev_out, total * sizeof(MatchOut), cudaMemcpyDeviceToHost, stream));
-        more = true;
+        if (expanded_early && total <= rb->staged) {
+          memcpy(r->host, rb->stage.matches, total * sizeof(MatchOut));
+        } else {
+          CV_CUDA(cudaMemcpyAsync(r->host, r->dev_out, total * sizeof(MatchOut), cudaMemcpyDeviceToHost, stream));
+          more = true;
+        }
       }
       uint32_t st2 = 0;
       if (nseg && total && !expanded_early)
@@ -653,12 +730,8 @@ void cv_free(void* handle) {
   if (magic == kMagicMaster) {
     cv_master* m = (cv_master*)handle;
     m->magic = 0;
-    if (m->slots) cudaFree(m->slots);
-    if (m->postings) cudaFree(m->postings);
-    if (m->bloom) cudaFree(m->bloom);
-    if (m->confirm) cudaFree(m->confirm);
-    if (m->keys0) cudaFree(m->keys0);
-    if (m->frag_l1) cudaFree(m->frag_l1);
+    void* const arrays[] = {m->slots, m->postings, m->bloom, m->confirm, m->keys0, m->frag_l1};
+    table_free(arrays, 6, m->dev);
     free(m);
   } else if (magic == kMagicResult) {
     cv_result* r = (cv_result*)handle;

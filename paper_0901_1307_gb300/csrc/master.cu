@@ -269,19 +269,19 @@ int sorted_from_hash(DevCtx* ctx, const uint4* slots, uint64_t n_slots, uint32_t
   CV_TRY(radix_sort_pairs(kfree, vr, kr, vfree, nu, 32, tmp, stream, &hk, &hv));
   void* out = nullptr;
   void* keys0 = nullptr;
-  CV_CUDA(cudaMalloc(&out, std::max<uint64_t>(nu, 1) * 32));
-  cudaError_t e = cudaMalloc(&keys0, std::max<uint64_t>(nu, 1) * 4);
-  if (e != cudaSuccess) {
-    cudaFree(out);
-    return cuda_fail(e);
+  CV_TRY(table_alloc(ctx, &out, std::max<uint64_t>(nu, 1) * 32, stream));
+  int rc = table_alloc(ctx, &keys0, std::max<uint64_t>(nu, 1) * 4, stream);
+  if (rc != CV_OK) {
+    cudaFreeAsync(out, stream);
+    return rc;
   }
   gather_slots_kernel<<<gu, 256, 0, stream>>>(slots, hv, nu, (uint4*)out);
-  e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && nu) e = cudaMemcpyAsync(keys0, hk, (uint64_t)nu * 4, cudaMemcpyDeviceToDevice, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
-    cudaFree(out);
-    cudaFree(keys0);
+    cudaFreeAsync(out, stream);
+    cudaFreeAsync(keys0, stream);
     return cuda_fail(e);
   }
   *slots_out = out;
@@ -371,20 +371,20 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       CV_CUDA(cudaMemcpyAsync(file_base_d, file_base.data(), (n_files + 1) * 8, cudaMemcpyHostToDevice, stream));
       CV_TRY(gather_master_units(ctx, files, n_files, file_base, U, tmp, stream, &arena));
       // long-lived table memory
-      CV_CUDA(cudaMalloc(&m->slots, n_slots * 32));
-      CV_CUDA(cudaMalloc(&m->postings, std::max<uint64_t>(M, 1) * 8));
+      CV_TRY(table_alloc(ctx, &m->slots, n_slots * 32, stream));
+      CV_TRY(table_alloc(ctx, &m->postings, std::max<uint64_t>(M, 1) * 8, stream));
       // Bloom blocks: 32 bytes for sector tables, one 32-bit word for fragment tables
       const uint64_t block_bytes = frag ? 4 : 32;
       uint64_t n_blocks = 0;
       if (bpk) {
         n_blocks = std::max<uint64_t>(next_pow2((M * bpk + block_bytes * 8 - 1) / (block_bytes * 8)), frag ? 8 : 1);
-        CV_CUDA(cudaMalloc(&m->bloom, n_blocks * block_bytes));
+        CV_TRY(table_alloc(ctx, &m->bloom, n_blocks * block_bytes, stream));
         CV_CUDA(cudaMemsetAsync(m->bloom, 0, n_blocks * block_bytes, stream));
       }
       if (frag) {
         // the shared-memory prefilter of a fragment table exists even when the table is empty
         // (all zero then: no window passes it)
-        CV_CUDA(cudaMalloc(&m->frag_l1, kFragL1Bytes));
+        CV_TRY(table_alloc(ctx, &m->frag_l1, kFragL1Bytes, stream));
         CV_CUDA(cudaMemsetAsync(m->frag_l1, 0, kFragL1Bytes, stream));
       }
       if (M) {
@@ -424,7 +424,7 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
                                         (uint2*)m->postings, member, tmp, stream));
       if (M && sig_is_weak(sig)) {
         // a copy of the kept master units in posting order, to confirm matches byte for byte
-        CV_CUDA(cudaMalloc(&m->confirm, M * U));
+        CV_TRY(table_alloc(ctx, &m->confirm, M * U, stream));
         if (hc[1]) {
           gather_units_kernel<<<grid_for(hc[1] * (U / 16), 256, ctx->sms), 256, 0, stream>>>(
               (const uint4*)arena, member, hc[1], (uint32_t)(U / 16), (uint4*)m->confirm);
@@ -438,7 +438,7 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
         void* sorted_slots = nullptr;
         CV_TRY(sorted_from_hash(ctx, (const uint4*)m->slots, n_slots, hc[2], tmp, stream, &sorted_slots, &m->keys0,
                                 &steps));
-        cudaFree(m->slots);
+        cudaFreeAsync(m->slots, stream);
         m->slots = sorted_slots;
       }
       m->tab.slots = (const uint4*)m->slots;
@@ -642,7 +642,8 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
     const bool always[6] = {true, true, false, false, false, false};  // the build allocates these even when empty
     for (int k = 0; k < 6; k++) {
       if (!sizes[k] && !always[k]) continue;
-      CV_CUDA(cudaMalloc(arrays[k], std::max<uint64_t>(sizes[k], 32)));
+      CV_TRY(table_alloc(ctx, arrays[k], std::max<uint64_t>(sizes[k], 32), stream));
+      CV_CUDA(cudaStreamSynchronize(stream));  // the copies below are not in the stream's order
       if (sizes[k]) CV_TRY(copy_from_file(f, *arrays[k], sizes[k]));
     }
     uint8_t extra;
@@ -734,7 +735,7 @@ int cvk::table_bloom(const TableView& tab, uint32_t bits_per_key, cudaStream_t s
   const uint64_t keys = std::max<uint64_t>(tab.n_keys, 1);
   const uint64_t n_blocks = next_pow2((keys * bits_per_key + 255) / 256);
   void* bloom = nullptr;
-  CV_CUDA(cudaMalloc(&bloom, n_blocks * 32));
+  CV_TRY(table_alloc(ctx, &bloom, n_blocks * 32, stream));
   cudaError_t e = cudaMemsetAsync(bloom, 0, n_blocks * 32, stream);
   if (e == cudaSuccess && n_records) {
     bloom_kernel<<<grid_for(n_records, 256, ctx->sms), 256, 0, stream>>>(tab.slots, (uint32_t)n_records,
@@ -743,7 +744,7 @@ int cvk::table_bloom(const TableView& tab, uint32_t bits_per_key, cudaStream_t s
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
-    cudaFree(bloom);
+    cudaFreeAsync(bloom, stream);
     return cuda_fail(e);
   }
   *bloom_out = bloom;

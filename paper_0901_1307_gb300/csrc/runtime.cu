@@ -68,6 +68,14 @@ int get_ctx(DevCtx** out) {
     CV_CUDA(cudaMemPoolCreate(&c.pool, &pp));
     uint64_t thr = UINT64_MAX;
     CV_CUDA(cudaMemPoolSetAttribute(c.pool, cudaMemPoolAttrReleaseThreshold, &thr));
+    CV_CUDA(cudaMemPoolCreate(&c.table_pool, &pp));
+    thr = kTablePoolKept;
+    CV_CUDA(cudaMemPoolSetAttribute(c.table_pool, cudaMemPoolAttrReleaseThreshold, &thr));
+    uint8_t* pinned = nullptr;
+    constexpr size_t stage_bytes = kStageCounts * 8 + kStageMatches * sizeof(MatchOut);
+    CV_CUDA(cudaMallocHost((void**)&pinned, kStages * stage_bytes));
+    for (int k = 0; k < kStages; k++, pinned += stage_bytes)
+      c.stage_free.push_back(Stage{(uint64_t*)pinned, (MatchOut*)(pinned + kStageCounts * 8)});
     CV_CUDA(cudaStreamCreateWithFlags(&c.copy_stream, cudaStreamNonBlocking));
     cudaDriverEntryPointQueryResult q;
     void* fn = nullptr;
@@ -117,6 +125,37 @@ int Temps::alloc_bytes(void** out, size_t bytes) {
   ptrs.push_back(p);
   *out = p;
   return CV_OK;
+}
+
+Stage DevCtx::take_stage() {
+  std::lock_guard<std::mutex> lk(stage_mutex);
+  if (stage_free.empty()) return Stage{nullptr, nullptr};
+  const Stage s = stage_free.back();
+  stage_free.pop_back();
+  return s;
+}
+
+void DevCtx::give_stage(Stage* s) {
+  if (!s->counts) return;
+  std::lock_guard<std::mutex> lk(stage_mutex);
+  stage_free.push_back(*s);
+  *s = Stage{nullptr, nullptr};
+}
+
+int table_alloc(DevCtx* ctx, void** out, size_t bytes, cudaStream_t stream) {
+  *out = nullptr;
+  CV_CUDA(cudaMallocFromPoolAsync(out, bytes ? bytes : 16, ctx->table_pool, stream));
+  return CV_OK;
+}
+
+void table_free(void* const* ptrs, int n, int dev) {
+  int current = -1;
+  if (cudaGetDevice(&current) == cudaSuccess && current != dev) cudaSetDevice(dev);
+  cudaDeviceSynchronize();  // scans on any stream may have read the table
+  for (int k = 0; k < n; k++)
+    if (ptrs[k]) cudaFreeAsync(ptrs[k], nullptr);
+  cudaGetLastError();
+  if (current >= 0 && current != dev) cudaSetDevice(current);
 }
 
 int DevCtx::take_events(cudaEvent_t* ev, int n) {

@@ -1,0 +1,88 @@
+"""What a call reads back in one wait: match counts below, at and above what is staged, scans from
+more threads than there are stages, and tables whose memory was another table's before."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+STAGED = 1 << 16  # matches that are read back without a second wait
+
+
+@pytest.fixture(scope="module")
+def cv(cuda_device):
+    import __graft_entry__
+
+    __graft_entry__.build()
+    from paper_0901_1307_gb300 import cv as cvmod
+
+    return cvmod
+
+
+@pytest.mark.parametrize("unit", [0, 1])
+@pytest.mark.parametrize("n", [1, 4096, 4097, STAGED - 1, STAGED, STAGED + 1])
+def test_counts_around_the_stage(cv, unit, n):
+    """n matches (one sector or fragment n times in one file), scanned three times: with no count to
+    go by, with the right one, and after a scan with one match."""
+    rng = np.random.default_rng(n)
+    size = 64 if unit else 512
+    key = rng.integers(0, 256, size, dtype=np.uint8)
+    img = np.concatenate([rng.integers(0, 256, 4096, dtype=np.uint8), key])
+    t = torch.from_numpy(img).cuda()
+    one = np.concatenate([key, np.tile(key, n - 1)]) if n > 1 else key
+    with cv.master_build([one], unit=unit) as m:
+        for _ in range(3):
+            with cv.scan(m, [t]) as r:
+                got = r.matches(0)
+                assert got.size == n and np.array_equal(got["file_sector"], np.arange(n))
+                assert (got["disk_sector"] == (1024 if unit else 8)).all()
+        with cv.scan(m, [t[:4096]]) as r:
+            assert r.matches(0).size == 0
+        with cv.scan(m, [t]) as r:
+            assert r.matches(0).size == n
+
+
+def test_more_threads_than_stages(cv):
+    rng = np.random.default_rng(1)
+    files = [rng.integers(0, 256, 512 * 40, dtype=np.uint8) for _ in range(10)]
+    images = [np.concatenate([rng.integers(0, 256, 51200, dtype=np.uint8), *[files[i] for i in rng.permutation(10)[:k]]])
+              for k in range(9)]
+    want = [oracle.match_hash(x, files) for x in images]
+    bad = []
+    with cv.master_build(files) as m:
+        devs = [torch.from_numpy(x).cuda() for x in images]
+        torch.cuda.synchronize()
+
+        def work(k):
+            s = torch.cuda.Stream()
+            for _ in range(20):
+                with cv.scan(m, [devs[k]], stream=s) as r:
+                    if not np.array_equal(r.matches(0), want[k]):
+                        bad.append(k)
+
+        threads = [threading.Thread(target=work, args=(k,)) for k in range(9)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    assert not bad
+
+
+def test_tables_in_used_memory(cv):
+    """Tables of changing size and kind, built on changing streams and freed, hold only their own
+    keys."""
+    rng = np.random.default_rng(2)
+    img = rng.integers(0, 256, 512 * 300, dtype=np.uint8)
+    t = torch.from_numpy(img).cuda()
+    torch.cuda.synchronize()
+    streams = [None, torch.cuda.Stream(), torch.cuda.Stream()]
+    for k in range(12):
+        files = [np.concatenate([img[512 * (20 * k):512 * (20 * k + 9)],
+                                 rng.integers(0, 256, 512 * int(rng.integers(1, 3000)), dtype=np.uint8)])]
+        kw = [{}, {"layout": cv.CV_LAYOUT_SORTED}, {"signature": 2}, {"bloom_bits_per_key": 0, "max_load": 0.9}][k % 4]
+        with cv.master_build(files, stream=streams[k % 3], **kw) as m, cv.scan(m, [t], stream=streams[(k + 1) % 3]) as r:
+            assert np.array_equal(r.matches(0), oracle.match_hash(img, files)), k

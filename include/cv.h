@@ -223,7 +223,7 @@ typedef struct {
   uint64_t hit_sectors;    /* disk sectors with at least one match (0 for fragment tables) */
   float kernel_ms;         /* device time of the hashing/probe launches */
   float total_ms;          /* device time from the first copy to the last result copy */
-  uint32_t kernel_launches; /* kernels the call launched (scan, offsets, expand) */
+  uint32_t kernel_launches; /* kernels the call launched */
   int32_t kernel_config;   /* the scan configuration used (cv_kernel_config_name), -1 for
                               fragment scans and results of the serving loop */
   uint64_t confirm_rejected; /* 64-bit signatures: candidate (disk sector, master sector or
@@ -338,7 +338,7 @@ int cv_selftest_wait_timeout(uint32_t timeout_us, void* stream);
  * Batched scans (a CUDA graph over many device images). The paper scans several drives at once
  * by multiplexing them onto one GPU (Section 3); a batch makes all of its images one work list
  * for one persistent scan launch (images in one device allocation share a tensor map), then
- * one offset pass and one expand pass, captured once as a CUDA graph and replayed per run.
+ * one pass that places and writes the matches, captured once as a CUDA graph and replayed per run.
  *
  * Images must be device buffers (16-byte aligned), borrowed for the life of the batch: each run
  * reads their current contents. Matches of the last run stay in device memory owned by the

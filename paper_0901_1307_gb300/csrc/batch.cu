@@ -2,7 +2,7 @@
 // graph. The paper scans several drives at once by multiplexing them onto one GPU (Section 3);
 // here all images of a batch are one work list: images that sit in one device allocation share
 // a tensor map, the persistent scan kernel takes tiles of every image in one launch, and one
-// offset pass and one expand pass produce every image's sorted matches. The whole sequence is
+// pass after it produces every image's sorted matches. The whole sequence is
 // captured once and replayed with a single graph launch per run.
 //
 // An optional autotuner times, on the batch itself, every kernel configuration (tile rows,
@@ -37,9 +37,7 @@ struct Buffers {
   uint4* hit_rec = nullptr;
   uint32_t* tile_nhit = nullptr;
   uint64_t* tile_ntrip = nullptr;
-  uint64_t* tile_off = nullptr;
-  uint64_t* off_scratch = nullptr;
-  uint64_t* counters_d = nullptr;  // seg_off[nseg], total, status
+  uint64_t* counters_d = nullptr;  // seg_off[nseg], total, status, triples per group of tiles
   MatchOut* out_d = nullptr;
   std::vector<void*> owned;
 
@@ -63,15 +61,13 @@ int make_buffers(const Job& job, const ScanCfg& cfg, uint64_t capacity, Buffers*
   CV_TRY(b->alloc((void**)&b->hit_rec, n_out * 32 * sizeof(uint4)));
   CV_TRY(b->alloc((void**)&b->tile_nhit, n_out * 4));
   CV_TRY(b->alloc((void**)&b->tile_ntrip, n_out * 8));
-  CV_TRY(b->alloc((void**)&b->tile_off, n_out * 8));
-  CV_TRY(b->alloc((void**)&b->off_scratch, tile_offsets_scratch_words(n_out) * 8));
-  CV_TRY(b->alloc((void**)&b->counters_d, (nseg + 2) * 8));
+  CV_TRY(b->alloc((void**)&b->counters_d, (nseg + 2 + finish_groups(n_out)) * 8));
   CV_TRY(b->alloc((void**)&b->out_d, std::max<uint64_t>(capacity, 1) * sizeof(MatchOut)));
   CV_CUDA(cudaMemcpy(b->segs_d, job.segs.data(), nseg * sizeof(Segment), cudaMemcpyHostToDevice));
   return CV_OK;
 }
 
-// Queue one complete run (status reset, scan, offsets, expand, counters to host) on stream.
+// Queue one complete run (status reset, scan, offsets and expansion, counters to host) on stream.
 int enqueue_run(DevCtx* ctx, int cfg_i, const TableView& tab, const Job& job, const Buffers& b, uint64_t capacity,
                 uint64_t* counters_h, cudaStream_t stream, cudaEvent_t ev0, cudaEvent_t ev1, int* launches) {
   int ncfg;
@@ -79,13 +75,16 @@ int enqueue_run(DevCtx* ctx, int cfg_i, const TableView& tab, const Job& job, co
   const size_t nseg = job.segs.size();
   const uint64_t n_out = job.n_tiles * (uint64_t)(cfg.T / 32);
   uint32_t* status = (uint32_t*)(b.counters_d + nseg + 1);
-  CV_CUDA(cudaMemsetAsync(status, 0, 8, stream));
+  unsigned long long* group_sum = (unsigned long long*)(b.counters_d + nseg + 2);
+  CV_CUDA(cudaMemsetAsync(status, 0, 8 + finish_groups(n_out) * 8ull, stream));
   ScanParams p;
   memset(&p, 0, sizeof p);
   p.tab = tab;
   p.hit_rec = b.hit_rec;
   p.tile_nhit = b.tile_nhit;
   p.tile_ntrip = b.tile_ntrip;
+  p.group_sum = group_sum;
+  p.group_log2 = finish_group_log2(n_out);
   p.status = status;
   // Under stream capture a plain record only orders the capture; the external flag makes it an
   // event-record node that every replay of the graph executes, so the timing events see each run.
@@ -106,17 +105,12 @@ int enqueue_run(DevCtx* ctx, int cfg_i, const TableView& tab, const Job& job, co
   cp.out = b.out_d;
   cp.out_cap = capacity;
   cp.status = status;
-  cp.tile_off = b.tile_off;
+  cp.group_sum = group_sum;
+  cp.group_log2 = p.group_log2;
+  cp.n_groups = finish_groups(n_out);
   cp.seg_off = b.counters_d;
   cp.total = b.counters_d + nseg;
-  if (n_out <= kFinishTiles) {
-    CV_CUDA((cudaError_t)launch_finish(cfg, cp, ctx->sms, stream));
-  } else {
-    CV_CUDA((cudaError_t)launch_tile_offsets(b.tile_ntrip, n_out, b.tile_off, cp.segs, (uint32_t)(cfg.T / 32),
-                                             cp.seg_off, cp.total, b.off_scratch, stream, status));
-    if (launches) *launches += 2;
-    CV_CUDA((cudaError_t)launch_expand(cfg, cp, ctx->sms, stream));
-  }
+  CV_CUDA((cudaError_t)launch_finish(cfg, cp, ctx->sms, stream));
   if (launches) *launches += 1;
   if (counters_h) CV_CUDA(cudaMemcpyAsync(counters_h, b.counters_d, (nseg + 2) * 8, cudaMemcpyDeviceToHost, stream));
   return CV_OK;

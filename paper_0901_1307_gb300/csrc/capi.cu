@@ -517,24 +517,21 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
         Segment* segs_d;
         uint4* hit_rec;
         uint32_t *tile_nhit, *status;
-        uint64_t *tile_ntrip, *tile_off = nullptr, *seg_off_d, *off_scratch = nullptr;
+        uint64_t *tile_ntrip, *seg_off_d;
         // compaction works on output tiles of 32 sectors, T / 32 per scan tile
         const uint64_t n_out = nt * (uint64_t)(cfg.T / 32);
-        const bool small = n_out <= kFinishTiles;  // offsets and expansion in one launch
+        const uint32_t n_groups = finish_groups(n_out);
         Carve carve;
         carve.add(&hit_rec, n_out * 32 * sizeof(uint4));
         carve.add(&tile_nhit, n_out * 4);
         carve.add(&tile_ntrip, n_out * 8);
-        if (!small) {
-          carve.add(&tile_off, n_out * 8);
-          carve.add(&off_scratch, tile_offsets_scratch_words(n_out) * 8);
-        }
-        // seg_off[nseg], total, status, hit sectors, rejected candidates
-        carve.add(&seg_off_d, (nseg + 4) * 8);
+        // seg_off[nseg], total, status, hit sectors, rejected candidates; triples per group of tiles
+        carve.add(&seg_off_d, (nseg + 4 + n_groups) * 8);
         CV_TRY(carve.commit(tmp));
         status = (uint32_t*)(seg_off_d + nseg + 1);
         status_keep = status;
-        CV_CUDA(cudaMemsetAsync(status, 0, 24, stream));
+        unsigned long long* group_sum = (unsigned long long*)(seg_off_d + nseg + 4);
+        CV_CUDA(cudaMemsetAsync(status, 0, 24 + n_groups * 8ull, stream));
         CV_TRY(job.segs_device(&segs_d, tmp, stream));
         ScanParams p;
         memset(&p, 0, sizeof p);
@@ -542,6 +539,8 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
         p.hit_rec = hit_rec;
         p.tile_nhit = tile_nhit;
         p.tile_ntrip = tile_ntrip;
+        p.group_sum = group_sum;
+        p.group_log2 = finish_group_log2(n_out);
         p.status = status;
         p.rejected = (unsigned long long*)(seg_off_d + nseg + 3);
         CV_CUDA(cudaEventRecord(ev[1], stream));
@@ -581,7 +580,9 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
         cp.n_out_tiles = n_out;
         cp.segs = seg_list(job.segs.data(), segs_d, nseg);
         cp.status = status;
-        cp.tile_off = tile_off;
+        cp.group_sum = group_sum;
+        cp.group_log2 = p.group_log2;
+        cp.n_groups = n_groups;
         cp.seg_off = seg_off_d;
         cp.total = seg_off_d + nseg;
         cp.nhit_sum = (unsigned long long*)(seg_off_d + nseg + 2);
@@ -589,33 +590,21 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
           CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, room * sizeof(MatchOut), ctx->pool, stream));
           cp.out = r->dev_out;
           cp.out_cap = room;
-          CV_CUDA((cudaError_t)(small ? launch_finish(cfg, cp, ctx->sms, stream)
-                                      : launch_expand(cfg, cp, ctx->sms, stream)));
+          CV_CUDA((cudaError_t)launch_finish(cfg, cp, ctx->sms, stream));
           r->launches += 1;
           return CV_OK;
         };
-        // the offsets, and the sectors with a match summed in the same pass
-        if (!small) {
-          CV_CUDA((cudaError_t)launch_tile_offsets(tile_ntrip, n_out, tile_off, cp.segs, (uint32_t)(cfg.T / 32),
-                                                   seg_off_d, cp.total, off_scratch, stream, status, tile_nhit,
-                                                   seg_off_d + nseg + 2));
-          r->launches += 2;
-        }
-        // The expand pass needs an output buffer before the exact count is known on the host.
-        // After a scan against the same table it is launched at once, with room for a quarter more
-        // than that scan's matches (one wait for the whole call); the exact count then tells
-        // whether the room sufficed (the pass writes nothing beyond it and flags the overflow),
-        // and only if not is it run again into an exact buffer. A small scan, whose offsets come
-        // from the same launch, has room for 4,096 matches at least.
+        // The last pass needs an output buffer before the exact count is known on the host: it is
+        // launched with room for a quarter more than the last scan's matches against the same table
+        // (4,096 at least), so that the call waits once; the exact count then tells whether the room
+        // sufficed (the pass writes nothing beyond it and flags the overflow), and only if not is it
+        // run again into an exact buffer.
         const uint64_t hint = __atomic_load_n(&const_cast<cv_master*>(m)->last_matches, __ATOMIC_RELAXED);
-        uint64_t room = 0;
-        if (hint || small) {
-          room = std::max<uint64_t>(hint + hint / 4 + 1024, small ? 4096 : 0);
-          CV_TRY(expand(room));
-        }
+        const uint64_t room = std::max<uint64_t>(hint + hint / 4 + 1024, 4096);
+        CV_TRY(expand(room));
         rb.emplace(ctx, seg_off.data(), seg_off_d, nseg + 4, stream);
         CV_TRY(rb->counts());
-        if (room && !r->on_device) CV_TRY(rb->matches(r->dev_out, room));
+        if (!r->on_device) CV_TRY(rb->matches(r->dev_out, room));
         // the call's end unless more work follows (then recorded again after it): in the common
         // case this one wait for the stream is the call's only one
         CV_CUDA(cudaEventRecord(ev[3], stream));

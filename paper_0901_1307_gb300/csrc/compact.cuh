@@ -1,12 +1,10 @@
 // Second half of the match compaction: the per-tile triple counts of the scan are turned into
-// output offsets by one exclusive scan, then every hit record of every tile is expanded into
-// its (disk_sector, file_id, file_sector) triples, in one kernel for scans of up to kFinishTiles
-// output tiles and in three for larger ones. Tiles are in sector order, the records of a
+// output offsets by an exclusive scan, and every hit record of every tile is expanded into
+// its (disk_sector, file_id, file_sector) triples. Tiles are in sector order, the records of a
 // tile are in sector order (ballot ranks), and each digest's postings are sorted by
-// (file_id, file_sector), so the output is sorted without a sort; the only waits between thread
-// blocks are the offset scan's bounded look-back. (The paper's Section 3.2 writes matches to a
-// host-visible buffer in no stated order; the sorted triple list is this library's output
-// format.)
+// (file_id, file_sector), so the output is sorted without a sort. (The paper's Section 3.2 writes
+// matches to a host-visible buffer in no stated order; the sorted triple list is this library's
+// output format.)
 #pragma once
 #include <stdint.h>
 
@@ -14,10 +12,10 @@
 
 namespace cvk {
 
-// Exclusive scan of the per-tile triple counts in one pass: each block scans a chunk and adds
-// its predecessors' published sums (decoupled look-back, every wait bounded). A second small pass
-// reads off each segment's first offset. (The kernels are in kernels_scan.cu; this header holds
-// the expand pass, instantiated with each configuration.)
+// Exclusive scan of per-tile counts in one pass, for the serving loop and the fragment scans: each
+// block scans a chunk and adds its predecessors' published sums (decoupled look-back, every wait
+// bounded). A second small pass reads off each segment's first offset. (These kernels are in
+// kernels_scan.cu; this header holds the passes instantiated with each configuration.)
 constexpr int kOffThreads = 1024;
 constexpr int kOffItems = 4;
 constexpr uint64_t kOffChunk = (uint64_t)kOffThreads * kOffItems;
@@ -34,8 +32,11 @@ struct CompactParams {
   MatchOut* out;
   uint64_t out_cap;
   uint32_t* status;
-  const uint64_t* tile_off;    // expand pass: output offset per tile
-  uint64_t* seg_off;           // one-kernel pass: out, the offset of every segment's first tile
+  const uint64_t* tile_off;    // expand_kernel: output offset per tile
+  const unsigned long long* group_sum;  // finish_kernel: triples per 2^group_log2 tiles
+  uint32_t group_log2;
+  uint32_t n_groups;           // at most kFinishGroups
+  uint64_t* seg_off;           // out, the offset of every segment's first tile
   uint64_t* total;             // out, the sum of the triple counts
   unsigned long long* nhit_sum;  // the sectors with a match are added to it (null: not counted)
 };
@@ -113,12 +114,10 @@ __device__ __forceinline__ void expand_group(const CompactParams& p, uint64_t u0
   }
 }
 
-// The hits of the group's tiles and their numbering: returns their number; my_n, my_first: this
-// lane's tile.
-__device__ __forceinline__ uint32_t group_hits(const CompactParams& p, uint64_t u0, uint32_t& my_n,
-                                               uint32_t& my_first) {
+// The numbering of the hits of the warp's tiles (this lane's has my_n): returns their number;
+// my_first: the first of this lane's.
+__device__ __forceinline__ uint32_t group_hits(uint32_t my_n, uint32_t& my_first) {
   const uint32_t lane = threadIdx.x & 31;
-  my_n = u0 + lane < p.n_out_tiles ? p.tile_nhit[u0 + lane] : 0u;
   uint32_t incl = my_n;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -129,122 +128,161 @@ __device__ __forceinline__ uint32_t group_hits(const CompactParams& p, uint64_t 
   return __shfl_sync(0xFFFFFFFFu, incl, 31);
 }
 
-// The second pass over offsets made before (larger scans). When the scan before it on the stream
-// failed (a wait timed out or a lookup ran past the probe bound: its hit records are not to be
-// trusted), the pass writes nothing.
+// The expansion alone, over offsets made before (the serving loop, whose host reads the counts in
+// between). When the scan before it on the stream failed (a wait timed out or a lookup ran past the
+// probe bound: its hit records are not to be trusted), the pass writes nothing.
 template <int T>
 __global__ void expand_kernel(const __grid_constant__ CompactParams p) {
   if (*(volatile const uint32_t*)p.status & (kStTimeout | kStProbeBound | kStBadTable)) return;
   const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
   for (uint64_t u0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; u0 < p.n_out_tiles;
        u0 += warps * 32) {
-    uint32_t my_n, my_first;
-    const uint32_t n_rec = group_hits(p, u0, my_n, my_first);
+    const uint64_t u = u0 + (threadIdx.x & 31);
+    const uint32_t my_n = u < p.n_out_tiles ? p.tile_nhit[u] : 0u;
+    uint32_t my_first;
+    const uint32_t n_rec = group_hits(my_n, my_first);
     if (n_rec == 0u) continue;
-    expand_group<T>(p, u0, my_n, my_first, n_rec, my_n ? p.tile_off[u0 + (threadIdx.x & 31)] : 0ull);
+    expand_group<T>(p, u0, my_n, my_first, n_rec, my_n ? p.tile_off[u] : 0ull);
   }
 }
 
-// Offsets and expansion in one launch, for scans of at most kFinishTiles output tiles: every block
-// sums all groups of 32 tiles and scans the sums itself (at most 1 MB, from L2), then expands its
-// share of the groups; block 0 writes the total and the segments' offsets. One launch in place of a
-// memset and three, whose gaps and latencies are what a small scan's second half consists of: 64 KiB
-// 6.6 us against 11.9 and the gaps (call 79 against 89 us), 1 GiB (65,540 tiles) 17.7 against 18.2
-// and the gaps (call 322 against 331). A warp loads eight groups' counts at a time: one by one the
-// 1 GiB scan's took 38 us. Above kFinishTiles every block's pass over all tiles costs more than
-// the three launches.
-constexpr uint64_t kFinishTiles = 1ull << 17;
-constexpr int kFinishThreads = 1024;
+// Offsets and expansion in one launch. The scan has summed its triples by groups of tiles (an atomic
+// for a tile that has any); every block scans these sums, at most kFinishGroups, and takes groups: a
+// thread per tile, 512 at a time, their counts scanned over the block, then a warp per 32 tiles
+// expands. What bounds it is latency: the sums, the counts, then for tiles with hits the record, the
+// posting and the write, each waiting for the one before it; so the counts of the next 512 tiles are
+// loaded before these are expanded (without that 7.2, 10.9 and 74 us where the last column says 6.2,
+// 9.6 and 64), and a group without triples is passed over. It took the place of a memset and three
+// launches (look-back offset scan, segments' offsets, expansion), the gaps between them not counted
+// here:            three launches       this one
+//   64 KiB         4.2 + 2.8 + 4.9 us   6.2 us
+//   1 GiB          8.2 + 2.7 + 7.3      9.1
+//   2 GiB, CRC64   10.5 + 2.6 + 7.7     9.6
+//   32 GiB, 1,000,000 matches: 64
+// 512 tiles to a group up to 2^21 tiles (32 GiB), more above, so that the sums' scan stays at most
+// 4,096 words a block.
+constexpr uint32_t kFinishGroups = 4096;
+constexpr int kFinishThreads = 512;
+constexpr uint32_t kFinishMinLog2 = 9;  // a group is whole chunks of kFinishThreads tiles
+static_assert((1 << kFinishMinLog2) == kFinishThreads, "chunks of a tile per thread");
 
-template <int T>
-__global__ void __launch_bounds__(kFinishThreads) finish_kernel(const __grid_constant__ CompactParams p) {
-  extern __shared__ uint64_t s_group[];  // per group: its triples, then the triples before it
-  __shared__ uint64_t s_warp[33];
+// The group size for n output tiles.
+inline uint32_t finish_group_log2(uint64_t n) {
+  uint32_t l = kFinishMinLog2;
+  while (((n + (1ull << l) - 1) >> l) > kFinishGroups) l++;
+  return l;
+}
+inline uint32_t finish_groups(uint64_t n) {
+  const uint32_t l = finish_group_log2(n);
+  return (uint32_t)((n + (1ull << l) - 1) >> l);
+}
+
+// Exclusive scan of x over the kFinishThreads threads of a block; *total gets the sum. buf: 17 words.
+__device__ __forceinline__ uint64_t finish_scan(uint64_t x, uint64_t* buf, uint64_t* total) {
   constexpr uint32_t kFull = 0xFFFFFFFFu;
-  constexpr uint32_t kWarps = kFinishThreads / 32;
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t n_groups = (uint32_t)((p.n_out_tiles + 31) / 32);
-  constexpr uint32_t kAhead = 8;  // groups whose counts a warp loads at a time
-  for (uint32_t g0 = warp; g0 < n_groups; g0 += kWarps * kAhead) {
-    uint64_t n[kAhead];
-#pragma unroll
-    for (uint32_t k = 0; k < kAhead; k++) {
-      const uint64_t u = 32ull * (g0 + k * kWarps) + lane;
-      n[k] = u < p.n_out_tiles ? p.tile_ntrip[u] : 0ull;
-    }
-#pragma unroll
-    for (uint32_t k = 0; k < kAhead; k++) {
-      uint64_t sum = __reduce_add_sync(kFull, (uint32_t)n[k] & 0xFFFFFFu);
-      if (__any_sync(kFull, (n[k] >> 24) != 0u)) {  // keys with very many postings
-        uint64_t high = n[k] >> 24;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) high += __shfl_xor_sync(kFull, (unsigned long long)high, d);
-        sum += high << 24;
-      }
-      if (lane == 0 && g0 + k * kWarps < n_groups) s_group[g0 + k * kWarps] = sum;
-    }
-  }
-  __syncthreads();
-  // exclusive scan of the groups' sums: `per` consecutive ones a thread
-  const uint32_t per = (n_groups + kFinishThreads - 1) / kFinishThreads;
-  uint64_t mine = 0;
-  for (uint32_t k = 0; k < per; k++)
-    if (tid * per + k < n_groups) mine += s_group[tid * per + k];
-  uint64_t incl = mine;
+  constexpr int kWarps = kFinishThreads / 32;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint64_t incl = x;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const uint64_t v = __shfl_up_sync(kFull, (unsigned long long)incl, d);
     if (lane >= (uint32_t)d) incl += v;
   }
-  if (lane == 31) s_warp[warp] = incl;
+  if (lane == 31) buf[warp] = incl;
   __syncthreads();
   if (warp == 0) {
-    const uint64_t w = s_warp[lane];
+    const uint64_t w = lane < (uint32_t)kWarps ? buf[lane] : 0ull;
     uint64_t wi = w;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
+    for (int d = 1; d < kWarps; d <<= 1) {
       const uint64_t v = __shfl_up_sync(kFull, (unsigned long long)wi, d);
       if (lane >= (uint32_t)d) wi += v;
     }
-    s_warp[lane] = wi - w;
-    if (lane == 31) s_warp[32] = wi;
+    if (lane < (uint32_t)kWarps) buf[lane] = wi - w;
+    if (lane == kWarps - 1) buf[kWarps] = wi;
   }
   __syncthreads();
-  uint64_t run = s_warp[warp] + incl - mine;
-  for (uint32_t k = 0; k < per; k++) {
-    if (tid * per + k >= n_groups) break;
-    const uint64_t v = s_group[tid * per + k];
-    s_group[tid * per + k] = run;
-    run += v;
+  *total = buf[kWarps];
+  const uint64_t r = buf[warp] + incl - x;
+  __syncthreads();  // buf may be used again
+  return r;
+}
+
+template <int T>
+__global__ void __launch_bounds__(kFinishThreads) finish_kernel(const __grid_constant__ CompactParams p) {
+  __shared__ uint64_t s_group[kFinishGroups];  // triples before the group
+  __shared__ uint64_t s_off[kFinishThreads];   // offsets of the chunk's tiles
+  __shared__ uint64_t s_buf[kFinishThreads / 32 + 1];
+  constexpr uint32_t kPer = kFinishGroups / kFinishThreads;
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  uint64_t g[kPer], mine = 0, total;
+#pragma unroll
+  for (uint32_t k = 0; k < kPer; k++) {
+    g[k] = tid * kPer + k < p.n_groups ? p.group_sum[tid * kPer + k] : 0ull;
+    mine += g[k];
   }
-  __syncthreads();
-  if (blockIdx.x == 0) {
-    if (tid == 0) *p.total = s_warp[32];
-    const Segment* const segs = p.segs.get();
-    for (uint32_t s = tid; s < p.segs.n; s += kFinishThreads) {
-      const uint64_t u = segs[s].tile_base * (T / 32);
-      uint64_t off = u < p.n_out_tiles ? s_group[u / 32] : s_warp[32];
-      if (u < p.n_out_tiles)
-        for (uint64_t q = u & ~31ull; q < u; q++) off += p.tile_ntrip[q];
-      p.seg_off[s] = off;
-    }
+  uint64_t run = finish_scan(mine, s_buf, &total);
+#pragma unroll
+  for (uint32_t k = 0; k < kPer; k++) {
+    s_group[tid * kPer + k] = run;
+    run += g[k];
   }
+  if (blockIdx.x == 0 && tid == 0) *p.total = total;
+  const Segment* const segs = p.segs.get();
   const bool failed = *(volatile const uint32_t*)p.status & (kStTimeout | kStProbeBound | kStBadTable);
   uint32_t hits = 0;
-  for (uint32_t g = blockIdx.x * kWarps + warp; g < n_groups && !failed; g += gridDim.x * kWarps) {
-    const uint64_t u0 = 32ull * g;
-    uint32_t my_n, my_first;
-    const uint32_t n_rec = group_hits(p, u0, my_n, my_first);
-    if (n_rec == 0u) continue;
-    hits += n_rec;
-    uint64_t off = my_n ? p.tile_ntrip[u0 + lane] : 0ull;  // a tile without hits has no triples
-    const uint64_t own = off;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint64_t v = __shfl_up_sync(kFull, (unsigned long long)off, d);
-      if (lane >= (uint32_t)d) off += v;
+  __syncthreads();
+  // The block's chunks one after another; a chunk's counts are loaded while the one before it is
+  // expanded.
+  uint32_t gi = blockIdx.x;
+  uint64_t c0 = (uint64_t)gi << p.group_log2;
+  uint64_t next_trip = 0, next_at = 0;
+  uint32_t next_hit = 0;
+  const auto load = [&](uint32_t g_, uint64_t c_) {
+    const uint64_t u = c_ + tid;
+    const bool in = g_ < p.n_groups && u < p.n_out_tiles;
+    next_trip = in ? p.tile_ntrip[u] : 0ull;
+    next_hit = in ? p.tile_nhit[u] : 0u;
+  };
+  if (gi < p.n_groups) next_at = s_group[gi];
+  load(gi, c0);
+  while (gi < p.n_groups) {
+    const uint64_t at = next_at, trip = next_trip, first_tile = c0;
+    const uint32_t my_n = next_hit;
+    const uint64_t end = min(((uint64_t)gi + 1) << p.group_log2, p.n_out_tiles);
+    const bool empty = (gi + 1 < p.n_groups ? s_group[gi + 1] : total) == s_group[gi];
+    c0 += kFinishThreads;
+    const bool same_group = c0 < end;
+    if (!same_group) {
+      gi += gridDim.x;
+      c0 = (uint64_t)gi << p.group_log2;
     }
-    expand_group<T>(p, u0, my_n, my_first, n_rec, s_group[g] + off - own);
+    load(gi, c0);
+    uint64_t sum = 0, off = at;
+    if (!empty) off += finish_scan(trip, s_buf, &sum);
+    next_at = same_group ? at + sum : gi < p.n_groups ? s_group[gi] : 0ull;
+    if (p.segs.n > 1 || first_tile == 0) {  // segments that begin in this chunk
+      s_off[tid] = off;
+      __syncthreads();
+      const uint64_t c1 = min(first_tile + kFinishThreads, end);
+      uint32_t lo = 0, hi = p.segs.n;  // the first segment at or after the chunk's first tile
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (segs[mid].tile_base * (T / 32) < first_tile) lo = mid + 1; else hi = mid;
+      }
+      for (uint32_t s = lo + tid; s < p.segs.n; s += kFinishThreads) {
+        const uint64_t first = segs[s].tile_base * (T / 32);
+        if (first >= c1) break;
+        p.seg_off[s] = s_off[first - first_tile];
+      }
+      __syncthreads();
+    }
+    if (!empty && !failed) {
+      uint32_t my_first;
+      const uint32_t n_rec = group_hits(my_n, my_first);
+      if (n_rec) expand_group<T>(p, first_tile + tid - lane, my_n, my_first, n_rec, off);
+      hits += n_rec;
+    }
   }
   if (p.nhit_sum && lane == 0 && hits) atomicAdd(p.nhit_sum, (unsigned long long)hits);
 }

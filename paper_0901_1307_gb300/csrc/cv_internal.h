@@ -153,6 +153,8 @@ struct ScanParams {
   SegList segs;                      // this launch's segments
   uint32_t map_base;
   uint32_t one;         // always 1 (an opaque multiplier for the MD5 additions)
+  uint32_t group_log2;
+  uint32_t pad;
   uint64_t tile_begin;  // global index of the first tile of this launch
   uint64_t n_tiles;     // tiles of this launch
   TableView tab;
@@ -160,6 +162,7 @@ struct ScanParams {
   uint4* hit_rec;        // 32 records per output tile {lane, post_off, post_cnt, triples emitted}
   uint32_t* tile_nhit;   // hit sectors per output tile
   uint64_t* tile_ntrip;  // triples per output tile
+  unsigned long long* group_sum;  // triples per 2^group_log2 output tiles, zero before (null: not summed)
   uint32_t* status;
   // digest outputs (digest mode): indexed by segment sector_base + row
   uint4* digests;

@@ -42,22 +42,21 @@ const ScanCfg& digest_config_for(int cfg_i, int sig, uint64_t sectors, int sms, 
 // The expand pass (see expand_kernel). Returns a CUDA error code.
 struct CompactParams;
 int launch_expand(const ScanCfg& cfg, const CompactParams& p, int sms, void* stream);
-// Offsets and expansion in one launch, for at most kFinishTiles output tiles (see finish_kernel).
+// Offsets and expansion in one launch (see finish_kernel).
 int launch_finish(const ScanCfg& cfg, const CompactParams& p, int sms, void* stream);
 // The tables' side of CompactParams.
 void compact_table(CompactParams* p, const TableView& tab);
 
-// Scratch (u64 words) the offset pass needs for n tiles.
+// Scratch (u64 words) the offset pass (serving loop, fragment scans) needs for n tiles.
 uint64_t tile_offsets_scratch_words(uint64_t n_tiles);
 
 // tile_off[i] = sum of tile_ntrip[0..i) over the n_tiles output tiles; *total = sum of all;
 // seg_off[s] = offset of segment s's first output tile (segment tile_base * scale). scratch:
 // tile_offsets_scratch_words(n_tiles) u64 words. status: the scan's status word (kStTimeout if
-// a wait of the pass gives up). With tile_nhit, the sum of the n_tiles hit counts is added to
-// *nhit_sum (device memory, zeroed by the caller). Returns a CUDA error code.
+// a wait of the pass gives up). Returns a CUDA error code.
 int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* tile_off, const SegList& segs,
                         uint32_t scale, uint64_t* seg_off, uint64_t* total, uint64_t* scratch, void* stream,
-                        uint32_t* status, const uint32_t* tile_nhit = nullptr, uint64_t* nhit_sum = nullptr);
+                        uint32_t* status);
 
 // ---------------------------------------------------------------- fragment scans (Section 5)
 uint64_t frag_windows(uint64_t n_bytes);       // 64-byte windows at 4-byte offsets in n_bytes

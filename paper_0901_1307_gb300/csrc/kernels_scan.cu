@@ -1,5 +1,5 @@
-// The scan configurations (assembled from scan_cfgs_*.cu), the offset pass and the launch of the
-// second compaction pass.
+// The scan configurations (assembled from scan_cfgs_*.cu), the offset pass of the serving loop and
+// the fragment scans, and the launches of the compaction passes.
 #include <string.h>
 
 #include <algorithm>
@@ -11,7 +11,7 @@
 
 namespace cvk {
 
-// ------------------------------------------------------------ offset pass (first of two)
+// ------------------------------------------------------------ offset pass
 // Block-wide inclusive scan of one u64 per thread (1024 threads).
 __device__ __forceinline__ uint64_t block_inclusive_scan(uint64_t x, uint64_t* warp_buf) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -42,15 +42,12 @@ __device__ __forceinline__ uint64_t block_inclusive_scan(uint64_t x, uint64_t* w
 // (decoupled look-back). A block only waits for chunks taken by blocks that started before it,
 // and each wait is bounded by timeout_ns (kStTimeout in *status on expiry; the block then
 // publishes what it has, so no wait depends on it for longer). state: chunks words, then the
-// ticket, all zero before the launch. With nhit, the sum of the n hit counts is added to
-// *nhit_sum in the same pass.
+// ticket, all zero before the launch.
 constexpr uint64_t kLbAgg = 1ull << 62, kLbIncl = 2ull << 62, kLbValue = (1ull << 62) - 1;
 
 __global__ void __launch_bounds__(kOffThreads) lookback_scan_kernel(const uint64_t* v, uint64_t n, uint64_t* out,
                                                                     uint64_t* total, uint64_t* state, uint64_t chunks,
-                                                                    const uint32_t* nhit,
-                                                                    unsigned long long* nhit_sum, uint32_t* status,
-                                                                    uint64_t timeout_ns) {
+                                                                    uint32_t* status, uint64_t timeout_ns) {
   __shared__ uint64_t wb[32];
   __shared__ uint64_t s_chunk, s_prefix;
   if (threadIdx.x == 0) s_chunk = atomicAdd(reinterpret_cast<unsigned long long*>(state + chunks), 1ull);
@@ -59,18 +56,10 @@ __global__ void __launch_bounds__(kOffThreads) lookback_scan_kernel(const uint64
   const uint64_t first = chunk * kOffChunk + (uint64_t)threadIdx.x * kOffItems;
   uint64_t x[kOffItems];
   uint64_t sum = 0;
-  unsigned long long h = 0;
 #pragma unroll
   for (int k = 0; k < kOffItems; k++) {
-    const bool in = first + k < n;
-    x[k] = in ? v[first + k] : 0ull;
+    x[k] = first + k < n ? v[first + k] : 0ull;
     sum += x[k];
-    if (nhit && in) h += nhit[first + k];
-  }
-  if (nhit) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) h += __shfl_xor_sync(0xFFFFFFFFu, h, d);
-    if ((threadIdx.x & 31) == 0 && h) atomicAdd(nhit_sum, h);
   }
   const uint64_t incl = block_inclusive_scan(sum, wb);
   if (threadIdx.x == kOffThreads - 1) {
@@ -220,14 +209,10 @@ int launch_expand(const ScanCfg& cfg, const CompactParams& p, int sms, void* str
 }
 
 int launch_finish(const ScanCfg& cfg, const CompactParams& p, int sms, void* stream) {
-  if (p.n_out_tiles > kFinishTiles) return (int)cudaErrorInvalidValue;
-  const uint64_t groups = (p.n_out_tiles + 31) / 32;
-  // a warp per group, up to 64 blocks: each block reads every tile's count
-  uint64_t g = (groups + kFinishThreads / 32 - 1) / (kFinishThreads / 32);
-  g = std::max<uint64_t>(1, std::min<uint64_t>(g, std::min(sms, 64)));
+  if (p.n_groups > kFinishGroups) return (int)cudaErrorInvalidValue;
+  const unsigned g = std::max(1u, std::min(p.n_groups, (unsigned)sms * 4));
   void* args[] = {const_cast<CompactParams*>(&p)};
-  return (int)cudaLaunchKernel(cfg.finish_fn, dim3((unsigned)g), dim3(kFinishThreads), args, groups * 8,
-                               (cudaStream_t)stream);
+  return (int)cudaLaunchKernel(cfg.finish_fn, dim3(g), dim3(kFinishThreads), args, 0, (cudaStream_t)stream);
 }
 
 int launch_wait_selftest(uint32_t* status, uint64_t timeout_ns, void* stream) {
@@ -251,8 +236,7 @@ int launch_lookback_selftest(uint64_t* words, uint32_t* status, uint64_t timeout
   if (e != cudaSuccess) return (int)e;
   const uint64_t one = 1;
   if ((e = cudaMemcpyAsync(state + 2, &one, 8, cudaMemcpyHostToDevice, stream)) != cudaSuccess) return (int)e;
-  lookback_scan_kernel<<<1, kOffThreads, 0, stream>>>(v, 2 * kOffChunk, out, total, state, 2, nullptr, nullptr,
-                                                      status, timeout_ns);
+  lookback_scan_kernel<<<1, kOffThreads, 0, stream>>>(v, 2 * kOffChunk, out, total, state, 2, status, timeout_ns);
   return (int)cudaGetLastError();
 }
 
@@ -260,7 +244,7 @@ uint64_t tile_offsets_scratch_words(uint64_t n_tiles) { return (n_tiles + kOffCh
 
 int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* tile_off, const SegList& segs,
                         uint32_t scale, uint64_t* seg_off, uint64_t* total, uint64_t* scratch, void* stream_,
-                        uint32_t* status, const uint32_t* tile_nhit, uint64_t* nhit_sum) {
+                        uint32_t* status) {
   cudaStream_t stream = (cudaStream_t)stream_;
   const uint64_t chunks = (n_tiles + kOffChunk - 1) / kOffChunk;
   cudaError_t e;
@@ -268,8 +252,7 @@ int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* 
     // the look-back words and the ticket start at zero
     if ((e = cudaMemsetAsync(scratch, 0, (chunks + 1) * 8, stream)) != cudaSuccess) return (int)e;
     lookback_scan_kernel<<<(unsigned)chunks, kOffThreads, 0, stream>>>(
-        tile_ntrip, n_tiles, tile_off, total, scratch, chunks, tile_nhit,
-        reinterpret_cast<unsigned long long*>(nhit_sum), status, kWaitTimeoutNs);
+        tile_ntrip, n_tiles, tile_off, total, scratch, chunks, status, kWaitTimeoutNs);
   } else if ((e = cudaMemsetAsync(total, 0, 8, stream)) != cudaSuccess) {
     return (int)e;
   }

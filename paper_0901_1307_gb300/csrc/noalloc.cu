@@ -14,7 +14,7 @@
 //   - An image may hold at most CV_NOALLOC_MAX_SECTORS whole sectors (256 MiB); larger
 //     requests are refused with CV_EINVAL before any work is queued.
 //   - Every call on a device uses the same array, and it keeps the previous call's contents.
-//     The status word is cleared at the start of each call; the kernels rewrite everything
+//     The status word and the sums are cleared at the start of each call; the kernels rewrite everything
 //     else they read. Two calls whose work overlaps on the GPU (different streams or host
 //     threads without ordering) race on the array and give wrong results: serialize them.
 //   - The first call on each device does a one-time set-up with that device current (the
@@ -44,11 +44,11 @@ namespace {
 // Scratch layout (offsets in bytes); sized for CV_NOALLOC_MAX_SECTORS with the smallest tile.
 constexpr uint64_t kMaxSectors = CV_NOALLOC_MAX_SECTORS;
 constexpr uint64_t kMaxTiles = kMaxSectors / 32 + 32;  // output tiles of 32 sectors, plus a ragged tile
-constexpr uint64_t kOffCounters = 256;                          // seg_off[1], total, status
-constexpr uint64_t kOffNhit = 512;                              // u32 per tile
+constexpr uint64_t kOffCounters = 256;  // seg_off[1], total, status, triples per group of tiles
+constexpr uint64_t kOffNhit = 1024;     // u32 per tile
 constexpr uint64_t kOffNtrip = kOffNhit + ((kMaxTiles * 4 + 255) / 256) * 256;  // u64 per tile
 constexpr uint64_t kOffHits = kOffNtrip + ((kMaxTiles * 8 + 255) / 256) * 256;  // uint4 per sector slot
-static_assert(kMaxTiles <= kFinishTiles, "offsets and expansion in one launch");
+static_assert(kOffCounters + 24 + (kMaxTiles / kFinishThreads + 1) * 8 <= kOffNhit, "counters");
 constexpr uint64_t kHitSlots = kMaxTiles * 32;
 constexpr uint64_t kNoAllocScratchBytes = kOffHits + kHitSlots * 16;
 
@@ -166,7 +166,8 @@ extern "C" int cv_scan_noalloc(const cv_master* m, const void* image, uint64_t n
   if (n_out_tiles > kMaxTiles) return CV_EINVAL;                   // tile wider than the layout allows
 
   cudaError_t e;
-  if ((e = cudaMemsetAsync(status_d, 0, 4, stream)) != cudaSuccess) return fail(e);
+  unsigned long long* group_sum = (unsigned long long*)(seg_off_d + 3);
+  if ((e = cudaMemsetAsync(status_d, 0, 8 + finish_groups(n_out_tiles) * 8ull, stream)) != cudaSuccess) return fail(e);
 
   p.segs = seg_list(&seg, nullptr, 1);
   p.map_base = 0;
@@ -177,6 +178,8 @@ extern "C" int cv_scan_noalloc(const cv_master* m, const void* image, uint64_t n
   p.hit_rec = hit_rec;
   p.tile_nhit = tile_nhit;
   p.tile_ntrip = tile_ntrip;
+  p.group_sum = group_sum;
+  p.group_log2 = finish_group_log2(n_out_tiles);
   p.status = status_d;
   void* sargs[] = {&p};
   if ((e = cudaLaunchKernel(cfg.scan_fn[table_kind(tab)], dim3((unsigned)n_tiles), dim3(cfg.threads), sargs, cfg.smem,
@@ -194,6 +197,9 @@ extern "C" int cv_scan_noalloc(const cv_master* m, const void* image, uint64_t n
   cp.out = (MatchOut*)out;
   cp.out_cap = out_capacity;
   cp.status = status_d;
+  cp.group_sum = group_sum;
+  cp.group_log2 = p.group_log2;
+  cp.n_groups = finish_groups(n_out_tiles);
   cp.seg_off = seg_off_d;
   cp.total = total_d;
   if ((e = (cudaError_t)launch_finish(cfg, cp, d->sms, stream)) != cudaSuccess) return fail(e);

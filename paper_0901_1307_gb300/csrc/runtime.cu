@@ -307,6 +307,8 @@ int launch_range(DevCtx* ctx, int cfg_i, bool digest, const Job& job, const Segm
     p.hit_rec = base.hit_rec;
     p.tile_nhit = base.tile_nhit;
     p.tile_ntrip = base.tile_ntrip;
+    p.group_sum = base.group_sum;
+    p.group_log2 = base.group_log2;
     p.status = base.status;
     p.digests = base.digests;
     p.trivial = base.trivial;

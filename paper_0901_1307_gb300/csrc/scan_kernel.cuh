@@ -517,6 +517,7 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
         if (lane == 0) {
           p.tile_nhit[u] = __popc(ballot);
           p.tile_ntrip[u] = wtrip;
+          if (wtrip && p.group_sum) atomicAdd(p.group_sum + (u >> p.group_log2), (unsigned long long)wtrip);
         }
       }
     }

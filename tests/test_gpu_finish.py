@@ -1,6 +1,7 @@
-"""The second half of a scan in one launch and in three: sizes around the limit between them, many
-postings per key, more matches than there is room for at first, images without matches, several
-images, and results that a first scan sized wrongly."""
+"""The second half of a scan, offsets and expansion in one launch over groups of 512 output tiles of 32
+sectors: sizes around a chunk, many groups and the end of the last one, many postings per key, more
+matches than there is room for at first, images without matches, several images, and results that a
+first scan sized wrongly."""
 import numpy as np
 import pytest
 
@@ -9,7 +10,7 @@ import oracle
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-LIMIT = (1 << 17) * 32  # sectors: output tiles of the one-launch form, 32 sectors each
+CHUNK = 512 * 32  # sectors of a group
 
 
 @pytest.fixture(scope="module")
@@ -22,8 +23,8 @@ def cv(cuda_device):
     return cvmod
 
 
-@pytest.mark.parametrize("n", [1, 31, 33, 128 * 32 + 5, LIMIT - 128, LIMIT, LIMIT + 1])
-def test_sizes_around_the_limit(cv, n):
+@pytest.mark.parametrize("n", [1, 31, 33, 128 * 32 + 5, CHUNK - 1, CHUNK, CHUNK + 1, 256 * CHUNK - 128, 256 * CHUNK + 1])
+def test_sizes_around_a_group(cv, n):
     """Matches in the first and last sector and every 4,097th between."""
     img = torch.randint(0, 256, (n * 512,), dtype=torch.uint8, device="cuda",
                         generator=torch.Generator("cuda").manual_seed(n))
@@ -74,3 +75,30 @@ def test_rejected_and_kept_postings_of_one_key(cv):
     with cv.master_build(files, signature=2) as m, cv.scan(m, [t]) as r:
         assert np.array_equal(r.matches(0), oracle.match_hash(img, files))
         assert r.stats()["confirm_rejected"] == 2 * 3 + 2 * 3
+
+
+@pytest.mark.parametrize("nosec", [4096 * 512 * 32 + 100])
+def test_groups_of_more_than_one_chunk(cv, nosec):
+    """Above 2^21 output tiles a group is 1,024 tiles: an offset follows from the chunk before it."""
+    if torch.cuda.mem_get_info()[0] < nosec * 600:
+        pytest.skip("not enough device memory")
+    img = torch.zeros(nosec * 512, dtype=torch.uint8, device="cuda")
+    at = sorted({*range(0, nosec, 99_991), *range(1024 * 32 * 7 - 40, 1024 * 32 * 7 + 40), nosec - 1})
+    rows = torch.randint(1, 256, (len(at), 512), dtype=torch.uint8, device="cuda",
+                         generator=torch.Generator("cuda").manual_seed(3))
+    img.view(nosec, 512)[torch.tensor(at, device="cuda")] = rows
+    cut = 64 << 20  # several images of one allocation: segments begin within groups
+    parts = [img[:512 * 1000], img[512 * 1000:512 * cut + 512 * 77], img[512 * cut + 512 * 77:]]
+    with cv.master_build([rows.reshape(-1)]) as m:
+        with cv.scan(m, [img]) as r:
+            got = r.matches(0)
+            assert got["disk_sector"].tolist() == at and got["file_sector"].tolist() == list(range(len(at)))
+        with cv.scan(m, parts) as r:
+            first, k = 0, 0
+            for i, p in enumerate(parts):
+                n = p.numel() // 512
+                want = [a - first for a in at if first <= a < first + n]
+                got = r.matches(i)
+                assert got["disk_sector"].tolist() == want
+                assert got["file_sector"].tolist() == list(range(k, k + len(want)))
+                first, k = first + n, k + len(want)

@@ -235,11 +235,12 @@ typedef struct {
 int cv_scan_get_stats(const cv_result* r, cv_scan_stats* st);
 
 /*
- * Lookup cost, counted exactly: what the scan of an image reads from the table (the paper's
- * occupancy study, Section 4, Figures 10-12). The scan's own lookups are replayed outside the
- * scan kernel (which keeps no counters): the Bloom test when the table has a filter, then
+ * Lookup cost, counted exactly: what the lookups of an image's sectors read from the table (the
+ * paper's occupancy study, Section 4, Figures 10-12), replayed outside the scan kernel (which
+ * keeps no counters): the Bloom test when the table has a filter, then
  * the linear-probing walk from the home slot of Eq. 3 up to the table's probe bound (hash
- * layout), or the bisection over the sorted key words and the comparison of the records that
+ * layout; in a table without a filter the scan itself walks a byte per slot and reads the
+ * slots whose byte agrees), or the bisection over the sorted key words and the comparison of the records that
  * share the sector's key word (sorted layout).
  *   image        device pointer, 16-byte aligned; n_bytes / 512 whole sectors are looked up.
  *   base_offset  as cv_scan_opts.base_offset (position-keyed tables).

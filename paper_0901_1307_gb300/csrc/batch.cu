@@ -123,10 +123,10 @@ struct TuneChoice {
 };
 std::map<std::string, TuneChoice> g_tune;  // key -> choice
 
-// table_kind: signature, layout and position keying of the table; unique and occupancy (in
+// table_key: signature, layout and position keying of the table; unique and occupancy (in
 // tenths of the slots): they change the probe's cost and so the choice.
 std::string tune_key(const char* gpu, int sms, uint64_t sectors, uint32_t images, uint64_t unique, uint32_t occupancy,
-                     bool bloom_avail, uint32_t table_kind) {
+                     bool bloom_avail, uint32_t table_key) {
   auto lg = [](uint64_t x) {
     int b = 0;
     while (x > 1) {
@@ -141,7 +141,7 @@ std::string tune_key(const char* gpu, int sms, uint64_t sectors, uint32_t images
     if (ch == ' ' || ch == '\t') ch = '_';
   char buf[256];
   snprintf(buf, sizeof buf, "%s|%d|s%d|i%d|u%d|o%u|b%d|t%u", name.c_str(), sms, lg(sectors), lg(images), lg(unique),
-           occupancy, bloom_avail ? 1 : 0, table_kind);
+           occupancy, bloom_avail ? 1 : 0, table_key);
   return buf;
 }
 
@@ -317,7 +317,7 @@ int cv_batch_create(const cv_master* m, const cv_buf* images, uint32_t n_images,
       CV_CUDA(cudaGetDeviceProperties(&prop, ctx->dev));
       const uint64_t n_slots = tab.layout == kLayoutSorted ? tab.n_keys : (uint64_t)tab.slot_mask + 1;
       const uint32_t tenths = (uint32_t)(10ull * tab.n_keys / std::max<uint64_t>(n_slots, 1));
-      const uint32_t tkey = (uint32_t)table_kind(tab) * 2u + (tab.tau_mask ? 1u : 0u);
+      const uint32_t tkey = (tab.sig + 4u * tab.layout) * 2u + (tab.tau_mask ? 1u : 0u);
       const std::string key =
           tune_key(prop.name, ctx->sms, total_sectors, n_images, tab.n_keys, tenths, bloom_avail, tkey);
       TuneChoice tc;

@@ -61,6 +61,9 @@ __host__ __device__ constexpr bool sig_is_weak(int sig) { return sig == kSigDjb2
 //   bloom: 8 u32 words (32 bytes) per block; block tau_block(d3, tau) & bloom_mask; in word j the bit
 //          (d1 >> 5j) & 31 for j < 6, (d2 >> 5(j-6)) & 31 for j = 6, 7.
 //   confirm: for 64-bit signatures, the master sector bytes of posting q at confirm + 512 q.
+//   tags: a byte per slot of a hash table without a filter, slot_tag(d2) or 0 for an empty slot (null:
+//          none): a lookup walks these and reads the slots whose byte is its own. Made from the
+//          slots, behind them in the same array, not part of a table file.
 //   sorted layout: slots holds n_keys records (no empty ones) in ascending order of
 //          h0 = tau_home(d0, tau), and keys0[q] is record q's h0: a lookup is a binary search of
 //          keys0 (the alternative to linear probing for high occupancy, Section 4), then a
@@ -76,6 +79,7 @@ struct TableView {
   const uint4* bloom;
   const uint8_t* confirm;
   const uint32_t* keys0;  // sorted layout only
+  const uint8_t* tags;      // hash layout of sector tables without a filter
   const uint32_t* frag_l1;  // fragment tables: the shared-memory filter (kFragL1Bytes)
   uint32_t slot_mask;
   uint32_t bloom_mask;
@@ -88,6 +92,12 @@ struct TableView {
   uint32_t n_keys;     // sorted layout: records in slots and keys0
   uint32_t unit;       // kUnitSector or kUnitFragment
 };
+
+// The tag byte of an occupied slot, and which tables have tags (a lookup reads 16 at a time).
+__host__ __device__ inline uint32_t slot_tag(uint32_t d2) { return d2 >> 24 ? d2 >> 24 : 1u; }
+inline bool table_has_tags(uint32_t unit, uint32_t layout, uint64_t bloom_bytes, uint64_t n_slots) {
+  return unit == kUnitSector && layout == kLayoutHash && bloom_bytes == 0 && n_slots >= 64;
+}
 
 // Position-keyed tables (Section 3.1: one table S_tau per sector position tau of an 8-sector
 // cluster) are stored as one open-addressing table whose key is (signature, tau): tau moves the

@@ -244,6 +244,20 @@ int gather_master_units(DevCtx* ctx, const cv_buf* files, uint32_t n_files, cons
   return rc;
 }
 
+// Bytes of the records of a table as they are held, with the tags or key words that belong to them.
+uint64_t table_records_bytes(const cv_master_info& in) {
+  if (in.layout == kLayoutSorted) return std::max<uint64_t>(in.n_unique, 1) * 36;
+  return in.n_slots * (table_has_tags(in.unit, in.layout, in.bloom_bytes, in.n_slots) ? 33 : 32);
+}
+
+// Device memory of a table: the records, a posting and, for 64-bit signatures, the unit's bytes per
+// master unit, the filters.
+uint64_t table_device_bytes(const cv_master_info& in) {
+  const bool frag = in.unit == kUnitFragment;
+  return table_records_bytes(in) + std::max<uint64_t>(in.n_sectors, 1) * 8 + in.bloom_bytes +
+         (sig_is_weak((int)in.signature) ? in.n_sectors * (frag ? kFrag : kSector) : 0) + (frag ? kFragL1Bytes : 0);
+}
+
 // The sorted layout of a hash table's occupied slots (Section 4: binary search for high
 // occupancy): the nu occupied records, compacted in slot order, then sorted by h0 =
 // tau_home(d0, tau) (a stable sort, so the order is deterministic), and their h0 words. The
@@ -371,7 +385,10 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       CV_CUDA(cudaMemcpyAsync(file_base_d, file_base.data(), (n_files + 1) * 8, cudaMemcpyHostToDevice, stream));
       CV_TRY(gather_master_units(ctx, files, n_files, file_base, U, tmp, stream, &arena));
       // long-lived table memory
-      CV_TRY(table_alloc(ctx, &m->slots, n_slots * 32, stream));
+      // (a table whose layout is the library's to choose has tags until it is sorted)
+      const bool tagged = table_has_tags(unit, layout == CV_LAYOUT_SORTED ? kLayoutSorted : kLayoutHash, bpk, n_slots);
+      CV_TRY(table_alloc(ctx, &m->slots, n_slots * (tagged ? 33 : 32), stream));
+      uint8_t* const tags = tagged ? (uint8_t*)m->slots + n_slots * 32 : nullptr;
       CV_TRY(table_alloc(ctx, &m->postings, std::max<uint64_t>(M, 1) * 8, stream));
       // Bloom blocks: 32 bytes for sector tables, one 32-bit word for fragment tables
       const uint64_t block_bytes = frag ? 4 : 32;
@@ -408,7 +425,7 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       CV_CUDA(cudaGetLastError());
       CV_TRY(scan_u32(first, chunks, sums, stream));
       table_slots_kernel<<<chunks, kSlotThreads, 0, stream>>>(
-          owner, extra, (uint32_t)n_slots, first, dig, tau, post, (uint4*)m->slots, (uint2*)m->postings, member,
+          owner, extra, (uint32_t)n_slots, first, dig, tau, post, (uint4*)m->slots, tags, (uint2*)m->postings, member,
           frag ? nullptr : (uint32_t*)m->bloom, bpk ? (uint32_t)(n_blocks - 1) : 0u, counters + 2);
       CV_CUDA(cudaGetLastError());
       if (M && frag)
@@ -444,6 +461,7 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       m->tab.slots = (const uint4*)m->slots;
       m->tab.keys0 = (const uint32_t*)m->keys0;
       m->tab.layout = layout;
+      m->tab.tags = layout == CV_LAYOUT_SORTED ? nullptr : tags;
       m->tab.n_keys = hc[2];
       m->tab.postings = (const uint2*)m->postings;
       m->tab.bloom = (const uint4*)m->bloom;
@@ -468,11 +486,8 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
       m->info.bloom_bytes = n_blocks * block_bytes;
       m->info.max_probe = layout == CV_LAYOUT_SORTED ? steps : hc[0] + 1;
       m->info.layout = layout;
-      const uint64_t table_bytes =
-          layout == CV_LAYOUT_SORTED ? std::max<uint64_t>(hc[2], 1) * 36 : n_slots * 32;
       if (layout == CV_LAYOUT_SORTED) m->info.n_slots = hc[2];
-      m->info.device_bytes = table_bytes + std::max<uint64_t>(M, 1) * 8 + n_blocks * block_bytes +
-                             (m->confirm ? M * U : 0) + (m->frag_l1 ? kFragL1Bytes : 0);
+      m->info.device_bytes = table_device_bytes(m->info);
       return CV_OK;
     };
     rc = body();
@@ -635,6 +650,7 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
   }
   m->magic = kMagicMaster;
   m->dev = ctx->dev;
+  const bool tagged = table_has_tags(h.unit, h.layout, in.bloom_bytes, in.n_slots);
   auto body = [&]() -> int {
     void** arrays[6] = {&m->slots, &m->postings, &m->bloom, &m->confirm, &m->keys0, &m->frag_l1};
     const uint64_t sizes[6] = {h.bytes_slots, h.bytes_postings, h.bytes_bloom, h.bytes_confirm, h.bytes_keys0,
@@ -642,7 +658,8 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
     const bool always[6] = {true, true, false, false, false, false};  // the build allocates these even when empty
     for (int k = 0; k < 6; k++) {
       if (!sizes[k] && !always[k]) continue;
-      CV_TRY(table_alloc(ctx, arrays[k], std::max<uint64_t>(sizes[k], 32), stream));
+      const uint64_t held = k == 0 && tagged ? n_records * 33 : sizes[k];
+      CV_TRY(table_alloc(ctx, arrays[k], std::max<uint64_t>(held, 32), stream));
       CV_CUDA(cudaStreamSynchronize(stream));  // the copies below are not in the stream's order
       if (sizes[k]) CV_TRY(copy_from_file(f, *arrays[k], sizes[k]));
     }
@@ -685,6 +702,14 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
     m->tab.n_keys = h.n_keys;
     m->tab.unit = h.unit;
     m->info = in;
+    if (tagged) {
+      uint8_t* const tags = (uint8_t*)m->slots + n_records * 32;
+      slot_tags_kernel<<<grid_for(n_records, 256, ctx->sms), 256, 0, stream>>>((const uint4*)m->slots, n_records, tags);
+      CV_CUDA(cudaGetLastError());
+      CV_CUDA(cudaStreamSynchronize(stream));
+      m->tab.tags = tags;
+    }
+    m->info.device_bytes = table_device_bytes(in);
     return CV_OK;
   };
   const int rc = body();
@@ -722,6 +747,7 @@ int cvk::table_sorted_copy(const TableView& tab, cudaStream_t stream, TableView*
   out->slots = (const uint4*)*slots_out;
   out->keys0 = (const uint32_t*)*keys0_out;
   out->layout = kLayoutSorted;
+  out->tags = nullptr;
   out->n_keys = nu;
   return CV_OK;
 }
@@ -752,5 +778,6 @@ int cvk::table_bloom(const TableView& tab, uint32_t bits_per_key, cudaStream_t s
   out->bloom = (const uint4*)bloom;
   out->bloom_mask = (uint32_t)(n_blocks - 1);
   out->use_bloom = 1u;
+  out->tags = nullptr;  // behind a filter the walk over the slots
   return CV_OK;
 }

@@ -6,7 +6,8 @@
 // lookups outside it. It computes the key words of every sector with the scan's own digest
 // pass, then a counting kernel runs the scan's own lookup functions for each sector with a
 // counter attached: the Bloom test (when the table has a filter), then either the
-// linear-probing walk from the home slot of Eq. 3 (hash layout) or the bisection over the
+// linear-probing walk from the home slot of Eq. 3 (hash layout; the table's own measure, a scan of a
+// table without a filter reads the tags instead of most of these slots) or the bisection over the
 // sorted keys and the comparison of the records that share the key word (sorted layout).
 #include <cuda_runtime.h>
 #include <stdint.h>

@@ -310,10 +310,11 @@ __device__ __forceinline__ void store_slot(uint4* p, uint4 a, uint4 b) {
 }
 
 // counters: [0] keys, [1] members of keys with several. post: posting per master index; member: the
-// master index of every posting (null: not wanted). bloom: null for none.
+// master index of every posting (null: not wanted). tags: a byte per slot (null: not wanted). bloom: null
+// for none.
 __global__ void __launch_bounds__(kSlotThreads) table_slots_kernel(
     const uint32_t* owners, const uint32_t* extra, uint32_t n_slots, const uint32_t* first, const uint4* dig, const uint8_t* tau,
-    const uint2* post, uint4* slots, uint2* postings, uint32_t* member, uint32_t* bloom, uint32_t bloom_mask,
+    const uint2* post, uint4* slots, uint8_t* tags, uint2* postings, uint32_t* member, uint32_t* bloom, uint32_t bloom_mask,
     uint32_t* counters) {
   constexpr int kWarps = kSlotThreads / 32;
   constexpr uint32_t kFull = 0xFFFFFFFFu;
@@ -359,6 +360,7 @@ __global__ void __launch_bounds__(kSlotThreads) table_slots_kernel(
     const uint64_t i = base + 32u * k;
     const uint32_t off = off0 + before[k];
     const uint32_t has = __ballot_sync(kFull, owner[k] != 0u);
+    if (tags && i < n_slots) tags[i] = cnt[k] ? (uint8_t)slot_tag(d[k].z) : 0;
     if (i < n_slots) store_slot(slots + 2 * i, d[k], make_uint4(owner[k] ? off : 0u, cnt[k], t[k], 0u));
     if (cnt[k] == 1u) {
       postings[off] = po[k];
@@ -473,6 +475,12 @@ __global__ void validate_slots_kernel(const uint4* slots, uint64_t n, uint64_t n
     const uint4 val = slots[2 * i + 1];
     if (val.y != 0u && (uint64_t)val.x + val.y > n_postings) atomicOr(status, kStBadTable);
   }
+}
+
+// The tags of a loaded table's slots.
+__global__ void slot_tags_kernel(const uint4* slots, uint64_t n, uint8_t* tags) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+    tags[i] = slots[2 * i + 1].y ? (uint8_t)slot_tag(slots[2 * i].z) : 0;
 }
 
 // ----------------------------------------------------------------------------- Bloom

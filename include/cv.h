@@ -240,8 +240,9 @@ int cv_scan_get_stats(const cv_result* r, cv_scan_stats* st);
  * keeps no counters): the Bloom test when the table has a filter, then
  * the linear-probing walk from the home slot of Eq. 3 up to the table's probe bound (hash
  * layout; in a table without a filter the scan itself walks a byte per slot and reads the
- * slots whose byte agrees), or the bisection over the sorted key words and the comparison of the records that
- * share the sector's key word (sorted layout).
+ * slots whose byte agrees), or the bisection over all the sorted key words and the comparison of
+ * the records that share the sector's key word (sorted layout; the scan's own bisection begins
+ * in the bucket of the key that an index gives).
  *   image        device pointer, 16-byte aligned; n_bytes / 512 whole sectors are looked up.
  *   base_offset  as cv_scan_opts.base_offset (position-keyed tables).
  *   st           st->struct_size = sizeof(cv_probe_stats); filled on success.

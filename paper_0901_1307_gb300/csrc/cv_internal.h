@@ -67,7 +67,9 @@ __host__ __device__ constexpr bool sig_is_weak(int sig) { return sig == kSigDjb2
 //   sorted layout: slots holds n_keys records (no empty ones) in ascending order of
 //          h0 = tau_home(d0, tau), and keys0[q] is record q's h0: a lookup is a binary search of
 //          keys0 (the alternative to linear probing for high occupancy, Section 4), then a
-//          comparison of the records whose h0 is equal.
+//          comparison of the records whose h0 is equal. key_start[b], behind the keys in the same
+//          array, is the first record whose h0 >> key_shift is b or more: the search begins between
+//          key_start[h0 >> key_shift] and the next. Made from the keys, not part of a table file.
 enum : uint32_t { kLayoutHash = 0, kLayoutSorted = 1 };
 // What a table's keys are: 512-byte sectors, or 64-byte fragments (a fragment table's Bloom
 // filter is one u32 word per block, 3 bits per key: frag_bloom_word and frag_bloom_bits).
@@ -78,7 +80,8 @@ struct TableView {
   const uint2* postings;
   const uint4* bloom;
   const uint8_t* confirm;
-  const uint32_t* keys0;  // sorted layout only
+  const uint32_t* keys0;      // sorted layout only
+  const uint32_t* key_start;  // sorted layout only
   const uint8_t* tags;      // hash layout of sector tables without a filter
   const uint32_t* frag_l1;  // fragment tables: the shared-memory filter (kFragL1Bytes)
   uint32_t slot_mask;
@@ -91,7 +94,19 @@ struct TableView {
   uint32_t layout;     // kLayout*
   uint32_t n_keys;     // sorted layout: records in slots and keys0
   uint32_t unit;       // kUnitSector or kUnitFragment
+  uint32_t key_shift;  // sorted layout
+  uint32_t pad;
 };
+
+// The index over a sorted table's n keys (n < 2^27): 2^(32 - shift) buckets of h0's top bits, of 1 to
+// 2 keys on average when they are spread evenly.
+inline uint32_t key_index_shift(uint32_t n) {
+  uint32_t bits = 1;
+  while ((2u << bits) <= n) bits++;
+  return 32 - bits;
+}
+// Words of the keys and their index together.
+inline uint64_t sorted_key_words(uint32_t n) { return (uint64_t)n + (1ull << (32 - key_index_shift(n))) + 1; }
 
 // The tag byte of an occupied slot, and which tables have tags (a lookup reads 16 at a time).
 __host__ __device__ inline uint32_t slot_tag(uint32_t d2) { return d2 >> 24 ? d2 >> 24 : 1u; }

@@ -244,9 +244,25 @@ int gather_master_units(DevCtx* ctx, const cv_buf* files, uint32_t n_files, cons
   return rc;
 }
 
+// The index over n sorted keys, behind them in the same array.
+void key_index(DevCtx* ctx, void* keys0, uint32_t n, cudaStream_t stream) {
+  const uint32_t shift = key_index_shift(n);
+  key_index_kernel<<<grid_for((1ull << (32 - shift)) + 1, 256, ctx->sms), 256, 0, stream>>>(
+      (const uint32_t*)keys0, n, shift, (uint32_t*)keys0 + n);
+}
+
+// The sorted layout's part of a view.
+void view_keys(TableView* tab, const void* keys0, uint32_t n) {
+  tab->n_keys = n;
+  tab->keys0 = (const uint32_t*)keys0;
+  tab->key_start = keys0 ? tab->keys0 + n : nullptr;
+  tab->key_shift = key_index_shift(n);
+}
+
 // Bytes of the records of a table as they are held, with the tags or key words that belong to them.
 uint64_t table_records_bytes(const cv_master_info& in) {
-  if (in.layout == kLayoutSorted) return std::max<uint64_t>(in.n_unique, 1) * 36;
+  if (in.layout == kLayoutSorted) 
+    return std::max<uint64_t>(in.n_unique, 1) * 32 + sorted_key_words((uint32_t)in.n_unique) * 4;
   return in.n_slots * (table_has_tags(in.unit, in.layout, in.bloom_bytes, in.n_slots) ? 33 : 32);
 }
 
@@ -261,7 +277,7 @@ uint64_t table_device_bytes(const cv_master_info& in) {
 // The sorted layout of a hash table's occupied slots (Section 4: binary search for high
 // occupancy): the nu occupied records, compacted in slot order, then sorted by h0 =
 // tau_home(d0, tau) (a stable sort, so the order is deterministic), and their h0 words. The
-// caller owns *slots_out (nu records of 32 bytes) and *keys0_out (nu words); *steps receives
+// caller owns *slots_out (nu records of 32 bytes) and *keys0_out (the words, then their index); *steps receives
 // ceil(log2 nu), the bisection steps of a lookup. Returns after the work has finished.
 int sorted_from_hash(DevCtx* ctx, const uint4* slots, uint64_t n_slots, uint32_t nu, Temps& tmp, cudaStream_t stream,
                      void** slots_out, void** keys0_out, uint32_t* steps) {
@@ -284,7 +300,7 @@ int sorted_from_hash(DevCtx* ctx, const uint4* slots, uint64_t n_slots, uint32_t
   void* out = nullptr;
   void* keys0 = nullptr;
   CV_TRY(table_alloc(ctx, &out, std::max<uint64_t>(nu, 1) * 32, stream));
-  int rc = table_alloc(ctx, &keys0, std::max<uint64_t>(nu, 1) * 4, stream);
+  int rc = table_alloc(ctx, &keys0, sorted_key_words(nu) * 4, stream);
   if (rc != CV_OK) {
     cudaFreeAsync(out, stream);
     return rc;
@@ -292,6 +308,10 @@ int sorted_from_hash(DevCtx* ctx, const uint4* slots, uint64_t n_slots, uint32_t
   gather_slots_kernel<<<gu, 256, 0, stream>>>(slots, hv, nu, (uint4*)out);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && nu) e = cudaMemcpyAsync(keys0, hk, (uint64_t)nu * 4, cudaMemcpyDeviceToDevice, stream);
+  if (e == cudaSuccess) {
+    key_index(ctx, keys0, nu, stream);
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
     cudaFreeAsync(out, stream);
@@ -459,10 +479,9 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
         m->slots = sorted_slots;
       }
       m->tab.slots = (const uint4*)m->slots;
-      m->tab.keys0 = (const uint32_t*)m->keys0;
+      view_keys(&m->tab, m->keys0, hc[2]);
       m->tab.layout = layout;
       m->tab.tags = layout == CV_LAYOUT_SORTED ? nullptr : tags;
-      m->tab.n_keys = hc[2];
       m->tab.postings = (const uint2*)m->postings;
       m->tab.bloom = (const uint4*)m->bloom;
       m->tab.slot_mask = mask;
@@ -658,7 +677,7 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
     const bool always[6] = {true, true, false, false, false, false};  // the build allocates these even when empty
     for (int k = 0; k < 6; k++) {
       if (!sizes[k] && !always[k]) continue;
-      const uint64_t held = k == 0 && tagged ? n_records * 33 : sizes[k];
+      const uint64_t held = k == 0 && tagged ? n_records * 33 : k == 4 ? sorted_key_words(h.n_keys) * 4 : sizes[k];
       CV_TRY(table_alloc(ctx, arrays[k], std::max<uint64_t>(held, 32), stream));
       CV_CUDA(cudaStreamSynchronize(stream));  // the copies below are not in the stream's order
       if (sizes[k]) CV_TRY(copy_from_file(f, *arrays[k], sizes[k]));
@@ -689,7 +708,6 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
     m->tab.postings = (const uint2*)m->postings;
     m->tab.bloom = (const uint4*)m->bloom;
     m->tab.confirm = (const uint8_t*)m->confirm;
-    m->tab.keys0 = (const uint32_t*)m->keys0;
     m->tab.frag_l1 = (const uint32_t*)m->frag_l1;
     m->tab.slot_mask = h.slot_mask;
     m->tab.bloom_mask = h.bloom_mask;
@@ -699,7 +717,7 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
     m->tab.tau_mask = h.tau_mask;
     m->tab.tau_add = 0;
     m->tab.layout = h.layout;
-    m->tab.n_keys = h.n_keys;
+    view_keys(&m->tab, m->keys0, h.n_keys);
     m->tab.unit = h.unit;
     m->info = in;
     if (tagged) {
@@ -708,6 +726,11 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
       CV_CUDA(cudaGetLastError());
       CV_CUDA(cudaStreamSynchronize(stream));
       m->tab.tags = tags;
+    }
+    if (m->keys0) {
+      key_index(ctx, m->keys0, h.n_keys, stream);
+      CV_CUDA(cudaGetLastError());
+      CV_CUDA(cudaStreamSynchronize(stream));
     }
     m->info.device_bytes = table_device_bytes(in);
     return CV_OK;
@@ -745,10 +768,9 @@ int cvk::table_sorted_copy(const TableView& tab, cudaStream_t stream, TableView*
   CV_CUDA(cudaStreamSynchronize(stream));  // temporaries returned
   *out = tab;
   out->slots = (const uint4*)*slots_out;
-  out->keys0 = (const uint32_t*)*keys0_out;
+  view_keys(out, *keys0_out, nu);
   out->layout = kLayoutSorted;
   out->tags = nullptr;
-  out->n_keys = nu;
   return CV_OK;
 }
 

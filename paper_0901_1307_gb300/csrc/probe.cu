@@ -8,7 +8,8 @@
 // counter attached: the Bloom test (when the table has a filter), then either the
 // linear-probing walk from the home slot of Eq. 3 (hash layout; the table's own measure, a scan of a
 // table without a filter reads the tags instead of most of these slots) or the bisection over the
-// sorted keys and the comparison of the records that share the key word (sorted layout).
+// sorted keys and the comparison of the records that share the key word (sorted layout; over all
+// keys: a scan begins in a bucket of an index over them).
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -25,7 +26,7 @@ namespace {
 
 constexpr uint64_t kProfileChunk = 1ull << 22;  // sectors per digest pass (64 MiB of key words)
 
-// Adds up the reads of the scan's own probe loops (table_probe, sorted_probe).
+// Adds up the reads of the lookups' loops (table_probe, sorted_find).
 struct ProbeCount {
   uint64_t* slots;
   uint64_t* keys;
@@ -45,7 +46,8 @@ __global__ void probe_profile_kernel(const uint4* dig, uint64_t n, uint64_t sect
     if (tab.use_bloom && !bloom_test(tab, d.y, d.z, d.w, tau)) continue;
     passed++;
     uint32_t post_off = 0;
-    const uint32_t c = tab.layout == kLayoutSorted ? sorted_probe(tab, d.x, d.y, d.z, d.w, tau, post_off, cnt)
+    const uint32_t c = tab.layout == kLayoutSorted ? sorted_find(tab, d.x, d.y, d.z, d.w, tau, 0u, tab.n_keys, post_off,
+                                                                 cnt)
                                                    : table_probe(tab, d.x, d.y, d.z, d.w, tau, post_off, cnt);
     if (c) found++;
   }

@@ -468,6 +468,21 @@ __global__ void gather_slots_kernel(const uint4* slots, const uint32_t* vals, ui
   }
 }
 
+// The index over the sorted keys: start[b] = the first key whose top bits are b or more, a search
+// per bucket.
+__global__ void key_index_kernel(const uint32_t* keys, uint32_t n, uint32_t shift, uint32_t* start) {
+  const uint64_t buckets = 1ull << (32 - shift);
+  for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b <= buckets;
+       b += (uint64_t)gridDim.x * blockDim.x) {
+    uint32_t lo = 0, hi = n;
+    while (lo < hi) {
+      const uint32_t mid = lo + (hi - lo) / 2;
+      if ((uint64_t)keys[mid] < (b << shift)) lo = mid + 1; else hi = mid;
+    }
+    start[b] = lo;
+  }
+}
+
 // ------------------------------------------------------------------- loaded tables
 // Every occupied record of a loaded table must name postings inside [0, n_postings).
 __global__ void validate_slots_kernel(const uint4* slots, uint64_t n, uint64_t n_postings, uint32_t* status) {

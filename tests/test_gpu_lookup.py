@@ -54,3 +54,18 @@ def test_tables_without_a_filter(cv, tmp_path, sig, n, cluster):
             with cv.batch_create(m, [t]) as b:
                 b.run()
                 assert np.array_equal(cv.device_matches_to_numpy(b.matches(0)), want)
+
+
+@pytest.mark.parametrize("sig", [2, 3])
+def test_sorted_keys_in_one_bucket(cv, sig):
+    """Signatures whose low words (the sorted keys) are nearly all in one bucket of the index: sectors of
+    zeros but for their last bytes."""
+    rng = np.random.default_rng(sig)
+    rows = np.zeros((9000, 512), np.uint8)
+    rows[:, 510:] = rng.permutation(65536)[:9000].astype(">u2").view(np.uint8).reshape(-1, 2)
+    image = np.concatenate([rows[::2], rng.integers(0, 256, (500, 512), dtype=np.uint8), rows[:7000:3]]).reshape(-1)
+    files = [rows[:4000].reshape(-1), rows[4000:6500].reshape(-1)]
+    t = torch.from_numpy(image).cuda()
+    with cv.master_build(files, signature=sig, layout=cv.CV_LAYOUT_SORTED, bloom_bits_per_key=0) as m:
+        with cv.scan(m, [t]) as r:
+            assert np.array_equal(r.matches(0), oracle.match_hash(image, files))

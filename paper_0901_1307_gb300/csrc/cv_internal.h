@@ -72,7 +72,7 @@ __host__ __device__ constexpr bool sig_is_weak(int sig) { return sig == kSigDjb2
 //          key_start[h0 >> key_shift] and the next. Made from the keys, not part of a table file.
 enum : uint32_t { kLayoutHash = 0, kLayoutSorted = 1 };
 // What a table's keys are: 512-byte sectors, or 64-byte fragments (a fragment table's Bloom
-// filter is one u32 word per block, 3 bits per key: frag_bloom_word and frag_bloom_bits).
+// filter is one u32 word per block, 3 or 5 bits per key: frag_bloom_word and frag_bloom_bit).
 enum : uint32_t { kUnitSector = 0, kUnitFragment = 1 };
 
 struct TableView {

@@ -102,12 +102,15 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
       : "memory");
 }
 
-// The one-word Bloom filter of a fragment table. MD5 keys are mixed already; a djb2-64 key is represented by g, the low word of h less
-// the initial value's share (what the scan rolls), spread by two odd multipliers.
+// The one-word Bloom filter of a fragment table. A djb2-64 key is represented by g, the low word of h less
+// the initial value's share (what the scan rolls), spread by two odd multipliers. An MD5 key is
+// represented by its first word, which is final three operations before the end of the last block:
+// the filter's bits from the third word, the block from the fourth, needed two of these three for
+// every window (1.347 ms for 256 MiB then, 1.336 so).
 template <int SIG>
-__device__ __forceinline__ uint32_t frag_bloom_word(uint32_t g, uint32_t d3, uint32_t mask) {
+__device__ __forceinline__ uint32_t frag_bloom_word(uint32_t g, uint32_t mask) {
   if constexpr (SIG == kSigDjb2) return __umulhi(g * 0x9E3779B1u + 0x7F4A7C15u, mask + 1u);
-  return d3 & mask;
+  return g & mask;
 }
 
 // The key's bits of its word: three bit numbers, for djb2-64 (where the test is off the scan's
@@ -116,16 +119,16 @@ template <int SIG>
 constexpr int kFragBloomBits = SIG == kSigDjb2 ? 5 : 3;
 
 template <int SIG>
-__device__ __forceinline__ uint32_t frag_bloom_bit(uint32_t g, uint32_t d2, int k) {
+__device__ __forceinline__ uint32_t frag_bloom_bit(uint32_t g, int k) {
   if constexpr (SIG == kSigDjb2) return (g * 0x85EBCA77u + 0x27D4EB2Fu) >> (27 - 5 * k);  // g = 0: zero windows
-  return d2 >> (5 * k);
+  return (g * 0x9E3779B1u) >> (27 - 5 * k);  // the top bits: g's low ones are the word's number
 }
 
 template <int SIG>
-__device__ __forceinline__ bool frag_bloom_hit(uint32_t v, uint32_t g, uint32_t d2) {
+__device__ __forceinline__ bool frag_bloom_hit(uint32_t v, uint32_t g) {
   uint32_t t = 1u;
 #pragma unroll
-  for (int k = 0; k < kFragBloomBits<SIG>; k++) t &= __funnelshift_r(v, 0u, frag_bloom_bit<SIG>(g, d2, k));
+  for (int k = 0; k < kFragBloomBits<SIG>; k++) t &= __funnelshift_r(v, 0u, frag_bloom_bit<SIG>(g, k));
   return t != 0u;
 }
 
@@ -251,15 +254,15 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
     for (uint32_t k = 0; k < n; k += 2) {  // two requests at a time
       const bool two = k + 1 < n;
       const uint32_t g0 = waiting[k], g1 = two ? waiting[k + 1] : 0u;
-      const uint32_t v0 = __ldg(bloom + frag_bloom_word<SIG>(g0, 0u, p.tab.bloom_mask));
-      const uint32_t v1 = two ? __ldg(bloom + frag_bloom_word<SIG>(g1, 0u, p.tab.bloom_mask)) : 0u;
+      const uint32_t v0 = __ldg(bloom + frag_bloom_word<SIG>(g0, p.tab.bloom_mask));
+      const uint32_t v1 = two ? __ldg(bloom + frag_bloom_word<SIG>(g1, p.tab.bloom_mask)) : 0u;
       const uint32_t b0 = fresh & (0u - fresh);
       fresh ^= b0;
-      if (frag_bloom_hit<SIG>(v0, g0, 0u)) cand |= b0;
+      if (frag_bloom_hit<SIG>(v0, g0)) cand |= b0;
       if (two) {
         const uint32_t b1 = fresh & (0u - fresh);
         fresh ^= b1;
-        if (frag_bloom_hit<SIG>(v1, g1, 0u)) cand |= b1;
+        if (frag_bloom_hit<SIG>(v1, g1)) cand |= b1;
       }
     }
     cand |= fresh;
@@ -272,8 +275,8 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
       uint32_t d[4];
       frag_key<SIG>(ws + w0 + i, d, p.one);
       if (!p.tab.use_bloom || frag_bloom_hit<SIG>(__ldg(reinterpret_cast<const uint32_t*>(p.tab.bloom) +
-                                                        frag_bloom_word<SIG>(d[0], d[3], p.tab.bloom_mask)),
-                                                  d[0], d[2]))
+                                                        frag_bloom_word<SIG>(d[0], p.tab.bloom_mask)),
+                                                  d[0]))
         cand |= 1u << i;
     }
     return cand;
@@ -648,8 +651,8 @@ __global__ void frag_bloom_kernel(const uint4* slots, uint32_t n_slots, uint32_t
     const uint32_t g = SIG == kSigDjb2 ? d.x - (uint32_t)kDjbInit : d.x;
     if (words) {
       uint32_t bits = 0;
-      for (int k = 0; k < kFragBloomBits<SIG>; k++) bits |= 1u << (frag_bloom_bit<SIG>(g, d.z, k) & 31);
-      atomicOr(words + frag_bloom_word<SIG>(g, d.w, mask), bits);
+      for (int k = 0; k < kFragBloomBits<SIG>; k++) bits |= 1u << (frag_bloom_bit<SIG>(g, k) & 31);
+      atomicOr(words + frag_bloom_word<SIG>(g, mask), bits);
     }
     atomicOr(l1 + frag_l1_word(g), frag_l1_bits(g));
   }

@@ -42,11 +42,13 @@ template <int SIG>
 struct FragGeom {
   static constexpr bool kRolled = SIG == kSigDjb2;
   // 32 warps per SM. The rolled kernel's blocks stay and share one copy of the filter; an MD5 warp
-  // hashes one tile (some 70 us) and a block of four such warps ends, so that the hardware deals the
+  // hashes one tile (some 70 us) and a block of two such warps ends, so that the hardware deals the
   // blocks out: with a fixed share of the tiles per warp the same kernel took 1,660 against 1,506 us
-  // (256 MiB), because the scheduler favours some warps of an SM.
-  static constexpr int kThreads = kRolled ? 1024 : 128;  // block size
-  static constexpr int kMinBlocks = kRolled ? 1 : 8;     // resident blocks per SM
+  // (256 MiB), because the scheduler favours some warps of an SM. Tiles with repeated windows are
+  // done earlier: blocks of four warps 1,231 us, of two 1,227, of one (of 29 windows a lane, for the
+  // blocks' shared memory) 1,244.
+  static constexpr int kThreads = kRolled ? 1024 : 64;   // block size
+  static constexpr int kMinBlocks = kRolled ? 1 : 16;     // resident blocks per SM
   static constexpr int kWarps = kThreads / 32;
   static constexpr int kWPT = kRolled ? 23 : 31;  // windows per lane per tile (odd)
   // Rolled: windows per lane that can wait for the second filter. They wait in the lane's part of
@@ -58,7 +60,9 @@ struct FragGeom {
   static constexpr uint32_t kTileBytes = kTileStep + 64;         // bytes staged per tile
   static constexpr bool kL1 = kRolled;                           // shared-memory filter
   static constexpr uint32_t kL1Off = kWarps * kTileBytes;  // filter after the warps' buffers
-  static constexpr uint32_t kSmemCount = kL1Off + (kL1 ? kFragL1Bytes : 0);
+  // not rolled: per warp the windows to be hashed (16-bit numbers) and the lanes' candidate masks
+  static constexpr uint32_t kListBytes = kRolled ? 0 : kTileWin * 2 + 128;
+  static constexpr uint32_t kSmemCount = kL1Off + (kL1 ? kFragL1Bytes : 0) + kWarps * kListBytes;
   static_assert(kWPT % 2 == 1 && kWPT <= 32 && (!kRolled || kQueue > 0), "odd window count, masks of 32 bits");
   static_assert(kTileBytes % 16 == 0 && kTileStep % 16 == 0, "bulk copies of whole 16-byte chunks");
   static_assert(kSmemCount <= 227 * 1024, "shared memory of one block");
@@ -197,6 +201,14 @@ __device__ __forceinline__ bool frag_equal(const uint32_t* x, const uint8_t* m) 
 // image. l1: the first filter, in shared or global memory (rolled kernels only). ws is the warp's
 // tile; the rolled kernels' waiting windows overwrite parts of it (FragGeom::kQueue).
 //
+// Not rolled (MD5): the hash is all of the cost (126 or 61 operations a window), so a window that equals
+// the one before it (fills; patterns of four bytes) is not hashed again. The lanes mark these (17
+// equal words), the others are listed and dealt out evenly over the warp, a candidate sets its bit in
+// its lane's mask, and the windows after it that equal it are candidates too. Where no two words at
+// the multiples of 16 and after are equal there is no such run, and the lanes hash their own windows.
+// 256 MiB of which 15% of the sectors are zeros 1,336 to 1,227 us, half of it zeros 1,312 to 728; random
+// bytes 1,342 to 1,347 (without the padding block 790 to 804).
+//
 // Rolled: the cost is instructions, not memory. A window takes one shared-memory word, two dp2a,
 // two multiply-adds and the filter (word address, load, two shifts by the low bits of g, which wrap
 // by themselves); its random load, 3.6 shared-memory cycles on average, sets the pace. The windows
@@ -212,7 +224,7 @@ __device__ __forceinline__ bool frag_equal(const uint32_t* x, const uint8_t* m) 
 // and each word is read a window ahead because no load may move past them.
 template <int SIG>
 __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_t* ws, uint32_t w0, uint32_t n_valid,
-                                                    const uint32_t* l1) {
+                                                    const uint32_t* l1, uint16_t* list, uint32_t* masks) {
   using G = FragGeom<SIG>;
   if constexpr (G::kRolled) {
     const uint32_t queue = smem_addr(ws + w0 + 15), queue_end = queue + 4u * G::kQueue;
@@ -269,17 +281,68 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
     // the windows after a candidate that share its entry: a carry through each run of them
     return cand | (((same + (same & (cand << 1))) ^ same) & same);
   } else {
+    constexpr uint32_t kFull = 0xFFFFFFFFu;
+    constexpr uint32_t kWords = G::kWPT + 15;  // of this lane's windows
+    const uint32_t lane = w0 / G::kWPT;
+    uint32_t same = 0;  // bit i: window w0 + i equals the one before it
+    // 17 equal words have one among them whose number is a multiple of 16, and the one after it
+    bool some = false;
+    for (uint32_t k = (w0 + 15u) & ~15u; k + 1 < w0 + kWords; k += 16) some |= ws[k] == ws[k + 1];
+    uint32_t rounds = n_valid, total = 0;
+    bool listed = false;
+    if (__any_sync(kFull, some)) {
+      // equal: bit k, word k + 1 is word k; window i is the one before it if bits i - 1 .. i + 14 are set
+      uint32_t lo = 0, hi = 0, before = ws[w0];
+#pragma unroll
+      for (uint32_t k = 0; k + 1 < kWords; k++) {
+        const uint32_t x = ws[w0 + k + 1];
+        if (x == before) {
+          if (k < 32) lo |= 1u << (k & 31);
+          else hi |= 1u << (k & 31);
+        }
+        before = x;
+      }
+      uint64_t equal = (uint64_t)hi << 32 | lo;
+#pragma unroll
+      for (int d = 1; d < 16; d <<= 1) equal &= equal >> d;
+      const uint32_t valid = (uint32_t)((1ull << n_valid) - 1u);
+      same = (uint32_t)equal << 1 & valid;
+      const uint32_t need = valid ^ same;
+      uint32_t at = __popc(need);
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t v = __shfl_up_sync(kFull, at, d);
+        if (lane >= (uint32_t)d) at += v;
+      }
+      total = __shfl_sync(kFull, at, 31);
+      at -= __popc(need);
+      listed = (total + 31) / 32 < __reduce_max_sync(kFull, n_valid);
+      if (listed) {
+        rounds = (total + 31 - lane) / 32;
+        masks[lane] = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < (uint32_t)G::kWPT; i++)
+          if (need >> i & 1u) list[at++] = (uint16_t)(w0 + i);
+        __syncwarp();
+      }
+    }
     uint32_t cand = 0;
 #pragma unroll 1
-    for (uint32_t i = 0; i < n_valid; i++) {
+    for (uint32_t r = 0; r < rounds; r++) {
+      const uint32_t w = listed ? list[32 * r + lane] : w0 + r;
       uint32_t d[4];
-      frag_key<SIG>(ws + w0 + i, d, p.one);
+      frag_key<SIG>(ws + w, d, p.one);
       if (!p.tab.use_bloom || frag_bloom_hit<SIG>(__ldg(reinterpret_cast<const uint32_t*>(p.tab.bloom) +
                                                         frag_bloom_word<SIG>(d[0], p.tab.bloom_mask)),
-                                                  d[0]))
-        cand |= 1u << i;
+                                                  d[0])) {
+        if (listed) atomicOr(masks + w / G::kWPT, 1u << (w % G::kWPT));
+        else cand |= 1u << r;
+      }
     }
-    return cand;
+    if (!listed) return cand;
+    __syncwarp();
+    cand = masks[lane];
+    return cand | (((same + (same & (cand << 1))) ^ same) & same);
   }
 }
 
@@ -411,6 +474,8 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBl
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t* l1 = G::kL1 ? reinterpret_cast<const uint32_t*>(fsm + G::kL1Off) : nullptr;
   uint8_t* buf = fsm + warp * G::kTileBytes;
+  uint32_t* const masks = G::kRolled ? nullptr : reinterpret_cast<uint32_t*>(fsm + G::kL1Off + warp * G::kListBytes);
+  uint16_t* const list = G::kRolled ? nullptr : reinterpret_cast<uint16_t*>(masks + 32);
   const uint32_t bar = smem_addr(&bars[warp]);
   const uint32_t bar_l1 = smem_addr(&bars[G::kWarps]);
   if (tid == 0) {
@@ -444,7 +509,7 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBl
     if ((tile + 1) * G::kTileStep + 64 > p.n_bytes) frag_tail<SIG>(p, tile, buf);  // warp-uniform
     uint32_t* ws = reinterpret_cast<uint32_t*>(buf);
     const uint32_t w0 = (uint32_t)lane * G::kWPT;
-    const uint32_t cand = frag_candidates<SIG>(p, ws, w0, frag_valid<SIG>(p, tile, w0), l1);
+    const uint32_t cand = frag_candidates<SIG>(p, ws, w0, frag_valid<SIG>(p, tile, w0), l1, list, masks);
     uint32_t rej = 0;
     uint32_t hits;
     uint64_t n = frag_thread_count<SIG, LAYOUT>(p, tile, ws, w0, cand, hits, &rej);

@@ -69,3 +69,27 @@ def test_candidates_that_are_all_rejected(cv):
     assert oracle.djb2_64(col) == oracle.djb2_64(frag)
     img = np.concatenate([np.tile(col, 300), frag, np.tile(frag, 40), np.tile(col, 50)])
     assert np.array_equal(scan(cv, [frag], img, signature=2), oracle.frag_match(img, [frag]))
+
+
+@pytest.mark.parametrize("sig", [0, 1, 2])
+@pytest.mark.parametrize("share", [0.02, 0.5, 0.95])
+def test_runs_of_equal_words(cv, sig, share):
+    """Runs of one word, 1 to 60 words and now and then some tiles long, anywhere: windows that equal the
+    one before are not hashed again, and match where that one does."""
+    rng = np.random.default_rng(int(100 * share))
+    word = np.frombuffer(b"\x11\x22\x33\x44", np.uint32)
+    parts, n = [], 0
+    while n < 40_000:
+        if rng.random() < share:
+            k = int(rng.integers(1, 61)) if rng.random() < 0.98 else int(rng.integers(900, 4000))
+            parts.append(np.full(k, rng.choice([0, word[0], 0xFFFFFFFF]), np.uint32))
+        else:
+            parts.append(rng.integers(0, 2**32, int(rng.integers(1, 40)), dtype=np.uint32))
+        n += parts[-1].size
+    img = np.concatenate(parts).view(np.uint8)
+    img = img[:img.size - int(rng.integers(0, 4))]
+    files = [np.tile(word, 16).view(np.uint8), img[1000 * 4:1000 * 4 + 640].copy()]
+    want = oracle.frag_match(img, files)
+    assert want.size > 10
+    for bloom in (0, 16):
+        assert np.array_equal(scan(cv, files, img, signature=sig, bloom_bits_per_key=bloom), want)

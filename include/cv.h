@@ -308,8 +308,8 @@ int cv_sector_signatures(const void* in, uint64_t n_sectors, uint32_t signature,
  * computed by the fragment scan's own code: window k is bytes [4k, 4k + 64), for every k with
  * 4k + 64 <= n_bytes. signature: CV_SIG_MD5 (the 64-byte message with its padding block),
  * CV_SIG_MD5_NOPAD (the state after the one data block) or CV_SIG_DJB2_64 (rolled from window
- * to window as in the scan: bytes 0-7 the value, little-endian, bytes 8-15 the library's mixing
- * of it); CV_SIG_CRC64 is refused with CV_EINVAL, as for fragment tables.
+ * to window, of which the scan's filters need the low word: bytes 0-7 the value, little-endian,
+ * bytes 8-15 the library's mixing of it); CV_SIG_CRC64 is refused with CV_EINVAL, as for fragment tables.
  *   image  device pointer, 16-byte aligned; out: device pointer, 16-byte aligned, 16 bytes per
  *          window. Fewer than 64 bytes: nothing to do.
  * Runs on stream and returns without waiting. Errors: CV_EINVAL, CV_ECUDA, CV_ENODEV.

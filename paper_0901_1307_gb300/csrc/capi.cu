@@ -2,8 +2,8 @@
 // batches (batch.cu), the server (server.cu) and the allocation-free scan (noalloc.cu).
 //
 // cv_scan  images -> segments (tensor maps over device memory, or host chunks copied into a
-//          double-buffered device ring on a side stream) -> scan launches -> tile offsets ->
-//          exact-size output -> expand -> per-image sorted matches; over a fragment table,
+//          double-buffered device ring on a side stream) -> scan launches -> offsets and
+//          expansion in one launch -> per-image sorted matches; over a fragment table,
 //          count -> offsets -> emit (fragments.cu).
 //
 // Temporaries come from a library-owned stream-ordered memory pool; results from the pool or

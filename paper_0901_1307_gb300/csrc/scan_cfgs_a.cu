@@ -2,8 +2,7 @@
 // sector per thread, two 64-byte ring stages, two of three MD5 operations adding on the FMA pipe,
 // register allocation bounded for four resident blocks per SM: with the stage loop unrolled in
 // fours, 48 registers and 32 hashing warps per SM measured 0.75% faster than 40 registers and 40
-// warps, 1.5% for MD5 without padding; hash tables whose lookups walk long probe runs, at 75-90%
-// occupancy without a filter, lose 9-17%, and the automatic layout takes the sorted one there),
+// warps, 1.5% for MD5 without padding),
 // then 480-sector tiles and the all-ALU pipe split.
 #include "scan_cfg_inst.cuh"
 

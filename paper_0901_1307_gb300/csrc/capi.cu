@@ -271,14 +271,14 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
     auto body = [&]() -> int {
       CV_TRY(ctx->take_events(ev, 4));
       CV_CUDA(cudaEventRecord(ev[0], stream));
-      uint64_t *tile_ntrip, *tile_off, *seg_off_d, *scratch;
+      uint64_t *tile_ntrip, *tile_off, *seg_off_d;
       FragHits hits;
       Segment* segs_d = nullptr;
       CV_TRY(tmp.alloc(&tile_ntrip, std::max<uint64_t>(T, 1) * 8));
       CV_TRY(tmp.alloc(&tile_off, std::max<uint64_t>(T, 1) * 8));
-      // seg_off[n], total, status, rejected, listed tiles of every image
-      CV_TRY(tmp.alloc(&seg_off_d, (2ull * n_images + 3) * 8));
-      CV_TRY(tmp.alloc(&scratch, tile_offsets_scratch_words(T) * 8 + 8));
+      // seg_off[n], total, status, rejected, listed tiles of every image, the offset pass's words
+      const uint64_t off_words = tile_offsets_scratch_words(T);
+      CV_TRY(tmp.alloc(&seg_off_d, (2ull * n_images + 3 + off_words) * 8));
       CV_TRY(tmp.alloc(&hits.tiles, T * 4));
       hits.mask_tiles = std::min(T, kFragMaskTiles);
       CV_TRY(tmp.alloc(&hits.masks, hits.mask_tiles * 32 * 4));
@@ -295,7 +295,7 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       uint32_t* status = (uint32_t*)(seg_off_d + n_images + 1);
       unsigned long long* rejected = (unsigned long long*)(seg_off_d + n_images + 2);
       uint64_t* listed = seg_off_d + n_images + 3;
-      CV_CUDA(cudaMemsetAsync(status, 0, 16 + n_images * 8ull, stream));
+      CV_CUDA(cudaMemsetAsync(status, 0, 16 + (n_images + off_words) * 8ull, stream));
       CV_CUDA(cudaEventRecord(ev[1], stream));
       for (uint32_t i = 0; i < n_images; i++) {
         if (tile_base[i + 1] == tile_base[i]) continue;
@@ -306,8 +306,9 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       }
       CV_CUDA(cudaEventRecord(ev[2], stream));
       CV_CUDA((cudaError_t)launch_tile_offsets(tile_ntrip, T, tile_off, seg_list(segs.data(), segs_d, n_images), 1,
-                                               seg_off_d, seg_off_d + n_images, scratch, stream, status));
-      r->launches += 2;
+                                               seg_off_d, seg_off_d + n_images, listed + n_images, stream, status,
+                                               true));
+      r->launches += 1;
       auto emit = [&](uint64_t room) -> int {
         CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, room * sizeof(MatchOut), ctx->pool, stream));
         for (uint32_t i = 0; i < n_images; i++) {

@@ -13,8 +13,8 @@
 namespace cvk {
 
 // Exclusive scan of per-tile counts in one pass, for the serving loop and the fragment scans: each
-// block scans a chunk and adds its predecessors' published sums (decoupled look-back, every wait
-// bounded). A second small pass reads off each segment's first offset. (These kernels are in
+// block scans a chunk, adds its predecessors' published sums (decoupled look-back, every wait
+// bounded) and writes the offsets of the segments that begin in the chunk. (This kernel is in
 // kernels_scan.cu; this header holds the passes instantiated with each configuration.)
 constexpr int kOffThreads = 1024;
 constexpr int kOffItems = 4;

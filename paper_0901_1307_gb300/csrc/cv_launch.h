@@ -56,10 +56,10 @@ uint64_t tile_offsets_scratch_words(uint64_t n_tiles);
 // tile_off[i] = sum of tile_ntrip[0..i) over the n_tiles output tiles; *total = sum of all;
 // seg_off[s] = offset of segment s's first output tile (segment tile_base * scale). scratch:
 // tile_offsets_scratch_words(n_tiles) u64 words. status: the scan's status word (kStTimeout if
-// a wait of the pass gives up). Returns a CUDA error code.
+// a wait of the pass gives up). zeroed: the scratch is zero already. Returns a CUDA error code.
 int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* tile_off, const SegList& segs,
                         uint32_t scale, uint64_t* seg_off, uint64_t* total, uint64_t* scratch, void* stream,
-                        uint32_t* status);
+                        uint32_t* status, bool zeroed = false);
 
 // ---------------------------------------------------------------- fragment scans (Section 5)
 uint64_t frag_windows(uint64_t n_bytes);       // 64-byte windows at 4-byte offsets in n_bytes

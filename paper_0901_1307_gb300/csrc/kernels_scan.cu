@@ -42,14 +42,18 @@ __device__ __forceinline__ uint64_t block_inclusive_scan(uint64_t x, uint64_t* w
 // (decoupled look-back). A block only waits for chunks taken by blocks that started before it,
 // and each wait is bounded by timeout_ns (kStTimeout in *status on expiry; the block then
 // publishes what it has, so no wait depends on it for longer). state: chunks words, then the
-// ticket, all zero before the launch.
+// ticket, all zero before the launch. The block of a segment's first value also writes that segment's
+// offset (value number tile_base * scale; the last block, those past the end): a pass of its own
+// for it took 3 us and the gap before it.
 constexpr uint64_t kLbAgg = 1ull << 62, kLbIncl = 2ull << 62, kLbValue = (1ull << 62) - 1;
 
 __global__ void __launch_bounds__(kOffThreads) lookback_scan_kernel(const uint64_t* v, uint64_t n, uint64_t* out,
                                                                     uint64_t* total, uint64_t* state, uint64_t chunks,
-                                                                    uint32_t* status, uint64_t timeout_ns) {
+                                                                    const __grid_constant__ SegList list, uint32_t scale,
+                                                                    uint64_t* seg_off, uint32_t* status,
+                                                                    uint64_t timeout_ns) {
   __shared__ uint64_t wb[32];
-  __shared__ uint64_t s_chunk, s_prefix;
+  __shared__ uint64_t s_chunk, s_prefix, s_end;
   if (threadIdx.x == 0) s_chunk = atomicAdd(reinterpret_cast<unsigned long long*>(state + chunks), 1ull);
   __syncthreads();
   const uint64_t chunk = s_chunk;
@@ -90,6 +94,7 @@ __global__ void __launch_bounds__(kOffThreads) lookback_scan_kernel(const uint64
       st[chunk] = kLbIncl | (prefix + incl);
     }
     s_prefix = prefix;
+    s_end = prefix + incl;
     if (chunk == chunks - 1) *total = prefix + incl;
   }
   __syncthreads();
@@ -99,15 +104,19 @@ __global__ void __launch_bounds__(kOffThreads) lookback_scan_kernel(const uint64
     if (first + k < n) out[first + k] = run;
     run += x[k];
   }
-}
-
-// seg_off[s] = offset of the first output tile of segment s (output tiles per scan tile: scale).
-__global__ void segment_offsets_kernel(const uint64_t* tile_off, uint64_t n, const __grid_constant__ SegList list,
-                                       uint32_t scale, const uint64_t* total, uint64_t* seg_off) {
+  if (list.n == 0u) return;
+  __syncthreads();  // the block's values are in place
   const Segment* const segs = list.get();
-  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < list.n; s += gridDim.x * blockDim.x) {
+  const uint64_t begin = chunk * kOffChunk, end = chunk == chunks - 1 ? ~0ull : begin + kOffChunk;
+  uint32_t lo = 0, hi = list.n;  // the first segment at or after the chunk's first value
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (segs[mid].tile_base * scale < begin) lo = mid + 1; else hi = mid;
+  }
+  for (uint32_t s = lo + threadIdx.x; s < list.n; s += kOffThreads) {
     const uint64_t u = segs[s].tile_base * scale;
-    seg_off[s] = u < n ? tile_off[u] : *total;
+    if (u >= end) break;
+    seg_off[s] = u < n ? out[u] : s_end;
   }
 }
 
@@ -236,7 +245,8 @@ int launch_lookback_selftest(uint64_t* words, uint32_t* status, uint64_t timeout
   if (e != cudaSuccess) return (int)e;
   const uint64_t one = 1;
   if ((e = cudaMemcpyAsync(state + 2, &one, 8, cudaMemcpyHostToDevice, stream)) != cudaSuccess) return (int)e;
-  lookback_scan_kernel<<<1, kOffThreads, 0, stream>>>(v, 2 * kOffChunk, out, total, state, 2, status, timeout_ns);
+  lookback_scan_kernel<<<1, kOffThreads, 0, stream>>>(v, 2 * kOffChunk, out, total, state, 2, SegList{}, 1u, nullptr, status,
+                                                      timeout_ns);
   return (int)cudaGetLastError();
 }
 
@@ -244,20 +254,19 @@ uint64_t tile_offsets_scratch_words(uint64_t n_tiles) { return (n_tiles + kOffCh
 
 int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* tile_off, const SegList& segs,
                         uint32_t scale, uint64_t* seg_off, uint64_t* total, uint64_t* scratch, void* stream_,
-                        uint32_t* status) {
+                        uint32_t* status, bool zeroed) {
   cudaStream_t stream = (cudaStream_t)stream_;
   const uint64_t chunks = (n_tiles + kOffChunk - 1) / kOffChunk;
   cudaError_t e;
   if (chunks) {
     // the look-back words and the ticket start at zero
-    if ((e = cudaMemsetAsync(scratch, 0, (chunks + 1) * 8, stream)) != cudaSuccess) return (int)e;
+    if (!zeroed && (e = cudaMemsetAsync(scratch, 0, (chunks + 1) * 8, stream)) != cudaSuccess) return (int)e;
     lookback_scan_kernel<<<(unsigned)chunks, kOffThreads, 0, stream>>>(
-        tile_ntrip, n_tiles, tile_off, total, scratch, chunks, status, kWaitTimeoutNs);
-  } else if ((e = cudaMemsetAsync(total, 0, 8, stream)) != cudaSuccess) {
-    return (int)e;
+        tile_ntrip, n_tiles, tile_off, total, scratch, chunks, segs, scale, seg_off, status, kWaitTimeoutNs);
+  } else {
+    if ((e = cudaMemsetAsync(total, 0, 8, stream)) != cudaSuccess) return (int)e;
+    if (segs.n && (e = cudaMemsetAsync(seg_off, 0, segs.n * 8ull, stream)) != cudaSuccess) return (int)e;
   }
-  if (segs.n)
-    segment_offsets_kernel<<<(segs.n + 255) / 256, 256, 0, stream>>>(tile_off, n_tiles, segs, scale, total, seg_off);
   return (int)cudaGetLastError();
 }
 

@@ -93,3 +93,22 @@ def test_runs_of_equal_words(cv, sig, share):
     assert want.size > 10
     for bloom in (0, 16):
         assert np.array_equal(scan(cv, files, img, signature=sig, bloom_bits_per_key=bloom), want)
+
+
+@pytest.mark.parametrize("n_images", [3, 7])
+def test_offsets_of_several_images(cv, n_images):
+    """Images of none, one and more than 4,096 tiles, the last without any, in one call."""
+    rng = np.random.default_rng(n_images)
+    frag = rng.integers(0, 256, 128, dtype=np.uint8)
+    sizes = [13 << 20, 40, 0, 64, 12_058_624 + 60, 100, 63][-n_images:]
+    images = [rng.integers(0, 256, s, dtype=np.uint8) for s in sizes]
+    for k, img in enumerate(images):
+        for at in (0, 4 * (img.size // 8), img.size // 4 * 4 - 64):
+            if 0 <= at <= img.size - 64:
+                img[at:at + 64] = frag[64 * (k % 2):][:64]
+    devs = [torch.from_numpy(img).cuda() if img.size else torch.empty(16, dtype=torch.uint8, device="cuda") for img in images]
+    for sig in (0, 2):
+        with cv.master_build([frag], unit=cv.CV_UNIT_FRAGMENT, signature=sig) as m, \
+                cv.scan(m, [(d.data_ptr(), img.size) for d, img in zip(devs, images)]) as r:
+            for k, img in enumerate(images):
+                assert np.array_equal(r.matches(k), oracle.frag_match(img, [frag])), (sig, k)

@@ -432,12 +432,15 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
           CV_TRY(job.add(ctx, cfg, arena, M, 0, 0, false));
           CV_TRY(digest_job(ctx, cfg_i, sig, job, dig, trivial, counters + 4, stream, tmp));
         }
-        const unsigned g = grid_for(M, 256, ctx->sms);
         unit_postings_kernel<<<grid_for((M + kPostRun - 1) / kPostRun * 32, 256, ctx->sms), 256, 0, stream>>>(
             file_base_d, n_files, M, post, tau);
         CV_CUDA(cudaGetLastError());
-        insert_kernel<<<g, 256, 0, stream>>>(dig, trivial, tau, M, owner, extra, slot_of, mask, counters, counters + 1,
-                                            counters + 4);
+        if (M >= kInsertChunksMin && 2 * M <= n_slots)
+          insert_chunks_kernel<<<(unsigned)((M + kInsertChunk - 1) / kInsertChunk), kInsertThreads, 0, stream>>>(
+              dig, trivial, tau, M, owner, extra, slot_of, mask, counters, counters + 1, counters + 4);
+        else
+          insert_kernel<<<grid_for(M, 256, ctx->sms), 256, 0, stream>>>(
+              dig, trivial, tau, M, owner, extra, slot_of, mask, counters, counters + 1, counters + 4);
         CV_CUDA(cudaGetLastError());
       }
       // also when there is no master unit: it clears the slots

@@ -58,9 +58,9 @@ __global__ void unit_postings_kernel(const uint64_t* file_base, uint32_t n_files
 
 // tau: per master sector position (position-keyed tables), or null for one table over all
 // positions (every tau 0). The key is (digest, tau). A slot's owner is the master index of its key's
-// first member + 1 (0: empty), its extra the number of other members. Bound by the random accesses:
-// 165 us for 4,194,304 keys while the owners (4 bytes a slot, 67 MB) stay in L2, against 248 us
-// with owner and count in one 8-byte word and 333 us with a second atomic that counts every member.
+// first member + 1 (0: empty), its extra the number of other members. Bound by the latency of
+// the random accesses (owner and count in one 8-byte word took 248 us against 165 for 4,194,304 keys,
+// and 333 us with a second atomic that counts every member).
 // (Claiming slots from the kernel that hashes the sectors saved nothing: waited for at once, the
 // atomics held up the hashing by 220 us; looked at a tile later, by 100, and the keys whose home was
 // taken still took 153.)
@@ -109,6 +109,116 @@ __global__ void insert_kernel(const uint4* dig, const uint8_t* trivial, const ui
   if ((threadIdx.x & 31) == 0 && kept) {
     atomicAdd(n_kept, kept);
     atomicMax(max_disp, longest);
+  }
+}
+
+// The same for many keys and at most half of the slots taken. What costs time above is that a thread
+// has one atomic in flight and a warp waits for its longest walk each time. Here a thread's six units
+// try their home slots together, and those that find an owner there are gathered in shared memory and
+// taken one per thread, each walking on by itself. Neighbours with one home slot (copies of a sector)
+// let the first of them try, or they would queue at one address. Both kernels, us:
+//   keys         load      one by one   here (4, 6, 12 units a thread)
+//   100,000      38%       13           18, 24, 31
+//   300,000      29%       18           15, 16, 25
+//   1,048,576    25%       42           21, 22, 28
+//   1,900,000    45%       65           49, 55, 60
+//   4,194,304    25%       178          120, 109, 101
+//   7,600,000    45%       327          258, 237, 266
+//   900,000      86%       290          425, 345, 420
+//   7,000,000    83%       1,140        768, 800, 830
+// so it is used from 2^18 keys on, and where walks are long, above half, not at all (the few longest
+// walks decide there, and the more keys are under way at once the longer they get).
+constexpr uint64_t kInsertChunksMin = 1ull << 18;
+constexpr int kInsertThreads = 128;
+constexpr int kInsertUnits = 6;   // per thread
+constexpr uint32_t kInsertChunk = kInsertThreads * kInsertUnits;
+
+__global__ void __launch_bounds__(kInsertThreads, 10)
+    insert_chunks_kernel(const uint4* dig, const uint8_t* trivial, const uint8_t* tau, uint64_t n, uint32_t* owner,
+                  uint32_t* extra, uint32_t* slot_of, uint32_t mask, uint32_t* max_disp, uint32_t* n_kept,
+                  uint32_t* status) {
+  __shared__ uint2 s_taken[kInsertChunk];  // units whose home slot has an owner: the unit, that owner
+  __shared__ uint32_t s_n, s_kept, s_longest;
+  const uint32_t none = mask + 1u;
+  const uint64_t c0 = (uint64_t)blockIdx.x * kInsertChunk + threadIdx.x;
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t kept = 0, longest = 0;
+  if (threadIdx.x == 0) s_n = s_kept = s_longest = 0;
+  uint32_t home[kInsertUnits], held[kInsertUnits];
+  bool live[kInsertUnits];
+#pragma unroll
+  for (int u = 0; u < kInsertUnits; u++) {
+    const uint64_t m = c0 + u * kInsertThreads;
+    live[u] = m < n && !trivial[m];
+    if (m < n && !live[u]) slot_of[m] = none;
+    home[u] = live[u] ? tau_home(dig[m].x, tau ? tau[m] : 0u) & mask : none;
+  }
+  __syncthreads();
+  // of neighbours with one home slot the first tries for all of them
+  uint32_t heads[kInsertUnits];
+#pragma unroll
+  for (int u = 0; u < kInsertUnits; u++) {
+    const uint32_t before = __shfl_up_sync(0xFFFFFFFFu, home[u], 1);
+    const bool head = lane == 0u || home[u] != before;
+    heads[u] = __ballot_sync(0xFFFFFFFFu, head);
+    held[u] = live[u] && head ? atomicCAS(owner + home[u], 0u, (uint32_t)(c0 + u * kInsertThreads) + 1u) : 0u;
+  }
+#pragma unroll
+  for (int u = 0; u < kInsertUnits; u++) {
+    const uint32_t m = (uint32_t)(c0 + u * kInsertThreads);
+    const uint32_t from = 31u - __clz(heads[u] << (31u - lane) >> (31u - lane));
+    const uint32_t by = __shfl_sync(0xFFFFFFFFu, held[u] ? held[u] : m + 1u, from);
+    if (from != lane) held[u] = by;
+  }
+#pragma unroll
+  for (int u = 0; u < kInsertUnits; u++) {
+    if (!live[u]) continue;
+    const uint32_t m = (uint32_t)(c0 + u * kInsertThreads);
+    if (held[u] == 0u) {
+      slot_of[m] = home[u];
+      kept++;
+    } else {
+      s_taken[atomicAdd(&s_n, 1u)] = make_uint2(m, held[u]);
+    }
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < s_n; i += kInsertThreads) {
+    const uint32_t m = s_taken[i].x;
+    const uint4 d = dig[m];
+    const uint32_t t = tau ? tau[m] : 0u;
+    uint32_t idx = tau_home(d.x, t) & mask, c = 0, by = s_taken[i].y;
+    while (by) {  // the slot has an owner: this key's, or the next slot is tried
+      const uint4 e = dig[by - 1u];
+      const uint32_t te = tau ? tau[by - 1u] : 0u;
+      if (e.x == d.x && e.y == d.y && e.z == d.z && e.w == d.w && te == t) {
+        atomicAdd(extra + idx, 1u);
+        break;
+      }
+      if (c == mask) {
+        atomicOr(status, kStTableFull);
+        idx = none;
+        break;
+      }
+      idx = (idx + 1u) & mask;
+      c++;
+      by = atomicCAS(owner + idx, 0u, m + 1u);
+    }
+    slot_of[m] = idx;
+    if (idx == none) continue;
+    longest = c > longest ? c : longest;
+    kept++;
+  }
+  // one update per block: a per-key atomic on one address serialises the whole build
+  kept = __reduce_add_sync(0xFFFFFFFFu, kept);
+  longest = __reduce_max_sync(0xFFFFFFFFu, longest);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s_kept, kept);
+    atomicMax(&s_longest, longest);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (s_kept) atomicAdd(n_kept, s_kept);
+    if (s_longest) atomicMax(max_disp, s_longest);
   }
 }
 
@@ -303,8 +413,10 @@ __global__ void __launch_bounds__(kSlotThreads) slot_sums_kernel(const uint32_t*
   if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
+// Evicted first, like the owners that have been read: the digests and postings that the slots gather
+// stay in L2 for longer (215 to 204 us for 16.8M slots).
 __device__ __forceinline__ void store_slot(uint4* p, uint4 a, uint4 b) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+  asm volatile("st.global.L2::evict_first.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
                "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
                : "memory");
 }
@@ -328,8 +440,8 @@ __global__ void __launch_bounds__(kSlotThreads) table_slots_kernel(
 #pragma unroll
   for (int k = 0; k < kSlotRows; k++) {
     const bool in = base + 32u * k < n_slots;
-    owner[k] = in ? owners[base + 32u * k] : 0u;
-    cnt[k] = in ? extra[base + 32u * k] + (owner[k] ? 1u : 0u) : 0u;
+    owner[k] = in ? __ldcs(owners + base + 32u * k) : 0u;
+    cnt[k] = in ? __ldcs(extra + base + 32u * k) + (owner[k] ? 1u : 0u) : 0u;
   }
 #pragma unroll
   for (int k = 0; k < kSlotRows; k++) {

@@ -57,3 +57,29 @@ def test_members_of_fragments(cv):
     for sig in (0, 2):
         with cv.master_build(parts, signature=sig, unit=cv.CV_UNIT_FRAGMENT) as m, cv.scan(m, [t]) as r:
             assert np.array_equal(r.matches(0), want)
+
+
+@pytest.mark.parametrize("n", [(1 << 18) - 1, 1 << 18, (1 << 18) + 767, 393_217])
+@pytest.mark.parametrize("copies", [0, 1, 1000])
+def test_inserts_of_many_keys(cv, n, copies):
+    """Around the number of keys from which the insert takes them by chunks of 768: sectors told apart by
+    their first bytes, runs of copies among them (within a warp and across), and fills left out."""
+    rng = np.random.default_rng(n)
+    ids = np.arange(n, dtype=np.uint32)
+    for at in rng.integers(0, n - 1100, 8 if copies else 0):
+        ids[at:at + copies + 1] = ids[at]
+    rows = np.zeros((n, 512), np.uint8)
+    rows[:, :4] = (ids[:, None] >> np.array([0, 8, 16, 24], np.uint32)).astype(np.uint8)
+    rows[:, 4] = 1
+    rows[5000] = 0
+    dev = torch.from_numpy(rows).cuda()
+    with cv.master_build([dev.view(-1)]) as m, cv.scan(m, [dev.view(-1)]) as r:
+        info, got = m.info(), r.matches(0)
+    live = np.delete(ids, 5000)
+    _, inverse, counts = np.unique(live, return_inverse=True, return_counts=True)
+    assert info["n_kept"] == n - 1 and info["n_unique"] == counts.size
+    assert got.size == int(counts[inverse].sum())
+    # every sector finds itself, and each match is of the sector's own bytes, in order
+    assert np.array_equal(ids[got["disk_sector"]], ids[got["file_sector"]])
+    assert (got["disk_sector"] == got["file_sector"]).sum() == n - 1
+    assert np.array_equal(np.lexsort((got["file_sector"], got["disk_sector"])), np.arange(got.size))

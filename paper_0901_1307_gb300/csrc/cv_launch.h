@@ -64,14 +64,17 @@ int launch_tile_offsets(const uint64_t* tile_ntrip, uint64_t n_tiles, uint64_t* 
 // ---------------------------------------------------------------- fragment scans (Section 5)
 uint64_t frag_windows(uint64_t n_bytes);       // 64-byte windows at 4-byte offsets in n_bytes
 uint64_t frag_tiles(int sig, uint64_t n_bytes);  // tiles of sig's fragment kernels over those windows
+// Which filters and count kernel a table with n_keys keys has.
+enum : int { kFragFewKeys = 0, kFragManyKeys = 1, kFragMostKeys = 2, kFragKeyClasses = 3 };
+int frag_key_class(int sig, uint64_t n_keys);
 bool frag_sig_supported(int sig);         // MD5, MD5 without padding, djb2-64
 
 // Key words and exclusion flags of n master fragments at arena (64 bytes each, 16-byte aligned).
 int frag_digests(int sig, const uint8_t* arena, uint64_t n, uint4* dig, uint8_t* trivial, int sms, void* stream);
 // The filters of a fragment table (zeroed by the caller): the one-word Bloom filter (words, null
 // for none; mask = words - 1) and the shared-memory filter l1 (kFragL1Bytes).
-int frag_bloom(int sig, const uint4* slots, uint32_t n_slots, uint32_t* words, uint32_t mask, uint32_t* l1, int sms,
-               void* stream);
+int frag_bloom(int sig, const uint4* slots, uint32_t n_slots, uint64_t n_keys, uint32_t* words, uint32_t mask,
+               uint32_t* l1, int sms, void* stream);
 // The hit lists of a scan's images: tiles has room for every tile of the scan, masks (32 words per
 // tile) for the first mask_tiles of them, an image's entries starting at its first tile; count is
 // the image's own counter.

@@ -31,6 +31,7 @@
 #include <stdint.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "cv_launch.h"
 #include "scan_kernel.cuh"
@@ -106,43 +107,74 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
       : "memory");
 }
 
-// The one-word Bloom filter of a fragment table. A djb2-64 key is represented by g, the low word of h less
-// the initial value's share (what the scan rolls), spread by two odd multipliers. An MD5 key is
-// represented by its first word, which is final three operations before the end of the last block:
-// the filter's bits from the third word, the block from the fourth, needed two of these three for
-// every window (1.347 ms for 256 MiB then, 1.336 so).
+// The one-word Bloom filter of a fragment table: a key's word comes from w, its bits from b (both
+// 32 bits, see the functions of that name below).
+//
+// KEYS is the table's class (frag_key_class). A djb2-64 key is represented by g, the low word of h less
+// the initial value's share (what the scan rolls), spread by two odd multipliers, in the largest
+// tables by both words of it. An MD5 key is represented by its first word, which is final three
+// operations before the end of the last block: the filter's bits from the third word, the block from
+// the fourth, needed two of these three for every window (1.347 ms for 256 MiB then, 1.336 so). 32
+// bits tell keys apart while these are few; 2^26 keys have 2^25 words, 7 bits are left to tell the
+// keys of a word apart, and by arithmetic one window in thirty passes instead of one in a hundred
+// and fifty. So the largest tables take the bits from the fourth word.
+struct FragFilterKey {
+  uint32_t w, b;
+};
+
 template <int SIG>
-__device__ __forceinline__ uint32_t frag_bloom_word(uint32_t g, uint32_t mask) {
-  if constexpr (SIG == kSigDjb2) return __umulhi(g * 0x9E3779B1u + 0x7F4A7C15u, mask + 1u);
-  return g & mask;
+__device__ __forceinline__ uint32_t frag_bloom_word(uint32_t w, uint32_t mask) {
+  if constexpr (SIG == kSigDjb2) return __umulhi(w, mask + 1u);
+  return w & mask;
 }
 
 // The key's bits of its word: three bit numbers, for djb2-64 (where the test is off the scan's
-// inner loop) five, each taken mod 32.
+// inner loop) five, each taken mod 32: the top bits of b first.
 template <int SIG>
 constexpr int kFragBloomBits = SIG == kSigDjb2 ? 5 : 3;
 
-template <int SIG>
-__device__ __forceinline__ uint32_t frag_bloom_bit(uint32_t g, int k) {
-  if constexpr (SIG == kSigDjb2) return (g * 0x85EBCA77u + 0x27D4EB2Fu) >> (27 - 5 * k);  // g = 0: zero windows
-  return (g * 0x9E3779B1u) >> (27 - 5 * k);  // the top bits: g's low ones are the word's number
-}
+__device__ __forceinline__ uint32_t frag_bloom_bit(uint32_t b, int k) { return b >> (27 - 5 * k); }
 
 template <int SIG>
-__device__ __forceinline__ bool frag_bloom_hit(uint32_t v, uint32_t g) {
+__device__ __forceinline__ bool frag_bloom_hit(uint32_t v, uint32_t b) {
   uint32_t t = 1u;
 #pragma unroll
-  for (int k = 0; k < kFragBloomBits<SIG>; k++) t &= __funnelshift_r(v, 0u, frag_bloom_bit<SIG>(g, k));
+  for (int k = 0; k < kFragBloomBits<SIG>; k++) t &= __funnelshift_r(v, 0u, frag_bloom_bit(b, k));
   return t != 0u;
 }
 
-// The shared-memory filter of a djb2 fragment table: two bits, from the low ten bits of g, of the
-// word that its top 15 bits select. Both bits are set for 0.09 of the windows at 173,751 keys,
+template <int KEYS>
+using FragRoll = typename std::conditional<KEYS == kFragMostKeys, uint64_t, uint32_t>::type;
+
+// g: h less the initial value's share, its low word unless KEYS is kFragMostKeys.
+template <int KEYS>
+__device__ __forceinline__ FragFilterKey frag_djb2_filter_key(FragRoll<KEYS> g) {
+  if constexpr (KEYS == kFragMostKeys) {
+    const uint32_t lo = (uint32_t)g, hi = (uint32_t)(g >> 32);
+    return {(uint32_t)((g * 0x9E3779B97F4A7C15ull) >> 32) + 0x7F4A7C15u, lo * 0x85EBCA77u + hi * 0x9E3779B1u + 0x27D4EB2Fu};
+  } else {
+    return {g * 0x9E3779B1u + 0x7F4A7C15u, g * 0x85EBCA77u + 0x27D4EB2Fu};  // g = 0: zero windows
+  }
+}
+
+template <int KEYS>
+__device__ __forceinline__ FragFilterKey frag_md5_filter_key(uint32_t d0, uint32_t d3) {
+  if constexpr (KEYS == kFragMostKeys) return {d0, d3};
+  return {d0, d0 * 0x9E3779B1u};  // the top bits: d0's low ones are the word's number
+}
+
+// The shared-memory filter of a djb2 fragment table: bits of the word that the top 15 bits of g
+// select, two from the low ten bits of g, or one where there are many keys (at 2^20 keys two bits
+// pass 0.75 of the windows, one 0.63). Both bits are set for 0.09 of the windows at 173,751 keys,
 // against 0.15 for one bit.
 __device__ __forceinline__ uint32_t frag_l1_word(uint32_t g) { return g >> 17; }
-__device__ __forceinline__ uint32_t frag_l1_bits(uint32_t g) { return (1u << (g & 31)) | (1u << ((g >> 5) & 31)); }
+template <int KEYS>
+__device__ __forceinline__ uint32_t frag_l1_bits(uint32_t g) {
+  return (1u << (g & 31)) | (KEYS == kFragFewKeys ? 1u << ((g >> 5) & 31) : 0u);
+}
+template <int KEYS>
 __device__ __forceinline__ uint32_t frag_l1_hit(uint32_t v, uint32_t g) {
-  return __funnelshift_r(v, 0u, g) & __funnelshift_r(v, 0u, g >> 5) & 1u;
+  return __funnelshift_r(v, 0u, g) & (KEYS == kFragFewKeys ? __funnelshift_r(v, 0u, g >> 5) : 1u) & 1u;
 }
 
 // djb2-64 of consecutive windows w0, w0 + 1, ... (ws: 32-bit words in shared memory), rolled:
@@ -222,11 +254,45 @@ __device__ __forceinline__ bool frag_equal(const uint32_t* x, const uint8_t* m) 
 // entry, so such runs need one place; a lane with more passing windows than places sends the rest
 // on unfiltered. The stores are predicated by hand (a branch per window cost more than they do),
 // and each word is read a window ahead because no load may move past them.
-template <int SIG>
+//
+// That holds while few windows pass the first filter. It has 2^20 bits whatever the table's size: at
+// 500,000 keys 0.38 of the windows pass and at 2^20 three of four, most lanes then have more than eight
+// of them, and each one sent on costs 16 words, the whole hash and a slot (1,564 and 6,350 us). With
+// many keys every window that passes asks for its Bloom word in the loop, four ahead of their tests,
+// and the tile stays as it is: 692 and 1,165 us. The most keys: nearly every window passes, so
+// the first filter is not looked at, and the Bloom words, from L2 and DRAM, are all of the cost. What
+// matters then is an even stream of requests: words asked for in rounds of 4, 8 and 23 took 3,780,
+// 3,835 and 4,370 us at 2^25 keys, four or six ahead 3,522 and 3,529, twelve ahead 3,772.
+template <int SIG, int KEYS>
 __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_t* ws, uint32_t w0, uint32_t n_valid,
                                                     const uint32_t* l1, uint16_t* list, uint32_t* masks) {
   using G = FragGeom<SIG>;
-  if constexpr (G::kRolled) {
+  if constexpr (G::kRolled && KEYS != kFragFewKeys) {
+    const uint32_t* const bloom = reinterpret_cast<const uint32_t*>(p.tab.bloom);
+    Djb2Roll<FragRoll<KEYS>> roll;
+    uint32_t cand = 0;
+    constexpr int kAhead = 4;
+    uint32_t v[kAhead], bits[kAhead];
+#pragma unroll
+    for (int i = 0; i < G::kWPT + kAhead; i++) {
+      if (i >= kAhead) {  // before window i takes its place
+        const int q = i - kAhead;
+        if (frag_bloom_hit<SIG>(v[q % kAhead], bits[q % kAhead])) cand |= 1u << q;
+      }
+      if (i < G::kWPT) {
+        if (i == 0) roll.first(ws, w0);
+        else roll.next(ws[w0 + i + 15], i);
+        const FragFilterKey key = frag_djb2_filter_key<KEYS>(roll.g);
+        bool pass = true;
+        if constexpr (KEYS != kFragMostKeys) pass = frag_l1_hit<KEYS>(l1[frag_l1_word(roll.g)], roll.g);
+        bits[i % kAhead] = key.b;
+        v[i % kAhead] = 0u;
+        if (pass) v[i % kAhead] = p.tab.use_bloom ? __ldg(bloom + frag_bloom_word<SIG>(key.w, p.tab.bloom_mask)) : ~0u;
+      }
+    }
+    // windows past the image's end come last
+    return n_valid < (uint32_t)G::kWPT ? cand & ((1u << n_valid) - 1u) : cand;
+  } else if constexpr (G::kRolled) {
     const uint32_t queue = smem_addr(ws + w0 + 15), queue_end = queue + 4u * G::kQueue;
     Djb2Roll<uint32_t> roll;
     uint32_t pass = 0, fresh = 0, at = queue, x = 0, before = 0;
@@ -250,7 +316,7 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
           "@first or.b32 %1, %1, %7;\n\t"
           "@hit or.b32 %2, %2, %7;\n\t}"
           : "+r"(at), "+r"(fresh), "+r"(pass)
-          : "r"(frag_l1_hit(l1[frag_l1_word(roll.g)], roll.g)), "r"(roll.g), "r"(before), "r"(queue_end), "r"(1u << i)
+          : "r"(frag_l1_hit<KEYS>(l1[frag_l1_word(roll.g)], roll.g)), "r"(roll.g), "r"(before), "r"(queue_end), "r"(1u << i)
           : "memory");
     }
     // windows past the image's end come last
@@ -265,16 +331,17 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
     uint32_t cand = 0;
     for (uint32_t k = 0; k < n; k += 2) {  // two requests at a time
       const bool two = k + 1 < n;
-      const uint32_t g0 = waiting[k], g1 = two ? waiting[k + 1] : 0u;
-      const uint32_t v0 = __ldg(bloom + frag_bloom_word<SIG>(g0, p.tab.bloom_mask));
-      const uint32_t v1 = two ? __ldg(bloom + frag_bloom_word<SIG>(g1, p.tab.bloom_mask)) : 0u;
+      const FragFilterKey k0 = frag_djb2_filter_key<KEYS>(waiting[k]);
+      const FragFilterKey k1 = frag_djb2_filter_key<KEYS>(two ? waiting[k + 1] : 0u);
+      const uint32_t v0 = __ldg(bloom + frag_bloom_word<SIG>(k0.w, p.tab.bloom_mask));
+      const uint32_t v1 = two ? __ldg(bloom + frag_bloom_word<SIG>(k1.w, p.tab.bloom_mask)) : 0u;
       const uint32_t b0 = fresh & (0u - fresh);
       fresh ^= b0;
-      if (frag_bloom_hit<SIG>(v0, g0)) cand |= b0;
+      if (frag_bloom_hit<SIG>(v0, k0.b)) cand |= b0;
       if (two) {
         const uint32_t b1 = fresh & (0u - fresh);
         fresh ^= b1;
-        if (frag_bloom_hit<SIG>(v1, g1)) cand |= b1;
+        if (frag_bloom_hit<SIG>(v1, k1.b)) cand |= b1;
       }
     }
     cand |= fresh;
@@ -332,9 +399,10 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
       const uint32_t w = listed ? list[32 * r + lane] : w0 + r;
       uint32_t d[4];
       frag_key<SIG>(ws + w, d, p.one);
+      const FragFilterKey key = frag_md5_filter_key<KEYS>(d[0], d[3]);
       if (!p.tab.use_bloom || frag_bloom_hit<SIG>(__ldg(reinterpret_cast<const uint32_t*>(p.tab.bloom) +
-                                                        frag_bloom_word<SIG>(d[0], p.tab.bloom_mask)),
-                                                  d[0])) {
+                                                        frag_bloom_word<SIG>(key.w, p.tab.bloom_mask)),
+                                                  key.b)) {
         if (listed) atomicOr(masks + w / G::kWPT, 1u << (w % G::kWPT));
         else cand |= 1u << r;
       }
@@ -348,10 +416,10 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
 
 // The 16 words of this thread's window w0 + i of the tile: in the tile, or, where the tile may be
 // overwritten, in the image.
-template <int SIG>
+template <int SIG, int KEYS>
 __device__ __forceinline__ const uint32_t* frag_words(const FragParams& p, uint64_t tile, const uint32_t* ws,
                                                       uint32_t w) {
-  if constexpr (FragGeom<SIG>::kRolled)
+  if constexpr (FragGeom<SIG>::kRolled && KEYS == kFragFewKeys)
     return reinterpret_cast<const uint32_t*>(p.image) + (tile * FragGeom<SIG>::kTileWin + w);
   return ws + w;
 }
@@ -390,7 +458,7 @@ __device__ __forceinline__ uint32_t frag_resolve(const FragParams& p, const uint
 
 // Triples of this thread's candidate windows; hits: the windows with any; *rejected adds the
 // candidates that the byte comparison dropped. Every lane of the warp calls it.
-template <int SIG, int LAYOUT>
+template <int SIG, int LAYOUT, int KEYS>
 __device__ __forceinline__ uint64_t frag_thread_count(const FragParams& p, uint64_t tile, const uint32_t* ws,
                                                       uint32_t w0, uint32_t cand, uint32_t& hits, uint32_t* rejected) {
   uint64_t n = 0;
@@ -400,7 +468,7 @@ __device__ __forceinline__ uint64_t frag_thread_count(const FragParams& p, uint6
     const uint32_t i = has ? (uint32_t)__ffs(cand) - 1u : 0u;
     cand &= cand - 1;
     uint32_t off, cnt;
-    const uint32_t k = frag_resolve<SIG, LAYOUT>(p, frag_words<SIG>(p, tile, ws, w0 + i), has, off, cnt);
+    const uint32_t k = frag_resolve<SIG, LAYOUT>(p, frag_words<SIG, KEYS>(p, tile, ws, w0 + i), has, off, cnt);
     n += k;
     if (k) hits |= 1u << i;
     *rejected += cnt - k;
@@ -465,8 +533,9 @@ __device__ __forceinline__ uint32_t frag_valid(const FragParams& p, uint64_t til
   return left < (uint64_t)G::kWPT ? (uint32_t)left : (uint32_t)G::kWPT;
 }
 
-template <int SIG, int LAYOUT>
-__global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBlocks) frag_count_kernel(const __grid_constant__ FragParams p) {
+template <int SIG, int LAYOUT, int KEYS>
+__global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBlocks)
+    frag_count_kernel(const __grid_constant__ FragParams p) {
   using G = FragGeom<SIG>;
   extern __shared__ __align__(128) uint8_t fsm[];
   __shared__ __align__(8) uint64_t bars[G::kWarps + 1];  // one per warp, the shared-memory filter
@@ -509,10 +578,10 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBl
     if ((tile + 1) * G::kTileStep + 64 > p.n_bytes) frag_tail<SIG>(p, tile, buf);  // warp-uniform
     uint32_t* ws = reinterpret_cast<uint32_t*>(buf);
     const uint32_t w0 = (uint32_t)lane * G::kWPT;
-    const uint32_t cand = frag_candidates<SIG>(p, ws, w0, frag_valid<SIG>(p, tile, w0), l1, list, masks);
+    const uint32_t cand = frag_candidates<SIG, KEYS>(p, ws, w0, frag_valid<SIG>(p, tile, w0), l1, list, masks);
     uint32_t rej = 0;
     uint32_t hits;
-    uint64_t n = frag_thread_count<SIG, LAYOUT>(p, tile, ws, w0, cand, hits, &rej);
+    uint64_t n = frag_thread_count<SIG, LAYOUT, KEYS>(p, tile, ws, w0, cand, hits, &rej);
     if (sig_is_weak(SIG) && rej && p.rejected) atomicAdd(p.rejected, (unsigned long long)rej);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) n += __shfl_xor_sync(0xFFFFFFFFu, n, d);
@@ -707,19 +776,22 @@ __global__ void frag_digest_kernel(const uint8_t* arena, uint64_t n, uint4* dig,
 
 // The filters of a fragment table from its occupied slots: the one-word Bloom filter (none when
 // words is null) and the shared-memory filter.
-template <int SIG>
+template <int SIG, int KEYS>
 __global__ void frag_bloom_kernel(const uint4* slots, uint32_t n_slots, uint32_t* words, uint32_t mask,
                                   uint32_t* l1) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_slots; i += gridDim.x * blockDim.x) {
     if (slots[2ull * i + 1].y == 0u) continue;
     const uint4 d = slots[2ull * i];
-    const uint32_t g = SIG == kSigDjb2 ? d.x - (uint32_t)kDjbInit : d.x;
+    const uint64_t g = ((uint64_t)d.y << 32 | d.x) - kDjbInit;  // djb2
     if (words) {
+      FragFilterKey key;
+      if constexpr (SIG == kSigDjb2) key = frag_djb2_filter_key<KEYS>((FragRoll<KEYS>)g);
+      else key = frag_md5_filter_key<KEYS>(d.x, d.w);
       uint32_t bits = 0;
-      for (int k = 0; k < kFragBloomBits<SIG>; k++) bits |= 1u << (frag_bloom_bit<SIG>(g, k) & 31);
-      atomicOr(words + frag_bloom_word<SIG>(g, mask), bits);
+      for (int k = 0; k < kFragBloomBits<SIG>; k++) bits |= 1u << (frag_bloom_bit(key.b, k) & 31);
+      atomicOr(words + frag_bloom_word<SIG>(key.w, mask), bits);
     }
-    atomicOr(l1 + frag_l1_word(g), frag_l1_bits(g));
+    if (SIG == kSigDjb2) atomicOr(l1 + frag_l1_word((uint32_t)g), frag_l1_bits<KEYS>((uint32_t)g));
   }
 }
 
@@ -734,27 +806,35 @@ struct Geom {
   uint32_t tile_win, smem_count;
 };
 
+template <int SIG, int LAYOUT>
+KernelFn count_fn(int keys) {
+  if (keys == kFragMostKeys) return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragMostKeys>;
+  if constexpr (FragGeom<SIG>::kRolled)
+    if (keys == kFragManyKeys) return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragManyKeys>;
+  return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragFewKeys>;
+}
+
 template <int SIG>
-Geom geom_t(uint32_t layout) {
+Geom geom_t(uint32_t layout, int keys) {
   using G = FragGeom<SIG>;
   const bool s = layout == kLayoutSorted;
-  return Geom{s ? (KernelFn)frag_count_kernel<SIG, kLayoutSorted> : (KernelFn)frag_count_kernel<SIG, kLayoutHash>,
+  return Geom{s ? count_fn<SIG, kLayoutSorted>(keys) : count_fn<SIG, kLayoutHash>(keys),
               s ? (KernelFn)frag_emit_kernel<SIG, kLayoutSorted> : (KernelFn)frag_emit_kernel<SIG, kLayoutHash>,
               G::kThreads, G::kTileWin, G::kSmemCount};
 }
 
-bool geom(int sig, uint32_t layout, Geom* g) {
+bool geom(int sig, uint32_t layout, int keys, Geom* g) {
   switch (sig) {
-    case kSigMd5: *g = geom_t<kSigMd5>(layout); return true;
-    case kSigMd5NoPad: *g = geom_t<kSigMd5NoPad>(layout); return true;
-    case kSigDjb2: *g = geom_t<kSigDjb2>(layout); return true;
+    case kSigMd5: *g = geom_t<kSigMd5>(layout, keys); return true;
+    case kSigMd5NoPad: *g = geom_t<kSigMd5NoPad>(layout, keys); return true;
+    case kSigDjb2: *g = geom_t<kSigDjb2>(layout, keys); return true;
     default: return false;
   }
 }
 
 struct FragDev {
   bool ready = false;
-  int count_blocks[3][2] = {};
+  int count_blocks[3][2][kFragKeyClasses] = {};
 };
 std::mutex g_frag_mu;
 FragDev g_frag_dev[64];
@@ -769,16 +849,17 @@ int frag_device(FragDev** out) {
   FragDev& d = g_frag_dev[dev];
   if (!d.ready) {
     for (int sig = 0; sig < 3; sig++)
-      for (uint32_t l = 0; l < 2; l++) {
+      for (int q = 0; q < 2 * kFragKeyClasses; q++) {
+        const int l = q & 1, keys = q >> 1;
         Geom g;
-        geom(sig, l, &g);
+        geom(sig, (uint32_t)l, keys, &g);
         if ((e = cudaFuncSetAttribute(g.count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem_count)) !=
             cudaSuccess)
           return (int)e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.count_blocks[sig][l], g.count, g.threads,
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.count_blocks[sig][l][keys], g.count, g.threads,
                                                                g.smem_count)) != cudaSuccess)
           return (int)e;
-        if (d.count_blocks[sig][l] < 1) return (int)cudaErrorInvalidConfiguration;
+        if (d.count_blocks[sig][l][keys] < 1) return (int)cudaErrorInvalidConfiguration;
       }
     d.ready = true;
   }
@@ -807,11 +888,29 @@ FragParams make_params(const TableView& tab, const uint8_t* image, uint64_t n_by
 
 }  // namespace
 
+int frag_key_class(int sig, uint64_t n_keys) {
+  // Where the count kernels measured equal on random images, us per scan:
+  //   djb2-64, 1 GiB       few     many    most
+  //     173,751 keys       368     446
+  //     250,000            466     485
+  //     300,000            519     472
+  //     500,000            1,564   692     1,872
+  //     4,194,304          12,607  1,911   1,932
+  //     16,777,216                 2,016   1,933
+  //     67,108,864                 6,448   6,080
+  //   MD5, 256 MiB (without the padding block)
+  //     262,144            1,376 (825)     1,382 (833)
+  //     1,048,576          1,405 (845)     1,383 (833)
+  //     67,108,864         1,879 (1,850)   1,570 (1,560)
+  if (sig != kSigDjb2) return n_keys > (1ull << 19) ? kFragMostKeys : kFragFewKeys;
+  return n_keys > (1ull << 22) ? kFragMostKeys : n_keys > (1ull << 18) ? kFragManyKeys : kFragFewKeys;
+}
+
 uint64_t frag_windows(uint64_t n_bytes) { return n_bytes >= 64 ? (n_bytes - 64) / kFragStride + 1 : 0; }
 
 uint64_t frag_tiles(int sig, uint64_t n_bytes) {
   Geom g;
-  if (!geom(sig, kLayoutHash, &g)) return 0;
+  if (!geom(sig, kLayoutHash, kFragFewKeys, &g)) return 0;
   return (frag_windows(n_bytes) + g.tile_win - 1) / g.tile_win;
 }
 
@@ -828,13 +927,18 @@ int frag_digests(int sig, const uint8_t* arena, uint64_t n, uint4* dig, uint8_t*
   return (int)cudaGetLastError();
 }
 
-int frag_bloom(int sig, const uint4* slots, uint32_t n_slots, uint32_t* words, uint32_t mask, uint32_t* l1, int sms,
-               void* stream) {
+int frag_bloom(int sig, const uint4* slots, uint32_t n_slots, uint64_t n_keys, uint32_t* words, uint32_t mask,
+               uint32_t* l1, int sms, void* stream) {
   const unsigned g = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(((uint64_t)n_slots + 255) / 256, (uint64_t)sms * 8));
+  const int keys = frag_key_class(sig, n_keys);
+  void (*fn)(const uint4*, uint32_t, uint32_t*, uint32_t, uint32_t*);
   if (sig == kSigDjb2)
-    frag_bloom_kernel<kSigDjb2><<<g, 256, 0, (cudaStream_t)stream>>>(slots, n_slots, words, mask, l1);
+    fn = keys == kFragMostKeys   ? frag_bloom_kernel<kSigDjb2, kFragMostKeys>
+         : keys == kFragManyKeys ? frag_bloom_kernel<kSigDjb2, kFragManyKeys>
+                                 : frag_bloom_kernel<kSigDjb2, kFragFewKeys>;
   else
-    frag_bloom_kernel<kSigMd5><<<g, 256, 0, (cudaStream_t)stream>>>(slots, n_slots, words, mask, l1);
+    fn = keys == kFragMostKeys ? frag_bloom_kernel<kSigMd5, kFragMostKeys> : frag_bloom_kernel<kSigMd5, kFragFewKeys>;
+  fn<<<g, 256, 0, (cudaStream_t)stream>>>(slots, n_slots, words, mask, l1);
   return (int)cudaGetLastError();
 }
 
@@ -880,10 +984,11 @@ int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uin
   int rc = frag_device(&d);
   if (rc) return rc;
   Geom g;
-  if (!geom((int)tab.sig, tab.layout, &g)) return (int)cudaErrorInvalidValue;
+  const int keys = frag_key_class((int)tab.sig, tab.n_keys);
+  if (!geom((int)tab.sig, tab.layout, keys, &g)) return (int)cudaErrorInvalidValue;
   if (tab.sig == kSigDjb2 && !tab.frag_l1) return (int)cudaErrorInvalidValue;  // the kernel copies it in
   p.tile_ntrip = tile_ntrip;
-  const uint64_t cap = tab.sig == kSigDjb2 ? (uint64_t)sms * (uint64_t)d->count_blocks[tab.sig][tab.layout] : INT32_MAX;
+  const uint64_t cap = tab.sig == kSigDjb2 ? (uint64_t)sms * (uint64_t)d->count_blocks[tab.sig][tab.layout][keys] : INT32_MAX;
   const uint64_t warps_per_block = (uint64_t)g.threads / 32;
   const unsigned grid = (unsigned)std::min<uint64_t>((p.n_tiles + warps_per_block - 1) / warps_per_block, cap);
   void* args[] = {&p};
@@ -896,7 +1001,7 @@ int frag_emit(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint
   FragParams p = make_params(tab, image, n_bytes, tile_base, hits, status);
   if (!p.n_tiles) return 0;
   Geom g;
-  if (!geom((int)tab.sig, tab.layout, &g)) return (int)cudaErrorInvalidValue;
+  if (!geom((int)tab.sig, tab.layout, kFragFewKeys, &g)) return (int)cudaErrorInvalidValue;
   p.tile_off = tile_off;
   p.out = out;
   p.out_cap = out_cap;

@@ -451,15 +451,15 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
           owner, extra, (uint32_t)n_slots, first, dig, tau, post, (uint4*)m->slots, tags, (uint2*)m->postings, member,
           frag ? nullptr : (uint32_t*)m->bloom, bpk ? (uint32_t)(n_blocks - 1) : 0u, counters + 2);
       CV_CUDA(cudaGetLastError());
-      if (M && frag)
-        CV_CUDA((cudaError_t)frag_bloom(sig, (const uint4*)m->slots, (uint32_t)n_slots, (uint32_t*)m->bloom,
-                                        bpk ? (uint32_t)(n_blocks - 1) : 0u, (uint32_t*)m->frag_l1, ctx->sms, stream));
       uint32_t hc[5];
       CV_CUDA(cudaMemcpyAsync(hc, counters, 20, cudaMemcpyDeviceToHost, stream));
       CV_CUDA(cudaStreamSynchronize(stream));
       if (hc[4] & kStTableFull) return CV_ETABLEFULL;
       if (hc[4] & kStTimeout) return CV_ETIMEOUT;
       if (hc[4]) return CV_ECORRUPT;
+      if (M && frag)  // which filters these are depends on the number of keys
+        CV_CUDA((cudaError_t)frag_bloom(sig, (const uint4*)m->slots, (uint32_t)n_slots, hc[2], (uint32_t*)m->bloom,
+                                        bpk ? (uint32_t)(n_blocks - 1) : 0u, (uint32_t*)m->frag_l1, ctx->sms, stream));
       if (hc[3]) CV_TRY(several_members(ctx, slot_of, M, n_slots, extra, (const uint4*)m->slots, hc[3], hc[1], post,
                                         (uint2*)m->postings, member, tmp, stream));
       if (M && sig_is_weak(sig)) {
@@ -703,8 +703,8 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
       // the scan kernel of this build, not to the file format
       CV_CUDA(cudaMemsetAsync(m->frag_l1, 0, h.bytes_l1, stream));
       if (h.bytes_bloom) CV_CUDA(cudaMemsetAsync(m->bloom, 0, h.bytes_bloom, stream));
-      CV_CUDA((cudaError_t)frag_bloom((int)h.sig, (const uint4*)m->slots, (uint32_t)n_records, (uint32_t*)m->bloom,
-                                      h.bloom_mask, (uint32_t*)m->frag_l1, ctx->sms, stream));
+      CV_CUDA((cudaError_t)frag_bloom((int)h.sig, (const uint4*)m->slots, (uint32_t)n_records, h.n_keys,
+                                      (uint32_t*)m->bloom, h.bloom_mask, (uint32_t*)m->frag_l1, ctx->sms, stream));
       CV_CUDA(cudaStreamSynchronize(stream));
     }
     m->tab.slots = (const uint4*)m->slots;

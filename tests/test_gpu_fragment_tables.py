@@ -1,0 +1,75 @@
+"""Fragment tables of every size: few, many and most keys have filters and count kernels of their own.
+Exact against the planted fragments, at the sizes between which the kernels change; a large table's
+scan is not out of proportion to a small one's."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cv(cuda_device):
+    import __graft_entry__
+
+    __graft_entry__.build()
+    from paper_0901_1307_gb300 import cv as cvmod
+
+    return cvmod
+
+
+def inputs(n_keys, size, seed):
+    """n_keys random fragments, a random image of size bytes and its matches (window, fragment): planted
+    ones, side by side, across the tiles' edges and up to the image's end, beside a fill."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    frags = torch.randint(0, 256, (n_keys, 64), generator=g, dtype=torch.uint8, device="cuda")
+    img = torch.randint(0, 256, (size,), generator=g, dtype=torch.uint8, device="cuda")
+    rng = np.random.default_rng(seed)
+    img[size // 2:size // 2 + 9000] = 0
+    last = (size - 64) // 4
+    at = [0, 16, 32, 32 * 23 - 3, 32 * 31 - 5, 5000, 5016, last - 16, last]
+    at += [6000 + 16 * k for k in range(64)]  # every sixteenth window of some lanes' tiles
+    rows = []
+    for w in at:
+        f = int(rng.integers(0, n_keys))
+        img[4 * w:4 * w + 64] = frags[f]
+        rows.append((w, f))
+    for f in (0, n_keys - 1):
+        w = int(rng.integers(8000, size // 8 - 16))
+        img[4 * w:4 * w + 64] = frags[f]
+        rows.append((w, f))
+    return frags, img, np.array(sorted(rows))
+
+
+@pytest.mark.parametrize("sig,n_keys", [(2, (1 << 18) - 1), (2, 1 << 18), (2, (1 << 18) + 1), (2, 1 << 20),
+                                        (2, 1 << 22), (2, (1 << 22) + 1), (0, 1 << 19), (0, (1 << 19) + 1),
+                                        (1, 1 << 19), (1, (1 << 19) + 1)])
+@pytest.mark.parametrize("size", [262_147, 1_048_576])
+def test_sizes_around_the_classes(cv, sig, n_keys, size, tmp_path):
+    frags, img, want = inputs(n_keys, size, sig + n_keys)
+    for kw in ({}, {"bloom_bits_per_key": 0}, {"layout": cv.CV_LAYOUT_SORTED}):
+        with cv.master_build([frags.view(-1)], signature=sig, unit=cv.CV_UNIT_FRAGMENT, **kw) as m:
+            with cv.scan(m, [img]) as r:
+                got = r.matches(0)
+            if not kw and size == 262_147:
+                cv.master_save(m, tmp_path / "t.cvt")
+        assert np.array_equal(np.stack([got["disk_sector"], got["file_sector"]], axis=1), want), kw
+    if size == 262_147:  # the filters are made again for the table's size
+        with cv.master_load(tmp_path / "t.cvt") as m, cv.scan(m, [img]) as r:
+            got = r.matches(0)
+        assert np.array_equal(np.stack([got["disk_sector"], got["file_sector"]], axis=1), want)
+
+
+def test_large_tables_keep_their_speed(cv):
+    """The count kernel against 2^20 djb2 fragments takes at most six times what it takes against 2^17."""
+    img = torch.randint(-2**31, 2**31 - 1, (1 << 26,), dtype=torch.int32, device="cuda").view(torch.uint8)
+    ms = []
+    for n_keys in (1 << 17, 1 << 20):
+        frags = torch.randint(0, 256, (n_keys * 64,), dtype=torch.uint8, device="cuda")
+        with cv.master_build([frags], signature=2, unit=cv.CV_UNIT_FRAGMENT) as m:
+            t = []
+            for _ in range(6):
+                with cv.scan(m, [img]) as r:
+                    t.append(r.stats()["kernel_ms"])
+        ms.append(min(t))
+    assert ms[1] < 6 * ms[0], ms

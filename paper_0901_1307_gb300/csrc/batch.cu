@@ -377,12 +377,12 @@ int cv_batch_create(const cv_master* m, const cv_buf* images, uint32_t n_images,
     if (layout_choice) CV_TRY(need_sorted());
     if (bloom && !bloom_avail) CV_TRY(need_bloom());
     if (!layout_choice && b->own_slots) {
-      cudaFreeAsync(b->own_slots, stream);  // used on this stream only so far
-      cudaFreeAsync(b->own_keys0, stream);
+      void* const arrays[] = {b->own_slots, b->own_keys0};
+      table_free(arrays, 2, b->dev);
       b->own_slots = b->own_keys0 = nullptr;
     }
     if (!bloom && b->own_bloom) {
-      cudaFreeAsync(b->own_bloom, stream);
+      table_free(&b->own_bloom, 1, b->dev);
       b->own_bloom = nullptr;
     }
     const TableView chosen = variant(layout_choice, bloom);

@@ -154,6 +154,7 @@ void table_free(void* const* ptrs, int n, int dev) {
   cudaDeviceSynchronize();  // scans on any stream may have read the table
   for (int k = 0; k < n; k++)
     if (ptrs[k]) cudaFreeAsync(ptrs[k], nullptr);
+  cudaStreamSynchronize(nullptr);  // a pool gives back what it does not keep at a wait after the free
   cudaGetLastError();
   if (current >= 0 && current != dev) cudaSetDevice(current);
 }

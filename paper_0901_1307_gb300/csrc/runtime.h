@@ -98,7 +98,8 @@ int get_ctx(DevCtx** out);
 
 constexpr uint64_t kTablePoolKept = 1ull << 30;
 // Table memory: allocated in order on stream; freed in order on a stream when only that one used
-// it, or, by the table's owner, once all work of its device is done.
+// it, or, by the table's owner, once all work of its device is done (table_free: what the pool does
+// not keep is free memory again when it returns).
 int table_alloc(DevCtx* ctx, void** out, size_t bytes, cudaStream_t stream);
 void table_free(void* const* ptrs, int n, int dev);
 

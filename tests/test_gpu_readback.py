@@ -86,3 +86,16 @@ def test_tables_in_used_memory(cv):
         kw = [{}, {"layout": cv.CV_LAYOUT_SORTED}, {"signature": 2}, {"bloom_bits_per_key": 0, "max_load": 0.9}][k % 4]
         with cv.master_build(files, stream=streams[k % 3], **kw) as m, cv.scan(m, [t], stream=streams[(k + 1) % 3]) as r:
             assert np.array_equal(r.matches(0), oracle.match_hash(img, files)), k
+
+
+def test_a_closed_table_is_free_memory(cv):
+    """What the library keeps of a table's memory is at most 1 GiB; the rest is free when close returns."""
+    data = torch.randint(0, 256, (1 << 20, 512), dtype=torch.uint8, device="cuda").view(-1)
+    cv.master_build([data[:5120]]).close()
+    torch.cuda.synchronize()
+    m = cv.master_build([data], signature=3, max_load=0.02)
+    size = m.info()["device_bytes"]
+    used = torch.cuda.mem_get_info()[0]
+    m.close()
+    freed = torch.cuda.mem_get_info()[0] - used
+    assert size > 2 << 30 and freed >= size - (1 << 30) - (64 << 20), (size, freed)

@@ -302,10 +302,7 @@ int cv_batch_create(const cv_master* m, const cv_buf* images, uint32_t n_images,
     };
     auto variant = [&](int sorted, int bl) {
       TableView t = sorted ? sorted_tab : tab;
-      if (bl && !bloom_avail) {  // the batch's own filter over the same keys
-        t.bloom = bloom_tab.bloom;
-        t.bloom_mask = bloom_tab.bloom_mask;
-      }
+      if (bl && !bloom_avail) view_bloom(&t, bloom_tab.bloom, bloom_tab.bloom_mask);  // the batch's own, same keys
       t.use_bloom = (uint32_t)bl;
       return t;
     };

@@ -114,6 +114,14 @@ inline bool table_has_tags(uint32_t unit, uint32_t layout, uint64_t bloom_bytes,
   return unit == kUnitSector && layout == kLayoutHash && bloom_bytes == 0 && n_slots >= 64;
 }
 
+// The view with a blocked Bloom filter over its keys: a lookup behind a filter walks the slots.
+inline void view_bloom(TableView* t, const uint4* bloom, uint32_t mask) {
+  t->bloom = bloom;
+  t->bloom_mask = mask;
+  t->use_bloom = 1u;
+  t->tags = nullptr;
+}
+
 // Position-keyed tables (Section 3.1: one table S_tau per sector position tau of an 8-sector
 // cluster) are stored as one open-addressing table whose key is (signature, tau): tau moves the
 // home slot and the Bloom block and is stored in the slot's third value word. tau = 0 leaves both

@@ -800,9 +800,6 @@ int cvk::table_bloom(const TableView& tab, uint32_t bits_per_key, cudaStream_t s
   }
   *bloom_out = bloom;
   *out = tab;
-  out->bloom = (const uint4*)bloom;
-  out->bloom_mask = (uint32_t)(n_blocks - 1);
-  out->use_bloom = 1u;
-  out->tags = nullptr;  // behind a filter the walk over the slots
+  view_bloom(out, (const uint4*)bloom, (uint32_t)(n_blocks - 1));
   return CV_OK;
 }

@@ -417,15 +417,25 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
   if (m->tab.unit == kUnitFragment) return frag_scan(ctx, m, images, n_images, flags, stream, out);
   int ncfg;
   scan_configs(&ncfg);
-  // what one launch scans: every device image, or a host image's chunk
-  uint64_t launch_sectors = 0;
-  for (uint32_t i = 0; i < n_images; i++) launch_sectors += images[i].n_bytes / kSector;
+  // what one launch scans: the device images, or a host image's chunk (with a 64-bit signature a host
+  // image is copied whole and scanned as a device image)
+  const int sig = (int)m->tab.sig;
+  std::vector<BufKind> kind(n_images);
+  uint64_t device_sectors = 0, launch_sectors = 0;
+  for (uint32_t i = 0; i < n_images; i++) {
+    const uint64_t ns = images[i].n_bytes / kSector;
+    if (ns == 0) continue;
+    if (!images[i].data) return CV_EINVAL;
+    CV_TRY(classify(ctx, images[i].data, &kind[i]));
+    if (kind[i] == kDevice || sig_is_weak(sig)) device_sectors += ns;
+    else launch_sectors = std::max(launch_sectors, std::min(ns, chunk / kSector));
+  }
+  launch_sectors = std::max(launch_sectors, device_sectors);
   int cfg_i = ctx->default_config(table_kind(m->tab), launch_sectors);
   if (opts && opts->kernel_config) {
     if (opts->kernel_config > (uint32_t)ncfg) return CV_EINVAL;
     cfg_i = (int)opts->kernel_config - 1;
   }
-  const int sig = (int)m->tab.sig;
   const ScanCfg& cfg = scan_config_for(cfg_i, table_kind(m->tab), &cfg_i);
   TableView tab = m->tab;  // disk sector g sits at cluster position (g - base_offset) mod 8
   tab.tau_add = (uint32_t)((8u - base_offset % 8u) % 8u);
@@ -434,7 +444,6 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
   Temps staging(ctx, stream);
 
   // ------------------------------------------------------------ plan the segments
-  std::vector<BufKind> kind(n_images);
   Job job;
   std::vector<size_t> first_seg(n_images + 1, 0);
   struct HostChunk {
@@ -447,8 +456,6 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
     first_seg[i] = job.segs.size();
     const uint64_t ns = images[i].n_bytes / kSector;
     if (ns == 0) continue;
-    if (!images[i].data) return CV_EINVAL;
-    CV_TRY(classify(ctx, images[i].data, &kind[i]));
     if (kind[i] == kHost && sig_is_weak(sig)) {
       uint8_t* copy;
       CV_TRY(staging.alloc(&copy, ns * kSector));

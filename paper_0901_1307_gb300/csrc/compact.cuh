@@ -51,6 +51,9 @@ struct CompactParams {
 // most tiles have no hit, and a tile's few hits would otherwise each wait in turn. A record's place
 // in the output is its tile's offset plus the triples of the records before it in the tile (a
 // segmented warp scan, carried across passes). out_cap bounds the writes (kStOverflow when exceeded).
+// A record's postings are written by one lane, bound by the latency of a posting's load while the next
+// had to wait for the store before it; loaded as read-only data, four in flight, 32 MiB with 128 copies
+// of each sector take 207 us instead of 573.
 template <int T>
 __device__ __forceinline__ void expand_group(const CompactParams& p, uint64_t u0, uint32_t my_n, uint32_t my_first,
                                              uint32_t n_rec, uint64_t my_off) {
@@ -99,17 +102,28 @@ __device__ __forceinline__ void expand_group(const CompactParams& p, uint64_t u0
     carry_b = last_b;
     if (!act) continue;
     uint64_t o = off_b + before;
-    const bool check = rec.w < rec.z;
-    const uint8_t* mine = check ? bytes_b + (uint64_t)rec.x * kSector : nullptr;
-    for (uint32_t k = 0; k < rec.z; k++) {
-      if (check && !sectors_equal(mine, p.confirm + (uint64_t)(rec.y + k) * kSector)) continue;
-      if (o < p.out_cap) {
-        const uint2 pf = p.postings[rec.y + k];
-        p.out[o] = MatchOut{sector_b + rec.x, pf.x, pf.y};
-      } else {
-        atomicOr(p.status, kStOverflow);
+    const uint2* const post = p.postings + rec.y;
+    MatchOut* const out = p.out + o;
+    const uint64_t room = o < p.out_cap ? p.out_cap - o : 0ull;
+    if (rec.w > room) atomicOr(p.status, kStOverflow);
+    if (rec.w == rec.z) {
+      const uint32_t n = rec.w < room ? rec.w : (uint32_t)room;
+#pragma unroll 4
+      for (uint32_t k = 0; k < n; k++) {
+        const uint2 pf = __ldg(post + k);
+        out[k] = MatchOut{sector_b + rec.x, pf.x, pf.y};
       }
-      o++;
+    } else {
+      const uint8_t* mine = bytes_b + (uint64_t)rec.x * kSector;
+      uint32_t n = 0;
+      for (uint32_t k = 0; k < rec.z; k++) {
+        if (!sectors_equal(mine, p.confirm + (uint64_t)(rec.y + k) * kSector)) continue;
+        if (n < room) {
+          const uint2 pf = __ldg(post + k);
+          out[n] = MatchOut{sector_b + rec.x, pf.x, pf.y};
+        }
+        n++;
+      }
     }
   }
 }
@@ -159,17 +173,27 @@ __global__ void expand_kernel(const __grid_constant__ CompactParams p) {
 //   1 GiB          8.2 + 2.7 + 7.3      9.1
 //   2 GiB, CRC64   10.5 + 2.6 + 7.7     9.6
 //   32 GiB, 1,000,000 matches: 64
-// 512 tiles to a group up to 2^21 tiles (32 GiB), more above, so that the sums' scan stays at most
-// 4,096 words a block.
+// A group is what one block expands, so few of them leave SMs idle where most sectors of a small image
+// match: a group has 32 tiles, or as many more (up to 512) as leave two groups per SM; 512 from 2.3 GiB to
+// 32 GiB, more above, so that the sums' scan stays at most 4,096 words a block. Offsets and expansion, us,
+// with groups of 512 tiles at least, and so (copies: of each matching sector in the master files):
+//   8 MiB, all of it matches, 16 copies    323    97
+//   32 MiB, 128 copies                     2,379  573
+//   256 MiB, 8 copies                      179    72
+//   1 GiB, one sector in 64 matches        19     19 to 21
+// (608 groups: 122 at 256 MiB, 23 at 1 GiB.) A block whose group has fewer tiles than threads has idle
+// warps, which costs nothing there.
 constexpr uint32_t kFinishGroups = 4096;
 constexpr int kFinishThreads = 512;
-constexpr uint32_t kFinishMinLog2 = 9;  // a group is whole chunks of kFinishThreads tiles
-static_assert((1 << kFinishMinLog2) == kFinishThreads, "chunks of a tile per thread");
+constexpr uint32_t kFinishMinLog2 = 5;    // a warp's tiles
+constexpr uint32_t kFinishChunkLog2 = 9;  // groups of as many tiles or more are whole chunks of kFinishThreads
+constexpr uint32_t kFinishFew = 304;      // groups of fewer tiles than a chunk, at most
+static_assert((1 << kFinishChunkLog2) == kFinishThreads, "chunks of a tile per thread");
 
 // The group size for n output tiles.
 inline uint32_t finish_group_log2(uint64_t n) {
   uint32_t l = kFinishMinLog2;
-  while (((n + (1ull << l) - 1) >> l) > kFinishGroups) l++;
+  while (((n + (1ull << l) - 1) >> l) > (l < kFinishChunkLog2 ? kFinishFew : kFinishGroups)) l++;
   return l;
 }
 inline uint32_t finish_groups(uint64_t n) {
@@ -240,7 +264,7 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const __grid_con
   uint32_t next_hit = 0;
   const auto load = [&](uint32_t g_, uint64_t c_) {
     const uint64_t u = c_ + tid;
-    const bool in = g_ < p.n_groups && u < p.n_out_tiles;
+    const bool in = g_ < p.n_groups && u < min(((uint64_t)g_ + 1) << p.group_log2, p.n_out_tiles);
     next_trip = in ? p.tile_ntrip[u] : 0ull;
     next_hit = in ? p.tile_nhit[u] : 0u;
   };

@@ -45,10 +45,10 @@ namespace {
 constexpr uint64_t kMaxSectors = CV_NOALLOC_MAX_SECTORS;
 constexpr uint64_t kMaxTiles = kMaxSectors / 32 + 32;  // output tiles of 32 sectors, plus a ragged tile
 constexpr uint64_t kOffCounters = 256;  // seg_off[1], total, status, triples per group of tiles
-constexpr uint64_t kOffNhit = 1024;     // u32 per tile
+constexpr uint64_t kOffNhit = 4096;     // u32 per tile
 constexpr uint64_t kOffNtrip = kOffNhit + ((kMaxTiles * 4 + 255) / 256) * 256;  // u64 per tile
 constexpr uint64_t kOffHits = kOffNtrip + ((kMaxTiles * 8 + 255) / 256) * 256;  // uint4 per sector slot
-static_assert(kOffCounters + 24 + (kMaxTiles / kFinishThreads + 1) * 8 <= kOffNhit, "counters");
+static_assert(kMaxTiles / kFinishThreads + 1 <= kFinishFew && kOffCounters + 24 + kFinishFew * 8 <= kOffNhit, "counters");
 constexpr uint64_t kHitSlots = kMaxTiles * 32;
 constexpr uint64_t kNoAllocScratchBytes = kOffHits + kHitSlots * 16;
 

@@ -31,6 +31,7 @@ struct CompactParams {
   const uint8_t* confirm;      // 64-bit signatures: the postings' master sectors, else null
   MatchOut* out;
   uint64_t out_cap;
+  uint32_t all_or_none;        // finish_kernel: nothing is written, nor tried, when out_cap is too little for all
   uint32_t* status;
   const uint64_t* tile_off;    // expand_kernel: output offset per tile
   const unsigned long long* group_sum;  // finish_kernel: triples per 2^group_log2 tiles
@@ -251,7 +252,11 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const __grid_con
     s_group[tid * kPer + k] = run;
     run += g[k];
   }
-  if (blockIdx.x == 0 && tid == 0) *p.total = total;
+  const bool no_room = p.all_or_none && total > p.out_cap;
+  if (blockIdx.x == 0 && tid == 0) {
+    *p.total = total;
+    if (no_room) atomicOr(p.status, kStOverflow);
+  }
   const Segment* const segs = p.segs.get();
   const bool failed = *(volatile const uint32_t*)p.status & (kStTimeout | kStProbeBound | kStBadTable);
   uint32_t hits = 0;
@@ -304,7 +309,7 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const __grid_con
     if (!empty && !failed) {
       uint32_t my_first;
       const uint32_t n_rec = group_hits(my_n, my_first);
-      if (n_rec) expand_group<T>(p, first_tile + tid - lane, my_n, my_first, n_rec, off);
+      if (n_rec && !no_room) expand_group<T>(p, first_tile + tid - lane, my_n, my_first, n_rec, off);
       hits += n_rec;
     }
   }

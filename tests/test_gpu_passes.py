@@ -1,0 +1,75 @@
+"""The passes after a scan, driven with the scratch that a caller of the C ABI has no say over (passes.cu):
+a finishing pass without room for every match."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+PACKAGE = os.path.join(os.path.dirname(HERE), "paper_0901_1307_gb300")
+ST_OVERFLOW = 8
+
+
+@pytest.fixture(scope="module")
+def cv(cuda_device):
+    import __graft_entry__
+
+    __graft_entry__.build()
+    from paper_0901_1307_gb300 import cv as cvmod
+
+    return cvmod
+
+
+@pytest.fixture(scope="module")
+def passes(cv, tmp_path_factory):
+    from paper_0901_1307_gb300 import build
+
+    lib = str(tmp_path_factory.mktemp("passes") / "passes.so")
+    cv.load()
+    subprocess.run([build._nvcc(), "-shared", "-cudart", "shared", *build.ARCH, *build.FLAGS,
+                    os.path.join(HERE, "passes.cu"), "-o", lib, "-L" + PACKAGE, "-lcv", "-Xlinker", "-rpath",
+                    "-Xlinker", PACKAGE], check=True)
+    return ctypes.CDLL(lib)
+
+
+def scan(passes, m, img, n, cap, all_or_none, room):
+    """(total, status, sectors with a match, output as int64[room, 2], -1 where nothing was written)."""
+    out = torch.full((room, 2), -1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    h = (ctypes.c_uint64 * 3)()
+    u64, vp = ctypes.c_uint64, ctypes.c_void_p
+    rc = passes.passes_scan(vp(m.handle), vp(img.data_ptr()), u64(n), u64(cap), ctypes.c_int(all_or_none),
+                            vp(out.data_ptr()), h)
+    assert rc == 0
+    return int(h[0]), int(h[1]) & 0xFFFFFFFF, int(h[2]), out
+
+
+@pytest.mark.parametrize("sig", [0, 2])
+@pytest.mark.parametrize("n", [40, 5000, 400_000])
+def test_room_for_all_or_none(cv, passes, sig, n):
+    """Without room for every match, one short or none at all, the pass writes nothing, says so, and has
+    counted; with room it writes all; where a part is wanted, that part."""
+    g = torch.Generator("cuda").manual_seed(n)
+    key = torch.randint(0, 256, (2, 512), generator=g, dtype=torch.uint8, device="cuda")
+    which = torch.arange(n, device="cuda") % 3
+    img = torch.where((which < 2)[:, None], key[which.clamp(max=1)], torch.zeros(512, dtype=torch.uint8, device="cuda"))
+    hits = int((which < 2).sum())
+    total = 3 * int((which == 0).sum()) + int((which == 1).sum())
+    with cv.master_build([key[0].repeat(3), key[1]], signature=sig) as m:
+        with cv.scan(m, [img.view(-1)], keep_on_device=True) as r:
+            want = torch.as_tensor(r.matches(0), device="cuda").view(torch.int64).clone()
+        assert want.shape[0] == total
+        for cap in (0, 1, total - 1):
+            t, status, h, out = scan(passes, m, img, n, cap, 1, total)
+            assert (t, status, h) == (total, ST_OVERFLOW, hits) and bool((out == -1).all())
+            t, status, h, out = scan(passes, m, img, n, cap, 0, total)
+            assert (t, status, h) == (total, ST_OVERFLOW, hits)
+            assert torch.equal(out[:cap], want[:cap]) and bool((out[cap:] == -1).all())
+        for part in (0, 1):
+            t, status, h, out = scan(passes, m, img, n, total, part, total)
+            assert (t, status, h) == (total, 0, hits) and torch.equal(out, want)

@@ -314,8 +314,8 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
         for (uint32_t i = 0; i < n_images; i++) {
           if (tile_base[i + 1] == tile_base[i]) continue;
           hits.count = (uint32_t*)(listed + i);
-          CV_CUDA((cudaError_t)frag_emit(m->tab, dptr[i], nbytes[i], tile_base[i], tile_off, hits, r->dev_out, room,
-                                         status, ctx->sms, stream));
+          CV_CUDA((cudaError_t)frag_emit(m->tab, dptr[i], nbytes[i], tile_base[i], tile_off,
+                                         seg_off_d + n_images, hits, r->dev_out, room, status, ctx->sms, stream));
           r->launches++;
         }
         return CV_OK;

@@ -93,10 +93,11 @@ int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uin
 // The 16-byte key of every 64-byte window at a 4-byte offset of a device image, through the
 // fragment kernels' own signature code (MD5, MD5 without padding, rolled djb2-64).
 int frag_window_sigs(int sig, const uint8_t* image, uint64_t n_bytes, uint4* out, int sms, void* stream);
-// The triples of the image's listed tiles, at out[tile_off[tile]..].
+// The triples of the image's listed tiles, at out[tile_off[tile]..]; none when *total (device memory,
+// the triples of all images) is above out_cap.
 int frag_emit(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base,
-              const uint64_t* tile_off, const FragHits& hits, MatchOut* out, uint64_t out_cap, uint32_t* status, int sms,
-              void* stream);
+              const uint64_t* tile_off, const uint64_t* total, const FragHits& hits, MatchOut* out, uint64_t out_cap,
+              uint32_t* status, int sms, void* stream);
 
 // One block whose single waiting thread waits on an mbarrier nothing completes (bounded by
 // timeout_ns): the status word gets the timeout bit. Returns a CUDA error code.

@@ -91,6 +91,7 @@ struct FragParams {
   uint32_t* hit_masks;           // per listed tile and lane: its windows with triples
   uint32_t* n_hit_tiles;         // their number (device), zero before the count
   uint32_t mask_cap;             // listed tiles that have masks
+  const uint64_t* total;         // emit: the triples of all images
   MatchOut* out;
   uint64_t out_cap;
   uint32_t* status;
@@ -624,13 +625,18 @@ __device__ __forceinline__ void frag_put(const FragParams& p, uint64_t pos, uint
 
 // A warp per listed tile: its windows with triples are numbered in window order (a lane's windows
 // follow one another) and taken 32 at a time, one per lane, so that the dependent loads of 32 of
-// them (words, slot, confirmation, posting) are in flight together. Bound by that latency.
+// them (words, slot, confirmation, posting) are in flight together. Bound by that latency. Without room
+// for the triples of all images nothing is looked up and the overflow is flagged once.
 constexpr int kEmitThreads = 256;
 
 template <int SIG, int LAYOUT>
 __global__ void __launch_bounds__(kEmitThreads) frag_emit_kernel(const __grid_constant__ FragParams p) {
   using G = FragGeom<SIG>;
   if (*(volatile const uint32_t*)p.status & (kStTimeout | kStProbeBound | kStBadTable)) return;
+  if (*p.total > p.out_cap) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(p.status, kStOverflow);
+    return;
+  }
   constexpr uint32_t kFull = 0xFFFFFFFFu;
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t n_list = *(volatile const uint32_t*)p.n_hit_tiles;
@@ -996,13 +1002,14 @@ int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uin
 }
 
 int frag_emit(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base,
-              const uint64_t* tile_off, const FragHits& hits, MatchOut* out, uint64_t out_cap, uint32_t* status, int sms,
-              void* stream) {
+              const uint64_t* tile_off, const uint64_t* total, const FragHits& hits, MatchOut* out, uint64_t out_cap,
+              uint32_t* status, int sms, void* stream) {
   FragParams p = make_params(tab, image, n_bytes, tile_base, hits, status);
   if (!p.n_tiles) return 0;
   Geom g;
   if (!geom((int)tab.sig, tab.layout, kFragFewKeys, &g)) return (int)cudaErrorInvalidValue;
   p.tile_off = tile_off;
+  p.total = total;
   p.out = out;
   p.out_cap = out_cap;
   const uint64_t warps_per_block = kEmitThreads / 32;

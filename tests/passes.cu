@@ -85,4 +85,50 @@ int passes_scan(const cv_master* m, const void* image, uint64_t n, uint64_t cap,
   return CV_OK;
 }
 
+// A fragment scan of n images (device): masks for mask_tiles listed tiles, room for cap triples at out.
+// h: total, status, then the images' first triples.
+int passes_fragments(const cv_master* m, const void* const* images, const uint64_t* bytes, uint32_t n, uint64_t mask_tiles,
+                     uint64_t cap, void* out, uint64_t* h) {
+  DevCtx* ctx;
+  TableView tab;
+  int dev;
+  CV_TRY(get_ctx(&ctx));
+  CV_TRY(master_view(m, &tab, &dev));
+  std::vector<uint64_t> base(n + 1, 0);
+  std::vector<Segment> segs(n);
+  for (uint32_t i = 0; i < n; i++) {
+    base[i + 1] = base[i] + frag_tiles((int)tab.sig, bytes[i]);
+    memset(&segs[i], 0, sizeof(Segment));
+    segs[i].tile_base = base[i];
+  }
+  if (n > kInlineSegs) return CV_EINVAL;
+  const uint64_t tiles = base[n];
+  Bufs b;
+  uint64_t *ntrip, *off, *words, *scratch;  // words: total, status, segment offsets, listed tiles per image
+  FragHits hits;
+  CV_TRY(b.get(&ntrip, tiles));
+  CV_TRY(b.get(&off, tiles));
+  CV_TRY(b.get(&words, 2 + 2 * n));
+  CV_TRY(b.get(&scratch, tile_offsets_scratch_words(tiles)));
+  CV_TRY(b.get(&hits.tiles, tiles));
+  hits.mask_tiles = mask_tiles < tiles ? mask_tiles : tiles;
+  CV_TRY(b.get(&hits.masks, hits.mask_tiles * 32));
+  uint32_t* const status = (uint32_t*)(words + 1);
+  CV_CUDA(cudaDeviceSynchronize());
+  for (uint32_t i = 0; i < n; i++) {
+    hits.count = (uint32_t*)(words + 2 + n + i);
+    CV_CUDA((cudaError_t)frag_count(tab, (const uint8_t*)images[i], bytes[i], base[i], ntrip, hits, status, nullptr,
+                                    ctx->sms, nullptr));
+  }
+  CV_CUDA((cudaError_t)launch_tile_offsets(ntrip, tiles, off, seg_list(segs.data(), nullptr, n), 1, words + 2, words,
+                                           scratch, nullptr, status));
+  for (uint32_t i = 0; i < n; i++) {
+    hits.count = (uint32_t*)(words + 2 + n + i);
+    CV_CUDA((cudaError_t)frag_emit(tab, (const uint8_t*)images[i], bytes[i], base[i], off, words, hits, (MatchOut*)out,
+                                   cap, status, ctx->sms, nullptr));
+  }
+  CV_CUDA(cudaMemcpy(h, words, (2 + n) * 8, cudaMemcpyDeviceToHost));
+  return CV_OK;
+}
+
 }  // extern "C"

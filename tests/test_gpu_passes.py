@@ -1,5 +1,5 @@
 """The passes after a scan, driven with the scratch that a caller of the C ABI has no say over (passes.cu):
-a finishing pass without room for every match."""
+passes without room for every match."""
 import ctypes
 import os
 import subprocess
@@ -73,3 +73,47 @@ def test_room_for_all_or_none(cv, passes, sig, n):
         for part in (0, 1):
             t, status, h, out = scan(passes, m, img, n, total, part, total)
             assert (t, status, h) == (total, 0, hits) and torch.equal(out, want)
+
+
+def fragments(passes, m, devs, sizes, mask_tiles, cap, room):
+    """(total, status, first triple of each image, output as int64[room, 2], -1 where nothing was written)."""
+    out = torch.full((room, 2), -1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    n, u64, vp = len(devs), ctypes.c_uint64, ctypes.c_void_p
+    h = (u64 * (2 + n))()
+    rc = passes.passes_fragments(vp(m.handle), (vp * n)(*[d.data_ptr() for d in devs]), (u64 * n)(*sizes), ctypes.c_uint32(n),
+                                 u64(mask_tiles), u64(cap), vp(out.data_ptr()), h)
+    assert rc == 0
+    return int(h[0]), int(h[1]) & 0xFFFFFFFF, [int(x) for x in h[2:]], out
+
+
+def fragment_case(sig):
+    """Three images (one without a match) of several tiles and a file of which fragments are planted, some
+    with two master copies; the master file."""
+    rng = np.random.default_rng(sig)
+    file = rng.integers(0, 256, 64 * 50, dtype=np.uint8)
+    file = np.concatenate([file, file[:640]])
+    images = []
+    for size, plants in ((30_011, 40), (9_000, 0), (70_000, 60)):
+        img = rng.integers(0, 256, size, dtype=np.uint8)
+        for w in rng.integers(0, (size - 64) // 4, plants):
+            k = int(rng.integers(0, 60))
+            img[4 * w:4 * w + 64] = file[64 * k:64 * k + 64]
+        images.append(img)
+    return images, file
+
+
+@pytest.mark.parametrize("sig", [0, 1, 2])
+def test_fragments_without_room(cv, passes, sig):
+    """Without room for every triple of all images none is written, and it is said so."""
+    images, file = fragment_case(sig)
+    devs = [torch.from_numpy(x).cuda() for x in images]
+    with cv.master_build([file], signature=sig, unit=cv.CV_UNIT_FRAGMENT) as m:
+        with cv.scan(m, devs, keep_on_device=True) as r:
+            want = torch.cat([torch.as_tensor(r.matches(i), device="cuda").view(torch.int64).clone() for i in (0, 2)])
+        total = want.shape[0]
+        assert total > 40
+        for cap in (0, 1, total - 1, total, total + 5):
+            t, status, first, out = fragments(passes, m, devs, [x.size for x in images], 1 << 22, cap, total)
+            assert t == total and status == (0 if cap >= total else ST_OVERFLOW)
+            assert torch.equal(out, want) if cap >= total else bool((out == -1).all())

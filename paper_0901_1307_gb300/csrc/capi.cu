@@ -16,6 +16,7 @@
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <mutex>
@@ -220,6 +221,17 @@ struct Readback {
   bool waited_ = false;
 };
 
+// The matches at dev into fresh memory of the host, queued on stream. The pages are touched first: one copy
+// in fifty (of 48 MB) into pages that the system had not yet provided took 43 ms instead of 4, and
+// providing them is paid for either way (median 7.46 ms for such a call without, 7.54 with; the mean
+// of 300 calls 7.78 to 8.02 and 7.57 to 7.62).
+int copy_matches(MatchOut* host, const MatchOut* dev, uint64_t n, cudaStream_t stream) {
+  static const uint64_t page = (uint64_t)std::max(4096l, sysconf(_SC_PAGESIZE));
+  for (uint64_t b = 0; b < n * sizeof(MatchOut); b += page) reinterpret_cast<volatile char*>(host)[b] = 0;
+  CV_CUDA(cudaMemcpyAsync(host, dev, n * sizeof(MatchOut), cudaMemcpyDeviceToHost, stream));
+  return CV_OK;
+}
+
 // cv_scan over a fragment table (Section 5): count kernel per image, one offset scan over all
 // tiles, emit kernel per image over its tiles with triples. Host images are copied whole.
 int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_images, uint32_t flags,
@@ -358,7 +370,7 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
         if (total <= rb.staged) {
           memcpy(r->host, rb.stage.matches, total * sizeof(MatchOut));
         } else {
-          CV_CUDA(cudaMemcpyAsync(r->host, r->dev_out, total * sizeof(MatchOut), cudaMemcpyDeviceToHost, stream));
+          CV_TRY(copy_matches(r->host, r->dev_out, total, stream));
           more = true;
         }
       }
@@ -654,7 +666,7 @@ int cv_scan(const cv_master* m, const cv_buf* images, uint32_t n_images, const c
         if (expanded_early && total <= rb->staged) {
           memcpy(r->host, rb->stage.matches, total * sizeof(MatchOut));
         } else {
-          CV_CUDA(cudaMemcpyAsync(r->host, r->dev_out, total * sizeof(MatchOut), cudaMemcpyDeviceToHost, stream));
+          CV_TRY(copy_matches(r->host, r->dev_out, total, stream));
           more = true;
         }
       }

@@ -1,6 +1,7 @@
 """What a call reads back in one wait: match counts below, at and above what is staged, scans from
 more threads than there are stages, and tables whose memory was another table's before."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -99,3 +100,20 @@ def test_a_closed_table_is_free_memory(cv):
     m.close()
     freed = torch.cuda.mem_get_info()[0] - used
     assert size > 2 << 30 and freed >= size - (1 << 30) - (64 << 20), (size, freed)
+
+
+def test_large_results_take_the_same_time_each(cv):
+    """48 MB of matches to the host, 600 times: no call (but one at most) takes five times the median."""
+    key = torch.randint(0, 256, (512,), dtype=torch.uint8, device="cuda")
+    img, file = key.repeat(1 << 16), key.repeat(48)
+    t = []
+    with cv.master_build([file]) as m:
+        for _ in range(600):
+            a = time.perf_counter()
+            with cv.scan(m, [img]) as r:
+                got = r.matches(0)
+            t.append(time.perf_counter() - a)
+            del r
+    assert got.size == 48 << 16 and np.array_equal(got["file_sector"][:48], np.arange(48))
+    slow = [x for x in t if x > 5 * np.median(t)]
+    assert len(slow) <= 1, (np.median(t), slow)

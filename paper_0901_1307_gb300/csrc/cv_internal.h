@@ -98,11 +98,11 @@ struct TableView {
   uint32_t pad;
 };
 
-// The index over a sorted table's n keys (n < 2^27): 2^(32 - shift) buckets of h0's top bits, of 1 to
-// 2 keys on average when they are spread evenly.
+// The index over a sorted table's n keys: 2^(32 - shift) buckets of h0's top bits, of 1 to 2 keys on
+// average when they are spread evenly.
 inline uint32_t key_index_shift(uint32_t n) {
   uint32_t bits = 1;
-  while ((2u << bits) <= n) bits++;
+  while ((2ull << bits) <= n) bits++;
   return 32 - bits;
 }
 // Words of the keys and their index together.

@@ -650,8 +650,8 @@ int cv_master_load(const char* path, void* stream_, cv_master** out) {
                   h.sig <= (uint32_t)kSigCrc64 && in.unit == h.unit && in.layout == h.layout &&
                   in.signature == h.sig && (h.tau_mask == 0u || h.tau_mask == 7u) && in.n_kept <= in.n_sectors &&
                   in.n_sectors < (1ull << 27) && in.n_unique <= in.n_kept && in.n_slots >= 1 &&
-                  in.n_slots <= (1ull << 31) &&
-                  (h.layout == kLayoutSorted ? h.n_keys == in.n_unique && in.n_slots == in.n_unique
+                  in.n_slots <= (1ull << 31) && h.n_keys == in.n_unique && in.n_unique <= in.n_slots &&
+                  (h.layout == kLayoutSorted ? in.n_slots == in.n_unique
                                              : ((uint64_t)h.slot_mask + 1 == in.n_slots &&
                                                 (in.n_slots & (in.n_slots - 1)) == 0 && h.max_probe <= in.n_slots)) &&
                   h.bytes_slots == n_records * 32 && h.bytes_postings == in.n_kept * 8 &&

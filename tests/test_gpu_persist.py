@@ -2,7 +2,10 @@
 from (and like the oracle); damaged or foreign files are refused with an error code, including a
 slot whose posting range points past the postings (checked on the device at load time)."""
 import ctypes
+import os
 import struct
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -12,6 +15,7 @@ from paper_0901_1307_gb300 import synth
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 
@@ -108,3 +112,27 @@ def test_damaged_files_refused(cv, tmp_path):
     with pytest.raises(cv.CVError) as e:
         cv.master_load(tmp_path / "missing.cvt")
     assert e.value.code == cv.CV_EIO
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(layout=1), dict(signature=2, unit=1)])
+@pytest.mark.parametrize("n_keys", [0x80000000, 0xFFFFFFFF, 1 << 27, -1, 1])
+def test_key_count_of_another_table_refused(cv, kw, n_keys, tmp_path):
+    """The header's number of keys is the table's number of distinct keys, whatever the layout (a search
+    index is sized by it, a sorted copy of the table made by it). -1, 1: one less, one more."""
+    rng = np.random.default_rng(84)
+    files = [rng.integers(0, 256, 512 * 40, dtype=np.uint8)]
+    path = tmp_path / "t.cvt"
+    with cv.master_build(files, **kw) as m:
+        cv.master_save(m, path)
+        unique = m.info()["n_unique"]
+    data = bytearray(path.read_bytes())
+    at = 8 + 4 + 4 + ctypes.sizeof(cv.cv_master_info) + 7 * 4
+    assert struct.unpack_from("<I", data, at)[0] == unique
+    struct.pack_into("<I", data, at, unique + n_keys if n_keys in (-1, 1) else n_keys)
+    path.write_bytes(bytes(data))
+    child = subprocess.run([sys.executable, "-c", "import sys; sys.path.insert(0, sys.argv[1])\n"
+                            "from paper_0901_1307_gb300 import cv\n"
+                            "try: cv.master_load(sys.argv[2])\n"
+                            "except cv.CVError as e: print('code', e.code)", ROOT, str(path)],
+                           capture_output=True, text=True, timeout=60)
+    assert child.stdout.split() == ["code", str(cv.CV_ECORRUPT)], (child.stdout, child.stderr)

@@ -59,24 +59,34 @@ int get_ctx(DevCtx** out) {
     if (prop.major < 10) return CV_ENODEV;
     c.dev = dev;
     c.sms = prop.multiProcessorCount;
+    c.cfg_index = -1;
+    const char* env = getenv("CV_SCAN_CONFIG");
+    if (env && *env) {
+      int k = find_cfg(env);
+      if (k < 0) return CV_EINVAL;
+      c.cfg_index = k;
+    }
+    // What is made here stays when a later step fails, and the next call goes on from there.
     cudaMemPoolProps pp;
     memset(&pp, 0, sizeof pp);
     pp.allocType = cudaMemAllocationTypePinned;
     pp.handleTypes = cudaMemHandleTypeNone;
     pp.location.type = cudaMemLocationTypeDevice;
     pp.location.id = dev;
-    CV_CUDA(cudaMemPoolCreate(&c.pool, &pp));
+    if (!c.pool) CV_CUDA(cudaMemPoolCreate(&c.pool, &pp));
     uint64_t thr = UINT64_MAX;
     CV_CUDA(cudaMemPoolSetAttribute(c.pool, cudaMemPoolAttrReleaseThreshold, &thr));
-    CV_CUDA(cudaMemPoolCreate(&c.table_pool, &pp));
+    if (!c.table_pool) CV_CUDA(cudaMemPoolCreate(&c.table_pool, &pp));
     thr = kTablePoolKept;
     CV_CUDA(cudaMemPoolSetAttribute(c.table_pool, cudaMemPoolAttrReleaseThreshold, &thr));
-    uint8_t* pinned = nullptr;
-    constexpr size_t stage_bytes = kStageCounts * 8 + kStageMatches * sizeof(MatchOut);
-    CV_CUDA(cudaMallocHost((void**)&pinned, kStages * stage_bytes));
-    for (int k = 0; k < kStages; k++, pinned += stage_bytes)
-      c.stage_free.push_back(Stage{(uint64_t*)pinned, (MatchOut*)(pinned + kStageCounts * 8)});
-    CV_CUDA(cudaStreamCreateWithFlags(&c.copy_stream, cudaStreamNonBlocking));
+    if (c.stage_free.empty()) {  // no call has taken one before the context is ready
+      uint8_t* pinned = nullptr;
+      constexpr size_t stage_bytes = kStageCounts * 8 + kStageMatches * sizeof(MatchOut);
+      CV_CUDA(cudaMallocHost((void**)&pinned, kStages * stage_bytes));
+      for (int k = 0; k < kStages; k++, pinned += stage_bytes)
+        c.stage_free.push_back(Stage{(uint64_t*)pinned, (MatchOut*)(pinned + kStageCounts * 8)});
+    }
+    if (!c.copy_stream) CV_CUDA(cudaStreamCreateWithFlags(&c.copy_stream, cudaStreamNonBlocking));
     cudaDriverEntryPointQueryResult q;
     void* fn = nullptr;
     CV_CUDA(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q));
@@ -101,13 +111,6 @@ int get_ctx(DevCtx** out) {
     }
     if (!cfgs[0].digest_fn[0]) return CV_ECUDA;  // the default configuration serves every digest pass
 
-    c.cfg_index = -1;
-    const char* env = getenv("CV_SCAN_CONFIG");
-    if (env && *env) {
-      int k = find_cfg(env);
-      if (k < 0) return CV_EINVAL;
-      c.cfg_index = k;
-    }
     c.ready = true;
   }
   *out = &c;

@@ -292,8 +292,17 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       const uint64_t off_words = tile_offsets_scratch_words(T);
       CV_TRY(tmp.alloc(&seg_off_d, (2ull * n_images + 3 + off_words) * 8));
       CV_TRY(tmp.alloc(&hits.tiles, T * 4));
+      // The masks spare the emit pass lookups, and the room for matches below a wait: without memory for
+      // either the scan does without.
+      const int before = last_cuda();
       hits.mask_tiles = std::min(T, kFragMaskTiles);
-      CV_TRY(tmp.alloc(&hits.masks, hits.mask_tiles * 32 * 4));
+      int got = tmp.alloc(&hits.masks, hits.mask_tiles * 32 * 4);
+      if (got == CV_ENOMEM) {
+        set_last_cuda(before);
+        hits.mask_tiles = 0;
+        got = tmp.alloc(&hits.masks, 0);
+      }
+      CV_TRY(got);
       std::vector<Segment> segs(n_images);
       memset(segs.data(), 0, segs.size() * sizeof(Segment));
       for (uint32_t i = 0; i < n_images; i++) {
@@ -322,6 +331,7 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
                                                true));
       r->launches += 1;
       auto emit = [&](uint64_t room) -> int {
+        r->dev_out = nullptr;
         CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, room * sizeof(MatchOut), ctx->pool, stream));
         for (uint32_t i = 0; i < n_images; i++) {
           if (tile_base[i + 1] == tile_base[i]) continue;
@@ -336,12 +346,18 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       // the table suggests, its outcome read back with the counts, and run again only if that
       // was too little.
       const uint64_t hint = __atomic_load_n(&const_cast<cv_master*>(m)->last_matches, __ATOMIC_RELAXED);
-      const uint64_t room = std::max<uint64_t>(hint + hint / 4 + 1024, 4096);
-      CV_TRY(emit(room));
+      uint64_t room = std::max<uint64_t>(hint + hint / 4 + 1024, 4096);
+      got = emit(room);
+      if (got == CV_ENOMEM && !r->dev_out) {  // the count is waited for
+        set_last_cuda(before);
+        room = 0;
+        got = CV_OK;
+      }
+      CV_TRY(got);
       std::vector<uint64_t> seg_off(n_images + 3, 0);
       Readback rb(ctx, seg_off.data(), seg_off_d, n_images + 3, stream);
       CV_TRY(rb.counts());
-      if (!r->on_device) CV_TRY(rb.matches(r->dev_out, room));
+      if (!r->on_device && room) CV_TRY(rb.matches(r->dev_out, room));
       CV_CUDA(cudaEventRecord(ev[3], stream));
       CV_TRY(rb.wait());
       uint32_t st = (uint32_t)seg_off[n_images + 1];
@@ -350,7 +366,7 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       const uint64_t total = seg_off[n_images];
       __atomic_store_n(&const_cast<cv_master*>(m)->last_matches, total, __ATOMIC_RELAXED);
       r->st.confirm_rejected = seg_off[n_images + 2];
-      if (total == 0 || total > room) {
+      if (r->dev_out && (total == 0 || total > room)) {
         CV_CUDA(cudaFreeAsync(r->dev_out, stream));
         r->dev_out = nullptr;
       }

@@ -7,6 +7,8 @@ import subprocess
 import numpy as np
 import pytest
 
+import oracle
+
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
@@ -117,3 +119,23 @@ def test_fragments_without_room(cv, passes, sig):
             t, status, first, out = fragments(passes, m, devs, [x.size for x in images], 1 << 22, cap, total)
             assert t == total and status == (0 if cap >= total else ST_OVERFLOW)
             assert torch.equal(out, want) if cap >= total else bool((out == -1).all())
+
+
+@pytest.mark.parametrize("sig", [0, 1, 2])
+@pytest.mark.parametrize("mask_tiles", [0, 1, 2, 9, 12, 1 << 20])
+def test_hit_lists_beyond_their_masks(cv, passes, sig, mask_tiles):
+    """Masks for none, some (ending within an image, at its first tile, before it) or all of the listed tiles:
+    the windows of the others are looked up again. The images' first triples are right as well."""
+    images, file = fragment_case(sig)
+    devs = [torch.from_numpy(x).cuda() for x in images]
+    want = [oracle.frag_match(x, [file]) for x in images]
+    total = sum(w.size for w in want)
+    for kw in ({}, {"bloom_bits_per_key": 0}, {"layout": cv.CV_LAYOUT_SORTED}):
+        with cv.master_build([file], signature=sig, unit=cv.CV_UNIT_FRAGMENT, **kw) as m:
+            t, status, first, out = fragments(passes, m, devs, [x.size for x in images], mask_tiles, total, total)
+        assert (t, status) == (total, 0)
+        assert first[:3] == [0, want[0].size, want[0].size]
+        got = out.cpu().numpy()
+        every = np.concatenate(want)
+        assert np.array_equal(got[:, 0], every["disk_sector"].astype(np.int64))
+        assert np.array_equal(got[:, 1] >> 32, every["file_sector"].astype(np.int64))

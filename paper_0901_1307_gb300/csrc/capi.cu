@@ -232,8 +232,8 @@ int copy_matches(MatchOut* host, const MatchOut* dev, uint64_t n, cudaStream_t s
   return CV_OK;
 }
 
-// cv_scan over a fragment table (Section 5): count kernel per image, one offset scan over all
-// tiles, emit kernel per image over its tiles with triples. Host images are copied whole.
+// cv_scan over a fragment table (Section 5): a count kernel over the images' tiles, an offset scan over
+// these, an emit kernel over the tiles with triples. Host images are copied whole.
 int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_images, uint32_t flags,
               cudaStream_t stream, cv_result** out) {
   NvtxRange nvtx_range("cv.scan.fragments");
@@ -288,9 +288,9 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       Segment* segs_d = nullptr;
       CV_TRY(tmp.alloc(&tile_ntrip, std::max<uint64_t>(T, 1) * 8));
       CV_TRY(tmp.alloc(&tile_off, std::max<uint64_t>(T, 1) * 8));
-      // seg_off[n], total, status, rejected, listed tiles of every image, the offset pass's words
+      // seg_off[n], total, status, rejected, listed tiles, the offset pass's words
       const uint64_t off_words = tile_offsets_scratch_words(T);
-      CV_TRY(tmp.alloc(&seg_off_d, (2ull * n_images + 3 + off_words) * 8));
+      CV_TRY(tmp.alloc(&seg_off_d, (n_images + 4ull + off_words) * 8));
       CV_TRY(tmp.alloc(&hits.tiles, T * 4));
       // The masks spare the emit pass lookups, and the room for matches below a wait: without memory for
       // either the scan does without.
@@ -316,30 +316,32 @@ int frag_scan(DevCtx* ctx, const cv_master* m, const cv_buf* images, uint32_t n_
       uint32_t* status = (uint32_t*)(seg_off_d + n_images + 1);
       unsigned long long* rejected = (unsigned long long*)(seg_off_d + n_images + 2);
       uint64_t* listed = seg_off_d + n_images + 3;
-      CV_CUDA(cudaMemsetAsync(status, 0, 16 + (n_images + off_words) * 8ull, stream));
-      CV_CUDA(cudaEventRecord(ev[1], stream));
-      for (uint32_t i = 0; i < n_images; i++) {
-        if (tile_base[i + 1] == tile_base[i]) continue;
-        hits.count = (uint32_t*)(listed + i);
-        CV_CUDA((cudaError_t)frag_count(m->tab, dptr[i], nbytes[i], tile_base[i], tile_ntrip, hits, status,
-                                        rejected, ctx->sms, stream));
-        r->launches++;
+      hits.count = (uint32_t*)listed;
+      std::vector<FragImage> with_tiles;
+      for (uint32_t i = 0; i < n_images; i++)
+        if (tile_base[i + 1] > tile_base[i])
+          with_tiles.push_back(FragImage{dptr[i], nbytes[i], frag_windows(nbytes[i]), tile_base[i]});
+      FragImage* with_tiles_d = nullptr;
+      if (with_tiles.size() > kInlineSegs) {
+        CV_TRY(tmp.alloc(&with_tiles_d, with_tiles.size() * sizeof(FragImage)));
+        CV_CUDA(cudaMemcpyAsync(with_tiles_d, with_tiles.data(), with_tiles.size() * sizeof(FragImage),
+                                cudaMemcpyHostToDevice, stream));
       }
+      const FragImages scanned = frag_images(with_tiles.data(), with_tiles_d, with_tiles.size());
+      CV_CUDA(cudaMemsetAsync(status, 0, 24 + off_words * 8ull, stream));
+      CV_CUDA(cudaEventRecord(ev[1], stream));
+      CV_CUDA((cudaError_t)frag_count(m->tab, scanned, T, tile_ntrip, hits, status, rejected, ctx->sms, stream));
+      if (T) r->launches++;
       CV_CUDA(cudaEventRecord(ev[2], stream));
       CV_CUDA((cudaError_t)launch_tile_offsets(tile_ntrip, T, tile_off, seg_list(segs.data(), segs_d, n_images), 1,
-                                               seg_off_d, seg_off_d + n_images, listed + n_images, stream, status,
-                                               true));
+                                               seg_off_d, seg_off_d + n_images, listed + 1, stream, status, true));
       r->launches += 1;
       auto emit = [&](uint64_t room) -> int {
         r->dev_out = nullptr;
         CV_CUDA(cudaMallocFromPoolAsync((void**)&r->dev_out, room * sizeof(MatchOut), ctx->pool, stream));
-        for (uint32_t i = 0; i < n_images; i++) {
-          if (tile_base[i + 1] == tile_base[i]) continue;
-          hits.count = (uint32_t*)(listed + i);
-          CV_CUDA((cudaError_t)frag_emit(m->tab, dptr[i], nbytes[i], tile_base[i], tile_off,
-                                         seg_off_d + n_images, hits, r->dev_out, room, status, ctx->sms, stream));
-          r->launches++;
-        }
+        CV_CUDA((cudaError_t)frag_emit(m->tab, scanned, T, tile_off, seg_off_d + n_images, hits, r->dev_out, room, status,
+                                       ctx->sms, stream));
+        if (T) r->launches++;
         return CV_OK;
       };
       // As in the sector scan: the emit pass is launched with the room that the last scan against

@@ -75,9 +75,23 @@ int frag_digests(int sig, const uint8_t* arena, uint64_t n, uint4* dig, uint8_t*
 // for none; mask = words - 1) and the shared-memory filter l1 (kFragL1Bytes).
 int frag_bloom(int sig, const uint4* slots, uint32_t n_slots, uint64_t n_keys, uint32_t* words, uint32_t mask,
                uint32_t* l1, int sms, void* stream);
-// The hit lists of a scan's images: tiles has room for every tile of the scan, masks (32 words per
-// tile) for the first mask_tiles of them, an image's entries starting at its first tile; count is
-// the image's own counter.
+// The images of a scan that have a tile, in order: their tiles are numbered through, an image's begin at
+// tile_base. Up to kInlineSegs of them travel in the kernels' parameters, as SegList's segments do.
+struct FragImage {
+  const uint8_t* data;  // device memory, 16-byte aligned
+  uint64_t n_bytes, n_windows, tile_base;
+};
+struct FragImages {
+  const FragImage* dev;  // device memory; not used (may be null) when n <= kInlineSegs
+  uint32_t n;
+  uint32_t pad;
+  FragImage in[kInlineSegs];
+  __host__ __device__ const FragImage* get() const { return n <= kInlineSegs ? in : dev; }
+};
+FragImages frag_images(const FragImage* host, const FragImage* dev, size_t n);
+
+// The hit list of a scan: tiles has room for every tile, masks (32 words per tile) for the first
+// mask_tiles that are listed.
 struct FragHits {
   uint32_t* tiles;
   uint32_t* masks;
@@ -85,19 +99,18 @@ struct FragHits {
   uint32_t* count;
 };
 constexpr uint64_t kFragMaskTiles = 1ull << 22;
-// Triples per tile of one device image (16-byte aligned) into tile_ntrip[tile_base ..) and its
-// hit list (*hits.count zero before); djb2 candidates dropped by the byte comparison are added to
-// *rejected (when non-null).
-int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base, uint64_t* tile_ntrip,
-               const FragHits& hits, uint32_t* status, unsigned long long* rejected, int sms, void* stream);
+// Triples per tile of the images (n_tiles in all) into tile_ntrip and their hit list (*hits.count zero
+// before); djb2 candidates dropped by the byte comparison are added to *rejected (when non-null).
+int frag_count(const TableView& tab, const FragImages& images, uint64_t n_tiles, uint64_t* tile_ntrip, const FragHits& hits,
+               uint32_t* status, unsigned long long* rejected, int sms, void* stream);
 // The 16-byte key of every 64-byte window at a 4-byte offset of a device image, through the
 // fragment kernels' own signature code (MD5, MD5 without padding, rolled djb2-64).
 int frag_window_sigs(int sig, const uint8_t* image, uint64_t n_bytes, uint4* out, int sms, void* stream);
-// The triples of the image's listed tiles, at out[tile_off[tile]..]; none when *total (device memory,
-// the triples of all images) is above out_cap.
-int frag_emit(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base,
-              const uint64_t* tile_off, const uint64_t* total, const FragHits& hits, MatchOut* out, uint64_t out_cap,
-              uint32_t* status, int sms, void* stream);
+// The triples of the listed tiles, at out[tile_off[tile]..]; none when *total (device memory, the triples
+// of all images) is above out_cap.
+int frag_emit(const TableView& tab, const FragImages& images, uint64_t n_tiles, const uint64_t* tile_off,
+              const uint64_t* total, const FragHits& hits, MatchOut* out, uint64_t out_cap, uint32_t* status, int sms,
+              void* stream);
 
 // One block whose single waiting thread waits on an mbarrier nothing completes (bounded by
 // timeout_ns): the status word gets the timeout bit. Returns a CUDA error code.

@@ -80,14 +80,11 @@ constexpr uint64_t kDjbInit = 5381ull * pow33(64);  // 5381 * 33^64: the initial
 
 struct FragParams {
   TableView tab;
-  const uint8_t* image;
-  uint64_t n_bytes;
-  uint64_t n_windows;
-  uint64_t n_tiles;
-  uint64_t tile_base;            // index of this image's first tile in tile_ntrip / tile_off
+  FragImages images;             // their tiles are numbered through
+  uint64_t n_tiles;              // of all images
   uint64_t* tile_ntrip;          // count: triples per tile
   const uint64_t* tile_off;      // emit: output offset per tile
-  uint32_t* hit_tiles;           // this image's tiles with triples, in any order (local indices)
+  uint32_t* hit_tiles;           // the tiles with triples, in any order
   uint32_t* hit_masks;           // per listed tile and lane: its windows with triples
   uint32_t* n_hit_tiles;         // their number (device), zero before the count
   uint32_t mask_cap;             // listed tiles that have masks
@@ -259,7 +256,7 @@ __device__ __forceinline__ bool frag_equal(const uint32_t* x, const uint8_t* m) 
 // That holds while few windows pass the first filter. It has 2^20 bits whatever the table's size: at
 // 500,000 keys 0.38 of the windows pass and at 2^20 three of four, most lanes then have more than eight
 // of them, and each one sent on costs 16 words, the whole hash and a slot (1,564 and 6,350 us). With
-// many keys every window that passes asks for its Bloom word in the loop, four ahead of their tests,
+// many keys every window that passes asks for its Bloom word in the loop, six ahead of their tests,
 // and the tile stays as it is: 692 and 1,165 us. The most keys: nearly every window passes, so
 // the first filter is not looked at, and the Bloom words, from L2 and DRAM, are all of the cost. What
 // matters then is an even stream of requests: words asked for in rounds of 4, 8 and 23 took 3,780,
@@ -272,7 +269,7 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
     const uint32_t* const bloom = reinterpret_cast<const uint32_t*>(p.tab.bloom);
     Djb2Roll<FragRoll<KEYS>> roll;
     uint32_t cand = 0;
-    constexpr int kAhead = 4;
+    constexpr int kAhead = 6;
     uint32_t v[kAhead], bits[kAhead];
 #pragma unroll
     for (int i = 0; i < G::kWPT + kAhead; i++) {
@@ -415,13 +412,26 @@ __device__ __forceinline__ uint32_t frag_candidates(const FragParams& p, uint32_
   }
 }
 
-// The 16 words of this thread's window w0 + i of the tile: in the tile, or, where the tile may be
-// overwritten, in the image.
+// The image of a tile.
+template <bool MULTI>
+__device__ __forceinline__ const FragImage& frag_image(const FragParams& p, uint64_t tile) {
+  if constexpr (!MULTI) return p.images.in[0];
+  const FragImage* const im = p.images.get();
+  uint32_t lo = 0, hi = p.images.n;
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (im[mid].tile_base <= tile) lo = mid; else hi = mid;
+  }
+  return im[lo];
+}
+
+// The 16 words of this thread's window w0 + i of the image's tile: in the staged tile, or, where that may
+// be overwritten, in the image.
 template <int SIG, int KEYS>
-__device__ __forceinline__ const uint32_t* frag_words(const FragParams& p, uint64_t tile, const uint32_t* ws,
+__device__ __forceinline__ const uint32_t* frag_words(const FragImage& im, uint64_t tile, const uint32_t* ws,
                                                       uint32_t w) {
   if constexpr (FragGeom<SIG>::kRolled && KEYS == kFragFewKeys)
-    return reinterpret_cast<const uint32_t*>(p.image) + (tile * FragGeom<SIG>::kTileWin + w);
+    return reinterpret_cast<const uint32_t*>(im.data) + (tile * FragGeom<SIG>::kTileWin + w);
   return ws + w;
 }
 
@@ -460,8 +470,8 @@ __device__ __forceinline__ uint32_t frag_resolve(const FragParams& p, const uint
 // Triples of this thread's candidate windows; hits: the windows with any; *rejected adds the
 // candidates that the byte comparison dropped. Every lane of the warp calls it.
 template <int SIG, int LAYOUT, int KEYS>
-__device__ __forceinline__ uint64_t frag_thread_count(const FragParams& p, uint64_t tile, const uint32_t* ws,
-                                                      uint32_t w0, uint32_t cand, uint32_t& hits, uint32_t* rejected) {
+__device__ __forceinline__ uint64_t frag_thread_count(const FragParams& p, const FragImage& im, uint64_t tile,
+                                                      const uint32_t* ws, uint32_t w0, uint32_t cand, uint32_t& hits, uint32_t* rejected) {
   uint64_t n = 0;
   hits = 0;
   while (__any_sync(0xFFFFFFFFu, cand != 0)) {
@@ -469,7 +479,7 @@ __device__ __forceinline__ uint64_t frag_thread_count(const FragParams& p, uint6
     const uint32_t i = has ? (uint32_t)__ffs(cand) - 1u : 0u;
     cand &= cand - 1;
     uint32_t off, cnt;
-    const uint32_t k = frag_resolve<SIG, LAYOUT>(p, frag_words<SIG, KEYS>(p, tile, ws, w0 + i), has, off, cnt);
+    const uint32_t k = frag_resolve<SIG, LAYOUT>(p, frag_words<SIG, KEYS>(im, tile, ws, w0 + i), has, off, cnt);
     n += k;
     if (k) hits |= 1u << i;
     *rejected += cnt - k;
@@ -498,43 +508,47 @@ __device__ __forceinline__ uint64_t warp_exclusive_u64(uint64_t v, uint64_t* tot
   return incl - v;
 }
 
-// Lane 0: issue tile `tile` into the buffer at smem address dst (completion on bar).
+// Lane 0: issue the image's tile `tile` into the buffer at smem address dst (completion on bar).
 template <int SIG>
-__device__ __forceinline__ void frag_issue(const FragParams& p, uint64_t tile, uint32_t dst, uint32_t bar,
+__device__ __forceinline__ void frag_issue(const FragImage& im, uint64_t tile, uint32_t dst, uint32_t bar,
                                            uint64_t policy) {
   using G = FragGeom<SIG>;
   const uint64_t start = tile * G::kTileStep;
-  const uint64_t left = p.n_bytes - start;
+  const uint64_t left = im.n_bytes - start;
   const uint32_t avail = left < G::kTileBytes ? (uint32_t)left : G::kTileBytes;
   const uint32_t bulk = avail & ~15u;
   mbar_arrive_expect_tx(bar, bulk);
-  if (bulk) bulk_load(dst, p.image + start, bulk, bar, policy);
+  if (bulk) bulk_load(dst, im.data + start, bulk, bar, policy);
 }
 
 // The bytes of the tile past its last whole 16-byte chunk (the bulk copy moves whole chunks
 // only), with plain loads by the warp's lanes; only the image's last tile has any. Ends with a
 // warp barrier.
 template <int SIG>
-__device__ __forceinline__ void frag_tail(const FragParams& p, uint64_t tile, uint8_t* buf) {
+__device__ __forceinline__ void frag_tail(const FragImage& im, uint64_t tile, uint8_t* buf) {
   using G = FragGeom<SIG>;
   const uint64_t start = tile * G::kTileStep;
-  const uint64_t left = p.n_bytes - start;
+  const uint64_t left = im.n_bytes - start;
   const uint32_t avail = left < G::kTileBytes ? (uint32_t)left : G::kTileBytes;
   const uint32_t b = (avail & ~15u) + (threadIdx.x & 31);
-  if (b < avail) buf[b] = p.image[start + b];
+  if (b < avail) buf[b] = im.data[start + b];
   __syncwarp();
 }
 
 template <int SIG>
-__device__ __forceinline__ uint32_t frag_valid(const FragParams& p, uint64_t tile, uint32_t w0) {
+__device__ __forceinline__ uint32_t frag_valid(const FragImage& im, uint64_t tile, uint32_t w0) {
   using G = FragGeom<SIG>;
   const uint64_t k0 = tile * G::kTileWin + w0;
-  if (k0 >= p.n_windows) return 0u;
-  const uint64_t left = p.n_windows - k0;
+  if (k0 >= im.n_windows) return 0u;
+  const uint64_t left = im.n_windows - k0;
   return left < (uint64_t)G::kWPT ? (uint32_t)left : (uint32_t)G::kWPT;
 }
 
-template <int SIG, int LAYOUT, int KEYS>
+// MULTI: several images, one after another in tile numbers; a tile's image is found by search. (With a
+// launch per image, small ones ran one after another, each on a few SMs, and as many emit launches behind
+// them: 200 images of 64 KiB without a match took 2,460 us, MD5 10,470; in one go 256 and 341.) For one
+// image its parameters are constants of the launch, which the kernels' registers are laid out for.
+template <int SIG, int LAYOUT, int KEYS, bool MULTI>
 __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBlocks)
     frag_count_kernel(const __grid_constant__ FragParams p) {
   using G = FragGeom<SIG>;
@@ -563,7 +577,11 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBl
     mbar_arrive_expect_tx(bar_l1, kFragL1Bytes);
     bulk_load(smem_addr(fsm + G::kL1Off), p.tab.frag_l1, kFragL1Bytes, bar_l1, policy);
   }
-  if (lane == 0 && first < p.n_tiles) frag_issue<SIG>(p, first, smem_addr(buf), bar, policy);
+  const auto issue = [&](uint64_t tile) {
+    const FragImage& im = frag_image<MULTI>(p, tile);
+    frag_issue<SIG>(im, tile - (MULTI ? im.tile_base : 0ull), smem_addr(buf), bar, policy);
+  };
+  if (lane == 0 && first < p.n_tiles) issue(first);
   bool ok = true;
   if constexpr (G::kL1) ok = mbar_wait(bar_l1, 0u, &abort_flag[G::kWarps], p.status);
   bool aborted = !__syncthreads_and(ok);  // the only block-wide barrier: the filter is in place
@@ -576,13 +594,15 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBl
       aborted = true;
       break;
     }
-    if ((tile + 1) * G::kTileStep + 64 > p.n_bytes) frag_tail<SIG>(p, tile, buf);  // warp-uniform
+    const FragImage& im = frag_image<MULTI>(p, tile);
+    const uint64_t local = tile - (MULTI ? im.tile_base : 0ull);
+    if ((local + 1) * G::kTileStep + 64 > im.n_bytes) frag_tail<SIG>(im, local, buf);  // warp-uniform
     uint32_t* ws = reinterpret_cast<uint32_t*>(buf);
     const uint32_t w0 = (uint32_t)lane * G::kWPT;
-    const uint32_t cand = frag_candidates<SIG, KEYS>(p, ws, w0, frag_valid<SIG>(p, tile, w0), l1, list, masks);
+    const uint32_t cand = frag_candidates<SIG, KEYS>(p, ws, w0, frag_valid<SIG>(im, local, w0), l1, list, masks);
     uint32_t rej = 0;
     uint32_t hits;
-    uint64_t n = frag_thread_count<SIG, LAYOUT, KEYS>(p, tile, ws, w0, cand, hits, &rej);
+    uint64_t n = frag_thread_count<SIG, LAYOUT, KEYS>(p, im, local, ws, w0, cand, hits, &rej);
     if (sig_is_weak(SIG) && rej && p.rejected) atomicAdd(p.rejected, (unsigned long long)rej);
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) n += __shfl_xor_sync(0xFFFFFFFFu, n, d);
@@ -595,11 +615,11 @@ __global__ void __launch_bounds__(FragGeom<SIG>::kThreads, FragGeom<SIG>::kMinBl
     }
     __syncwarp();  // every lane is done with the buffer
     if (lane == 0) {
-      p.tile_ntrip[p.tile_base + tile] = n;
+      p.tile_ntrip[tile] = n;
       const uint64_t next = tile + n_warps;
       if (next < p.n_tiles) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        frag_issue<SIG>(p, next, smem_addr(buf), bar, policy);
+        issue(next);
       }
     }
     __syncwarp();
@@ -642,11 +662,13 @@ __global__ void __launch_bounds__(kEmitThreads) frag_emit_kernel(const __grid_co
   const uint32_t n_list = *(volatile const uint32_t*)p.n_hit_tiles;
   const uint32_t n_warps = gridDim.x * (kEmitThreads / 32);
   for (uint32_t j = blockIdx.x * (kEmitThreads / 32) + (threadIdx.x >> 5); j < n_list; j += n_warps) {
-    const uint64_t tile = p.hit_tiles[j];
+    const uint64_t numbered = p.hit_tiles[j];
+    const FragImage& im = frag_image<true>(p, numbered);
+    const uint64_t tile = numbered - im.tile_base;
     // beyond the masks' room every window is looked up
-    const uint32_t valid = frag_valid<SIG>(p, tile, lane * G::kWPT);
+    const uint32_t valid = frag_valid<SIG>(im, tile, lane * G::kWPT);
     const uint32_t mask = j < p.mask_cap ? p.hit_masks[32ull * j + lane] : (uint32_t)((1ull << valid) - 1u);
-    uint64_t at = p.tile_off[p.tile_base + tile];
+    uint64_t at = p.tile_off[numbered];
     const uint32_t n = (uint32_t)__popc(mask);
     uint32_t first = n;
 #pragma unroll
@@ -669,7 +691,7 @@ __global__ void __launch_bounds__(kEmitThreads) frag_emit_kernel(const __grid_co
       if (!has) k = 0;
       for (; k > 0; k--) m &= m - 1;
       const uint64_t w = tile * G::kTileWin + src * G::kWPT + (has ? (uint32_t)__ffs(m) - 1u : 0u);
-      const uint32_t* x = reinterpret_cast<const uint32_t*>(p.image) + w;
+      const uint32_t* x = reinterpret_cast<const uint32_t*>(im.data) + w;
       uint32_t off, cnt;
       const uint32_t put = frag_resolve<SIG, LAYOUT>(p, x, has, off, cnt);
       uint64_t sum;
@@ -812,35 +834,38 @@ struct Geom {
   uint32_t tile_win, smem_count;
 };
 
-template <int SIG, int LAYOUT>
+template <int SIG, int LAYOUT, bool MULTI>
 KernelFn count_fn(int keys) {
-  if (keys == kFragMostKeys) return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragMostKeys>;
+  if (keys == kFragMostKeys) return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragMostKeys, MULTI>;
   if constexpr (FragGeom<SIG>::kRolled)
-    if (keys == kFragManyKeys) return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragManyKeys>;
-  return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragFewKeys>;
+    if (keys == kFragManyKeys) return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragManyKeys, MULTI>;
+  return (KernelFn)frag_count_kernel<SIG, LAYOUT, kFragFewKeys, MULTI>;
 }
 
 template <int SIG>
-Geom geom_t(uint32_t layout, int keys) {
+Geom geom_t(uint32_t layout, int keys, bool multi) {
   using G = FragGeom<SIG>;
   const bool s = layout == kLayoutSorted;
-  return Geom{s ? count_fn<SIG, kLayoutSorted>(keys) : count_fn<SIG, kLayoutHash>(keys),
+  const KernelFn count = multi ? s ? count_fn<SIG, kLayoutSorted, true>(keys) : count_fn<SIG, kLayoutHash, true>(keys)
+                         : s   ? count_fn<SIG, kLayoutSorted, false>(keys)
+                               : count_fn<SIG, kLayoutHash, false>(keys);
+  return Geom{count,
               s ? (KernelFn)frag_emit_kernel<SIG, kLayoutSorted> : (KernelFn)frag_emit_kernel<SIG, kLayoutHash>,
               G::kThreads, G::kTileWin, G::kSmemCount};
 }
 
-bool geom(int sig, uint32_t layout, int keys, Geom* g) {
+bool geom(int sig, uint32_t layout, int keys, bool multi, Geom* g) {
   switch (sig) {
-    case kSigMd5: *g = geom_t<kSigMd5>(layout, keys); return true;
-    case kSigMd5NoPad: *g = geom_t<kSigMd5NoPad>(layout, keys); return true;
-    case kSigDjb2: *g = geom_t<kSigDjb2>(layout, keys); return true;
+    case kSigMd5: *g = geom_t<kSigMd5>(layout, keys, multi); return true;
+    case kSigMd5NoPad: *g = geom_t<kSigMd5NoPad>(layout, keys, multi); return true;
+    case kSigDjb2: *g = geom_t<kSigDjb2>(layout, keys, multi); return true;
     default: return false;
   }
 }
 
 struct FragDev {
   bool ready = false;
-  int count_blocks[3][2][kFragKeyClasses] = {};
+  int count_blocks[3][2][kFragKeyClasses][2] = {};
 };
 std::mutex g_frag_mu;
 FragDev g_frag_dev[64];
@@ -855,17 +880,17 @@ int frag_device(FragDev** out) {
   FragDev& d = g_frag_dev[dev];
   if (!d.ready) {
     for (int sig = 0; sig < 3; sig++)
-      for (int q = 0; q < 2 * kFragKeyClasses; q++) {
-        const int l = q & 1, keys = q >> 1;
+      for (int q = 0; q < 4 * kFragKeyClasses; q++) {
+        const int l = q & 1, multi = q >> 1 & 1, keys = q >> 2;
         Geom g;
-        geom(sig, (uint32_t)l, keys, &g);
+        geom(sig, (uint32_t)l, keys, multi != 0, &g);
         if ((e = cudaFuncSetAttribute(g.count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem_count)) !=
             cudaSuccess)
           return (int)e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.count_blocks[sig][l][keys], g.count, g.threads,
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.count_blocks[sig][l][keys][multi], g.count, g.threads,
                                                                g.smem_count)) != cudaSuccess)
           return (int)e;
-        if (d.count_blocks[sig][l][keys] < 1) return (int)cudaErrorInvalidConfiguration;
+        if (d.count_blocks[sig][l][keys][multi] < 1) return (int)cudaErrorInvalidConfiguration;
       }
     d.ready = true;
   }
@@ -873,19 +898,16 @@ int frag_device(FragDev** out) {
   return 0;
 }
 
-FragParams make_params(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base,
-                       const FragHits& hits, uint32_t* status) {
+FragParams make_params(const TableView& tab, const FragImages& images, uint64_t n_tiles, const FragHits& hits,
+                       uint32_t* status) {
   FragParams p;
   memset(&p, 0, sizeof p);
   p.tab = tab;
-  p.image = image;
-  p.n_bytes = n_bytes;
-  p.n_windows = frag_windows(n_bytes);
-  p.n_tiles = frag_tiles((int)tab.sig, n_bytes);
-  p.tile_base = tile_base;
-  p.hit_tiles = hits.tiles + tile_base;
-  p.hit_masks = hits.masks + 32 * std::min(tile_base, hits.mask_tiles);
-  p.mask_cap = (uint32_t)std::min(p.n_tiles, hits.mask_tiles - std::min(tile_base, hits.mask_tiles));
+  p.images = images;
+  p.n_tiles = n_tiles;
+  p.hit_tiles = hits.tiles;
+  p.hit_masks = hits.masks;
+  p.mask_cap = (uint32_t)hits.mask_tiles;
   p.n_hit_tiles = hits.count;
   p.status = status;
   p.one = 1u;
@@ -916,7 +938,7 @@ uint64_t frag_windows(uint64_t n_bytes) { return n_bytes >= 64 ? (n_bytes - 64) 
 
 uint64_t frag_tiles(int sig, uint64_t n_bytes) {
   Geom g;
-  if (!geom(sig, kLayoutHash, kFragFewKeys, &g)) return 0;
+  if (!geom(sig, kLayoutHash, kFragFewKeys, false, &g)) return 0;
   return (frag_windows(n_bytes) + g.tile_win - 1) / g.tile_win;
 }
 
@@ -981,33 +1003,44 @@ int frag_window_sigs(int sig, const uint8_t* image, uint64_t n_bytes, uint4* out
   return (int)cudaLaunchKernel(fn, dim3(grid), dim3(256), args, smem, (cudaStream_t)stream);
 }
 
-int frag_count(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base, uint64_t* tile_ntrip,
-               const FragHits& hits, uint32_t* status, unsigned long long* rejected, int sms, void* stream) {
-  FragParams p = make_params(tab, image, n_bytes, tile_base, hits, status);
+FragImages frag_images(const FragImage* host, const FragImage* dev, size_t n) {
+  FragImages l;
+  memset(&l, 0, sizeof l);
+  l.dev = dev;
+  l.n = (uint32_t)n;
+  for (size_t k = 0; k < n && n <= kInlineSegs; k++) l.in[k] = host[k];
+  return l;
+}
+
+int frag_count(const TableView& tab, const FragImages& images, uint64_t n_tiles, uint64_t* tile_ntrip, const FragHits& hits,
+               uint32_t* status, unsigned long long* rejected, int sms, void* stream) {
+  FragParams p = make_params(tab, images, n_tiles, hits, status);
   p.rejected = rejected;
   if (!p.n_tiles) return 0;
+  const bool multi = images.n > 1;
   FragDev* d;
   int rc = frag_device(&d);
   if (rc) return rc;
   Geom g;
   const int keys = frag_key_class((int)tab.sig, tab.n_keys);
-  if (!geom((int)tab.sig, tab.layout, keys, &g)) return (int)cudaErrorInvalidValue;
+  if (!geom((int)tab.sig, tab.layout, keys, multi, &g)) return (int)cudaErrorInvalidValue;
   if (tab.sig == kSigDjb2 && !tab.frag_l1) return (int)cudaErrorInvalidValue;  // the kernel copies it in
   p.tile_ntrip = tile_ntrip;
-  const uint64_t cap = tab.sig == kSigDjb2 ? (uint64_t)sms * (uint64_t)d->count_blocks[tab.sig][tab.layout][keys] : INT32_MAX;
+  const uint64_t cap =
+      tab.sig == kSigDjb2 ? (uint64_t)sms * (uint64_t)d->count_blocks[tab.sig][tab.layout][keys][multi] : INT32_MAX;
   const uint64_t warps_per_block = (uint64_t)g.threads / 32;
   const unsigned grid = (unsigned)std::min<uint64_t>((p.n_tiles + warps_per_block - 1) / warps_per_block, cap);
   void* args[] = {&p};
   return (int)cudaLaunchKernel(g.count, dim3(grid), dim3(g.threads), args, g.smem_count, (cudaStream_t)stream);
 }
 
-int frag_emit(const TableView& tab, const uint8_t* image, uint64_t n_bytes, uint64_t tile_base,
-              const uint64_t* tile_off, const uint64_t* total, const FragHits& hits, MatchOut* out, uint64_t out_cap,
-              uint32_t* status, int sms, void* stream) {
-  FragParams p = make_params(tab, image, n_bytes, tile_base, hits, status);
+int frag_emit(const TableView& tab, const FragImages& images, uint64_t n_tiles, const uint64_t* tile_off,
+              const uint64_t* total, const FragHits& hits, MatchOut* out, uint64_t out_cap, uint32_t* status, int sms,
+              void* stream) {
+  FragParams p = make_params(tab, images, n_tiles, hits, status);
   if (!p.n_tiles) return 0;
   Geom g;
-  if (!geom((int)tab.sig, tab.layout, kFragFewKeys, &g)) return (int)cudaErrorInvalidValue;
+  if (!geom((int)tab.sig, tab.layout, kFragFewKeys, false, &g)) return (int)cudaErrorInvalidValue;
   p.tile_off = tile_off;
   p.total = total;
   p.out = out;

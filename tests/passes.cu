@@ -104,29 +104,25 @@ int passes_fragments(const cv_master* m, const void* const* images, const uint64
   if (n > kInlineSegs) return CV_EINVAL;
   const uint64_t tiles = base[n];
   Bufs b;
-  uint64_t *ntrip, *off, *words, *scratch;  // words: total, status, segment offsets, listed tiles per image
+  uint64_t *ntrip, *off, *words, *scratch;  // words: total, status, segment offsets, listed tiles
   FragHits hits;
   CV_TRY(b.get(&ntrip, tiles));
   CV_TRY(b.get(&off, tiles));
-  CV_TRY(b.get(&words, 2 + 2 * n));
+  CV_TRY(b.get(&words, 3 + n));
   CV_TRY(b.get(&scratch, tile_offsets_scratch_words(tiles)));
   CV_TRY(b.get(&hits.tiles, tiles));
   hits.mask_tiles = mask_tiles < tiles ? mask_tiles : tiles;
   CV_TRY(b.get(&hits.masks, hits.mask_tiles * 32));
   uint32_t* const status = (uint32_t*)(words + 1);
+  hits.count = (uint32_t*)(words + 2 + n);
+  std::vector<FragImage> list;
+  for (uint32_t i = 0; i < n; i++) list.push_back(FragImage{(const uint8_t*)images[i], bytes[i], frag_windows(bytes[i]), base[i]});
+  const FragImages scanned = frag_images(list.data(), nullptr, n);
   CV_CUDA(cudaDeviceSynchronize());
-  for (uint32_t i = 0; i < n; i++) {
-    hits.count = (uint32_t*)(words + 2 + n + i);
-    CV_CUDA((cudaError_t)frag_count(tab, (const uint8_t*)images[i], bytes[i], base[i], ntrip, hits, status, nullptr,
-                                    ctx->sms, nullptr));
-  }
+  CV_CUDA((cudaError_t)frag_count(tab, scanned, tiles, ntrip, hits, status, nullptr, ctx->sms, nullptr));
   CV_CUDA((cudaError_t)launch_tile_offsets(ntrip, tiles, off, seg_list(segs.data(), nullptr, n), 1, words + 2, words,
                                            scratch, nullptr, status));
-  for (uint32_t i = 0; i < n; i++) {
-    hits.count = (uint32_t*)(words + 2 + n + i);
-    CV_CUDA((cudaError_t)frag_emit(tab, (const uint8_t*)images[i], bytes[i], base[i], off, words, hits, (MatchOut*)out,
-                                   cap, status, ctx->sms, nullptr));
-  }
+  CV_CUDA((cudaError_t)frag_emit(tab, scanned, tiles, off, words, hits, (MatchOut*)out, cap, status, ctx->sms, nullptr));
   CV_CUDA(cudaMemcpy(h, words, (2 + n) * 8, cudaMemcpyDeviceToHost));
   return CV_OK;
 }

@@ -51,9 +51,14 @@ def test_sizes_around_the_classes(cv, sig, n_keys, size, tmp_path):
         with cv.master_build([frags.view(-1)], signature=sig, unit=cv.CV_UNIT_FRAGMENT, **kw) as m:
             with cv.scan(m, [img]) as r:
                 got = r.matches(0)
+            part = 200_000  # a second image of fewer tiles before it, and one too short for a window
+            with cv.scan(m, [img[:part], img[:40], img]) as r:
+                two = [r.matches(0), r.matches(2)]
+                assert r.count(1) == 0
             if not kw and size == 262_147:
                 cv.master_save(m, tmp_path / "t.cvt")
         assert np.array_equal(np.stack([got["disk_sector"], got["file_sector"]], axis=1), want), kw
+        assert np.array_equal(two[1], got) and np.array_equal(two[0], got[got["disk_sector"] * 4 + 64 <= part]), kw
     if size == 262_147:  # the filters are made again for the table's size
         with cv.master_load(tmp_path / "t.cvt") as m, cv.scan(m, [img]) as r:
             got = r.matches(0)

@@ -13,7 +13,7 @@
 //
 // Tiles are handed out as blocks get to them: the grid has one block per tile, the blocks that
 // become resident stay, and each takes the next tile over from a block that has not started yet
-// (cluster launch control), asking for it one tile ahead. With a fixed share of the tiles per
+// (cluster launch control), asking for it while it stages one. With a fixed share of the tiles per
 // block the scheduler's preference among the blocks of an SM let some finish early, and the SM
 // ran a quarter short of warps on average (27.5 of 36 active; 1 GiB image).
 //
@@ -380,7 +380,13 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
     bool ok = true, more = true;
     const Segment* const segs = p.segs.get();
     while (more && ok) {
-      clc_ask(base + L::kClcOff, bar_clc);  // the next tile; answered while this one is staged
+      // The next tile is asked for half-way through the staging of this one, early enough for the answer
+      // and no earlier: a block that asked as soon as it could took a tile over from one that had not
+      // started yet and would have had the room, and then one more while it still hashed its first. With
+      // 155,648 sectors, one round of blocks, 128-sector tiles took 34.0 us and without the padding block
+      // 32.0, now 27.8 and 27.5; 160,000 in 256-sector tiles 34.8 and 37.6, now 30.0 and 28.5. Asked for with
+      // the last stage, the answer came late: 4 GiB without a filter 845 us, 837 at first, 839 now.
+      bool asked = false;
       const uint64_t tile = p.tile_begin + lt;
       const Segment& seg = segs[find_segment(segs, p.segs.n, tile)];
       const CUtensorMap* map = &p.maps[seg.map - p.map_base];
@@ -391,6 +397,10 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
         if (j >= (uint32_t)NS && !mbar_wait(bar_empty + 8 * s, ((j / NS) - 1) & 1, s_abort, p.status)) {
           ok = false;
           break;
+        }
+        if (c == kChunks / 2) {
+          clc_ask(base + L::kClcOff, bar_clc);
+          asked = true;
         }
         // published by the arrive below (release), seen after the matching wait (acquire); the
         // entry is rewritten for the tile after next, whose first copy waits for every hashing
@@ -408,6 +418,7 @@ __global__ void __launch_bounds__(T / SPT + 32, MINB) scan_kernel(const __grid_c
           tma_load_2d(base + s * L::kStageBytes + k * kBoxRows * BOXB, map, c * (BOXB / 4), row0 + k * kBoxRows,
                       bar_full + 8 * s, policy);
       }
+      if (!asked) break;  // gave up before
       // the answer, also when giving up: it must not land after the block exits
       if (!mbar_wait(bar_clc, answers & 1, s_abort, p.status)) {
         volatile uint32_t never = 0;

@@ -98,8 +98,9 @@ typedef struct cv_result cv_result; /* the results of one scan */
 #define CV_LAYOUT_HASH 0u
 #define CV_LAYOUT_SORTED 1u
 /* CV_LAYOUT_AUTO: the hash layout, turned into the sorted one when the built table's occupancy
- * (distinct keys / slots) exceeds 0.8 with a Bloom filter or 0.5 without one, where linear
- * probing measured slower than bisection on GB300. cv_master_info.layout reports the choice. */
+ * (distinct keys / slots) exceeds 0.8 with a Bloom filter or 0.5 without one: from there on linear
+ * probing measured slower than bisection on GB300 (without a filter with the 64-bit signatures from
+ * about 0.65 on, by at most 2% faster below). cv_master_info.layout reports the choice. */
 #define CV_LAYOUT_AUTO 2u
 
 /* What the master files are cut into (cv_master_opts.unit).
@@ -339,7 +340,7 @@ int cv_selftest_wait_timeout(uint32_t timeout_us, void* stream);
 /*
  * Batched scans (a CUDA graph over many device images). The paper scans several drives at once
  * by multiplexing them onto one GPU (Section 3); a batch makes all of its images one work list
- * for one persistent scan launch (images in one device allocation share a tensor map), then
+ * for one scan launch (images in one device allocation share a tensor map), then
  * one pass that places and writes the matches, captured once as a CUDA graph and replayed per run.
  *
  * Images must be device buffers (16-byte aligned), borrowed for the life of the batch: each run

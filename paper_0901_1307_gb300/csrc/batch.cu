@@ -1,7 +1,7 @@
 // Batched scans: many device-resident images against one master table, replayed as one CUDA
 // graph. The paper scans several drives at once by multiplexing them onto one GPU (Section 3);
 // here all images of a batch are one work list: images that sit in one device allocation share
-// a tensor map, the persistent scan kernel takes tiles of every image in one launch, and one
+// a tensor map, one scan launch takes the tiles of every image, and one
 // pass after it produces every image's sorted matches. The whole sequence is
 // captured once and replayed with a single graph launch per run.
 //

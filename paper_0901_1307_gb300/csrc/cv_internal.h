@@ -189,7 +189,6 @@ struct ScanParams {
   uint32_t group_log2;
   uint32_t pad;
   uint64_t tile_begin;  // global index of the first tile of this launch
-  uint64_t n_tiles;     // tiles of this launch
   TableView tab;
   // scan outputs, indexed by global output tile (32 sectors)
   uint4* hit_rec;        // 32 records per output tile {lane, post_off, post_cnt, triples emitted}

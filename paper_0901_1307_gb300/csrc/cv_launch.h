@@ -112,12 +112,12 @@ int frag_emit(const TableView& tab, const FragImages& images, uint64_t n_tiles, 
               const uint64_t* total, const FragHits& hits, MatchOut* out, uint64_t out_cap, uint32_t* status, int sms,
               void* stream);
 
-// One block whose single waiting thread waits on an mbarrier nothing completes (bounded by
-// timeout_ns): the status word gets the timeout bit. Returns a CUDA error code.
 // The offset scan's look-back wait running out (words: lookback_selftest_words() u64).
 int launch_lookback_selftest(uint64_t* words, uint32_t* status, uint64_t timeout_ns, void* stream);
 constexpr uint64_t lookback_selftest_words() { return 4 * 4096 + 4; }
 
+// One block whose single waiting thread waits on an mbarrier nothing completes (bounded by
+// timeout_ns): the status word gets the timeout bit. Returns a CUDA error code.
 int launch_wait_selftest(uint32_t* status, uint64_t timeout_ns, void* stream);
 
 }  // namespace cvk

@@ -14,15 +14,15 @@
 //   P(x_{k+q}) 33^{4 (15 - q)}, so g(W_{k+1}) = 33^4 g(W_k) - 33^64 P(x_k) + P(x_{k+16})
 //   (mod 2^64): after a lane's first window each one costs one word and a few multiply-adds.
 //   The same recurrence holds mod 2^32, so the count kernel rolls only the low word of h: two
-//   multiply-adds a window. Its filters are functions of that word: two bits of one word of a
-//   2^20-bit filter in shared memory (loaded once per block), then, for the windows that pass, one
-//   word of a Bloom filter in global memory. What is left computes its whole h and is looked up.
+//   multiply-adds a window. Its filters are functions of that word (but see frag_key_class): two bits
+//   of one word of a 2^20-bit filter in shared memory (loaded once per block), then, for the windows
+//   that pass, one word of a Bloom filter in global memory. What is left computes its whole h and is looked up.
 //   MD5 is computed per window (two compressions, or one without the padding block); there the
 //   hash dominates and the global Bloom word is tested directly.
 //
-// Passes. The count kernel hashes every window, filters it, resolves the candidates (probe; byte
-// confirmation for djb2), writes each tile's triple count and, for a tile with triples, an entry
-// of the image's hit list: which windows of each lane have any. An exclusive scan gives every tile
+// Passes, over the tiles of all images of a call. The count kernel hashes every window, filters it,
+// resolves the candidates (probe; byte confirmation for djb2), writes each tile's triple count and, for
+// a tile with triples, an entry of the hit list: which windows of each lane have any. An exclusive scan gives every tile
 // its output offset; the emit kernel looks the listed windows up again and writes their triples
 // in window order. (Hit records instead of lookups done twice would need room for every window.)
 // The lists' masks take 128 bytes per tile, 4.3% of the image for djb2 and 3.2% for MD5, and at
@@ -226,10 +226,9 @@ __device__ __forceinline__ bool frag_equal(const uint32_t* x, const uint8_t* m) 
   return diff == 0;
 }
 
-// Candidate windows of this thread (bit i: window w0 + i passed the filters; every valid window
-// when the table has no Bloom filter and no first filter). n_valid: the thread's windows inside the
-// image. l1: the first filter, in shared or global memory (rolled kernels only). ws is the warp's
-// tile; the rolled kernels' waiting windows overwrite parts of it (FragGeom::kQueue).
+// Candidate windows of this thread (bit i: window w0 + i passed the filters that the table has). n_valid: the thread's windows inside the
+// image. l1: the first filter (rolled kernels only). ws is the warp's tile; the waiting windows of the
+// rolled kernel for few keys overwrite parts of it (FragGeom::kQueue).
 //
 // Not rolled (MD5): the hash is all of the cost (126 or 61 operations a window), so a window that equals
 // the one before it (fills; patterns of four bytes) is not hashed again. The lanes mark these (17

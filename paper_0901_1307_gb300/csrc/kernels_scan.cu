@@ -135,9 +135,10 @@ __global__ void wait_timeout_selftest_kernel(uint32_t* status, uint64_t timeout_
 }
 
 
-// The configurations in table order. The first and the 128-byte-stage one have digest-mode kernels; every one has scan
-// kernels for all eight table kinds (four signatures x two layouts), so the batch autotuner can
-// pick any of them for any table. The kernels are instantiated in scan_cfgs_{a,b,c}.cu, which
+// The configurations in table order. The first and the one of 128-byte stages of 128-sector tiles have
+// digest-mode kernels; every one has scan kernels for all eight table kinds (table_kind: four
+// signatures, looked up in the slots or otherwise), so the batch autotuner can pick any of them for any
+// table. The kernels are instantiated in scan_cfgs_{a,b,c}.cu, which
 // compile in parallel.
 static const std::vector<ScanCfg>& all_configs() {
   static const std::vector<ScanCfg> v = [] {
@@ -198,6 +199,7 @@ int preferred_config(int kind, uint64_t sectors, int sms) {
 const ScanCfg& digest_config_for(int cfg_i, int sig, uint64_t sectors, int sms, int* used) {
   int n;
   const ScanCfg* c = scan_configs(&n);
+  // MD5 without padding from 1 GiB on prefers a configuration without digest kernels and gets the first
   if (cfg_i < 0) cfg_i = preferred_config(sig, sectors, sms);
   if (cfg_i >= n || sig < 0 || sig > kSigCrc64 || !c[cfg_i].digest_fn[sig]) cfg_i = 0;
   if (used) *used = cfg_i;

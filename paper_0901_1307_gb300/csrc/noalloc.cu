@@ -173,7 +173,6 @@ extern "C" int cv_scan_noalloc(const cv_master* m, const void* image, uint64_t n
   p.map_base = 0;
   p.one = 1u;
   p.tile_begin = 0;
-  p.n_tiles = n_tiles;
   p.tab = tab;
   p.hit_rec = hit_rec;
   p.tile_nhit = tile_nhit;

@@ -323,11 +323,11 @@ int launch_range(DevCtx* ctx, int cfg_i, bool digest, const Job& job, const Segm
     p.segs = seg_list(job.segs.data() + a, segs_d ? segs_d + a : nullptr, b - a);
     p.tile_begin = job.segs[a].tile_base;
     const uint64_t tile_end = (b < job.segs.size()) ? job.segs[b].tile_base : job.n_tiles;
-    p.n_tiles = tile_end - p.tile_begin;
-    if (p.n_tiles) {
-      if (p.n_tiles > (uint64_t)INT32_MAX) return CV_EINVAL;  // one block per tile
+    const uint64_t n_tiles = tile_end - p.tile_begin;
+    if (n_tiles) {
+      if (n_tiles > (uint64_t)INT32_MAX) return CV_EINVAL;  // one block per tile
       void* args[] = {&p};
-      CV_CUDA(cudaLaunchKernel(fn, dim3((unsigned)p.n_tiles), dim3(cfg.threads), args, cfg.smem, stream));
+      CV_CUDA(cudaLaunchKernel(fn, dim3((unsigned)n_tiles), dim3(cfg.threads), args, cfg.smem, stream));
       if (launches) (*launches)++;
     }
     a = b;

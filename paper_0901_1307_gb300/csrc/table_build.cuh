@@ -59,7 +59,7 @@ __global__ void unit_postings_kernel(const uint64_t* file_base, uint32_t n_files
 // tau: per master sector position (position-keyed tables), or null for one table over all
 // positions (every tau 0). The key is (digest, tau). A slot's owner is the master index of its key's
 // first member + 1 (0: empty), its extra the number of other members. Bound by the latency of
-// the random accesses (owner and count in one 8-byte word took 248 us against 165 for 4,194,304 keys,
+// the random accesses (owner and count in one 8-byte word took 248 us against 178 for 4,194,304 keys,
 // and 333 us with a second atomic that counts every member).
 // (Claiming slots from the kernel that hashes the sectors saved nothing: waited for at once, the
 // atomics held up the hashing by 220 us; looked at a tile later, by 100, and the keys whose home was
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kRsThreads) rs_scatter_kernel(const uint32_t* 
 // Bound by memory: 8 bytes read and 32 written per slot (4,194,304 keys in 2^24 slots: 671 MB),
 // two random sectors read per key, a Bloom block updated per key. A slot record is one 32-byte store.
 // Of a key's eight Bloom bits eight lanes each set one, so that the block is one update in L2. This
-// and the sums take 245 us, where sorting (slot, master) pairs, filling postings and slots, a pass
+// takes 204 us and the sums 25, where sorting (slot, master) pairs, filling postings and slots, a pass
 // for the Bloom filter and clearing the slots and counts took 804.
 constexpr int kSlotThreads = 256;
 constexpr int kSlotRows = 4;

@@ -302,7 +302,7 @@ int sorted_from_hash(DevCtx* ctx, const uint4* slots, uint64_t n_slots, uint32_t
   CV_TRY(table_alloc(ctx, &out, std::max<uint64_t>(nu, 1) * 32, stream));
   int rc = table_alloc(ctx, &keys0, sorted_key_words(nu) * 4, stream);
   if (rc != CV_OK) {
-    cudaFreeAsync(out, stream);
+    cudaFree(out);
     return rc;
   }
   gather_slots_kernel<<<gu, 256, 0, stream>>>(slots, hv, nu, (uint4*)out);
@@ -314,8 +314,8 @@ int sorted_from_hash(DevCtx* ctx, const uint4* slots, uint64_t n_slots, uint32_t
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
-    cudaFreeAsync(out, stream);
-    cudaFreeAsync(keys0, stream);
+    cudaFree(out);
+    cudaFree(keys0);
     return cuda_fail(e);
   }
   *slots_out = out;
@@ -481,7 +481,7 @@ int cv_master_build(const cv_buf* files, uint32_t n_files, const cv_master_opts*
         void* sorted_slots = nullptr;
         CV_TRY(sorted_from_hash(ctx, (const uint4*)m->slots, n_slots, hc[2], tmp, stream, &sorted_slots, &m->keys0,
                                 &steps));
-        cudaFreeAsync(m->slots, stream);
+        cudaFree(m->slots);  // the sort is done with it
         m->slots = sorted_slots;
       }
       m->tab.slots = (const uint4*)m->slots;
@@ -798,7 +798,7 @@ int cvk::table_bloom(const TableView& tab, uint32_t bits_per_key, cudaStream_t s
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) {
-    cudaFreeAsync(bloom, stream);
+    cudaFree(bloom);
     return cuda_fail(e);
   }
   *bloom_out = bloom;

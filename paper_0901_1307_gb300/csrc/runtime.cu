@@ -147,7 +147,10 @@ void DevCtx::give_stage(Stage* s) {
 
 int table_alloc(DevCtx* ctx, void** out, size_t bytes, cudaStream_t stream) {
   *out = nullptr;
-  CV_CUDA(cudaMallocFromPoolAsync(out, bytes ? bytes : 16, ctx->table_pool, stream));
+  if (bytes > kTablePoolKept)
+    CV_CUDA(cudaMalloc(out, bytes));
+  else
+    CV_CUDA(cudaMallocFromPoolAsync(out, bytes ? bytes : 16, ctx->table_pool, stream));
   return CV_OK;
 }
 
@@ -156,7 +159,7 @@ void table_free(void* const* ptrs, int n, int dev) {
   if (cudaGetDevice(&current) == cudaSuccess && current != dev) cudaSetDevice(dev);
   cudaDeviceSynchronize();  // scans on any stream may have read the table
   for (int k = 0; k < n; k++)
-    if (ptrs[k]) cudaFreeAsync(ptrs[k], nullptr);
+    if (ptrs[k]) cudaFree(ptrs[k]);
   cudaStreamSynchronize(nullptr);  // a pool gives back what it does not keep at a wait after the free
   cudaGetLastError();
   if (current >= 0 && current != dev) cudaSetDevice(current);

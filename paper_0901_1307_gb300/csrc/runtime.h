@@ -68,7 +68,7 @@ struct DevCtx {
   int dev = -1;
   int sms = 0;
   cudaMemPool_t pool = nullptr;      // stream-ordered temporaries and results
-  // Tables: at most kTablePoolKept bytes stay with the pool when they are freed. A cudaMalloc and
+  // Tables: at most kTablePoolKept bytes stay with the pool when they are freed (see table_alloc). A cudaMalloc and
   // cudaFree of a 4,194,304-sector table's arrays took 660 us of a 1,910 us build and scan.
   cudaMemPool_t table_pool = nullptr;
   cudaStream_t copy_stream = nullptr;  // host-to-device copies of streamed images
@@ -97,9 +97,10 @@ struct DevCtx {
 int get_ctx(DevCtx** out);
 
 constexpr uint64_t kTablePoolKept = 1ull << 30;
-// Table memory: allocated in order on stream; freed in order on a stream when only that one used
-// it, or, by the table's owner, once all work of its device is done (table_free: what the pool does
-// not keep is free memory again when it returns).
+// Table memory: from the pool, in order on stream, or, an array that the pool could not keep, from
+// cudaMalloc: mapping it for the pool and giving it back took longer (a build and free of 8,000,000
+// djb2-64 sectors, 4.5 GiB, 10.8 ms by the pool, 5.2 so). It is freed once all work of its device is done, and
+// what the pool does not keep is free memory again when table_free returns.
 int table_alloc(DevCtx* ctx, void** out, size_t bytes, cudaStream_t stream);
 void table_free(void* const* ptrs, int n, int dev);
 

@@ -64,3 +64,22 @@ def test_equal_sectors_do_not_queue(cv):
             t.append(time.perf_counter() - a)
         best.append(min(t))
     assert best[1] < 2.5 * best[0], best
+
+
+def test_large_tables_are_not_paid_for_twice(cv):
+    """A table with an array of more than 1 GiB (the sectors' copies of a 64-bit signature) is built and freed
+    in less than four and a half times what one of half the sectors takes, which fits what is kept."""
+    best = []
+    for n in (1_500_000, 3_000_000):
+        table = torch.randint(-2**31, 2**31 - 1, (n * 128,), dtype=torch.int32, device="cuda").view(torch.uint8)
+        t = []
+        for _ in range(8):
+            torch.cuda.synchronize()
+            a = time.perf_counter()
+            m = cv.master_build([table], signature=2)
+            info = m.info()
+            m.close()
+            t.append(time.perf_counter() - a)
+        best.append(min(t))
+        assert info["n_unique"] == n
+    assert best[1] < 4.5 * best[0], best
